@@ -146,19 +146,30 @@ __device__ __forceinline__ void load_rows(const T* G, int64_t ld, int nrows, int
 // memory: the LU of its hs x hs diagonal block without pivoting, blocked by 32
 // columns, and U's rows right of the block (columns hs .. wt).  Per block of
 // 32 columns:
-//   (i)  the block's columns, one at a time: the multipliers of the column (a
-//        thread per row, dividing by the pivot as in the definition), then a
-//        rank-1 update of the rows below it within the block's columns (a
-//        thread per row); two barriers per column;
-//   (i') the block's rows right of the block (U's rows there) by forward
-//        substitution with the block's L, a thread per column;
+//   (a)  the 32 x 32 diagonal block, by one warp, a lane per row with the
+//        row's 32 columns in registers: column by column, the pivot's lane
+//        writes its row (U) to shared memory, every lane below it divides by
+//        the pivot (as in the definition) and subtracts its multiple of the row;
+//   (b)  the rows below the block, a thread per row, by the same elimination
+//        against the block's finished U, and beside them, on other warps,
+//        (i') U's rows right of the block by forward substitution with the
+//        block's L, a thread per column;
 //   (ii) a rank-32 update of the rows below the block and the columns right
-//        of it (register tiles).
+//        of it, in 32 x 32 tiles, a warp per tile (8 x 4 per thread, 16-byte
+//        operand loads).  Warp 0 takes the next diagonal block's tile first
+//        and factors that block at once, so that (a) runs under the other
+//        warps' tiles.
+// Every element gets the same products in the same order as column-by-column
+// rank-1 updates of the 32-column block would give it.
 // Then, for the rows below the slab, (iii) the inverses of U's 32 x 32
-// diagonal blocks (a warp per block), written to uinv.
-// The loops stay rolled, with their shared-memory loads batched ahead of the
-// products: the kernel runs once per launch on one SM, where a long
-// straight-line body would be fetched from L2 at every block.
+// diagonal blocks (a warp per block, a lane per column), written to uinv while
+// the other warps write the slab back.
+// What bounds it: the chain of hs dependent columns on one SM.  Column steps
+// across the whole CTA cost two barriers and a round through shared memory
+// each (about 900 cycles); within a warp the step is a broadcast and a
+// division.  The register arrays are indexed statically in bodies of eight
+// columns that a rolled loop runs four times, the registers moved down by
+// eight in between: a fully unrolled block would be fetched from L2.
 // A zero pivot lowers *info to its absolute column + 1 (kabs = D's first
 // column) and skips its scaling.  With sp.flag set it is a stage of a pivoted
 // panel's diagonal-pivot check: the first slab (first != 0) saves its rows to
@@ -168,20 +179,221 @@ __device__ __forceinline__ void load_rows(const T* G, int64_t ld, int nrows, int
 // restore_rows, then flag[0]).  It returns at once when an earlier stage or
 // panel failed.
 constexpr int SL_THREADS = 256;
+constexpr int SL_WARPS = SL_THREADS / 32;
 
 // Row stride of the slab in shared memory, in elements: at least the width
 // and whole 32-column blocks, and VN (mod 2 VN) for VN elements per 16 bytes,
-// so that each thread's 16-byte piece of its own row falls in banks of its
-// own within a quarter-warp.
+// so that the 16-byte pieces that a quarter-warp reads from eight consecutive
+// rows fall in different banks.
 __host__ __device__ inline int slab_wp(int hs, int wt, int tsize) {
   const int vn = 16 / tsize;
   const int w = wt > ((hs + 31) & ~31) ? wt : ((hs + 31) & ~31);
   return (w + 2 * vn - 1) / (2 * vn) * (2 * vn) + vn;
 }
-// shared memory of one slab: rows, the pivot row's block columns, the
-// multipliers, and a 32 x 33 scratch per diagonal block for its U's inverse
-inline size_t slab_smem_bytes(int hs, int wt, int tsize) {
-  return ((size_t)hs * slab_wp(hs, wt, tsize) + 32 + (size_t)hs + (size_t)((hs + 31) / 32) * 32 * 33) * tsize;
+inline size_t slab_smem_bytes(int hs, int wt, int tsize) { return (size_t)hs * slab_wp(hs, wt, tsize) * tsize; }
+
+// VN consecutive elements of shared memory (16-byte aligned) from / to registers
+template <typename T>
+__device__ __forceinline__ void s16_get(const T* p, T* out) {
+  v16_get<T>(*reinterpret_cast<const typename V16<T>::type*>(p), out);
+}
+template <typename T>
+__device__ __forceinline__ void s16_put(T* p, const T* e) {
+  *reinterpret_cast<typename V16<T>::type*>(p) = v16_make<T>(e);
+}
+
+// Eliminate the 32 columns c0 .. c0 + bw of this thread's row (at `row`, the
+// row's column c0; bw < 32 only for a ragged last block) against the rows of
+// U of the diagonal block at Ub (row stride wp).  DIAG: the warp's lanes are
+// the diagonal block's own rows, lane j publishing row j before column j's
+// step; `live` lanes hold a row.
+template <typename T, bool DIAG>
+__device__ __forceinline__ void slab_eliminate(T* Ub, int wp, T* row, bool live, int bw, bool spec, int* info, int kcol,
+                                               bool& bad) {
+  constexpr int VN = V16<T>::n;
+  const int lane = threadIdx.x & 31;
+  T a[32];
+#pragma unroll
+  for (int g = 0; g < 32 / VN; ++g) {
+    if (live) {
+      s16_get<T>(row + g * VN, a + g * VN);
+    } else {
+#pragma unroll
+      for (int e = 0; e < VN; ++e) a[g * VN + e] = T(0);
+    }
+  }
+#pragma unroll 1
+  for (int jb = 0; jb < 32; jb += 8) {
+    if (jb >= bw) break;
+    const int left = 32 - jb;  // columns jb .. 31 are in a[0 .. left)
+#pragma unroll
+    for (int jj = 0; jj < 8; ++jj) {
+      const int j = jb + jj;
+      if (j < bw) {
+        T* urow = Ub + (size_t)j * wp + jb;
+        if (DIAG) {
+          if (lane == j) {
+#pragma unroll
+            for (int g = jj / VN; g < 32 / VN; ++g)
+              if (g * VN < left) s16_put<T>(urow + g * VN, a + g * VN);
+          }
+          __syncwarp();
+        }
+        T u[32];
+#pragma unroll
+        for (int g = jj / VN; g < 32 / VN; ++g)
+          if (g * VN < left) s16_get<T>(urow + g * VN, u + g * VN);
+        const T piv = u[jj];
+        const bool pz = !(piv != T(0));
+        if (DIAG && lane == 0) {
+          if (spec) {
+            if (!finite_nonzero(piv)) bad = true;
+          } else if (pz) {
+            atomicMin(info, kcol + j + 1);
+          }
+        }
+        if (live && (!DIAG || lane > j)) {
+          T l = a[jj];
+          if (!pz) l = l / piv;
+          if (spec && !spec_ok_mult(l)) bad = true;
+          a[jj] = l;
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            if (g * 8 < left) {  // uniform
+#pragma unroll
+              for (int e = 0; e < 8; ++e)
+                if (g * 8 + e > jj) a[g * 8 + e] = fma(-l, u[g * 8 + e], a[g * 8 + e]);
+            }
+          }
+        }
+      }
+    }
+    if (live) {
+#pragma unroll
+      for (int g = 0; g < 8 / VN; ++g) s16_put<T>(row + jb + g * VN, a + g * VN);
+    }
+#pragma unroll
+    for (int i = 0; i < 24; ++i) a[i] = a[i + 8];
+  }
+  if (DIAG) __syncwarp();
+}
+
+// Column of U's 32 rows right of a diagonal block: x <- L^-1 x, x_t at
+// x[t * wp], L (unit lower, 32 x 32) at Lb.
+template <typename T>
+__device__ __forceinline__ void slab_top_column(const T* Lb, int wp, T* xcol) {
+  constexpr int VN = V16<T>::n;
+  T x[32];
+#pragma unroll
+  for (int t = 0; t < 32; ++t) x[t] = xcol[(size_t)t * wp];
+#pragma unroll 1
+  for (int sb = 0; sb < 32; sb += 8) {
+    const int left = 32 - sb;  // rows sb .. 31 are in x[0 .. left)
+#pragma unroll
+    for (int i = 1; i < 32; ++i) {
+      if (i < left) {  // uniform
+        T l[8];
+#pragma unroll
+        for (int g = 0; g < 8 / VN; ++g) s16_get<T>(Lb + (size_t)(sb + i) * wp + sb + g * VN, l + g * VN);
+#pragma unroll
+        for (int s = 0; s < 8; ++s)
+          if (s < i) x[i] = fma(-l[s], x[s], x[i]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) xcol[(size_t)(sb + i) * wp] = x[i];
+#pragma unroll
+    for (int i = 0; i < 24; ++i) x[i] = x[i + 8];
+  }
+}
+
+// One warp: the 32 x 32 tile of A at rows rr.., columns cc.. -= (the rows'
+// columns c0 .. c0 + 31) x (rows c0 .. c0 + 31's columns).  Thread = rows
+// rr + (lane >> 3) + 4 i, columns cc + 4 (lane & 7) ..: the four row groups'
+// 16-byte pieces fall in different banks.
+template <typename T>
+__device__ __forceinline__ void slab_update_tile(T* A, int wp, int c0, int rr, int cc, int hs, int wt) {
+  constexpr int VN = V16<T>::n;
+  const int lane = threadIdx.x & 31;
+  const int r0 = rr + (lane >> 3), cj = cc + 4 * (lane & 7);
+  if (cj >= wt) return;  // (columns past wt but below its 16-byte piece's end are padding of the row)
+  T acc[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[i][q] = T(0);
+  const T* ar[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) ar[i] = A + (size_t)min(r0 + 4 * i, hs - 1) * wp + c0;
+  const T* br = A + (size_t)c0 * wp + cj;
+#pragma unroll 1
+  for (int k = 0; k < 32; k += VN) {
+    T av[8][VN];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s16_get<T>(ar[i] + k, av[i]);
+#pragma unroll
+    for (int e = 0; e < VN; ++e) {
+      T bv[4];
+#pragma unroll
+      for (int q = 0; q < 4; q += VN) s16_get<T>(br + (size_t)(k + e) * wp + q, bv + q);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[i][q] = fma(av[i][e], bv[q], acc[i][q]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = r0 + 4 * i;
+    if (r < hs) {
+      T* p = A + (size_t)r * wp + cj;
+#pragma unroll
+      for (int q = 0; q < 4; q += VN) {
+        T y[VN];
+        s16_get<T>(p + q, y);
+#pragma unroll
+        for (int e = 0; e < VN; ++e) y[e] -= acc[i][q + e];
+        s16_put<T>(p + q, y);
+      }
+    }
+  }
+}
+
+// One warp: the inverse of the upper bw x bw block Ub (row stride wp) to out
+// (32 x 32, row-major; the identity outside a ragged block).  Lane = a column
+// of the inverse: back substitution with the division by U's diagonal.
+template <typename T>
+__device__ __forceinline__ void slab_inverse(const T* Ub, int wp, int bw, T* out) {
+  const int lane = threadIdx.x & 31;
+  T z[32];  // row tb + i of the column at z[24 + i]
+#pragma unroll
+  for (int t = 0; t < 32; ++t) z[t] = t == lane ? T(1) : T(0);
+#pragma unroll 1
+  for (int tb = 24; tb >= 0; tb -= 8) {
+#pragma unroll
+    for (int jj = 7; jj >= 0; --jj) {
+      const int t = tb + jj;
+      if (t < bw) {  // uniform
+        const T* ucol = Ub + t;  // U(q, t) at ucol[q * wp]
+        const T zt = z[24 + jj] / ucol[(size_t)t * wp];
+        z[24 + jj] = zt;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          if (g * 8 >= 24 - tb) {  // uniform: rows tb - 24 + 8 g .. exist
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const int i = g * 8 + e;  // row q = tb - 24 + i
+              if (i < 24 + jj) z[i] = z[i] - ucol[(size_t)(tb - 24 + i) * wp] * zt;
+            }
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) out[(tb + i) * 32 + lane] = z[24 + i];
+#pragma unroll
+    for (int i = 31; i >= 8; --i) z[i] = z[i - 8];
+  }
 }
 
 template <typename T>
@@ -209,147 +421,51 @@ __global__ void __launch_bounds__(SL_THREADS) slab_lu_kernel(T* D, int64_t ld, i
     if (tid == 0) sp.perm[0] = 0;
   }
   __syncthreads();
-  T* pr = A + (size_t)hs * wp;  // [32]: the pivot row's block columns right of the pivot, zero elsewhere
-  T* lcol = pr + 32;            // [hs]: the current column's multipliers
+  if (warp == 0)
+    slab_eliminate<T, true>(A, wp, A + (size_t)lane * wp, lane < hs, min(32, hs), spec, info, kabs, bad);
+  __syncthreads();
   for (int c0 = 0; c0 < hs; c0 += 32) {
     const int bw = min(32, hs - c0);
     const int r1 = c0 + bw;
-    // (i) the block's columns, one at a time.  Column cj: (a) a thread per
-    //     row below the pivot divides by the pivot (as in the definition),
-    //     and the last warp copies the pivot row's block columns right of cj;
-    //     (b) a thread per row below cj applies the rank-1 update to its
-    //     row's 32 block columns in 16-byte pieces (the copy's zeros leave
-    //     the columns at and left of cj as they are).
-    for (int j = 0; j < bw; ++j) {
-      const int cj = c0 + j;
-      const T piv = A[cj * wp + cj];
-      const bool pz = !(piv != T(0));
-      if (tid == 0) {
-        if (spec) {
-          if (!finite_nonzero(piv)) bad = true;
-        } else if (pz) {
-          atomicMin(info, kabs + cj + 1);
-        }
-      }
-      for (int r = cj + 1 + tid; r < hs; r += SL_THREADS) {
-        T l = A[r * wp + cj];
-        if (!pz) l = l / piv;
-        if (spec && !spec_ok_mult(l)) bad = true;
-        A[r * wp + cj] = l;
-        lcol[r] = l;
-      }
-      if (warp == SL_THREADS / 32 - 1) {  // (never a row thread: a slab has at most 128 rows)
-        const int k = c0 + lane;
-        pr[lane] = (k > cj && k < r1) ? A[cj * wp + k] : T(0);
-      }
-      __syncthreads();
-      for (int r = cj + 1 + tid; r < hs; r += SL_THREADS) {
-        const T nl = -lcol[r];
-        VT* y = reinterpret_cast<VT*>(A + r * wp + c0);
-        const VT* x = reinterpret_cast<const VT*>(pr);
-#pragma unroll
-        for (int v = 0; v < 32 / VN; ++v) {
-          T yv[VN], xv[VN];
-          v16_get<T>(y[v], yv);
-          v16_get<T>(x[v], xv);
-#pragma unroll
-          for (int e = 0; e < VN; ++e) yv[e] = fma(nl, xv[e], yv[e]);
-          y[v] = v16_make<T>(yv);
-        }
-      }
-      __syncthreads();
-    }
-    // (i') the block's rows right of the block: forward substitution with the
-    //      block's unit lower L, a thread per column -- the same products in
-    //      the same order as rank-1 updates column by column would apply them
-    for (int k = r1 + tid; k < wt; k += SL_THREADS) {
-      for (int t = c0 + 1; t < r1; ++t) {
-        T v = A[t * wp + k];
-        for (int s0 = c0; s0 < t; s0 += 8) {
-          T lv[8], xv[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int ss = s0 + u < t ? s0 + u : t - 1;
-            lv[u] = A[t * wp + ss];
-            xv[u] = A[ss * wp + k];
-          }
-#pragma unroll
-          for (int u = 0; u < 8; ++u)
-            if (s0 + u < t) v = fma(-lv[u], xv[u], v);
-        }
-        A[t * wp + k] = v;
-      }
-    }
-    __syncthreads();
-    // (ii) rank-bw update of rows [r1, hs) x columns [r1, wt): a thread per
-    //       4 rows x 4 columns 32 apart (the warp reads consecutive columns)
+    T* Ub = A + (size_t)c0 * wp + c0;
+    // (b), (i'): rows below, then columns right of the block (a column exists
+    // only beside a whole 32-column block)
     const int nr = hs - r1, nc = wt - r1;
-    if (nr > 0 && nc > 0) {
-      const int ntr = (nr + 3) / 4, ncg = (nc + 127) / 128;
-      for (int it = tid; it < ntr * ncg * 32; it += SL_THREADS) {
-        const int cl = it & 31, g = (it >> 5) % ncg, tr = (it >> 5) / ncg;
-        const int rr = r1 + 4 * tr, cc = r1 + 128 * g + cl;
-        T acc[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) acc[i][q] = T(0);
-#pragma unroll 4
-        for (int j = 0; j < bw; ++j) {
-          T av[4], bv[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) av[i] = rr + i < hs ? A[(rr + i) * wp + c0 + j] : T(0);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) bv[q] = cc + 32 * q < wt ? A[(c0 + j) * wp + cc + 32 * q] : T(0);
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[i][q] = fma(av[i], bv[q], acc[i][q]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (rr + i < hs && cc + 32 * q < wt) A[(rr + i) * wp + cc + 32 * q] -= acc[i][q];
-      }
+    for (int it = tid; it < nr + nc; it += SL_THREADS) {
+      if (it < nr)
+        slab_eliminate<T, false>(Ub, wp, A + (size_t)(r1 + it) * wp + c0, true, bw, spec, info, kabs + c0, bad);
+      else
+        slab_top_column<T>(Ub, wp, A + (size_t)c0 * wp + r1 + (it - nr));
     }
     __syncthreads();
-  }
-  for (int r = warp; r < hs; r += SL_THREADS / 32)
-    for (int c = lane; c < wt; c += 32) D[(int64_t)r * ld + c] = A[r * wp + c];
-  // (iii) for the rows below the slab: the inverse of each 32 x 32 diagonal
-  //       block of U, a warp per block, a lane per column of the inverse:
-  //       back substitution with the division by U's diagonal; uinv[b]
-  //       (32 x 32, row-major), the identity outside a ragged last block
-  if (uinv != nullptr) {
-    T* Zs = lcol + hs;
-    for (int b = warp; 32 * b < hs; b += SL_THREADS / 32) {
-      const int c0 = 32 * b, bw = min(32, hs - c0);
-      T* Z = Zs + (size_t)b * 32 * 33;  // [32][33]
-      const T* Ub = A + (size_t)c0 * wp + c0;
-      for (int t = 0; t < 32; ++t) Z[t * 33 + lane] = (t == lane) ? T(1) : T(0);
-      __syncwarp();
-      for (int t = bw - 1; t >= 0; --t) {
-        const T zt = Z[t * 33 + lane] / Ub[t * wp + t];
-        Z[t * 33 + lane] = zt;
-        for (int q0 = 0; q0 < t; q0 += 8) {
-          T uq[8], zq[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int q = q0 + u < t ? q0 + u : t - 1;
-            uq[u] = Ub[q * wp + t];
-            zq[u] = Z[q * 33 + lane];
-          }
-#pragma unroll
-          for (int u = 0; u < 8; ++u)
-            if (q0 + u < t) Z[(q0 + u) * 33 + lane] = zq[u] - uq[u] * zt;
-        }
+    if (nr > 0) {
+      // (ii), and (a) of the next block on warp 0
+      const int tc = (nc + 31) / 32, tiles = ((nr + 31) / 32) * tc;
+      if (warp == 0) {
+        slab_update_tile<T>(A, wp, c0, r1, r1, hs, wt);
         __syncwarp();
+        slab_eliminate<T, true>(A + (size_t)r1 * wp + r1, wp, A + (size_t)min(r1 + lane, hs - 1) * wp + r1,
+                                r1 + lane < hs, min(32, hs - r1), spec, info, kabs + r1, bad);
       }
-      T* ub = uinv + (size_t)b * 1024;
-      for (int t = 0; t < 32; ++t) ub[t * 32 + lane] = Z[t * 33 + lane];
+      for (int t = warp == 0 ? tiles : warp; t < tiles; t += SL_WARPS - 1)
+        slab_update_tile<T>(A, wp, c0, r1 + 32 * (t / tc), r1 + 32 * (t % tc), hs, wt);
+      __syncthreads();
     }
   }
+  // (iii) on the first warps while the others write the slab back
+  const int nblk = uinv != nullptr ? (hs + 31) / 32 : 0;
+  const int w0 = nblk < SL_WARPS ? nblk : 0;
+  if (warp >= w0) {
+    const bool vec = ((reinterpret_cast<uintptr_t>(D) & 15) == 0) && ((ld * (int64_t)sizeof(T)) & 15) == 0;
+    const int nvec = vec ? wt / VN : 0;
+    for (int r = warp - w0; r < hs; r += SL_WARPS - w0) {
+      for (int v = lane; v < nvec; v += 32)
+        reinterpret_cast<VT*>(D + (int64_t)r * ld)[v] = *reinterpret_cast<const VT*>(A + (size_t)r * wp + v * VN);
+      for (int c = nvec * VN + lane; c < wt; c += 32) D[(int64_t)r * ld + c] = A[(size_t)r * wp + c];
+    }
+  }
+  for (int b = warp; b < nblk; b += SL_WARPS)
+    slab_inverse<T>(A + (size_t)(32 * b) * wp + 32 * b, wp, min(32, hs - 32 * b), uinv + (size_t)b * 1024);
   if (spec && __syncthreads_or(bad) && tid == 0) {
     sp.flag[1] = tag;
     sp.flag[2] = restore_rows;
