@@ -146,30 +146,35 @@ __device__ __forceinline__ void load_rows(const T* G, int64_t ld, int nrows, int
 // memory: the LU of its hs x hs diagonal block without pivoting, blocked by 32
 // columns, and U's rows right of the block (columns hs .. wt).  Per block of
 // 32 columns:
-//   (a)  the 32 x 32 diagonal block, by one warp, a lane per row with the
-//        row's 32 columns in registers: column by column, the pivot's lane
-//        writes its row (U) to shared memory, every lane below it divides by
-//        the pivot (as in the definition) and subtracts its multiple of the row;
-//   (b)  the rows below the block, a thread per row, by the same elimination
-//        against the block's finished U, and beside them, on other warps,
+//   (a)  the 32 x 32 diagonal block, by one warp, a lane per row, in
+//        sub-blocks of eight columns held in registers: per column the pivot
+//        row comes by shuffles, every lane below divides by the pivot (as in
+//        the definition) and subtracts its multiple of the row; then the
+//        sub-block's rows of U to its right (a lane per column) and a rank-8
+//        update of the rows below (a lane per row);
+//   (b)  the rows below the block, two or four lanes per row, by the same
+//        elimination against the block's finished U, and beside them, on other warps,
 //        (i') U's rows right of the block by forward substitution with the
-//        block's L, a thread per column;
+//        block's L, a thread per column, both by sub-blocks of eight;
 //   (ii) a rank-32 update of the rows below the block and the columns right
 //        of it, in 32 x 32 tiles, a warp per tile (8 x 4 per thread, 16-byte
-//        operand loads).  Warp 0 takes the next diagonal block's tile first
-//        and factors that block at once, so that (a) runs under the other
-//        warps' tiles.
+//        operand loads).  Warps 0 to 3 share the next diagonal block's tile
+//        first and warp 0 factors that block at once, so that (a) runs under
+//        the other warps' tiles.
 // Every element gets the same products in the same order as column-by-column
 // rank-1 updates of the 32-column block would give it.
 // Then, for the rows below the slab, (iii) the inverses of U's 32 x 32
 // diagonal blocks (a warp per block, a lane per column), written to uinv while
 // the other warps write the slab back.
-// What bounds it: the chain of hs dependent columns on one SM.  Column steps
-// across the whole CTA cost two barriers and a round through shared memory
-// each (about 900 cycles); within a warp the step is a broadcast and a
-// division.  The register arrays are indexed statically in bodies of eight
-// columns that a rolled loop runs four times, the registers moved down by
-// eight in between: a fully unrolled block would be fetched from L2.
+// What bounds it: the chain of hs dependent columns on one SM (clock stamps,
+// 128 x 256 FP32 slab: 240 cycles a column in (a), 5000 to 7600 per block in
+// (b) and (i'), 9000 for the inverses and the write-back).  Alone on the GPU a
+// 128 x 256 slab takes 47 us and a 128 x 128 one 41 us; with each column step
+// across the whole CTA, two barriers and a round through shared memory a
+// column, they took 112 and 87 us.
+// The loops over sub-blocks stay rolled and their bodies short and free of
+// branches: a 32-column elimination with every column in registers measured
+// 440 cycles a column, most of them at the ends of its many short branches.
 // A zero pivot lowers *info to its absolute column + 1 (kabs = D's first
 // column) and skips its scaling.  With sp.flag set it is a stage of a pivoted
 // panel's diagonal-pivot check: the first slab (first != 0) saves its rows to
@@ -178,7 +183,7 @@ __device__ __forceinline__ void load_rows(const T* G, int64_t ld, int nrows, int
 // a zero or non-finite pivot, records the failure (flag[1] = tag, flag[2] =
 // restore_rows, then flag[0]).  It returns at once when an earlier stage or
 // panel failed.
-constexpr int SL_THREADS = 256;
+constexpr int SL_THREADS = 512;
 constexpr int SL_WARPS = SL_THREADS / 32;
 
 // Row stride of the slab in shared memory, in elements: at least the width
@@ -190,7 +195,10 @@ __host__ __device__ inline int slab_wp(int hs, int wt, int tsize) {
   const int w = wt > ((hs + 31) & ~31) ? wt : ((hs + 31) & ~31);
   return (w + 2 * vn - 1) / (2 * vn) * (2 * vn) + vn;
 }
-inline size_t slab_smem_bytes(int hs, int wt, int tsize) { return (size_t)hs * slab_wp(hs, wt, tsize) * tsize; }
+// shared memory of one slab: its rows, and 32 x 32 scratch per diagonal block for its U's inverse
+inline size_t slab_smem_bytes(int hs, int wt, int tsize) {
+  return ((size_t)hs * slab_wp(hs, wt, tsize) + (size_t)((hs + 31) / 32) * 1024) * tsize;
+}
 
 // VN consecutive elements of shared memory (16-byte aligned) from / to registers
 template <typename T>
@@ -202,148 +210,236 @@ __device__ __forceinline__ void s16_put(T* p, const T* e) {
   *reinterpret_cast<typename V16<T>::type*>(p) = v16_make<T>(e);
 }
 
-// Eliminate the 32 columns c0 .. c0 + bw of this thread's row (at `row`, the
-// row's column c0; bw < 32 only for a ragged last block) against the rows of
-// U of the diagonal block at Ub (row stride wp).  DIAG: the warp's lanes are
-// the diagonal block's own rows, lane j publishing row j before column j's
-// step; `live` lanes hold a row.
-template <typename T, bool DIAG>
-__device__ __forceinline__ void slab_eliminate(T* Ub, int wp, T* row, bool live, int bw, bool spec, int* info, int kcol,
-                                               bool& bad) {
+// a / p from r = 1 / p (rounded): P. Markstein's quotient correction ("Computation
+// of elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
+// Develop. 34, 1990): q = a r, then q + (a - p q) r, which rounds as the division
+// does while p, a and q stay clear of the ends of the exponent range.  Outside
+// that (slab_recip gives r = 0 then) the division itself.
+template <typename T>
+__device__ __forceinline__ T slab_recip(T p) {
+  const T lim = sizeof(T) == 4 ? T(1.0e18) : T(1.0e150);
+  const T m = p < T(0) ? -p : p;
+  return (m < lim && m * lim > T(1)) ? T(1) / p : T(0);
+}
+template <typename T>
+__device__ __forceinline__ T slab_quot(T a, T p, T r) {
+  if (r == T(0)) return a / (p != T(0) ? p : T(1));  // uniform: p and r are the column's
+  const T q = a * r;
+  const T l = fma(fma(-p, q, a), r, q);
+  return l - l == T(0) ? l : q;  // (an overflowed q stays)
+}
+
+// Eight columns of a row, y (registers) -= a x (eight rows of U at u, row stride wp)
+template <typename T>
+__device__ __forceinline__ void slab_rank8(T* y, const T (&a)[8], const T* u, int wp) {
+  constexpr int VN = V16<T>::n;
+  T yv[8];
+#pragma unroll
+  for (int g = 0; g < 8; g += VN) s16_get<T>(y + g, yv + g);
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    T uv[8];
+#pragma unroll
+    for (int g = 0; g < 8; g += VN) s16_get<T>(u + (size_t)t * wp + g, uv + g);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) yv[e] = fma(-a[t], uv[e], yv[e]);
+  }
+#pragma unroll
+  for (int g = 0; g < 8; g += VN) s16_put<T>(y + g, yv + g);
+}
+
+// One column's eight entries x (row stride wp) <- their part of L^-1 x for the
+// 8 x 8 unit-lower block at L; xv keeps them
+template <typename T>
+__device__ __forceinline__ void slab_tri8(T* x, const T* L, int wp, T (&xv)[8]) {
+  constexpr int VN = V16<T>::n;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) xv[t] = x[(size_t)t * wp];
+#pragma unroll
+  for (int t = 1; t < 8; ++t) {
+    T l[8];
+#pragma unroll
+    for (int g = 0; g < t; g += VN) s16_get<T>(L + (size_t)t * wp + g, l + g);
+#pragma unroll
+    for (int q = 0; q < t; ++q) xv[t] = fma(-l[q], xv[q], xv[t]);
+  }
+#pragma unroll
+  for (int t = 1; t < 8; ++t) x[(size_t)t * wp] = xv[t];
+}
+
+// (a) One warp: LU of the bw x bw diagonal block at Ub (row stride wp; bw < 32
+// only for a ragged last block), lane = row, by sub-blocks of eight columns;
+// the reciprocals of its pivots to rinv.
+template <typename T>
+__device__ __forceinline__ void slab_diag(T* Ub, int wp, int bw, bool spec, int* info, int kcol, T* rinv, bool& bad) {
   constexpr int VN = V16<T>::n;
   const int lane = threadIdx.x & 31;
-  T a[32];
-#pragma unroll
-  for (int g = 0; g < 32 / VN; ++g) {
-    if (live) {
-      s16_get<T>(row + g * VN, a + g * VN);
-    } else {
-#pragma unroll
-      for (int e = 0; e < VN; ++e) a[g * VN + e] = T(0);
-    }
-  }
+  const bool live = lane < bw;
+  T* row = Ub + (size_t)lane * wp;
 #pragma unroll 1
-  for (int jb = 0; jb < 32; jb += 8) {
-    if (jb >= bw) break;
-    const int left = 32 - jb;  // columns jb .. 31 are in a[0 .. left)
+  for (int jb = 0; jb < bw; jb += 8) {
+    T a[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) a[e] = T(0);
+    if (live) {
+#pragma unroll
+      for (int g = 0; g < 8; g += VN) s16_get<T>(row + jb + g, a + g);
+    }
+    // lanes at or above the pivot (and lanes without a row) take part with the
+    // multiplier's uses masked: no branch inside a column step
+    const int below = live ? lane - jb : -1;  // columns jb + jj < lane are this row's
+    const int jn = bw - jb;
+    bool big = false;
 #pragma unroll
     for (int jj = 0; jj < 8; ++jj) {
-      const int j = jb + jj;
-      if (j < bw) {
-        T* urow = Ub + (size_t)j * wp + jb;
-        if (DIAG) {
-          if (lane == j) {
+      T u[8];
 #pragma unroll
-            for (int g = jj / VN; g < 32 / VN; ++g)
-              if (g * VN < left) s16_put<T>(urow + g * VN, a + g * VN);
-          }
-          __syncwarp();
-        }
-        T u[32];
+      for (int e = jj; e < 8; ++e) u[e] = __shfl_sync(0xffffffffu, a[e], jb + jj);
+      const T l = a[jj] / (u[jj] != T(0) ? u[jj] : T(1));
+      const bool upd = below > jj && jj < jn;
+      big |= upd && !spec_ok_mult(l);
 #pragma unroll
-        for (int g = jj / VN; g < 32 / VN; ++g)
-          if (g * VN < left) s16_get<T>(urow + g * VN, u + g * VN);
-        const T piv = u[jj];
-        const bool pz = !(piv != T(0));
-        if (DIAG && lane == 0) {
-          if (spec) {
-            if (!finite_nonzero(piv)) bad = true;
-          } else if (pz) {
-            atomicMin(info, kcol + j + 1);
-          }
-        }
-        if (live && (!DIAG || lane > j)) {
-          T l = a[jj];
-          if (!pz) l = l / piv;
-          if (spec && !spec_ok_mult(l)) bad = true;
-          a[jj] = l;
+      for (int e = jj + 1; e < 8; ++e) a[e] = upd ? fma(-l, u[e], a[e]) : a[e];
+      a[jj] = upd ? l : a[jj];
+    }
+    if (spec && big) bad = true;
+    if (below >= 0 && below < 8) {  // this lane's row holds a pivot of the sub-block
+      T piv = a[0];
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            if (g * 8 < left) {  // uniform
-#pragma unroll
-              for (int e = 0; e < 8; ++e)
-                if (g * 8 + e > jj) a[g * 8 + e] = fma(-l, u[g * 8 + e], a[g * 8 + e]);
-            }
-          }
-        }
+      for (int e = 1; e < 8; ++e) piv = below == e ? a[e] : piv;
+      rinv[lane] = slab_recip(piv);
+      if (spec) {
+        if (!finite_nonzero(piv)) bad = true;
+      } else if (!(piv != T(0))) {
+        atomicMin(info, kcol + lane + 1);
       }
     }
     if (live) {
 #pragma unroll
-      for (int g = 0; g < 8 / VN; ++g) s16_put<T>(row + jb + g * VN, a + g * VN);
+      for (int g = 0; g < 8; g += VN) s16_put<T>(row + jb + g, a + g);
     }
-#pragma unroll
-    for (int i = 0; i < 24; ++i) a[i] = a[i + 8];
+    __syncwarp();
+    if (jb + 8 < bw) {
+      // the sub-block's rows of U right of it (lane = column), then the rows below it
+      if (jb + 8 + lane < 32) {
+        T x[8];
+        slab_tri8<T>(Ub + (size_t)jb * wp + jb + 8 + lane, Ub + (size_t)jb * wp + jb, wp, x);
+      }
+      __syncwarp();
+      if (live && lane >= jb + 8) {
+#pragma unroll 1
+        for (int cb = jb + 8; cb < 32; cb += 8) slab_rank8<T>(row + cb, a, Ub + (size_t)jb * wp + cb, wp);
+      }
+      __syncwarp();
+    }
   }
-  if (DIAG) __syncwarp();
 }
 
-// Column of U's 32 rows right of a diagonal block: x <- L^-1 x, x_t at
-// x[t * wp], L (unit lower, 32 x 32) at Lb.
+// (b) Two neighbouring lanes per row: the 32 columns of a row below the
+// diagonal block at Ub eliminated against its U (its pivots' reciprocals at
+// rinv).  Each lane divides the sub-block's eight columns itself; the 8-column
+// chunks right of them are dealt to the two lanes.
 template <typename T>
-__device__ __forceinline__ void slab_top_column(const T* Lb, int wp, T* xcol) {
+__device__ __forceinline__ void slab_left_row(const T* Ub, int wp, const T* rinv, T* row, bool live, int part, bool spec,
+                                              bool& bad) {
   constexpr int VN = V16<T>::n;
-  T x[32];
-#pragma unroll
-  for (int t = 0; t < 32; ++t) x[t] = xcol[(size_t)t * wp];
 #pragma unroll 1
-  for (int sb = 0; sb < 32; sb += 8) {
-    const int left = 32 - sb;  // rows sb .. 31 are in x[0 .. left)
+  for (int jb = 0; jb < 32; jb += 8) {
+    const T* ub = Ub + (size_t)jb * wp + jb;
+    T a[8];
+    if (live) {
 #pragma unroll
-    for (int i = 1; i < 32; ++i) {
-      if (i < left) {  // uniform
-        T l[8];
+      for (int g = 0; g < 8; g += VN) s16_get<T>(row + jb + g, a + g);
 #pragma unroll
-        for (int g = 0; g < 8 / VN; ++g) s16_get<T>(Lb + (size_t)(sb + i) * wp + sb + g * VN, l + g * VN);
+      for (int jj = 0; jj < 8; ++jj) {
+        T u[8];
 #pragma unroll
-        for (int s = 0; s < 8; ++s)
-          if (s < i) x[i] = fma(-l[s], x[s], x[i]);
+        for (int g = jj / VN * VN; g < 8; g += VN) s16_get<T>(ub + (size_t)jj * wp + g, u + g);
+        const T l = slab_quot(a[jj], u[jj], rinv[jb + jj]);
+        if (spec && !spec_ok_mult(l)) bad = true;
+        a[jj] = l;
+#pragma unroll
+        for (int e = jj + 1; e < 8; ++e) a[e] = fma(-l, u[e], a[e]);
       }
     }
+    __syncwarp();  // every lane of the row has read the sub-block
+    if (live) {
+      if (part == 0) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) xcol[(size_t)(sb + i) * wp] = x[i];
-#pragma unroll
-    for (int i = 0; i < 24; ++i) x[i] = x[i + 8];
+        for (int g = 0; g < 8; g += VN) s16_put<T>(row + jb + g, a + g);
+      }
+#pragma unroll 1
+      for (int cb = jb + 8 + 8 * part; cb < 32; cb += 16) slab_rank8<T>(row + cb, a, ub + (cb - jb), wp);
+    }
+    __syncwarp();
   }
 }
 
-// One warp: the 32 x 32 tile of A at rows rr.., columns cc.. -= (the rows'
+// (i') One thread: a column of U's 32 rows right of the diagonal block,
+// x <- L^-1 x with x_t at x[t * wp] and L at Lb.
+template <typename T>
+__device__ __forceinline__ void slab_top_column(const T* Lb, int wp, T* x) {
+  constexpr int VN = V16<T>::n;
+#pragma unroll 1
+  for (int sb = 0; sb < 32; sb += 8) {
+    T xv[8];
+    slab_tri8<T>(x + (size_t)sb * wp, Lb + (size_t)sb * wp + sb, wp, xv);
+#pragma unroll 1
+    for (int rb = sb + 8; rb < 32; rb += 8) {
+      T y[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) y[t] = x[(size_t)(rb + t) * wp];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        T l[8];
+#pragma unroll
+        for (int g = 0; g < 8; g += VN) s16_get<T>(Lb + (size_t)(rb + t) * wp + sb + g, l + g);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) y[t] = fma(-l[q], xv[q], y[t]);
+      }
+#pragma unroll
+      for (int t = 0; t < 8; ++t) x[(size_t)(rb + t) * wp] = y[t];
+    }
+  }
+}
+
+// One warp: the 4 RI x 32 tile of A at rows rr.., columns cc.. -= (the rows'
 // columns c0 .. c0 + 31) x (rows c0 .. c0 + 31's columns).  Thread = rows
 // rr + (lane >> 3) + 4 i, columns cc + 4 (lane & 7) ..: the four row groups'
 // 16-byte pieces fall in different banks.
-template <typename T>
+template <typename T, int RI>
 __device__ __forceinline__ void slab_update_tile(T* A, int wp, int c0, int rr, int cc, int hs, int wt) {
   constexpr int VN = V16<T>::n;
   const int lane = threadIdx.x & 31;
   const int r0 = rr + (lane >> 3), cj = cc + 4 * (lane & 7);
   if (cj >= wt) return;  // (columns past wt but below its 16-byte piece's end are padding of the row)
-  T acc[8][4];
+  T acc[RI][4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < RI; ++i)
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[i][q] = T(0);
-  const T* ar[8];
+  const T* ar[RI];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) ar[i] = A + (size_t)min(r0 + 4 * i, hs - 1) * wp + c0;
+  for (int i = 0; i < RI; ++i) ar[i] = A + (size_t)min(r0 + 4 * i, hs - 1) * wp + c0;
   const T* br = A + (size_t)c0 * wp + cj;
 #pragma unroll 1
   for (int k = 0; k < 32; k += VN) {
-    T av[8][VN];
+    T av[RI][VN];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) s16_get<T>(ar[i] + k, av[i]);
+    for (int i = 0; i < RI; ++i) s16_get<T>(ar[i] + k, av[i]);
 #pragma unroll
     for (int e = 0; e < VN; ++e) {
       T bv[4];
 #pragma unroll
       for (int q = 0; q < 4; q += VN) s16_get<T>(br + (size_t)(k + e) * wp + q, bv + q);
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < RI; ++i)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[i][q] = fma(av[i][e], bv[q], acc[i][q]);
     }
   }
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < RI; ++i) {
     const int r = r0 + 4 * i;
     if (r < hs) {
       T* p = A + (size_t)r * wp + cj;
@@ -361,39 +457,79 @@ __device__ __forceinline__ void slab_update_tile(T* A, int wp, int c0, int rr, i
 
 // One warp: the inverse of the upper bw x bw block Ub (row stride wp) to out
 // (32 x 32, row-major; the identity outside a ragged block).  Lane = a column
-// of the inverse: back substitution with the division by U's diagonal.
+// of the inverse, held in Z (32 x 32): back substitution with the division by
+// U's diagonal, by sub-blocks of eight rows.
 template <typename T>
-__device__ __forceinline__ void slab_inverse(const T* Ub, int wp, int bw, T* out) {
+__device__ __forceinline__ void slab_inverse(T* Ub, int wp, int bw, const T* rinv, T* Z, T* out) {
+  constexpr int VN = V16<T>::n;
   const int lane = threadIdx.x & 31;
-  T z[32];  // row tb + i of the column at z[24 + i]
-#pragma unroll
-  for (int t = 0; t < 32; ++t) z[t] = t == lane ? T(1) : T(0);
+  for (int t = 0; t < 32; ++t) Z[t * 32 + lane] = t == lane ? T(1) : T(0);  // (a lane reads its own column only)
+  if (bw < 32) {  // the padding right of a ragged block's columns couples to nothing
+    for (int r = 0; r < bw; ++r)
+      if (lane >= bw) Ub[(size_t)r * wp + lane] = T(0);
+    __syncwarp();
+  }
 #pragma unroll 1
   for (int tb = 24; tb >= 0; tb -= 8) {
+    // the 8 x 8 block of U on the diagonal, the identity past a ragged block
+    T z[8], u[8][8];
 #pragma unroll
-    for (int jj = 7; jj >= 0; --jj) {
-      const int t = tb + jj;
-      if (t < bw) {  // uniform
-        const T* ucol = Ub + t;  // U(q, t) at ucol[q * wp]
-        const T zt = z[24 + jj] / ucol[(size_t)t * wp];
-        z[24 + jj] = zt;
+    for (int i = 0; i < 8; ++i) z[i] = Z[(tb + i) * 32 + lane];
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          if (g * 8 >= 24 - tb) {  // uniform: rows tb - 24 + 8 g .. exist
+    for (int i = 0; i < 8; ++i) {
+      const bool in = tb + i < bw;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const int i = g * 8 + e;  // row q = tb - 24 + i
-              if (i < 24 + jj) z[i] = z[i] - ucol[(size_t)(tb - 24 + i) * wp] * zt;
-            }
-          }
+      for (int g = i / VN * VN; g < 8; g += VN) {
+        if (in) {
+          s16_get<T>(Ub + (size_t)(tb + i) * wp + tb + g, &u[i][g]);
+        } else {
+#pragma unroll
+          for (int e = g; e < g + VN; ++e) u[i][e] = e == i ? T(1) : T(0);
         }
       }
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) out[(tb + i) * 32 + lane] = z[24 + i];
+    for (int jj = 7; jj >= 0; --jj) {
+      z[jj] = slab_quot(z[jj], u[jj][jj], tb + jj < bw ? rinv[tb + jj] : T(1));
 #pragma unroll
-    for (int i = 31; i >= 8; --i) z[i] = z[i - 8];
+      for (int i = 0; i < jj; ++i) z[i] = fma(-u[i][jj], z[jj], z[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) out[(tb + i) * 32 + lane] = z[i];
+    if (tb >= bw) continue;
+#pragma unroll 1
+    for (int qb = tb - 8; qb >= 0; qb -= 8) {
+      T y[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) y[i] = Z[(qb + i) * 32 + lane];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        T uq[8];
+#pragma unroll
+        for (int g = 0; g < 8; g += VN) s16_get<T>(Ub + (size_t)(qb + i) * wp + tb + g, uq + g);
+#pragma unroll
+        for (int jj = 7; jj >= 0; --jj) y[i] = fma(-uq[jj], z[jj], y[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) Z[(qb + i) * 32 + lane] = y[i];
+    }
   }
+}
+
+// rows [0, nrows) x columns [0, ncol) of G (row-major, ld) into S (row stride
+// sld, a multiple of 16 bytes): asynchronous 16-byte copies when G's rows are
+// 16-byte aligned, all in flight together
+template <typename T>
+__device__ __forceinline__ void slab_load(const T* G, int64_t ld, int nrows, int ncol, T* S, int sld) {
+  constexpr int VN = V16<T>::n;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool vec = ((reinterpret_cast<uintptr_t>(G) & 15) == 0) && ((ld * (int64_t)sizeof(T)) & 15) == 0;
+  const int nvec = vec ? ncol / VN : 0;
+  for (int r = warp; r < nrows; r += SL_WARPS) {
+    for (int v = lane; v < nvec; v += 32) cp_async<16>(S + (size_t)r * sld + v * VN, G + (int64_t)r * ld + v * VN);
+    for (int c = nvec * VN + lane; c < ncol; c += 32) cp_async<sizeof(T)>(S + (size_t)r * sld + c, G + (int64_t)r * ld + c);
+  }
+  cp_async_wait_all();
 }
 
 template <typename T>
@@ -405,6 +541,7 @@ __global__ void __launch_bounds__(SL_THREADS) slab_lu_kernel(T* D, int64_t ld, i
   using VT = typename V16<T>::type;
   const int wp = slab_wp(hs, wt, sizeof(T));
   T* A = reinterpret_cast<T*>(smem_raw);  // [hs][wp]
+  __shared__ T rinv[128];                 // the reciprocals of the pivots
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool spec = sp.flag != nullptr;
   bool bad = false;
@@ -415,14 +552,20 @@ __global__ void __launch_bounds__(SL_THREADS) slab_lu_kernel(T* D, int64_t ld, i
       return;
     }
   }
-  load_rows<T, SL_THREADS>(D, ld, hs, hs, wt, A, wp, (spec && first) ? sp.backup : nullptr);
+  slab_load<T>(D, ld, hs, wt, A, wp);
   if (spec && first) {
     for (int j = tid; j < wt; j += SL_THREADS) sp.ipiv[kabs + j] = kabs + j + 1;
     if (tid == 0) sp.perm[0] = 0;
   }
   __syncthreads();
-  if (warp == 0)
-    slab_eliminate<T, true>(A, wp, A + (size_t)lane * wp, lane < hs, min(32, hs), spec, info, kabs, bad);
+  if (warp == 0) {
+    slab_diag<T>(A, wp, min(32, hs), spec, info, kabs, rinv, bad);
+  } else if (spec && first) {
+    // the rows as they were (D itself is written at the end)
+    for (int r = warp - 1; r < hs; r += SL_WARPS - 1)
+#pragma unroll 4
+      for (int c = lane; c < wt; c += 32) sp.backup[(int64_t)r * wt + c] = D[(int64_t)r * ld + c];
+  }
   __syncthreads();
   for (int c0 = 0; c0 < hs; c0 += 32) {
     const int bw = min(32, hs - c0);
@@ -431,24 +574,27 @@ __global__ void __launch_bounds__(SL_THREADS) slab_lu_kernel(T* D, int64_t ld, i
     // (b), (i'): rows below, then columns right of the block (a column exists
     // only beside a whole 32-column block)
     const int nr = hs - r1, nc = wt - r1;
-    for (int it = tid; it < nr + nc; it += SL_THREADS) {
-      if (it < nr)
-        slab_eliminate<T, false>(Ub, wp, A + (size_t)(r1 + it) * wp + c0, true, bw, spec, info, kabs + c0, bad);
-      else
-        slab_top_column<T>(Ub, wp, A + (size_t)c0 * wp + r1 + (it - nr));
+    const int ritems = (nr * 2 + 31) & ~31;  // whole warps
+    for (int it = tid; it < ritems + nc; it += SL_THREADS) {
+      if (it < ritems) {
+        const int r = it >> 1;
+        slab_left_row<T>(Ub, wp, rinv + c0, A + (size_t)(r1 + min(r, nr - 1)) * wp + c0, r < nr, it & 1, spec, bad);
+      } else {
+        slab_top_column<T>(Ub, wp, A + (size_t)c0 * wp + r1 + (it - ritems));
+      }
     }
     __syncthreads();
     if (nr > 0) {
-      // (ii), and (a) of the next block on warp 0
+      // (ii), and (a) of the next block on warp 0 once warps 0..3 have updated its tile
       const int tc = (nc + 31) / 32, tiles = ((nr + 31) / 32) * tc;
-      if (warp == 0) {
-        slab_update_tile<T>(A, wp, c0, r1, r1, hs, wt);
-        __syncwarp();
-        slab_eliminate<T, true>(A + (size_t)r1 * wp + r1, wp, A + (size_t)min(r1 + lane, hs - 1) * wp + r1,
-                                r1 + lane < hs, min(32, hs - r1), spec, info, kabs + r1, bad);
+      if (warp < 4) {
+        slab_update_tile<T, 2>(A, wp, c0, r1 + 8 * warp, r1, min(hs, r1 + 32), wt);
+        asm volatile("bar.sync 1, 128;" ::: "memory");
       }
-      for (int t = warp == 0 ? tiles : warp; t < tiles; t += SL_WARPS - 1)
-        slab_update_tile<T>(A, wp, c0, r1 + 32 * (t / tc), r1 + 32 * (t % tc), hs, wt);
+      if (warp == 0)
+        slab_diag<T>(A + (size_t)r1 * wp + r1, wp, min(32, hs - r1), spec, info, kabs + r1, rinv + r1, bad);
+      for (int t = warp == 0 ? tiles : SL_WARPS - warp; t < tiles; t += SL_WARPS - 1)
+        slab_update_tile<T, 8>(A, wp, c0, r1 + 32 * (t / tc), r1 + 32 * (t % tc), hs, wt);
       __syncthreads();
     }
   }
@@ -465,7 +611,8 @@ __global__ void __launch_bounds__(SL_THREADS) slab_lu_kernel(T* D, int64_t ld, i
     }
   }
   for (int b = warp; b < nblk; b += SL_WARPS)
-    slab_inverse<T>(A + (size_t)(32 * b) * wp + 32 * b, wp, min(32, hs - 32 * b), uinv + (size_t)b * 1024);
+    slab_inverse<T>(A + (size_t)(32 * b) * wp + 32 * b, wp, min(32, hs - 32 * b), rinv + 32 * b,
+                    A + (size_t)hs * wp + (size_t)b * 1024, uinv + (size_t)b * 1024);
   if (spec && __syncthreads_or(bad) && tid == 0) {
     sp.flag[1] = tag;
     sp.flag[2] = restore_rows;
