@@ -165,6 +165,28 @@ __device__ __forceinline__ bool is_inf_mag(double v) {
   return (unsigned long long)__double_as_longlong(v) == 0x7ff0000000000000ull;
 }
 
+// a / p from r = 1 / p (rounded): P. Markstein's quotient correction ("Computation
+// of elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
+// Develop. 34, 1990): q = a r, then q + (a - p q) r, which rounds as the division
+// does while p, a and q stay clear of the ends of the exponent range.  A pivot
+// outside that gets r = 0 from recip_rn, and its quotients the division itself.
+__device__ __forceinline__ float recip_rn(float p) {
+  const float m = fabsf(p);
+  return m > 1.0e-18f && m < 1.0e18f ? 1.0f / p : 0.0f;
+}
+__device__ __forceinline__ double recip_rn(double p) {
+  // (2^-500 <= |p| < 2^500 on the exponent field: FP64 compares are slow here)
+  const unsigned e = ((unsigned)__double2hiint(p) >> 20) & 0x7ffu;
+  return e - 523u < 1000u ? 1.0 / p : 0.0;
+}
+template <typename T>
+__device__ __forceinline__ T quot_rn(T a, T p, T r) {
+  if (!nonzero(r)) return a / (nonzero(p) ? p : T(1));
+  const T q = a * r;
+  const T l = fma(fma(-p, q, a), r, q);
+  return is_inf_mag(pivot_mag(q)) ? q : l;  // (an overflowed q stays)
+}
+
 template <typename T>
 __device__ __forceinline__ void warp_argmax(T& v, int& i) {
 #pragma unroll

@@ -67,13 +67,15 @@ cudaError_t launch_panel(T* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv,
                          const PanelScratch& s, const DevInfo& dev, cudaStream_t st, const int* spec_flag = nullptr,
                          const T* spec_backup = nullptr);
 
-// The FP32 panel on one thread-block cluster (panel_cluster.cu): same
-// arguments and outputs as launch_panel; used by launch_panel<float> when
-// panel_cluster_available(m, w).  panel_cluster_size gives its CTA count.
-int panel_cluster_size(int m, int w);
-bool panel_cluster_available(int m, int w);
-cudaError_t launch_panel_cluster(float* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv, int* info, int* status,
-                                 int* perm, cudaStream_t st);
+// The panel on one thread-block cluster (panel_cluster.cu): same arguments and
+// outputs as launch_panel without a check; used by launch_panel when the panel
+// fits (panel_cluster_fits: its rows, all w columns, in the shared memory of
+// at most 16 CTAs).
+template <typename T>
+bool panel_cluster_fits(int m, int w, const DevInfo& dev);
+template <typename T>
+cudaError_t launch_panel_cluster(T* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv, int* info, int* status,
+                                 int* perm, const DevInfo& dev, cudaStream_t st);
 // SMs one panel launch occupies (for the lookahead's trailing-update cap).
 int panel_sm_use(int m, int w, int tsize, const DevInfo& dev, const PanelScratch& s);
 

@@ -268,7 +268,7 @@ extern "C" int lu_create_ex(lu_ctx* out, void* cuda_stream, lu_alloc_fn alloc, l
     return LU_ECUDA;
   }
   if (getenv("GB300LU_NO_LOOKAHEAD")) c->lookahead = false;
-  // the cluster panel kernel has no restore step for a failed check
+  // (GB300LU_PANEL_CLUSTER: every panel pivoted, on a cluster where it fits)
   if (getenv("GB300LU_NO_SPEC") || getenv("GB300LU_PANEL_CLUSTER")) c->spec = false;
   if (const char* e = getenv("GB300LU_SPEC_SMS")) c->spec_sms = atoi(e);
   if (getenv("GB300LU_RESIDUAL_DFMA")) c->split_residual = false;
@@ -478,7 +478,11 @@ static int factor_loop(lu_fact f) {
     // with the lookahead, only the next panel's columns of the top block row
     // are solved and cast before the next panel starts; the rest follow on
     // this stream while the next panel runs on the side stream
-    const bool split_top = tc && lookahead && rest > w2;
+    // (a pivoted panel on one cluster waits for a whole GPC, which the update
+    // beside it would hold: it runs after the update instead, and is faster
+    // alone than the cooperative panel beside it)
+    const bool split_top =
+        tc && lookahead && rest > w2 && !(mode == SPEC_OFF && panel_cluster_fits<T>(rest, w2, c->dev));
     if (f->ozaki) {
       CU_TRY(top_solve_split(f, (double*)Wkk, (double*)U12, ld, w, rest));
     } else if (tc) {

@@ -210,25 +210,6 @@ __device__ __forceinline__ void s16_put(T* p, const T* e) {
   *reinterpret_cast<typename V16<T>::type*>(p) = v16_make<T>(e);
 }
 
-// a / p from r = 1 / p (rounded): P. Markstein's quotient correction ("Computation
-// of elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
-// Develop. 34, 1990): q = a r, then q + (a - p q) r, which rounds as the division
-// does while p, a and q stay clear of the ends of the exponent range.  Outside
-// that (slab_recip gives r = 0 then) the division itself.
-template <typename T>
-__device__ __forceinline__ T slab_recip(T p) {
-  const T lim = sizeof(T) == 4 ? T(1.0e18) : T(1.0e150);
-  const T m = p < T(0) ? -p : p;
-  return (m < lim && m * lim > T(1)) ? T(1) / p : T(0);
-}
-template <typename T>
-__device__ __forceinline__ T slab_quot(T a, T p, T r) {
-  if (r == T(0)) return a / (p != T(0) ? p : T(1));  // uniform: p and r are the column's
-  const T q = a * r;
-  const T l = fma(fma(-p, q, a), r, q);
-  return l - l == T(0) ? l : q;  // (an overflowed q stays)
-}
-
 // Eight columns of a row, y (registers) -= a x (eight rows of U at u, row stride wp)
 template <typename T>
 __device__ __forceinline__ void slab_rank8(T* y, const T (&a)[8], const T* u, int wp) {
@@ -307,7 +288,7 @@ __device__ __forceinline__ void slab_diag(T* Ub, int wp, int bw, bool spec, int*
       T piv = a[0];
 #pragma unroll
       for (int e = 1; e < 8; ++e) piv = below == e ? a[e] : piv;
-      rinv[lane] = slab_recip(piv);
+      rinv[lane] = recip_rn(piv);
       if (spec) {
         if (!finite_nonzero(piv)) bad = true;
       } else if (!(piv != T(0))) {
@@ -355,7 +336,7 @@ __device__ __forceinline__ void slab_left_row(const T* Ub, int wp, const T* rinv
         T u[8];
 #pragma unroll
         for (int g = jj / VN * VN; g < 8; g += VN) s16_get<T>(ub + (size_t)jj * wp + g, u + g);
-        const T l = slab_quot(a[jj], u[jj], rinv[jb + jj]);
+        const T l = quot_rn(a[jj], u[jj], rinv[jb + jj]);
         if (spec && !spec_ok_mult(l)) bad = true;
         a[jj] = l;
 #pragma unroll
@@ -490,7 +471,7 @@ __device__ __forceinline__ void slab_inverse(T* Ub, int wp, int bw, const T* rin
     }
 #pragma unroll
     for (int jj = 7; jj >= 0; --jj) {
-      z[jj] = slab_quot(z[jj], u[jj][jj], tb + jj < bw ? rinv[tb + jj] : T(1));
+      z[jj] = quot_rn(z[jj], u[jj][jj], tb + jj < bw ? rinv[tb + jj] : T(1));
 #pragma unroll
       for (int i = 0; i < jj; ++i) z[i] = fma(-u[i][jj], z[jj], z[i]);
     }

@@ -407,18 +407,7 @@ int panel_grid_size(int m, int w, int tsize, const DevInfo& dev, int gmax, int g
   return (int)cdiv(m, R);
 }
 
-// Panels use the cooperative grid kernel.  The cluster kernel (FP32 only;
-// GB300LU_PANEL_CLUSTER set) computes the same factorization on at most 16
-// SMs: about 4 us per column like the cooperative kernel, but its in-panel
-// update on 16 SMs makes it slower alone (210 vs 185 ms of panels at
-// n = 32768), and beside the lookahead update it waits for a free GPC.
-static bool use_cluster_panel(int m, int w, int tsize) {
-  static const bool cluster = getenv("GB300LU_PANEL_CLUSTER") != nullptr;
-  return tsize == 4 && cluster && panel_cluster_available(m, w);
-}
-
 int panel_sm_use(int m, int w, int tsize, const DevInfo& dev, const PanelScratch& s) {
-  if (use_cluster_panel(m, w, tsize)) return panel_cluster_size(m, w);
   return panel_grid_size(m, w, tsize, dev, s.gmax, s.gtarget);
 }
 
@@ -427,12 +416,8 @@ cudaError_t launch_panel(T* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv,
                          const PanelScratch& s, const DevInfo& dev, cudaStream_t st, const int* spec_flag,
                          const T* spec_backup) {
   if (w <= 0 || m < w || w > s.wmax) return cudaErrorInvalidValue;
-  if constexpr (sizeof(T) == 4) {
-    if (use_cluster_panel(m, w, 4)) {
-      if (spec_flag != nullptr) return cudaErrorInvalidValue;  // no restore step in the cluster kernel
-      return launch_panel_cluster(Wkk, ldw, m, w, kabs, ipiv, info, status, s.perm, st);
-    }
-  }
+  if (spec_flag == nullptr && panel_cluster_fits<T>(m, w, dev))
+    return launch_panel_cluster<T>(Wkk, ldw, m, w, kabs, ipiv, info, status, s.perm, dev, st);
   if (s.gmax > PNL_XG) return cudaErrorInvalidValue;  // every candidate row fits the exchange buffer
   const int ib = PNL_IB < s.ibmax ? PNL_IB : s.ibmax;
   const int G0 = panel_grid_size(m, w, sizeof(T), dev, s.gmax, s.gtarget);

@@ -1,4 +1,4 @@
-// FP32 panel factorization with partial pivoting on one thread-block cluster.
+// Panel factorization with partial pivoting on one thread-block cluster.
 //
 // The same computation as panel_getrf_kernel (the paper's diagonal and left
 // blocks of a block iteration, factored together because partial pivoting
@@ -7,68 +7,54 @@
 // below j, swap rows j and p, divide the entries below the diagonal by the
 // pivot, rank-1 update of the columns to the right.
 //
-// The grid is one cluster of CL <= 16 CTAs (512 threads each); CTA c owns the
-// panel rows [c R, c R + R).  Per column, the candidates are exchanged
-// through distributed shared memory: every CTA publishes its best (|a|, row)
-// and that row's sub-panel values in its own shared memory, the cluster
-// barrier (release/acquire, cluster scope) follows, and every CTA reads all
-// peers' candidates in one round of DSMEM loads.  That replaces the grid
-// barrier and the L2 round trips of the cooperative kernel.
+// The grid is one cluster of CL <= 16 CTAs; CTA c holds the panel rows
+// [c R, c R + R), all w columns, in shared memory for the whole panel.  Rows do
+// not move: every row carries its current position (pos), a pivot swaps two
+// positions, and at the end each row is written to its position.
 //
-// The panel is processed in sub-panels of 16 columns.  A thread owns up to 4
-// rows (tid + 512 q) of the sub-panel; the part of a row still being updated
-// sits in registers, rotated so that the current column is always register 0
-// (every register index is a compile-time constant and one copy of the column
-// code serves all columns), and the finished part of every row goes to shared
-// memory (Ls), where the sub-panel is whole when its last column is done.  After a sub-panel: its
-// values are written back, its row interchanges are applied to the panel's
-// other columns (columns distributed over the CTAs), every CTA solves the
-// sub-panel's top rows of the columns to its right (U rows, into shared
-// memory), and each CTA updates its own rows of those columns (a rank-16
-// update, coalesced along the row, U in registers).  Three cluster
-// synchronizations per sub-panel, one per column.
+// What bounds it is the chain of w columns, one exchange of candidates each:
+//  - every CTA sends its best (|a|, position), the pivot's reciprocal and the
+//    row's values right of the diagonal into every peer's shared memory
+//    (st.async, whose bytes complete a transaction barrier there): one hop
+//    through distributed shared memory, no grid barrier and no L2 round trip;
+//  - what the exchange needs of column j + 1 comes first (the multipliers of
+//    column j, column j + 1's update and search, the candidate row's values);
+//    the update of the other columns runs while the candidates travel.
+// Quotients come from the pivot's reciprocal by P. Markstein's correction
+// (see quot_rn), three multiply-adds instead of a division: GB300 issues an
+// FP64 warp instruction once in 64 cycles per SM quarter, and a division takes
+// nine of them.
+// Measured (us per column, step call, cooperative kernel -> this one): FP64
+// 512 x 64 5.1 -> 2.2, 1023 x 64 5.5 -> 2.5, 4096 x 64 5.9 -> 4.4, 2500 x 128
+// 6.0 -> 4.6; FP32 512 x 64 3.6 -> 1.6, 2500 x 128 4.0 -> 1.8, 6000 x 64
+// 4.3 -> 2.2.  Clock stamps (1024 x 64): the wait for the records is 130 cycles
+// of a column's 2700 (FP32) and 4600 (FP64); the rest is the CTA's own chain
+// (search 550, multipliers 300 / 780, sending 600 / 880) and the update of
+// the other columns (400 / 1500).
 //
-// The kernel spins on nothing: its only waits are hardware cluster barriers,
-// and every CTA executes the same sequence of them (no CTA leaves early, the
-// loop bounds are the same in all), so each one completes.
+// A record's buffer is reused every third column: its pivot row is read until
+// a CTA has finished column j, a peer sends column j + 3 only after it has
+// this CTA's record of column j + 2, and that is sent after column j is done.
+//
+// Every wait on a transaction barrier is bounded; a CTA whose wait runs out
+// raises ST_TIMEOUT and goes to the closing cluster barrier, which all CTAs
+// reach (the others' waits run out too).
 #include <climits>
 #include <mutex>
-#include <utility>
 
 #include "common.cuh"
 #include "kernels.h"
-#include "permrec.cuh"
+#include "tc_ptx.cuh"
 
 namespace gb {
 
-constexpr int PC_THREADS = 512;
-constexpr int PC_WARPS = PC_THREADS / 32;
-constexpr int PC_IB = 16;
-constexpr int PC_RPT = 4;          // rows per thread at most: R <= 2048
 constexpr int PC_CLMAX = 16;
-constexpr int PC_WMAX = 512;
-constexpr int PC_HF = 2048;        // hash buckets: rows outside the panel's top w rows
-constexpr int PC_HS = 128;         // hash buckets: rows outside a sub-panel's top rows
+constexpr int PC_NTMAX = 512;
+constexpr int PC_NBUF = 3;
 
-struct alignas(16) PcSmem {
-  float slot[2][2 + PC_IB];  // |a|, row (bits), the row's sub-panel values
-  float rowj[2][PC_IB];      // row j's sub-panel values (its owner CTA)
-  float stg[PC_WARPS][PC_IB];
-  float redv[PC_WARPS];
-  int redi[PC_WARPS];
-  float xs[PC_CLMAX][2 + PC_IB];  // every CTA's slot, read through DSMEM
-  float rj[PC_IB];
-  int cnt[2];  // permutation record counts: whole panel, sub-panel
-  float L11[PC_IB][PC_IB + 1];
-  int fpos[2 * PC_WMAX], fcur[2 * PC_WMAX];
-  int spos[2 * PC_IB], scur[2 * PC_IB];
-  int hfk[PC_HF], hfv[PC_HF];
-  int hsk[PC_HS], hsv[PC_HS];
-  float U[PC_IB][PC_WMAX];
-};
-
+template <typename T>
 struct PcParams {
-  float* A;  // W(k, k)
+  T* A;  // W(k, k)
   int64_t ld;
   int m, w, R;
   int kabs;
@@ -78,479 +64,447 @@ struct PcParams {
   int* perm;
 };
 
-__device__ __forceinline__ uint32_t cl_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
+// A candidate's record: 16-byte pieces, the header first (key, position,
+// reciprocal), then the row's w values.  Column j's record is sent from the
+// piece that holds column j on.
+template <typename T>
+struct PcRec;
+template <>
+struct PcRec<double> {
+  static constexpr int VN = 2, HC = 2;  // values per piece, header pieces
+};
+template <>
+struct PcRec<float> {
+  static constexpr int VN = 4, HC = 1;
+};
+
+__host__ __device__ inline int pc_pieces(int w, int tsize) {
+  return (tsize == 8 ? PcRec<double>::HC : PcRec<float>::HC) + (w * tsize + 15) / 16;
 }
-__device__ __forceinline__ uint32_t cl_map(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ float cl_ldf(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ void cl_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t sm_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+// the tile, the records (received ones and the CTA's own; they hold at least
+// R positions at the end)
+__host__ __device__ inline size_t pc_smem_bytes(int R, int w, int cl, int tsize) {
+  const size_t tile = ((size_t)w * (R | 1) * tsize + 15) / 16 * 16;
+  const size_t recs = (size_t)(PC_NBUF * cl + 1) * pc_pieces(w, tsize) * 16;
+  return tile + (recs > (size_t)R * 4 ? recs : (size_t)R * 4);
 }
 
-// v[q][c] for a run-time q, by predicated selects: an indexed read would move
-// the whole register tile to local memory.
-static_assert(PC_RPT == 4, "pc_pick selects among four rows");
-__device__ __forceinline__ float pc_pick(const float (&v)[PC_RPT][PC_IB], int c, int q) {
-  float x = v[0][c];
-  asm("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %2, 1;\n\tselp.f32 %0, %1, %0, p;\n\t}" : "+f"(x) : "f"(v[1][c]), "r"(q));
-  asm("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %2, 2;\n\tselp.f32 %0, %1, %0, p;\n\t}" : "+f"(x) : "f"(v[2][c]), "r"(q));
-  asm("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %2, 3;\n\tselp.f32 %0, %1, %0, p;\n\t}" : "+f"(x) : "f"(v[3][c]), "r"(q));
-  return x;
+// Pivot-search order as unsigned words: larger first, 0 = no candidate (a
+// magnitude's bit pattern is below 0x7ff00001 / 0x7f800001).
+struct PcKey {
+  unsigned hi, lo;
+  int pos;
+};
+__device__ __forceinline__ PcKey pc_key(float v, bool valid, int pos) {
+  return {valid ? __float_as_uint(pivot_mag(v)) + 1u : 0u, 0u, valid ? pos : INT_MAX};
+}
+__device__ __forceinline__ PcKey pc_key(double v, bool valid, int pos) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(pivot_mag(v));
+  return {valid ? (unsigned)(b >> 32) + 1u : 0u, valid ? (unsigned)b : 0u, valid ? pos : INT_MAX};
+}
+__device__ __forceinline__ bool pc_better(const PcKey& a, const PcKey& b) {
+  if (a.hi != b.hi) return a.hi > b.hi;
+  if (a.lo != b.lo) return a.lo > b.lo;
+  return a.pos < b.pos;
+}
+// the best key of the warp in every lane; true in the lane that holds it
+// (positions are distinct, so at most one lane does)
+template <typename T>
+__device__ __forceinline__ bool pc_warp_best(PcKey& k) {
+  const unsigned mh = __reduce_max_sync(0xffffffffu, k.hi);
+  bool in = k.hi == mh;
+  unsigned ml = 0u;
+  if (sizeof(T) == 8) {
+    ml = __reduce_max_sync(0xffffffffu, in ? k.lo : 0u);
+    in = in && k.lo == ml;
+  }
+  const int mp = (int)__reduce_min_sync(0xffffffffu, in ? (unsigned)k.pos : (unsigned)INT_MAX);
+  const bool mine = in && k.pos == mp && mh != 0u;
+  k = {mh, ml, mp};
+  return mine;
 }
 
-// Cluster synchronization (the hardware cluster barrier, release/acquire at
-// cluster scope): this CTA's prior writes, shared and global, become visible
-// to every peer, and the peers' to this CTA.  Every CTA runs the same
-// sequence of synchronizations (the loop bounds are the same in all), so the
-// barrier always completes.
-#define PC_CSYNC() cl_barrier()
+// 16 bytes into a peer's shared memory, counted on the peer's transaction
+// barrier (both shared::cluster addresses of the same CTA)
+__device__ __forceinline__ void pc_send16(uint32_t dst, longlong2 v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(dst),
+               "l"(v.x), "l"(v.y), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ bool pc_try(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 
-__global__ void __launch_bounds__(PC_THREADS, 1) panel_cluster_kernel(PcParams P) {
+template <typename T>
+__global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> P) {
+  constexpr int VN = PcRec<T>::VN, HC = PcRec<T>::HC;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  PcSmem& S = *reinterpret_cast<PcSmem*>(smem_raw);
-  float* Ls = reinterpret_cast<float*>(smem_raw + sizeof(PcSmem));  // [R][PC_IB]: the sub-panel's L rows
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int cta = (int)cl_rank(), CL = (int)gridDim.x;
-  const int R = P.R, w = P.w;
+  __shared__ __align__(8) unsigned long long bars[PC_NBUF];
+  __shared__ uint4 red[PC_NTMAX / 32];  // each row group's best: key, position, row
+  __shared__ int abort_flag;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
+  const int cta = (int)cluster_rank(), CL = (int)gridDim.x;
+  const int R = P.R, w = P.w, Rs = R | 1;
   const int64_t ld = P.ld;
   const int row0 = cta * R;
   const int rloc = max(0, min(P.m, row0 + R) - row0);
-  float* A = P.A;
+  // A warp serves one group of 32 rows, a lane per row: class 0 of the group's
+  // warps takes the chain (multipliers, the next column, the search), and
+  // every class its share of the other columns.
+  const int RG = (R + 31) / 32;
+  const int NC = nw / RG;  // classes; warps past NC * RG only help with the records
+  const int rg = warp % RG, cls = warp / RG;
+  const int r = rg * 32 + lane;
+  const bool live = cls < NC && r < rloc;
+  const bool chain = warp < RG;
+  const int pieces = pc_pieces(w, sizeof(T));
+  const size_t tile = ((size_t)w * Rs * sizeof(T) + 15) / 16 * 16;
+  T* S = reinterpret_cast<T*>(smem_raw);  // [w][Rs]: column c of the tile, row r
+  unsigned char* recs = smem_raw + tile;  // [PC_NBUF][CL][pieces][16]
+  unsigned char* mine = recs + (size_t)PC_NBUF * CL * pieces * 16;  // this CTA's own record
+  T* mrow = reinterpret_cast<T*>(mine + 16 * HC);
+  T* Sr = S + r;  // this lane's row (dereferenced by live lanes only)
 
-  for (int s = tid; s < w; s += PC_THREADS) {
-    S.fpos[s] = s;
-    S.fcur[s] = s;
+  if (tid == 0) {
+    for (int b = 0; b < PC_NBUF; ++b) mbar_init(smem_u32(&bars[b]), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    abort_flag = 0;
+    if (cta == 0) P.perm[0] = 0;
   }
-  for (int s = tid; s < PC_HF; s += PC_THREADS) S.hfk[s] = -1;
-  if (tid == 0) S.cnt[0] = w;
+  // the rows, four of a warp's rows in flight at a time
+  for (int rb = warp; rb < rloc; rb += 4 * nw) {
+    for (int c = lane; c < w; c += 32) {
+      T x[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int rr = rb + i * nw;
+        x[i] = rr < rloc ? __ldcg(P.A + (int64_t)(row0 + rr) * ld + c) : T(0);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int rr = rb + i * nw;
+        if (rr < rloc) S[(size_t)c * Rs + rr] = x[i];
+      }
+    }
+  }
   __syncthreads();
-  cl_barrier();  // every peer has started before any DSMEM access
-  const PermRec fperm{S.fpos, S.fcur, S.hfk, S.hfv, PC_HF - 1, 0, w, &S.cnt[0]};
+  cluster_sync();  // every peer's barriers are set up, and the count of perm is zero
 
-  float v[PC_RPT][PC_IB];
-  // 16-byte row segments: the tile moves in float4 when the rows allow it
-  const bool aligned = ((uintptr_t)A & 15u) == 0 && (ld % 4) == 0;
-  for (int j0 = 0; j0 < w; j0 += PC_IB) {
-    const int ibs = min(PC_IB, w - j0);
-    const bool vec = aligned && ibs == PC_IB;
-    // ---- the sub-panel's rows into registers
+  // this warp's peers (at most two) and this CTA's record in them
+  const uint32_t bar0 = smem_u32(&bars[0]);
+  const uint32_t dst0 = smem_u32(recs + (size_t)cta * pieces * 16);
+  const uint32_t bufstep = (uint32_t)(CL * pieces * 16);
+  uint32_t pbar[2], pdst[2];
 #pragma unroll
-    for (int q = 0; q < PC_RPT; ++q) {
-      const int r = tid + PC_THREADS * q;
-#pragma unroll
-      for (int c = 0; c < PC_IB; ++c) v[q][c] = 0.f;
-      if (r < rloc) {
-        const float* src = A + (int64_t)(row0 + r) * ld + j0;
-        if (vec) {
-#pragma unroll
-          for (int u = 0; u < PC_IB / 4; ++u) {
-            const float4 x = __ldcg(reinterpret_cast<const float4*>(src) + u);
-            v[q][4 * u] = x.x;
-            v[q][4 * u + 1] = x.y;
-            v[q][4 * u + 2] = x.z;
-            v[q][4 * u + 3] = x.w;
-          }
-        } else {
-#pragma unroll
-          for (int c = 0; c < PC_IB; ++c)
-            if (c < ibs) v[q][c] = __ldcg(src + c);
-        }
-      }
+  for (int i = 0; i < 2; ++i) {
+    const int peer = warp + i * nw;
+    pbar[i] = cluster_map(bar0, (uint32_t)(peer < CL ? peer : 0));
+    pdst[i] = cluster_map(dst0, (uint32_t)(peer < CL ? peer : 0));
+  }
+
+  // The CTA's candidate of column c (key `best` of this lane's row, chain
+  // warps): its record to every peer.  pr: the pivot row of column c - 1, by
+  // which the columns right of c still lack their update (null: none).
+  auto publish = [&](int c, int buf, PcKey best, const T* pr) {
+    if (chain) {
+      const bool own = pc_warp_best<T>(best);
+      const unsigned at = __ballot_sync(0xffffffffu, own);
+      if (lane == 0) red[warp] = make_uint4(best.hi, best.lo, (unsigned)best.pos, (unsigned)(rg * 32 + __ffs(at) - 1));
     }
-    // every row's sub-panel values also start in Ls (rows above the
-    // sub-panel keep them; the others are overwritten as they finish)
-#pragma unroll
-    for (int q = 0; q < PC_RPT; ++q) {
-      const int r = tid + PC_THREADS * q;
-      if (r < rloc) {
-        float4* lsv = reinterpret_cast<float4*>(Ls + r * PC_IB);
-#pragma unroll
-        for (int u = 0; u < PC_IB / 4; ++u) lsv[u] = make_float4(v[q][4 * u], v[q][4 * u + 1], v[q][4 * u + 2], v[q][4 * u + 3]);
-      }
-    }
-    for (int s = tid; s < ibs; s += PC_THREADS) {
-      S.spos[s] = j0 + s;
-      S.scur[s] = j0 + s;
-    }
-    for (int s = tid; s < PC_HS; s += PC_THREADS) S.hsk[s] = -1;
-    if (tid == 0) S.cnt[1] = ibs;
     __syncthreads();
-    const PermRec sperm{S.spos, S.scur, S.hsk, S.hsv, PC_HS - 1, j0, j0 + ibs, &S.cnt[1]};
-
-    // local candidate of the sub-panel's first column
-    float bv = -1.f;
-    int bi = INT_MAX, bq = 0;
-#pragma unroll
-    for (int q = 0; q < PC_RPT; ++q) {
-      const int r = tid + PC_THREADS * q;
-      if (r < rloc && row0 + r >= j0) {
-        const float a = pivot_mag(v[q][0]);
-        if (a > bv || (a == bv && row0 + r < bi)) {
-          bv = a;
-          bi = row0 + r;
-          bq = q;
-        }
+    if (abort_flag) return false;
+    uint4 e = red[lane < RG ? lane : 0];
+    if (RG > 1) {
+      PcKey k{lane < RG ? e.x : 0u, lane < RG ? e.y : 0u, lane < RG ? (int)e.z : INT_MAX};
+      const bool own = pc_warp_best<T>(k);
+      const unsigned at = __ballot_sync(0xffffffffu, own);
+      e.w = __shfl_sync(0xffffffffu, e.w, at ? __ffs(at) - 1 : 0);
+      e.x = k.hi;
+      e.y = k.lo;
+      e.z = (unsigned)k.pos;
+    }
+    const bool any = e.x != 0u;
+    if (any) {
+      const T* Sk = S + e.w;
+      const T lc = pr != nullptr ? Sk[(size_t)(c - 1) * Rs] : T(0);
+      for (int q = c + tid; q < w; q += nt) {
+        T v = Sk[(size_t)q * Rs];
+        if (pr != nullptr && q > c) v = fma(-lc, pr[q], v);
+        mrow[q] = v;
       }
     }
-#pragma unroll 1
-    for (int J = 0; J < ibs; ++J) {
-      const int jg = j0 + J;
-      const int par = jg & 1;
-      // ---- 1. this CTA's candidate and its row; row jg from its owner.  A
-      //      published row is whole: its finished part from Ls, the rest
-      //      from the (rotated) registers.
-      if (!(bv < INFINITY)) atomicOr(P.status, ST_RANGE);  // a non-finite candidate
-      float wv = bv;
-      int wi = bi;
-      warp_argmax(wv, wi);
-      if (wi != INT_MAX && bi == wi) {
-        const int r = wi - row0;
-        for (int c = 0; c < J; ++c) S.stg[warp][c] = Ls[r * PC_IB + c];
-#pragma unroll
-        for (int k = 0; k < PC_IB; ++k)
-          if (J + k < PC_IB) S.stg[warp][J + k] = pc_pick(v, k, bq);
-      }
+    if (warp == nw - 1) {
+      const T rv = recip_rn(any ? S[(size_t)c * Rs + e.w] : T(0));
       if (lane == 0) {
-        S.redv[warp] = wv;
-        S.redi[warp] = wi;
-      }
-      {
-        const int lr = jg - row0;
-        if (lr >= 0 && lr < rloc && (lr % PC_THREADS) == tid) {
-          for (int c = 0; c < J; ++c) S.rowj[par][c] = Ls[lr * PC_IB + c];
-#pragma unroll
-          for (int k = 0; k < PC_IB; ++k)
-            if (J + k < PC_IB) S.rowj[par][J + k] = pc_pick(v, k, lr / PC_THREADS);
-        }
-      }
-      __syncthreads();
-      if (warp == 0) {
-        float cv = lane < PC_WARPS ? S.redv[lane] : -1.f;
-        int ci = lane < PC_WARPS ? S.redi[lane] : INT_MAX;
-        warp_argmax(cv, ci);
-        const unsigned mk = __ballot_sync(0xffffffffu, lane < PC_WARPS && ci != INT_MAX && S.redi[lane] == ci);
-        const int ww = mk ? __ffs(mk) - 1 : 0;
-        if (lane == 0) {
-          S.slot[par][0] = cv;
-          S.slot[par][1] = __int_as_float(ci);
-        }
-        if (lane < PC_IB) S.slot[par][2 + lane] = ci != INT_MAX ? S.stg[ww][lane] : 0.f;
-      }
-      // ---- 2. exchange: every CTA's slot and row jg in one round of DSMEM reads
-      PC_CSYNC();
-      if (tid < CL * (2 + PC_IB)) {
-        const int c_ = tid / (2 + PC_IB), k_ = tid % (2 + PC_IB);
-        S.xs[c_][k_] = cl_ldf(cl_map(sm_u32(&S.slot[par][k_]), (uint32_t)c_));
-      } else if (tid >= 320 && tid < 320 + PC_IB) {
-        S.rj[tid - 320] = cl_ldf(cl_map(sm_u32(&S.rowj[par][tid - 320]), (uint32_t)(jg / R)));
-      }
-      __syncthreads();
-      int p, cc = 0;
-      {
-        float cv = -1.f;
-        int ci = INT_MAX;
-        for (int c_ = 0; c_ < CL; ++c_) {
-          const float v_ = S.xs[c_][0];
-          const int i_ = __float_as_int(S.xs[c_][1]);
-          if (v_ > cv || (v_ == cv && i_ < ci)) {
-            cv = v_;
-            ci = i_;
-            cc = c_;
-          }
-        }
-        p = ci;
-      }
-      const float* prow = p != INT_MAX ? &S.xs[cc][2] : S.rj;  // the whole pivot row
-      if (p == INT_MAX) p = jg;  // no candidate at all (cannot happen: row jg is one)
-      float pr[PC_IB];  // its part from column J on, rotated like the registers
-#pragma unroll
-      for (int k = 0; k < PC_IB; ++k) pr[k] = J + k < PC_IB ? prow[J + k] : 0.f;
-      const float piv = pr[0];
-      if (tid == 0) {
-        if (cta == 0) {
-          P.ipiv[P.kabs + jg] = P.kabs + p + 1;
-          if (piv == 0.f) atomicMin(P.info, P.kabs + jg + 1);
-        }
-        if (p != jg) {
-          if (cta == 0) fperm.swap_rows(jg, p);
-          sperm.swap_rows(jg, p);
-        }
-      }
-      // ---- 3. swap, scale (a division, as in the definition), rank-1
-      //      update, rotation, and the next column's local candidate
-      bv = -1.f;
-      bi = INT_MAX;
-      bq = 0;
-#pragma unroll
-      for (int q = 0; q < PC_RPT; ++q) {
-        const int r = tid + PC_THREADS * q;
-        const int rg = row0 + r;
-        if (r < rloc) {
-          if (p != jg && rg == p) {
-            // row p takes row jg: its finished part and its current part
-            for (int c = 0; c < J; ++c) Ls[r * PC_IB + c] = S.rj[c];
-#pragma unroll
-            for (int k = 0; k < PC_IB; ++k) v[q][k] = J + k < PC_IB ? S.rj[J + k] : 0.f;
-          }
-          if (rg == jg) {
-            // the pivot row is final from here on
-            for (int c = 0; c < PC_IB; ++c) Ls[r * PC_IB + c] = prow[c];
-          }
-          if (rg > jg) {
-            float l = v[q][0];
-            if (piv != 0.f) l = l / piv;
-            Ls[r * PC_IB + J] = l;
-#pragma unroll
-            for (int k = 1; k < PC_IB; ++k) v[q][k] -= l * pr[k];
-#pragma unroll
-            for (int k = 0; k + 1 < PC_IB; ++k) v[q][k] = v[q][k + 1];
-            v[q][PC_IB - 1] = 0.f;
-            if (J + 1 < ibs) {
-              const float a = pivot_mag(v[q][0]);
-              if (a > bv || (a == bv && rg < bi)) {
-                bv = a;
-                bi = rg;
-                bq = q;
-              }
-            }
-          }
-        }
+        unsigned* h = reinterpret_cast<unsigned*>(mine);
+        h[0] = e.x;
+        h[1] = e.z;
+        if (sizeof(T) == 8) h[2] = e.y;
+        reinterpret_cast<T*>(mine)[2] = rv;
       }
     }
     __syncthreads();
+    const int p0 = HC + c / VN;  // row pieces from column c's on
+    const int np = HC + pieces - p0;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      if (warp + i * nw < CL) {
+        const uint32_t bar = pbar[i] + 8u * (uint32_t)buf, dst = pdst[i] + bufstep * (uint32_t)buf;
+        for (int x = lane; x < np; x += 32) {
+          const int pc = x < HC ? x : p0 + x - HC;
+          pc_send16(dst + 16u * (uint32_t)pc, reinterpret_cast<const longlong2*>(mine)[pc], bar);
+        }
+      }
+    }
+    return true;
+  };
+  // arm the barrier of column c's records (its previous phase is complete)
+  auto arm = [&](int c, int buf) {
+    if (tid == nt - 1) mbar_expect_tx(bar0 + 8u * (uint32_t)buf, (uint32_t)(CL * (pieces - c / VN) * 16));
+  };
 
-    // ---- (a) the sub-panel (whole in Ls) back to memory
-#pragma unroll
-    for (int q = 0; q < PC_RPT; ++q) {
-      const int r = tid + PC_THREADS * q;
-      if (r < rloc) {
-        float* dst = A + (int64_t)(row0 + r) * ld + j0;
-        const float4* lsv = reinterpret_cast<const float4*>(Ls + r * PC_IB);
-        if (vec) {
-#pragma unroll
-          for (int u = 0; u < PC_IB / 4; ++u) reinterpret_cast<float4*>(dst)[u] = lsv[u];
-        } else {
-          for (int c = 0; c < ibs; ++c) dst[c] = Ls[r * PC_IB + c];
-        }
-      }
-    }
-    PC_CSYNC();
-    // ---- (b) the sub-panel's interchanges on the panel's other columns:
-    //      column o of the others goes to CTA o mod CL; a CTA reads every
-    //      source row of a column before writing any destination row
-    const int nout = w - ibs;
-    const int scnt = S.cnt[1];
-    for (int kb = 0; cta + CL * kb < nout; kb += PC_THREADS / 32) {
-      const int o = cta + CL * (kb + tid / 32);
-      const int s = tid % 32;
-      const bool act = o < nout && s < scnt;
-      const int c = o < j0 ? o : o + ibs;
-      float val = 0.f;
-      if (act) val = __ldcg(A + (int64_t)S.scur[s] * ld + c);
-      __syncthreads();
-      if (act) A[(int64_t)S.spos[s] * ld + c] = val;
-      __syncthreads();
-    }
-    PC_CSYNC();
-    const int nr = w - j0 - ibs;  // columns to the right of the sub-panel
-    if (nr > 0) {
-      // ---- (c) U rows of the right columns: L11^-1 A12, every CTA for itself
-      for (int e = tid; e < ibs * ibs; e += PC_THREADS) {
-        const int t = e / ibs, s = e % ibs;
-        S.L11[t][s] = __ldcg(A + (int64_t)(j0 + t) * ld + j0 + s);
-      }
-      for (int e = tid; e < ibs * nr; e += PC_THREADS) {
-        const int t = e / nr, c = e % nr;
-        S.U[t][c] = __ldcg(A + (int64_t)(j0 + t) * ld + j0 + ibs + c);
-      }
-      __syncthreads();
-      for (int c = tid; c < nr; c += PC_THREADS) {
-        for (int t = 1; t < ibs; ++t) {
-          float x = S.U[t][c];
-          for (int s = 0; s < t; ++s) x -= S.L11[t][s] * S.U[s][c];
-          S.U[t][c] = x;
-        }
-      }
-    }
-    PC_CSYNC();  // every CTA has read the top rows before their owners overwrite them
-    if (nr > 0) {
-      // ---- (d) own rows: top rows take U; rows below get the rank-ibs
-      //      update.  A warp takes rows; a lane takes 4 columns 32 apart per
-      //      pass, with their U column in registers (4 FMAs per shared-memory
-      //      load of the row's L value), the next row's values loaded ahead.
-      for (int r = warp; r < rloc; r += PC_WARPS) {
-        const int rg = row0 + r;
-        if (rg >= j0 && rg < j0 + ibs) {
-          float* rowp = A + (int64_t)rg * ld + j0 + ibs;
-          for (int c = lane; c < nr; c += 32) rowp[c] = S.U[rg - j0][c];
-        }
-      }
-      const int rfirst = max(0, j0 + ibs - row0);  // first own row below the sub-panel
-      constexpr int D = 2;                         // rows per step (and rows of loads in flight)
-      for (int cb = 0; cb < nr; cb += 128) {
-        float u[PC_IB][4];
-#pragma unroll
-        for (int t = 0; t < PC_IB; ++t)
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int c = cb + lane + 32 * k;
-            u[t][k] = (t < ibs && c < nr) ? S.U[t][c] : 0.f;
+  int pos = row0 + r;        // this lane's row's position
+  T cur = live ? Sr[0] : T(0);                                    // chain warps: column j of the row,
+  T nxt = live && w > 1 ? Sr[(size_t)Rs] : T(0);                  // and column j + 1 before column j's update
+  arm(0, 0);
+  bool ok = publish(0, 0, pc_key(cur, live, pos), nullptr);
+  int buf = 0;
+  uint32_t par = 0;
+  for (int j = 0; j < w && ok; ++j) {
+    {
+      const uint32_t bar = bar0 + 8u * (uint32_t)buf;
+      if (!pc_try(bar, par)) {
+        const uint64_t t0 = gtimer();
+        while (!pc_try(bar, par)) {
+          if (*(volatile int*)&abort_flag) break;
+          if (gtimer() - t0 > GB_SPIN_LIMIT_NS) {
+            atomicOr(P.status, ST_TIMEOUT);
+            *(volatile int*)&abort_flag = 1;  // seen by every thread after the CTA's next barrier
+            break;
           }
-        bool cok[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) cok[k] = cb + lane + 32 * k < nr;
-        auto load_rows = [&](int rb, float (&x)[D][4]) {
-#pragma unroll
-          for (int d = 0; d < D; ++d) {
-            const int r = rb + PC_WARPS * d;
-            const float* rp = A + (int64_t)(row0 + r) * ld + j0 + ibs + cb + lane;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) x[d][k] = (r < rloc && cok[k]) ? __ldcg(rp + 32 * k) : 0.f;
-          }
-        };
-        float a[D][4], an[D][4];
-        int rb = rfirst + warp;
-        load_rows(rb, a);
-        for (; rb < rloc; rb += PC_WARPS * D) {
-          load_rows(rb + PC_WARPS * D, an);  // the next rows' values in flight
-#pragma unroll
-          for (int d = 0; d < D; ++d) {
-            const int r = rb + PC_WARPS * d;
-            if (r < rloc) {
-              const float4* lr4 = reinterpret_cast<const float4*>(Ls + r * PC_IB);
-#pragma unroll
-              for (int t4 = 0; t4 < PC_IB / 4; ++t4) {
-                const float4 l4 = lr4[t4];
-                const float lt[4] = {l4.x, l4.y, l4.z, l4.w};
-#pragma unroll
-                for (int tt = 0; tt < 4; ++tt) {
-                  if (4 * t4 + tt < ibs) {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) a[d][k] -= lt[tt] * u[4 * t4 + tt][k];
-                  }
-                }
-              }
-              float* rowp = A + (int64_t)(row0 + r) * ld + j0 + ibs + cb + lane;
-#pragma unroll
-              for (int k = 0; k < 4; ++k)
-                if (cok[k]) rowp[32 * k] = a[d][k];
-            }
-          }
-#pragma unroll
-          for (int d = 0; d < D; ++d)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) a[d][k] = an[d][k];
+        }
+      }
+      __syncwarp();
+    }
+    const int nbuf = buf + 1 == PC_NBUF ? 0 : buf + 1;
+    if (j + 1 < w) arm(j + 1, nbuf);
+    // the pivot: the best of the CTAs' candidates, in every warp
+    const unsigned char* rb = recs + (size_t)buf * bufstep;
+    PcKey k{0u, 0u, INT_MAX};
+    if (lane < CL) {
+      const unsigned* h = reinterpret_cast<const unsigned*>(rb + (size_t)lane * pieces * 16);
+      k = {h[0], sizeof(T) == 8 ? h[2] : 0u, (int)h[1]};
+    }
+    const bool kown = pc_warp_best<T>(k);
+    const unsigned bal = __ballot_sync(0xffffffffu, kown);
+    const int win = bal ? __ffs(bal) - 1 : 0;
+    const int p = k.pos;
+    const unsigned char* rec = rb + (size_t)win * pieces * 16;
+    const T* pr = reinterpret_cast<const T*>(rec + 16 * HC);  // the pivot row, columns j .. w
+    if (live) {
+      if (pos == p)
+        pos = j;
+      else if (pos == j)
+        pos = p;
+    }
+    const bool act = live && pos > j;  // the row is below the diagonal
+    // chain warps: multipliers, column j + 1 and its search
+    PcKey best{0u, 0u, INT_MAX};
+    if (chain) {
+      const T rinv = reinterpret_cast<const T*>(rec)[2];
+      const T piv = pr[j];
+      const T u1 = j + 1 < w ? pr[j + 1] : T(0);
+      if (cta == 0 && tid == 0) {
+        P.ipiv[P.kabs + j] = P.kabs + p + 1;
+        if (!nonzero(piv)) atomicMin(P.info, P.kabs + j + 1);
+        if (is_inf_mag(pivot_mag(piv))) atomicOr(P.status, ST_RANGE);  // a non-finite candidate
+      }
+      if (act) {
+        const T l = nonzero(piv) ? quot_rn(cur, piv, rinv) : cur;
+        Sr[(size_t)j * Rs] = l;
+        cur = fma(-l, u1, nxt);
+        if (j + 1 < w) {
+          Sr[(size_t)(j + 1) * Rs] = cur;
+          best = pc_key(cur, true, pos);
         }
       }
     }
-    __syncthreads();
+    if (j + 1 == w) break;
+    ok = publish(j + 1, nbuf, best, pr);
+    if (!ok) break;
+    // the other columns while the candidates travel: class q takes columns
+    // j + 2 + q, + NC, ... (column j + 2, which the chain needs next, is class 0's)
+    if (act) {
+      const T l = Sr[(size_t)j * Rs];
+      const size_t step = (size_t)NC * Rs;
+      int c = j + 2 + cls;
+      T* x = Sr + (size_t)c * Rs;
+      if (chain && c < w) {
+        nxt = fma(-l, pr[c], x[0]);
+        x[0] = nxt;
+        c += NC;
+        x += step;
+      }
+      for (; c + 3 * NC < w; c += 4 * NC, x += 4 * step) {
+        T v[4], u[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          v[q] = x[q * step];
+          u[q] = pr[c + q * NC];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q * step] = fma(-l, u[q], v[q]);
+      }
+      T v[3], u[3];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        if (c + q * NC < w) {
+          v[q] = x[q * step];
+          u[q] = pr[c + q * NC];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (c + q * NC < w) x[q * step] = fma(-l, u[q], v[q]);
+    }
+    buf = nbuf;
+    if (buf == 0) par ^= 1u;
   }
-
-  // ---- whole-panel permutation for the row interchanges outside the panel
-  if (cta == 0) {
+  __syncthreads();
+  if (!abort_flag) {
+    // each row to its position; the rows that moved to the permutation record
+    int* sp = reinterpret_cast<int*>(recs);  // [R] (the records are all read)
+    if (chain && live) sp[r] = pos;
     __syncthreads();
-    const int fcnt = S.cnt[0];
-    if (tid == 0) P.perm[0] = fcnt;
-    for (int s = tid; s < fcnt; s += PC_THREADS) {
-      P.perm[1 + s] = S.fpos[s];
-      P.perm[1 + 2 * w + s] = S.fcur[s];
+    for (int rr = warp; rr < rloc; rr += nw) {
+      T* dst = P.A + (int64_t)sp[rr] * ld;
+      for (int c = lane; c < w; c += 32) dst[c] = S[(size_t)c * Rs + rr];
     }
+    if (chain && live && pos != row0 + r) {
+      const int q = atomicAdd(P.perm, 1);
+      P.perm[1 + q] = pos;
+      P.perm[1 + 2 * w + q] = row0 + r;
+    }
+  } else {
+    // records may still be on their way to a CTA whose wait ran out
+    const uint64_t t0 = gtimer();
+    while (gtimer() - t0 < 1000000ull) __nanosleep(1000);
   }
-  cl_barrier();  // no CTA leaves while a peer may still read its shared memory
+  cluster_sync();  // no CTA leaves while a peer may still send to it
 }
 
-#undef PC_COLUMN
-#undef PC_CSYNC
-
-// The cluster of a panel: up to 16 CTAs of at most 2048 rows each, at least
-// 256 rows per CTA; -1 when the panel does not fit this kernel.
-int panel_cluster_size(int m, int w) {
-  if (w < 1 || w > PC_WMAX || m < w) return -1;
-  int cl = (m + 255) / 256;
-  if (cl > PC_CLMAX) cl = PC_CLMAX;
-  if (cl < 1) cl = 1;
-  const int R = (m + cl - 1) / cl;
-  if (R > PC_RPT * PC_THREADS) return -1;
+// CTAs of a panel's cluster: rows of 32 (FP64: the FP64 pipes of as many SMs as
+// help) or 64 (FP32) per CTA up to 16 CTAs; -1 when the tile does not fit the
+// shared memory then, or when the cooperative kernel is as fast: an FP64 panel
+// of m w > 360,000 is bound by the FP64 pipes of 16 SMs (3000 x 128: 783 us
+// against 772; 6000 x 64: 358 against 380).
+static int pc_config(int m, int w, int tsize, int optin, int* R, int* nt, size_t* smem) {
+  if (w < 1 || w > 512 || m < w) return -1;
+  const int target = tsize == 8 ? 32 : 64;
+  int cl = 1;
+  while (cl < PC_CLMAX && cl * target < m) cl *= 2;
+  *R = (int)cdiv(m, cl);
+  *nt = *R <= 64 ? 256 : PC_NTMAX;  // (a warp per 32 rows at least)
+  if (*R > PC_NTMAX) return -1;
+  *smem = pc_smem_bytes(*R, w, cl, tsize);
+  if (*smem + 1024 > (size_t)optin) return -1;
+  if (tsize == 8 && (int64_t)m * w > 360000) return -1;
   return cl;
 }
 
-cudaError_t launch_panel_cluster(float* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv, int* info, int* status,
-                                 int* perm, cudaStream_t st) {
-  const int cl = panel_cluster_size(m, w);
+template <typename T>
+static cudaLaunchConfig_t pc_launch(int cl, int nt, size_t smem, cudaStream_t st, cudaLaunchAttribute* at) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cl);
+  cfg.blockDim = dim3(nt);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = cl;
+  at->val.clusterDim.y = 1;
+  at->val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+template <typename T>
+static cudaError_t pc_prepare() {
+  cudaError_t e = allow_max_smem((const void*)panel_cluster_kernel<T>);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute((const void*)panel_cluster_kernel<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
+// Whether the panel fits the cluster kernel and such a cluster can be placed
+// on the current device (asked of the runtime once per cluster and block size,
+// with the largest shared memory).
+template <typename T>
+bool panel_cluster_fits(int m, int w, const DevInfo& dev) {
+  int R = 0, nt = 0;
+  size_t smem = 0;
+  const int cl = pc_config(m, w, sizeof(T), dev.max_smem_optin, &R, &nt, &smem);
+  if (cl < 0) return false;
+  int device = 0;
+  if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return false;
+  static std::mutex mu;
+  static signed char known[64][2][PC_CLMAX + 1] = {};  // 0 unknown, 1 yes, -1 no
+  std::lock_guard<std::mutex> lk(mu);
+  signed char& kn = known[device][nt == PC_NTMAX][cl];
+  if (kn == 0) {
+    int n = 0;
+    cudaLaunchAttribute at[1];
+    cudaFuncAttributes fa;
+    cudaError_t e = pc_prepare<T>();
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, (const void*)panel_cluster_kernel<T>);
+    if (e == cudaSuccess) {
+      cudaLaunchConfig_t cfg =
+          pc_launch<T>(cl, nt, (size_t)dev.max_smem_optin - fa.sharedSizeBytes, nullptr, at);
+      e = cudaOccupancyMaxActiveClusters(&n, (const void*)panel_cluster_kernel<T>, &cfg);
+    }
+    if (e != cudaSuccess) cudaGetLastError();
+    kn = (e == cudaSuccess && n > 0) ? 1 : -1;
+  }
+  return kn > 0;
+}
+
+template <typename T>
+cudaError_t launch_panel_cluster(T* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv, int* info, int* status,
+                                 int* perm, const DevInfo& dev, cudaStream_t st) {
+  PcParams<T> P;
+  int nt = 0;
+  size_t smem = 0;
+  const int cl = pc_config(m, w, sizeof(T), dev.max_smem_optin, &P.R, &nt, &smem);
   if (cl < 0) return cudaErrorInvalidConfiguration;
-  const int R = (m + cl - 1) / cl;
-  const size_t smem = sizeof(PcSmem) + (size_t)R * PC_IB * sizeof(float);
-  cudaError_t e = allow_max_smem((const void*)panel_cluster_kernel);
+  cudaError_t e = pc_prepare<T>();
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute((const void*)panel_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
-  PcParams P;
   P.A = Wkk;
   P.ld = ldw;
   P.m = m;
   P.w = w;
-  P.R = R;
   P.kabs = kabs;
   P.ipiv = ipiv;
   P.info = info;
   P.status = status;
   P.perm = perm;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cl);
-  cfg.blockDim = dim3(PC_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cl;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, panel_cluster_kernel, P);
+  const cudaLaunchConfig_t cfg = pc_launch<T>(cl, nt, smem, st, at);
+  return cudaLaunchKernelEx(&cfg, panel_cluster_kernel<T>, P);
 }
 
-// Whether a cluster of `cl` such CTAs can be placed on this device.
-bool panel_cluster_available(int m, int w) {
-  const int cl = panel_cluster_size(m, w);
-  if (cl < 0) return false;
-  static std::mutex mu;
-  static int known[PC_CLMAX + 1] = {};  // 0 unknown, 1 yes, -1 no
-  std::lock_guard<std::mutex> lk(mu);
-  if (known[cl] == 0) {
-    allow_max_smem((const void*)panel_cluster_kernel);
-    cudaFuncSetAttribute((const void*)panel_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    const int R = PC_RPT * PC_THREADS;  // the largest shared-memory need
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cl);
-    cfg.blockDim = dim3(PC_THREADS);
-    cfg.dynamicSmemBytes = sizeof(PcSmem) + (size_t)R * PC_IB * sizeof(float);
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = cl;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, (const void*)panel_cluster_kernel, &cfg);
-    if (e != cudaSuccess) cudaGetLastError();
-    known[cl] = (e == cudaSuccess && n > 0) ? 1 : -1;
-  }
-  return known[cl] > 0;
-}
+#define GB_INST(T)                                                                                            \
+  template bool panel_cluster_fits<T>(int, int, const DevInfo&);                                              \
+  template cudaError_t launch_panel_cluster<T>(T*, int64_t, int, int, int, int*, int*, int*, int*,            \
+                                               const DevInfo&, cudaStream_t);
+GB_INST(double)
+GB_INST(float)
+#undef GB_INST
 
 }  // namespace gb
