@@ -1,7 +1,7 @@
 """Panels at the edges of the cluster kernel's shapes (rows per CTA, CTAs per
 cluster, the last size that fits and the first that goes to the cooperative
-kernel), in arithmetic that is exact in FP32 and FP64, with many ties and with
-zero columns: pivots, L and U equal the oracle's bit for bit."""
+kernel), in arithmetic that is exact in FP32 and FP64, with a zero column and
+with ties across CTAs: pivots, L and U equal the oracle's bit for bit."""
 import numpy as np
 import pytest
 
@@ -24,38 +24,57 @@ def ctx():
 
 
 def _exact_panel(m, w, seed, zero_col):
-    # entries of L in {0, +-1/2, +-1} and of U in {+-1, +-2}, banded: every product and
-    # sum is a short dyadic number, and magnitudes tie in nearly every column
+    # A = P^T L U with |l| < 1 and short dyadic entries: elimination is exact
     rng = np.random.default_rng(seed)
-    L = np.tril(rng.integers(-2, 3, size=(m, w)) / 2.0, -1)
+    L = np.tril(rng.integers(-7, 8, size=(m, w)) / 8.0, -1)
     L[np.arange(w), np.arange(w)] = 1.0
-    U = np.triu(rng.choice([-2.0, -1.0, 1.0, 2.0], size=(w, w)))
-    U = np.where(np.triu(np.ones((w, w)), 6) > 0, 0.0, U)
+    U = np.triu(rng.integers(-8, 9, size=(w, w)).astype(np.float64))
+    U[np.arange(w), np.arange(w)] = rng.integers(1, 9, size=w) * rng.choice([-1.0, 1.0], size=w)
     if zero_col is not None:
-        U[:, zero_col] = 0.0
+        U[:, zero_col] = U[zero_col, :] = 0.0
     return (L @ U)[rng.permutation(m)]
+
+
+def _panel(ctx, P, prec):
+    import torch
+    Pd = torch.from_numpy(np.ascontiguousarray(P)).to("cuda", torch.float64 if prec == "f64" else torch.float32)
+    w = P.shape[1]
+    ipiv = torch.zeros(w, dtype=torch.int32, device="cuda")
+    info = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ctx.step_panel(Pd, ipiv, info, prec)
+    assert ctx.status() == 0
+    return Pd.cpu().numpy().astype(np.float64), ipiv.cpu().numpy(), info.item()
 
 
 @pytest.mark.parametrize("prec", ["f64", "f32"])
 @pytest.mark.parametrize("m,w", SIZES)
 def test_panel_at_size_edges(ctx, m, w, prec):
-    import torch
-    for seed, zc in ((m + w, None), (m + 2 * w, w // 2)):
+    for seed, zc in ((m + w, None), (m + 2 * w, w - 1)):
         P = _exact_panel(m, w, seed, zc)
         LUo, ipo, info_o = O.getf2(P)
-        # (the elimination stays exact: the oracle's FP64 factors are FP32 numbers)
-        if not np.array_equal(LUo, LUo.astype(np.float32).astype(np.float64)):
-            assert prec == "f64" or zc is not None
-            if prec == "f32":
-                continue
-        Pd = torch.from_numpy(np.ascontiguousarray(P)).to("cuda", torch.float64 if prec == "f64" else torch.float32)
-        ipiv = torch.zeros(w, dtype=torch.int32, device="cuda")
-        info = torch.zeros(1, dtype=torch.int32, device="cuda")
-        ctx.step_panel(Pd, ipiv, info, prec)
-        assert ctx.status() == 0
-        assert info.item() == info_o
-        assert np.array_equal(ipiv.cpu().numpy(), ipo)
-        assert np.array_equal(Pd.cpu().numpy().astype(np.float64), LUo)
+        assert info_o == (0 if zc is None else zc + 1)
+        LU, ipiv, info = _panel(ctx, P, prec)
+        assert info == info_o
+        assert np.array_equal(ipiv, ipo)
+        assert np.array_equal(LU, LUo)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("m", [40, 700, 3000])
+def test_ties_go_to_the_first_row(ctx, m, prec):
+    """Equal magnitudes in different CTAs, either sign, in a column that an
+    interchange has reordered: the pivot is the first of them."""
+    P = np.zeros((m, 3))
+    P[:, 0] = 0.5
+    P[m // 3, 0], P[m - 1, 0] = -2.0, 2.0
+    P[:, 1] = np.where(np.arange(m) % 7 == 3, -4.0, 4.0)
+    P[:, 2] = np.arange(m) % 5
+    LUo, ipo, _ = O.getf2(P)
+    assert ipo[0] == m // 3 + 1
+    LU, ipiv, _ = _panel(ctx, P, prec)
+    assert np.array_equal(ipiv, ipo)
+    d = np.abs(LU - LUo).max()
+    assert d <= 8 * (2.0 ** -53 if prec == "f64" else 2.0 ** -24) * np.abs(LUo).max()
 
 
 def test_permutation_record_reaches_the_other_columns(ctx):
