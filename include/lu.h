@@ -35,7 +35,9 @@ extern "C" {
 #endif
 
 /* Factor precision.  LU_F64: FP64 panel, FP64 trailing update (the plain
- * FP64 solve).  LU_BF16 / LU_FP16: FP32 working matrix and panel, trailing
+ * FP64 solve; large updates run as certified split products, see
+ * LU_FACTOR_OZAKI: an element whose split error bound would exceed the FP64
+ * dot product's, k 2^-53 sum_k |a b|, is updated on the FP64 CUDA cores).  LU_BF16 / LU_FP16: FP32 working matrix and panel, trailing
  * update on the tensor cores with BF16 / FP16 operands and FP32 accumulation;
  * solutions are brought to FP64 accuracy by lu_refine.  LU_F32: FP32 panel and
  * FP32 trailing update on the CUDA cores. */
@@ -116,10 +118,10 @@ int lu_factor(lu_ctx ctx, int n, const double *dA, int lda, lu_prec prec, int nb
  * C -= L21 U12 (section "Base Implementation", the inner blocks) runs on the
  * BF16 tensor cores by error-free splitting (Ozaki scheme): each operand row
  * or column is scaled by a power of two and cut into 8 slices of 7-bit
- * integers, the 36 slice products with p + q <= 7 are exact in the FP32
+ * integers (balanced digits), the 36 slice products with p + q <= 7 are exact in the FP32
  * accumulator, and they are combined exactly in 64-bit integers before one
  * FP64 rounding.  The error of an update element C - sum_k a b is below
- * 2^-53 * ((1.13 k + 4) * 2^(e_i + f_j) + sum_k |a b| + |result|), with 2^e_i and
+ * 2^-53 * ((0.35 k + 4) * 2^(e_i + f_j) + sum_k |a b| + |result|), with 2^e_i and
  * 2^f_j the powers of two just above the largest |L21| of row i and |U12| of
  * column j: the order of an FP64 dot product's error bound.  Non-finite
  * operands fail with LU_ERANGE. */

@@ -11,14 +11,17 @@
 // tcgen05 has no FP64 kind.
 //
 // Splitting.  Row i of A is scaled by 2^-e_i (2^e_i the power of two just
-// above its largest |a|) and cut into S = 8 slices of 7-bit integers d_p:
-//   a = 2^e_i * sum_p d_p 2^(-7(p+1))  + (remainder below 2^(e_i - 56)).
+// above its largest |a|), rounded to 56 bits and cut into S = 8 slices of
+// balanced base-128 digits d_p:
+//   a = 2^e_i * sum_p d_p 2^(-7(p+1))  + (remainder at most 2^(e_i - 57)).
 // Column j of B likewise (2^f_j, slices g_q).  Every slice is an integer in
-// [-127, 127], exact in BF16.
+// [-64, 63], the leading one in [-128, 128], exact in BF16.  Balanced digits
+// keep the dropped products small and of either sign: digits of one sign
+// (truncation) made them add up within each element.
 //
 // Products.  For each slice pair (p, q) with t = p + q <= S - 1 (36 pairs) the
 // tensor cores form G = sum_k d_p(i,k) g_q(k,j) over the full k <= 256: an
-// integer of magnitude < 256 * 127^2 < 2^22, exact in the FP32 accumulator.
+// integer of magnitude at most 256 * 128^2 = 2^22, exact in the FP32 accumulator.
 //
 // Combination, exact and in integers.  G + 1.5 * 2^23 is exact in FP32 and
 // its bit pattern is 0x4B400000 + G; the epilogue adds that pattern, shifted
@@ -30,8 +33,9 @@
 // one in the subtraction.
 //
 // Error of I * 2^(e_i + f_j - 54) against the exact sum of products, in units
-// of 2^-53 * 2^(e_i + f_j): dropped pairs (t >= 8) < 0.87 k, splitting
-// remainders < 0.25 k, rounded shifts <= 3.75; so below (1.13 k + 4).  The
+// of 2^-53 * 2^(e_i + f_j): dropped pairs (t >= 8) < 0.222 k (seven pairs of at
+// most 64^2 2^-70 for t = 8, a 128th of that beyond), splitting remainders
+// < 0.126 k, rounded shifts <= 3.82; so below (0.35 k + 4).  The
 // conversion adds at most 2^-53 sum_k |a b|, the subtraction 2^-53 |result|:
 // the order of the rounding error bound of a k-term FP64 dot product.
 //
@@ -51,7 +55,20 @@
 // a tile then takes the products of slices 0 and 4 only (12 instead of 36),
 // each epilogue warp weights its quarter by that quarter's slice order, and
 // the four quarters' exact partial sums are added before the FP64 update,
-// which every quarter applies to a quarter of the columns.  Every mbarrier
+// which every quarter applies to a quarter of the columns.
+//
+// Certified update (the plain FP64 factorizations).  The bound above is in
+// terms of the lines' largest elements; an FP64 dot product's is in terms of
+// sum_k |a b|, which badly scaled rows can leave far below.  The certified
+// form therefore takes one more product first, of the leading digits'
+// magnitudes (a ninth slice of each operand): G = sum_k |d_0 g_0| gives
+// sum_k |a b| >= G 2^(e_i + f_j - 14), so G >= (0.35 + 4 / 64) 2^14 makes the
+// bound at most k 2^-53 sum_k |a b|, the dot product's own (k >= 64).  A block of 32
+// rows x 64 columns with an element below that is left alone and listed, and
+// gemm_list_kernel updates the listed blocks in plain FP64.  When nearly every
+// block of an update failed, the rest of the factorization goes to that kernel
+// whole (a device flag, which the split and product kernels read first).
+// Every mbarrier
 // wait is bounded; on timeout the kernel raises ST_TIMEOUT, lets issued copies
 // and MMAs land, frees TMEM and returns.
 #include <cuda_bf16.h>
@@ -66,7 +83,10 @@ namespace gb {
 
 constexpr int OZ_S = 8;        // slices per operand
 constexpr int OZ_BITS = 7;     // bits per slice
-constexpr int OZ_KMAX = 256;   // exactness bound on k (k * 127^2 < 2^22)
+constexpr int OZ_KMAX = 256;   // exactness bound on k (k * 128^2 <= 2^22)
+constexpr int OZ_MAG = OZ_S;   // the ninth slice of a certified update: magnitudes of slice 0
+constexpr float OZ_CERT_MIN = 6759.0f;  // (0.35 + 4 / 64) 2^14, rounded up
+constexpr int OZ_ZERO_LINE = -(1 << 20);  // exponent that marks an all-zero line
 constexpr int OZ_F = 40;       // fraction bits of the integer sum below the t = 0 term
 constexpr int OZ_BM = 128, OZ_BN = 128, OZ_BK = 64;
 constexpr int OZ_CHUNK = OZ_BM * OZ_BK * 2;          // 16 KB: one 128 x 64 BF16 box (A or B)
@@ -86,35 +106,50 @@ constexpr size_t OZ_SMEM = 1024 + 2 * (size_t)OZ_ABUF + (size_t)OZ_BSTAGES * OZ_
 constexpr uint32_t OZ_MAGIC_BITS = 0x4B400000u;  // bit pattern of 1.5 * 2^23
 constexpr float OZ_MAGIC = 12582912.0f;
 
-static_assert(OZ_KMAX * 127 * 127 < (1 << 22), "a slice-pair product must stay below 2^22");
+static_assert(OZ_KMAX * 128 * 128 <= (1 << 22), "a slice-pair product must stay within 2^22");
+static_assert(OZ_S == 8 && OZ_F == 40 && OZ_BITS == 7, "oz_acc32's rounding of the two smallest orders");
 static_assert(OZ_SMEM <= 232448, "shared memory per CTA");
 
 // ------------------------------------------------------------ splitting
-// The slices of x with |x| < 2^e: d_p = trunc(128 r_p), r_{p+1} = 128 r_p - d_p,
-// r_0 = x 2^-e.  Every step is exact in FP64, so d_p is digit p of the base-128
-// expansion of |x| 2^-e with x's sign; it is taken here from the bit pattern
-// (integer operations only: GB300's FP64 rate would make the FP64 form the
-// cost of the split).  The 56-bit magnitude M = floor(|x| 2^(56 - e)) holds the
-// eight digits, d_p = (M >> (49 - 7p)) & 127.
+// The slices of x with |x| < 2^e: the balanced base-128 digits of |x| 2^-e
+// rounded to 56 bits, with x's sign.  They are taken from the bit pattern
+// (integer operations: GB300's FP64 rate would make the FP64 form the cost of
+// the split).  M = |x| 2^(56 - e) rounded to the nearest integer, at most 2^56;
+// adding 64 in each of the seven lower digit places turns the digits of the
+// sum into the balanced ones plus 64.
 __device__ __forceinline__ uint64_t oz_fixed56(uint64_t bits, int e) {
   const int field = (int)((bits >> 52) & 0x7ff);
   uint64_t mant = bits & 0xfffffffffffffull;
   if (field) mant |= 1ull << 52;
   const int sh = (field ? field : 1) - 1075 + 56 - e;  // |x| = mant 2^(field' - 1075)
   if (sh >= 0) return sh < 64 ? mant << sh : 0ull;
-  return -sh < 64 ? mant >> (-sh) : 0ull;
+  return -sh < 64 ? ((mant >> (-sh - 1)) + 1) >> 1 : 0ull;
 }
-
-// BF16 pattern of the integer sign * d, 0 <= d <= 127 (exact: <= 7 significant bits)
-__device__ __forceinline__ uint32_t oz_bf16_digit(uint32_t d, uint32_t sign) {
-  if (d == 0) return 0u;
-  const int k = 31 - __clz(d);  // leading bit
-  return sign | ((127u + (uint32_t)k) << 7) | ((d << (7 - k)) & 0x7fu);
+constexpr uint64_t oz_places64() {
+  uint64_t h = 0;
+  for (int p = 1; p < OZ_S; ++p) h |= 64ull << (7 * (OZ_S - 1 - p));
+  return h;
 }
+constexpr uint64_t OZ_H = oz_places64();
 
-// e with |x| < 2^e <= 2|x| for the largest |x| of a line, from its pattern (0 for 0)
+// BF16 patterns (in the upper half) of digit p of the sum Mh = M + OZ_H, and of
+// the magnitude M's leading digit; sign = x's sign bit.  An integer of at most
+// eight bits under the exponent of 2^23, less the offset, is the digit in FP32,
+// whose upper half is exact.
+__device__ __forceinline__ uint32_t oz_digit(uint64_t Mh, int p, uint32_t sign) {
+  const uint32_t u = p == 0 ? (uint32_t)(Mh >> 49) : (uint32_t)(Mh >> (49 - OZ_BITS * p)) & 127u;
+  const float f = __uint_as_float(0x4B000000u | u) - (p == 0 ? 8388608.0f : 8388608.0f + 64.0f);
+  return __float_as_uint(f) ^ sign;
+}
+__device__ __forceinline__ uint32_t oz_lead(uint64_t M) {
+  return __float_as_uint(__uint_as_float(0x4B000000u | (uint32_t)(M >> 49)) - 8388608.0f);
+}
+__device__ __forceinline__ uint32_t oz_pack(uint32_t lo, uint32_t hi) { return __byte_perm(lo, hi, 0x7632); }
+
+// e with |x| < 2^e <= 2|x| for the largest |x| of a line, from its pattern
+// (every digit of an all-zero line is 0, whatever its exponent)
 __device__ __forceinline__ int oz_expo(uint64_t absbits) {
-  if (absbits == 0) return 0;
+  if (absbits == 0) return OZ_ZERO_LINE;
   const int field = (int)(absbits >> 52);
   if (field) return field - 1022;
   return (63 - __clzll((long long)absbits)) - 1074 + 1;  // subnormal
@@ -124,7 +159,9 @@ __device__ __forceinline__ int oz_expo(uint64_t absbits) {
 // One warp per row; a lane takes element pairs (2 lane + 64 u, + 1).
 __global__ void __launch_bounds__(256) oz_split_rows_kernel(const double* __restrict__ A, int64_t lda, int m, int k,
                                                             int kpad, __nv_bfloat16* __restrict__ As,
-                                                            int* __restrict__ ea, int* status) {
+                                                            int* __restrict__ ea, int* status, int mag,
+                                                            const int* off) {
+  if (off != nullptr && __ldcg(off)) return;
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (i >= m) return;
@@ -160,14 +197,11 @@ __global__ void __launch_bounds__(256) oz_split_rows_kernel(const double* __rest
     if (c >= kpad) break;
     const uint64_t M0 = zero ? 0ull : oz_fixed56(v[u][0], e);
     const uint64_t M1 = zero ? 0ull : oz_fixed56(v[u][1], e);
-    const uint32_t s0 = (uint32_t)(v[u][0] >> 48) & 0x8000u, s1 = (uint32_t)(v[u][1] >> 48) & 0x8000u;
+    const uint32_t s0 = (uint32_t)(v[u][0] >> 32) & 0x80000000u, s1 = (uint32_t)(v[u][1] >> 32) & 0x80000000u;
 #pragma unroll
-    for (int p = 0; p < OZ_S; ++p) {
-      const int sh = 49 - OZ_BITS * p;
-      const uint32_t w = oz_bf16_digit((uint32_t)(M0 >> sh) & 127u, s0) |
-                         (oz_bf16_digit((uint32_t)(M1 >> sh) & 127u, s1) << 16);
-      out[(((int64_t)p * m + i) * kpad + c) >> 1] = w;
-    }
+    for (int p = 0; p < OZ_S; ++p)
+      out[(((int64_t)p * m + i) * kpad + c) >> 1] = oz_pack(oz_digit(M0 + OZ_H, p, s0), oz_digit(M1 + OZ_H, p, s1));
+    if (mag) out[(((int64_t)OZ_MAG * m + i) * kpad + c) >> 1] = oz_pack(oz_lead(M0), oz_lead(M1));
   }
 }
 
@@ -175,7 +209,9 @@ __global__ void __launch_bounds__(256) oz_split_rows_kernel(const double* __rest
 // fb[j] = f_j.  CTA = 32 columns; 64-row blocks go through shared memory.
 __global__ void __launch_bounds__(256) oz_split_cols_kernel(const double* __restrict__ B, int64_t ldb, int k, int n,
                                                             int kpad, __nv_bfloat16* __restrict__ Bs,
-                                                            int* __restrict__ fb, int* status) {
+                                                            int* __restrict__ fb, int* status, int mag,
+                                                            const int* off) {
+  if (off != nullptr && __ldcg(off)) return;
   __shared__ uint64_t tile[OZ_BK][33];
   __shared__ uint64_t red[8][32];
   __shared__ int fe[32];
@@ -217,14 +253,12 @@ __global__ void __launch_bounds__(256) oz_split_cols_kernel(const double* __rest
       const uint64_t x0 = tile[2 * lane][c], x1 = tile[2 * lane + 1][c];
       const uint64_t M0 = e == ZERO_COL ? 0ull : oz_fixed56(x0, e);
       const uint64_t M1 = e == ZERO_COL ? 0ull : oz_fixed56(x1, e);
-      const uint32_t s0 = (uint32_t)(x0 >> 48) & 0x8000u, s1 = (uint32_t)(x1 >> 48) & 0x8000u;
+      const uint32_t s0 = (uint32_t)(x0 >> 32) & 0x80000000u, s1 = (uint32_t)(x1 >> 32) & 0x80000000u;
 #pragma unroll
-      for (int q = 0; q < OZ_S; ++q) {
-        const int sh = 49 - OZ_BITS * q;
-        const uint32_t w = oz_bf16_digit((uint32_t)(M0 >> sh) & 127u, s0) |
-                           (oz_bf16_digit((uint32_t)(M1 >> sh) & 127u, s1) << 16);
-        out[(((int64_t)q * n + jj) * kpad + r0 + 2 * lane) >> 1] = w;
-      }
+      for (int q = 0; q < OZ_S; ++q)
+        out[(((int64_t)q * n + jj) * kpad + r0 + 2 * lane) >> 1] =
+            oz_pack(oz_digit(M0 + OZ_H, q, s0), oz_digit(M1 + OZ_H, q, s1));
+      if (mag) out[(((int64_t)OZ_MAG * n + jj) * kpad + r0 + 2 * lane) >> 1] = oz_pack(oz_lead(M0), oz_lead(M1));
     }
     __syncthreads();
   }
@@ -244,6 +278,10 @@ struct OzParams {
   const int* fb;   // column exponents f_j of this update's columns
   int vec_ok;      // C rows 16-byte aligned (vector loads and stores)
   int stacked;     // m == 32: an A box holds four consecutive slices (see the kernel)
+  int cert;        // certified update: the magnitude product first, failing blocks listed
+  const int* off;  // certified update: the device flag that sends every block to gemm_list_kernel
+  int* cnt;        // ... the number of listed blocks
+  int* list;       // ... the blocks: (row / 32) * ceil(n / 64) + column / 64
   long long* scratch;  // per CTA: the previous tile's sums (OZ_BM x OZ_BN)
   uint32_t idesc;
   int* status;
@@ -274,10 +312,14 @@ __device__ __forceinline__ void oz_add64(uint32_t& l, uint32_t& h, uint32_t xl, 
 // (hi:lo)[j] += pattern of (G_j + 1.5 * 2^23) shifted by 40 - 7t (64-bit sums
 // kept as two 32-bit words).  t <= 1 touches the high word only; t = 6, 7 are
 // right shifts rounded to nearest: half a unit of the shifted result rides in
-// the float constant (G + 1.5 * 2^23 + 2^(r-1) is still exact), and since the
+// the float constant (G + 1.5 * 2^23 + half is still exact), and since the
 // constant's pattern has 22 low zero bits, the shifted pattern is the shifted
-// constant plus floor((G + 2^(r-1)) / 2^r).
-__device__ __forceinline__ void oz_acc32(uint32_t* lo, uint32_t* hi, const uint32_t* v, int t) {
+// constant plus floor((G + half) / 2^r).  Halves at t = 6 (a shift by two) are
+// frequent, and rounding them one way in every pair would add the same error to
+// every element of every update: pairs with an even A slice p round them up,
+// odd ones down, and the fourth even pair's eighth of a unit is taken back in
+// pair (7, 0).
+__device__ __forceinline__ void oz_acc32(uint32_t* lo, uint32_t* hi, const uint32_t* v, int t, int p) {
   const int sh = OZ_F - OZ_BITS * t;
   if (sh >= 32) {
     const uint32_t mul = 1u << (sh - 32);
@@ -292,7 +334,8 @@ __device__ __forceinline__ void oz_acc32(uint32_t* lo, uint32_t* hi, const uint3
     }
   } else {
     const int r = -sh;
-    const float M = OZ_MAGIC + (float)(1 << (r - 1));
+    const int half = t == 6 ? (1 << (r - 1)) - (p & 1) : (p == 7 ? 192 : 1 << (r - 1));
+    const float M = OZ_MAGIC + (float)half;
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
       const uint32_t b = __float_as_uint(__uint_as_float(v[j]) + M);
@@ -326,6 +369,7 @@ __device__ __forceinline__ double oz_sub(double c, long long I, int E) {
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, OzParams P) {
   extern __shared__ unsigned char smem_raw[];
+  if (P.cert && __ldcg(P.off)) return;
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char* gbase = smem_raw + (base - raw);
@@ -352,7 +396,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   // four 32-row quarters, so one product with B slice q serves the pairs
   // (p + g, q), g = 0..3: the tile walks p = 0, 4 (12 products instead of 36)
   // and each epilogue warp weights its quarter by that quarter's slice order.
-  const int pstep = P.stacked ? 4 : 1;
+  // A certified tile starts with the magnitude slices' product.
+  // The tile's A slices in order, i = 0 .. na - 1, and each one's B slices:
+  const int na = P.cert ? OZ_S + 1 : (P.stacked ? 2 : OZ_S);
+  auto a_slice = [&](int i) { return P.cert ? (i == 0 ? OZ_MAG : i - 1) : (P.stacked ? 4 * i : i); };
+  auto b_count = [&](int p) { return p == OZ_MAG ? 1 : OZ_S - p; };
 
   if (threadIdx.x == 0) {
     for (int a = 0; a < 2; ++a) {
@@ -398,7 +446,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       uint32_t ph = 0, abph = 0;
       bool ok = true;
       // A slices load one slice ahead, into the buffer the MMA released last:
-      // slice (tile, p + pstep) is issued once the B chunks of (p, q = 0) are.
+      // the next slice is issued once the B chunks of (p, q = 0) are.
       auto load_a = [&](int tile, int p) -> bool {
         if (!mbar_wait(bar_aempty + 8 * ab, abph ^ 1u, P.status, abort_flag)) return false;
         int tm, tn_unused;
@@ -414,19 +462,21 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         }
         return true;
       };
-      if ((int)blockIdx.x < ntiles) ok = load_a(blockIdx.x, 0);
+      if ((int)blockIdx.x < ntiles) ok = load_a(blockIdx.x, a_slice(0));
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         int tm_unused, tn;
         oz_tile(t, P.tiles_m, P.tiles_n, tm_unused, tn);
-        for (int p = 0; p < OZ_S && ok; p += pstep) {
-          for (int q = 0; q < OZ_S - p && ok; ++q) {
+        for (int ai = 0; ai < na && ok; ++ai) {
+          const int p = a_slice(ai);
+          for (int q = 0; q < b_count(p) && ok; ++q) {
+            const int bq = p == OZ_MAG ? OZ_MAG : q;
             for (int kc = 0; kc < P.kchunks; ++kc) {
               if (!mbar_wait(bar_bempty + 8 * s, ph ^ 1u, P.status, abort_flag)) {
                 ok = false;
                 break;
               }
               mbar_expect_tx(bar_bfull + 8 * s, OZ_CHUNK);
-              tma_load_2d(sB + s * OZ_CHUNK, &tmB, kc * OZ_BK, q * P.b_rows + P.b_col0 + tn * OZ_BN,
+              tma_load_2d(sB + s * OZ_CHUNK, &tmB, kc * OZ_BK, bq * P.b_rows + P.b_col0 + tn * OZ_BN,
                           bar_bfull + 8 * s);
               bpar[s] = (int)ph;
               if (++s == OZ_BSTAGES) {
@@ -435,10 +485,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
               }
             }
             if (ok && q == 0) {
-              if (p + pstep < OZ_S)
-                ok = load_a(t, p + pstep);
+              if (ai + 1 < na)
+                ok = load_a(t, a_slice(ai + 1));
               else if (t + (int)gridDim.x < ntiles)
-                ok = load_a(t + gridDim.x, 0);
+                ok = load_a(t + gridDim.x, a_slice(0));
             }
           }
         }
@@ -466,14 +516,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       uint32_t ph = 0, abph = 0, tph = 0;
       bool ok = true, issued = false;
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        for (int p = 0; p < OZ_S && ok; p += pstep) {
+        for (int ai = 0; ai < na && ok; ++ai) {
+          const int p = a_slice(ai);
           if (!mbar_wait(bar_afull + 8 * ab, abph, P.status, abort_flag)) {
             ok = false;
             break;
           }
           tc_fence_after();
           const uint32_t a0 = sA + ab * OZ_ABUF;
-          for (int q = 0; q < OZ_S - p && ok; ++q) {
+          for (int q = 0; q < b_count(p) && ok; ++q) {
             if (!mbar_wait(bar_tempty + 8 * acc, tph ^ 1u, P.status, abort_flag)) {
               ok = false;
               break;
@@ -598,7 +649,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       int tm, tn;
       oz_tile(t, P.tiles_m, P.tiles_n, tm, tn);
       const int row = P.stacked ? lane : tm * OZ_BM + quarter * 32 + lane;
-      const bool rok = row < P.m;
+      bool rok = row < P.m;
       const int col0 = tn * OZ_BN + half * 64;
       double* crow = P.C + (int64_t)row * P.ldc + col0;
       uint32_t lo[64], hi[64];
@@ -606,14 +657,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       for (int j = 0; j < 64; ++j) lo[j] = hi[j] = 0u;
       unsigned long long corr = 0ull;
       int pi = 0;  // slice pair index within the tile
-      for (int p = 0; p < OZ_S && ok; p += pstep) {
+      for (int ai = 0; ai < na && ok; ++ai) {
+        const int p = a_slice(ai);
         if (p == (P.stacked ? 4 : 6) && rok) {
           // bring this tile's C segment into L2 for its deferred update
 #pragma unroll
           for (int c = 0; c < 64; c += 16)
             if (col0 + c < P.n) asm volatile("prefetch.global.L2::evict_last [%0];" ::"l"(crow + c));
         }
-        for (int q = 0; q < OZ_S - p; ++q, ++pi) {
+        for (int q = 0; q < b_count(p); ++q, ++pi) {
           int okw = 1;
           if (lane == 0) okw = mbar_wait(bar_tfull + 8 * acc, tph, P.status, abort_flag) ? 1 : 0;
           okw = __shfl_sync(0xffffffffu, okw, 0);
@@ -623,20 +675,50 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           }
           tc_fence_after();
           const int tt = p + gq + q;
-          if (tt < OZ_S) {
+          if (p == OZ_MAG) {
+            // G of this warp's 32 rows x 64 columns: all of them large enough, or
+            // the block goes to the list (all-zero lines pass: their part is 0)
+            const uint32_t taddr = tmem_base + lane_addr + (uint32_t)(acc * OZ_BN + half * 64);
+            const bool zrow = rok && P.ea[row] == OZ_ZERO_LINE;
+            bool small = false;
+#pragma unroll 1
+            for (int h = 0; h < 64; h += 32) {
+              uint32_t v[32];
+              TMEM_LD_X16(taddr + h, v);
+              TMEM_LD_X16(taddr + h + 16, (v + 16));
+              tmem_wait_ld();
+              const int nc = rok && !zrow ? P.n - col0 - h : 0;
+              bool low = false;
+#pragma unroll
+              for (int j = 0; j < 32; ++j) low |= j < nc && __uint_as_float(v[j]) < OZ_CERT_MIN;
+              if (low) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                  if (j < nc && __uint_as_float(v[j]) < OZ_CERT_MIN) small |= P.fb[col0 + h + j] != OZ_ZERO_LINE;
+              }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_tempty + 8 * acc);
+            if (__any_sync(0xffffffffu, small)) {
+              if (lane == 0)
+                P.list[atomicAdd(P.cnt, 1)] = (tm * (OZ_BM / 32) + quarter) * ((P.n + 63) / 64) + tn * (OZ_BN / 64) + half;
+              rok = false;
+            }
+          } else if (tt < OZ_S) {
             const uint32_t taddr = tmem_base + lane_addr + (uint32_t)(acc * OZ_BN + half * 64);
             uint32_t v[32];
             TMEM_LD_X16(taddr, v);
             TMEM_LD_X16(taddr + 16, (v + 16));
             tmem_wait_ld();
-            oz_acc32(lo, hi, v, tt);
+            oz_acc32(lo, hi, v, tt, p + gq);
             TMEM_LD_X16(taddr + 32, v);
             TMEM_LD_X16(taddr + 48, (v + 16));
             tmem_wait_ld();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_tempty + 8 * acc);
-            oz_acc32(lo + 32, hi + 32, v, tt);
+            oz_acc32(lo + 32, hi + 32, v, tt, p + gq);
             corr += oz_corr(tt);
           } else {
             // a stacked quarter whose pair order is past the last kept one
@@ -722,9 +804,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 // ------------------------------------------------------------ host side
 static size_t al1k(size_t b) { return (b + 1023) / 1024 * 1024; }
 
-size_t ozaki_ws_bytes(int m, int n, int k, int sm_count) {
+size_t ozaki_ws_bytes(int m, int n, int k, int sm_count, bool cert) {
   const size_t kpad = (size_t)cdiv(k > 0 ? k : 1, OZ_BK) * OZ_BK;
-  return al1k((size_t)OZ_S * m * kpad * 2) + al1k((size_t)OZ_S * n * kpad * 2) + al1k((size_t)m * 4) +
+  const size_t sl = OZ_S + (cert ? 1 : 0);
+  return al1k(sl * m * kpad * 2) + al1k(sl * n * kpad * 2) + al1k((size_t)m * 4) +
          al1k((size_t)n * 4) + (size_t)sm_count * OZ_BM * OZ_BN * 8;
 }
 
@@ -735,14 +818,15 @@ struct OzLayout {
   int kpad;
 };
 
-static OzLayout oz_layout(void* ws, int m, int n, int k) {
+static OzLayout oz_layout(void* ws, int m, int n, int k, bool cert) {
   OzLayout L;
+  const size_t sl = OZ_S + (cert ? 1 : 0);
   L.kpad = (int)cdiv(k, OZ_BK) * OZ_BK;
   char* p = (char*)ws;
   L.As = (__nv_bfloat16*)p;
-  p += al1k((size_t)OZ_S * m * L.kpad * 2);
+  p += al1k(sl * m * L.kpad * 2);
   L.Bs = (__nv_bfloat16*)p;
-  p += al1k((size_t)OZ_S * n * L.kpad * 2);
+  p += al1k(sl * n * L.kpad * 2);
   L.ea = (int*)p;
   p += al1k((size_t)m * 4);
   L.fb = (int*)p;
@@ -752,14 +836,16 @@ static OzLayout oz_layout(void* ws, int m, int n, int k) {
 }
 
 cudaError_t ozaki_split(const double* A, int64_t lda, const double* B, int64_t ldb, int m, int n, int k, void* ws,
-                        int* status, cudaStream_t st) {
+                        int* status, cudaStream_t st, const OzCert* cert) {
   if (m <= 0 || n <= 0 || k <= 0) return cudaSuccess;
   if (k > OZ_KMAX || ws == nullptr) return cudaErrorInvalidValue;
-  const OzLayout L = oz_layout(ws, m, n, k);
-  oz_split_rows_kernel<<<(unsigned)cdiv(m, 8), 256, 0, st>>>(A, lda, m, k, L.kpad, L.As, L.ea, status);
+  const OzLayout L = oz_layout(ws, m, n, k, cert != nullptr);
+  const int mag = cert != nullptr;
+  const int* off = cert ? cert->off : nullptr;
+  oz_split_rows_kernel<<<(unsigned)cdiv(m, 8), 256, 0, st>>>(A, lda, m, k, L.kpad, L.As, L.ea, status, mag, off);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  oz_split_cols_kernel<<<(unsigned)cdiv(n, 32), 256, 0, st>>>(B, ldb, k, n, L.kpad, L.Bs, L.fb, status);
+  oz_split_cols_kernel<<<(unsigned)cdiv(n, 32), 256, 0, st>>>(B, ldb, k, n, L.kpad, L.Bs, L.fb, status, mag, off);
   return cudaGetLastError();
 }
 
@@ -794,12 +880,13 @@ static bool oz_map(CUtensorMap* map, const void* ptr, int64_t rows, int kpad) {
 }
 
 cudaError_t ozaki_gemm(double* C, int64_t ldc, const void* ws, int m, int n, int k, int col0, int ncols, int* status,
-                       const DevInfo& dev, cudaStream_t st, int max_ctas) {
+                       const DevInfo& dev, cudaStream_t st, int max_ctas, const OzCert* cert) {
   if (m <= 0 || ncols <= 0 || k <= 0) return cudaSuccess;
   if (k > OZ_KMAX || col0 < 0 || col0 + ncols > n || ws == nullptr) return cudaErrorInvalidValue;
-  const OzLayout L = oz_layout(const_cast<void*>(ws), m, n, k);
+  const OzLayout L = oz_layout(const_cast<void*>(ws), m, n, k, cert != nullptr);
+  const int64_t sl = OZ_S + (cert ? 1 : 0);
   CUtensorMap ma, mb;
-  if (!oz_map(&ma, L.As, (int64_t)OZ_S * m, L.kpad) || !oz_map(&mb, L.Bs, (int64_t)OZ_S * n, L.kpad))
+  if (!oz_map(&ma, L.As, sl * m, L.kpad) || !oz_map(&mb, L.Bs, sl * n, L.kpad))
     return cudaErrorInvalidValue;
   cudaError_t e = allow_max_smem((const void*)oz_gemm_kernel);
   if (e != cudaSuccess) return e;
@@ -825,7 +912,11 @@ cudaError_t ozaki_gemm(double* C, int64_t ldc, const void* ws, int m, int n, int
   P.scratch = L.scratch;
   P.idesc = tc_idesc_mn(1u, OZ_BM, OZ_BN);
   P.vec_ok = (((uintptr_t)C & 15u) == 0 && (ldc % 2) == 0) ? 1 : 0;
-  P.stacked = m == 32 ? 1 : 0;  // the slices of a 32-row A are 32 rows apart: four per 128-row box
+  P.cert = cert ? 1 : 0;
+  P.off = cert ? cert->off : nullptr;
+  P.cnt = cert ? cert->cnt : nullptr;
+  P.list = cert ? cert->list : nullptr;
+  P.stacked = m == 32 && !cert ? 1 : 0;  // the slices of a 32-row A are 32 rows apart: four per 128-row box
   P.status = status;
   const int ntiles = P.tiles_m * P.tiles_n;
   int grid = ntiles < dev.sm_count ? ntiles : dev.sm_count;

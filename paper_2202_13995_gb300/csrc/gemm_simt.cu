@@ -97,6 +97,88 @@ cudaError_t launch_gemm_simt(T* C, int64_t ldc, const T* A, int64_t lda, const T
   return cudaGetLastError();
 }
 
+// The blocks that a certified split update left alone (gemm_ozaki.cu):
+// 32 rows x 64 columns of C -= A B each, 2 x 4 elements per thread, bound by
+// FP64 issue like gemm_simt_kernel.  Persistent CTAs walk the list; with none
+// listed (the usual case) the launch costs a few microseconds.
+constexpr int GL_BM = 32, GL_BN = 64, GL_BK = 32;
+
+__global__ void __launch_bounds__(256) gemm_list_kernel(double* __restrict__ C, int64_t ldc,
+                                                        const double* __restrict__ A, int64_t lda,
+                                                        const double* __restrict__ B, int64_t ldb, int m, int n, int k,
+                                                        int* off, int tag, const int* cnt, const int* list) {
+  __shared__ double As[GL_BK][GL_BM + 1];
+  __shared__ double Bs[GL_BK][GL_BN];
+  const int nbn = (n + GL_BN - 1) / GL_BN;
+  const int all = ((m + GL_BM - 1) / GL_BM) * nbn;
+  // (raised by an earlier update, never by this launch's own block 0)
+  const int raised = __ldcg(off);
+  const bool whole = raised != 0 && raised != tag;
+  const int count = whole ? all : min(__ldcg(cnt), all);
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  for (int it = blockIdx.x; it < count; it += gridDim.x) {
+    const int b = whole ? it : list[it];
+    const int m0 = (b / nbn) * GL_BM, n0 = (b % nbn) * GL_BN;
+    double acc[2][4] = {};
+    for (int k0 = 0; k0 < k; k0 += GL_BK) {
+      double ra[GL_BM * GL_BK / 256], rb[GL_BN * GL_BK / 256];
+#pragma unroll
+      for (int q = 0; q < GL_BM * GL_BK / 256; ++q) {
+        const int e = tid + 256 * q, r = m0 + e / GL_BK, c = k0 + e % GL_BK;
+        ra[q] = r < m && c < k ? A[(int64_t)r * lda + c] : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < GL_BN * GL_BK / 256; ++q) {
+        const int e = tid + 256 * q, r = k0 + e / GL_BN, c = n0 + e % GL_BN;
+        rb[q] = r < k && c < n ? B[(int64_t)r * ldb + c] : 0.0;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < GL_BM * GL_BK / 256; ++q) {
+        const int e = tid + 256 * q;
+        As[e % GL_BK][e / GL_BK] = ra[q];
+      }
+#pragma unroll
+      for (int q = 0; q < GL_BN * GL_BK / 256; ++q) {
+        const int e = tid + 256 * q;
+        Bs[e / GL_BN][e % GL_BN] = rb[q];
+      }
+      __syncthreads();
+#pragma unroll 8
+      for (int kk = 0; kk < GL_BK; ++kk) {
+        const double a0 = As[kk][ty], a1 = As[kk][ty + 16];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const double bv = Bs[kk][tx + 16 * j];
+          acc[0][j] = fma(a0, bv, acc[0][j]);
+          acc[1][j] = fma(a1, bv, acc[1][j]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int r = m0 + ty + 16 * i;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = n0 + tx + 16 * j;
+        if (r < m && c < n) C[(int64_t)r * ldc + c] -= acc[i][j];
+      }
+    }
+  }
+  // (the split update costs about a twentieth of the plain one, so it pays
+  // until nearly every block comes here)
+  if (blockIdx.x == 0 && tid == 0 && !whole && (int64_t)count * 10 > (int64_t)all * 9) *off = tag;
+}
+
+cudaError_t launch_gemm_list(double* C, int64_t ldc, const double* A, int64_t lda, const double* B, int64_t ldb, int m,
+                             int n, int k, const OzCert& cert, const DevInfo& dev, cudaStream_t st) {
+  if (m <= 0 || n <= 0 || k <= 0) return cudaSuccess;
+  const int64_t blocks = (int64_t)oz_cert_blocks(m, n);
+  const int grid = (int)(blocks < 4 * dev.sm_count ? blocks : 4 * dev.sm_count);
+  gemm_list_kernel<<<grid, 256, 0, st>>>(C, ldc, A, lda, B, ldb, m, n, k, cert.off, cert.tag, cert.cnt, cert.list);
+  return cudaGetLastError();
+}
+
 template cudaError_t launch_gemm_simt<double>(double*, int64_t, const double*, int64_t, const double*, int64_t, int,
                                               int, int, cudaStream_t);
 template cudaError_t launch_gemm_simt<float>(float*, int64_t, const float*, int64_t, const float*, int64_t, int, int,

@@ -151,6 +151,11 @@ template <typename T>
 cudaError_t launch_gemm_simt(T* C, int64_t ldc, const T* A, int64_t lda, const T* B, int64_t ldb, int m, int n,
                              int k, cudaStream_t st);
 
+// The listed 32 x 64 blocks of C -= A B in FP64 (every block when cert.off is set).
+struct OzCert;
+cudaError_t launch_gemm_list(double* C, int64_t ldc, const double* A, int64_t lda, const double* B, int64_t ldb, int m,
+                             int n, int k, const OzCert& cert, const DevInfo& dev, cudaStream_t st);
+
 // ---------------------------------------------------------------- gemm_tc.cu
 // Operand casts for the tensor-core update (kind 1 = BF16, 2 = FP16):
 //   Aop[i*kpad + t] = L21(i, t)     (K-major, m x k)
@@ -174,11 +179,24 @@ cudaError_t tc_gemm_run(int kind, float* C, int64_t ldc, const void* Aop, const 
 // that runs it); ozaki_gemm then updates columns
 // [col0, col0 + ncols) of the m x n product into C (row-major FP64, column 0
 // of C is column col0 of the product).  Non-finite operands set ST_RANGE.
-size_t ozaki_ws_bytes(int m, int n, int k, int sm_count);
+// With a certificate the update is certified (see gemm_ozaki.cu): blocks of 32
+// rows x 64 columns whose error bound would exceed the FP64 dot product's are
+// left alone and listed (off: the flag that skips the split kernels; cnt, zero
+// at the call: the number listed; list: room for oz_cert_blocks(m, n)), and
+// launch_gemm_list updates them in plain FP64 and raises the flag when more
+// than nine in ten failed.
+struct OzCert {
+  int* off;  // 0, or the tag of the update that raised it
+  int* cnt;
+  int* list;
+  int tag;   // this update's tag, not 0, another for each update that shares off
+};
+inline size_t oz_cert_blocks(int m, int n) { return (size_t)((m + 31) / 32) * (size_t)((n + 63) / 64); }
+size_t ozaki_ws_bytes(int m, int n, int k, int sm_count, bool cert = false);
 cudaError_t ozaki_split(const double* A, int64_t lda, const double* B, int64_t ldb, int m, int n, int k, void* ws,
-                        int* status, cudaStream_t st);
+                        int* status, cudaStream_t st, const OzCert* cert = nullptr);
 cudaError_t ozaki_gemm(double* C, int64_t ldc, const void* ws, int m, int n, int k, int col0, int ncols, int* status,
-                       const DevInfo& dev, cudaStream_t st, int max_ctas = 0);
+                       const DevInfo& dev, cudaStream_t st, int max_ctas = 0, const OzCert* cert = nullptr);
 // M (w x w, row-major) = I - L^-1 for the unit-lower block L (w <= 256), so that
 // the top block solve L^-1 A12 is the split update A12 - M A12.
 cudaError_t launch_unit_lower_inv_comp(const double* L, int64_t ldl, int w, double* M, int64_t ldm, cudaStream_t st);

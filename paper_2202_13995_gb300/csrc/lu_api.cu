@@ -164,6 +164,7 @@ struct lu_fact_s {
   bool ozaki = false;   // FP64 trailing update by error-free splitting
   void* oz_ws = nullptr;
   double* oz_minv = nullptr;  // nb x nb: I - L11^-1 of the current block
+  int* oz_cert = nullptr;     // plain FP64 with certified split updates: flag, counts per step, block list
   int* spec_flag = nullptr;   // diagonal-pivot check flags (SpecArgs), FP32 panels
   void* spec_backup = nullptr;  // n x nb FP32: a checked panel's rows before the check
   void* uinv = nullptr;         // nb x 32: inverses of the diagonal blocks of a block column's U
@@ -427,6 +428,36 @@ static cudaError_t panel_step(lu_fact f, int mode, T* Wkk, int m, int w, int kab
 // SMs; a shared context's (server slots) keep to gemm_ctas.
 static int gemm_cap(lu_ctx c) { return c->gemm_ctas > 0 ? c->gemm_ctas : c->dev.sm_count; }
 
+// The plain FP64 factorization's trailing update: certified split products
+// (gemm_ozaki.cu) for a full block width of at least 64 (below that the
+// certificate's sum is short and fails on dense matrices too) and from
+// kCertRest remaining rows on, where they win over the FP64 CUDA cores (all
+// updates of a factorization: n = 8192, nb = 192, 290 -> 26 ms; n = 2048,
+// nb = 64, 6.0 -> 3.1 ms; n = 600, nb = 64, where two updates lie above the
+// line, 0.7 ms either way); the CUDA cores otherwise.
+constexpr int kCertNb = 64, kCertRest = 384;
+static bool cert_applies(int n, int nb) { return nb >= kCertNb && nb <= 256 && n - nb >= kCertRest; }
+static size_t cert_ints(int n, int nb) { return 1 + (size_t)(n / nb + 1) + oz_cert_blocks(n, n); }
+
+static int update_f64(lu_fact f, double* A22, const double* L21, const double* U12, int rest, int w, int step) {
+  lu_ctx c = f->ctx;
+  cudaStream_t st = c->stream;
+  const int64_t ld = f->ldw;
+  if (f->oz_cert == nullptr || w < kCertNb || rest < kCertRest) {
+    CU_TRY(PHASE(c, PH_GEMM, 1, launch_gemm_simt<double>(A22, ld, L21, ld, U12, ld, rest, rest, w, st)));
+    return LU_OK;
+  }
+  OzCert cert;
+  cert.off = f->oz_cert;
+  cert.cnt = f->oz_cert + 1 + step;
+  cert.list = f->oz_cert + 1 + (f->n / f->nb + 1);
+  cert.tag = step + 1;
+  CU_TRY(PHASE(c, PH_CAST, 2, ozaki_split(L21, ld, U12, ld, rest, rest, w, f->oz_ws, c->d_status, st, &cert)));
+  CU_TRY(PHASE(c, PH_GEMM, 1, ozaki_gemm(A22, ld, f->oz_ws, rest, rest, w, 0, rest, c->d_status, c->dev, st, 0, &cert)));
+  CU_TRY(PHASE(c, PH_GEMM, 1, launch_gemm_list(A22, ld, L21, ld, U12, ld, rest, rest, w, cert, c->dev, st)));
+  return LU_OK;
+}
+
 template <typename T>
 static int factor_loop(lu_fact f) {
   lu_ctx c = f->ctx;
@@ -497,6 +528,11 @@ static int factor_loop(lu_fact f) {
                                                f->oz_ws, c->d_status, st)));
       CU_TRY(PHASE(c, PH_GEMM, 1, ozaki_gemm((double*)A22, ld, f->oz_ws, rest, rest, w, 0, rest, c->d_status, c->dev,
                                               st)));
+      continue;
+    }
+    if constexpr (sizeof(T) == 8) {
+      const int rc = update_f64(f, A22, L21, U12, rest, w, k / nb);
+      if (rc) return rc;
       continue;
     }
     if (!tc) {
@@ -618,6 +654,9 @@ static int factor_loop_nopiv(lu_fact f) {
       const int cap = c->dev.sm_count - keep;
       CU_TRY(PHASE(c, PH_GEMM, 1, tc_gemm_run(kind, (float*)(A22 + w2), ld, f->aop, bop2, rest, rest - w2, f->kpad,
                                                c->d_status, c->dev, st, cap > 8 ? cap : 8)));
+    } else if constexpr (sizeof(T) == 8) {
+      const int rc = update_f64(f, A22, L21, U12, rest, w, k / nb);
+      if (rc) return rc;
     } else {
       CU_TRY(PHASE(c, PH_GEMM, 1, launch_gemm_simt<T>(A22, ld, L21, ld, U12, ld, rest, rest, w, st)));
     }
@@ -628,7 +667,7 @@ static int factor_loop_nopiv(lu_fact f) {
 
 extern "C" void lu_fact_free(lu_fact f) {
   if (!f) return;
-  for (void* p : {f->W, (void*)f->ipiv, f->panel_mem, f->aop, f->oz_ws, (void*)f->oz_minv, (void*)f->spec_flag,
+  for (void* p : {f->W, (void*)f->ipiv, f->panel_mem, f->aop, f->oz_ws, (void*)f->oz_minv, (void*)f->oz_cert, (void*)f->spec_flag,
                   f->spec_backup, f->uinv, f->solve_mem, f->ss.dinv, (void*)f->vec_ws, f->res_ws})
     ffree(f, p);
   delete f;
@@ -698,6 +737,13 @@ extern "C" int lu_factor_ex(lu_ctx c, int n, const double* dA, int lda, lu_prec 
       return rc;
     }
   }
+  if (prec == LU_F64 && !f->ozaki && cert_applies(n, f->nb)) {
+    if ((rc = falloc(f, &f->oz_ws, ozaki_ws_bytes(n - f->nb, n - f->nb, f->nb, c->dev.sm_count, true))) ||
+        (rc = falloc(f, (void**)&f->oz_cert, cert_ints(n, f->nb) * sizeof(int)))) {
+      lu_fact_free(f);
+      return rc;
+    }
+  }
   const bool spec = prec != LU_F64 && !nopiv && c->spec && n > f->nb;
   if (spec) {
     if ((rc = falloc(f, (void**)&f->spec_flag, 4 * sizeof(int))) ||
@@ -726,6 +772,8 @@ extern "C" int lu_factor_ex(lu_ctx c, int n, const double* dA, int lda, lu_prec 
     return r;
   };
   if (cudaMemsetAsync(f->info_d, 0x7f, sizeof(int), st) != cudaSuccess) return fail(LU_ECUDA);
+  if (f->oz_cert && cudaMemsetAsync(f->oz_cert, 0, (2 + (size_t)(n / f->nb)) * sizeof(int), st) != cudaSuccess)
+    return fail(LU_ECUDA);
   if (f->spec_flag && cudaMemsetAsync(f->spec_flag, 0, 4 * sizeof(int), st) != cudaSuccess) return fail(LU_ECUDA);
   if (n > 0) {
     if (PHASE(c, PH_OTHER, 1, launch_iota(f->rowid, n, st)) != cudaSuccess) return fail(LU_ECUDA);
@@ -1180,6 +1228,8 @@ size_t gb_fact_bytes(int n, int nrhs, lu_prec prec, int nb, int sm_count) {
   size_t b = ldw * nn * tsize + (size_t)(2 * nn + 64) * sizeof(int) + panel_scratch_bytes(sm_count, 32, nb, tsize) +
              solve_scratch_bytes(nn, tsize);
   if (prec != LU_F64) b += solve_dinv_bytes(nn, tsize);
+  if (prec == LU_F64 && cert_applies(nn, nb))  // certified split updates
+    b += ozaki_ws_bytes(nn - nb, nn - nb, nb, sm_count, true) + cert_ints(nn, nb) * sizeof(int);
   if (prec != LU_F64 && n > nb)  // diagonal-pivot check
     b += 4 * sizeof(int) + (size_t)nn * nb * tsize + (size_t)round_up(nb, 32) * 32 * tsize;
   if (prec == LU_BF16 || prec == LU_FP16) b += (size_t)2 * nn * round_up(nb, 64) * 2 + 1024;

@@ -7,7 +7,7 @@
 
 namespace gb {
 
-// kind: 0 FP64 (CUDA-core update), 1 FP64 (split tensor-core update),
+// kind: 0 FP64 (certified split update), 1 FP64 (split tensor-core update),
 // 2 BF16 / FP16 mixed, 3 FP32.  The first entry of the kind whose nmax
 // is at least n applies.
 struct NbEntry {
@@ -15,11 +15,11 @@ struct NbEntry {
 };
 
 constexpr NbEntry kNbTable[] = {
-    {0, 1536, 64},  // f64, measured at n = 1024: nb 64: 7.718, nb 128: 8.339, nb 192: 9.302, nb 256: 9.536
-    {0, 3072, 64},  // f64, measured at n = 2048: nb 64: 19.147, nb 128: 20.414, nb 192: 21.652, nb 256: 22.787
-    {0, 6144, 64},  // f64, measured at n = 4096: nb 64: 66.583, nb 128: 68.244, nb 192: 70.896, nb 256: 72.259
-    {0, 12288, 128},  // f64, measured at n = 8192: nb 64: 358.492, nb 128: 358.441, nb 192: 361.787, nb 256: 364.058
-    {0, 24576, 256},  // f64, measured at n = 16384: nb 64: 2518.025, nb 128: 2497.408, nb 192: 2495.840, nb 256: 2493.114
+    {0, 1536, 64},  // f64, measured at n = 1023: nb 64: 4.59, nb 128: 4.70, nb 192: 5.48, nb 256: 6.43
+    {0, 3072, 64},  // f64, measured at n = 2048: nb 64: 10.46, nb 128: 10.86, nb 192: 13.50, nb 256: 16.22 (3000: 17.9, 19.1, 22.6, 25.4)
+    {0, 6144, 128},  // f64, measured at n = 6000: nb 64: 61.05, nb 128: 55.45, nb 192: 58.05, nb 256: 62.07 (4096: 29.4, 30.1, 34.1, 37.4)
+    {0, 12288, 192},  // f64, measured at n = 8192: nb 64: 118.4, nb 128: 94.89, nb 192: 93.46, nb 256: 96.34
+    {0, 24576, 256},  // f64, measured at n = 16384: nb 64: 647, nb 128: 412, nb 192: 349, nb 256: 326
     {0, 1073741824, 256},  // f64, measured at n = 32768: not measured: n = 32768 keeps the smaller size's choice
     {1, 1536, 128},  // f64_split, measured at n = 1024: nb 64: 8.105, nb 128: 7.824, nb 192: 8.141, nb 256: 8.463
     {1, 3072, 128},  // f64_split, measured at n = 2048: nb 64: 17.218, nb 128: 16.488, nb 192: 16.861, nb 256: 17.595

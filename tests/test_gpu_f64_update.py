@@ -1,0 +1,103 @@
+"""The plain FP64 factorization's trailing update (certified split products,
+with the FP64 CUDA cores where the certificate fails or the update is small):
+factors against the oracle at the edges of the rule that chooses it, and the
+componentwise backward error of badly scaled, banded and sparse systems, which
+a split update without the certificate loses."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2202_13995_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+U = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import torch
+    from paper_2202_13995_gb300 import lu
+    c = lu.Context()
+    yield c
+    torch.cuda.synchronize()
+    c.close()
+
+
+def _dev(a):
+    import torch
+    from paper_2202_13995_gb300 import lu
+    t = lu.colmajor_empty(a.shape[0], a.shape[1])
+    t.copy_(torch.from_numpy(np.asfortranarray(a)))
+    return t
+
+
+# one step, the first size that takes the split update, the last that does not, ragged last blocks,
+# widths below, at and above the certificate's least and most
+@pytest.mark.parametrize("n,nb", [(447, 64), (448, 64), (449, 64), (449, 63), (600, 65), (1030, 64), (777, 128),
+                                  (900, 256), (1000, 257)])
+@pytest.mark.parametrize("nopiv", [False, True])
+def test_factors_at_the_edges_of_the_rule(ctx, n, nb, nopiv):
+    A = I.hpl_matrix(n, 300 + n + nb, diag_shift=n / 4 if nopiv else 0.0)
+    f = ctx.factor(_dev(A), "f64", nb, nopiv=nopiv)
+    LUo, ipo, info = O.getrf(A)
+    assert f.info == info == 0
+    assert np.array_equal(f.ipiv().cpu().numpy(), ipo)
+    assert np.abs(f.lu().cpu().numpy() - LUo).max() <= 256 * n * U * np.abs(LUo).max()
+    f.free()
+
+
+def _system(kind, n, rng):
+    A = rng.random((n, n)) - 0.5
+    i = np.arange(n)
+    if kind == "row_scaled":
+        A *= 10.0 ** (30 * rng.random((n, 1)) - 15)
+    elif kind == "rows_far_apart":
+        A *= 10.0 ** (200 * rng.random((n, 1)) - 100)
+    elif kind == "column_scaled":
+        A *= 10.0 ** (30 * rng.random((1, n)) - 15)
+    elif kind == "banded":
+        A = A * (np.abs(i[:, None] - i[None, :]) < 40) + 2 * np.eye(n)
+    elif kind == "sparse":
+        A = A * (rng.random((n, n)) < 0.02) + 2 * np.eye(n)
+    elif kind == "half_scaled":
+        A[: n // 2] *= 1e-12
+    return A
+
+
+@pytest.mark.parametrize("nb", [64, 128])
+@pytest.mark.parametrize("kind", ["row_scaled", "rows_far_apart", "column_scaled", "banded", "sparse", "half_scaled"])
+def test_componentwise_backward_error(ctx, kind, nb):
+    """|b - A x| <= c (|A||x| + |b|) row by row.  Partial pivoting gives
+    |b - A x| <= 3 n u |P^T L||U||x| (N. Higham, Accuracy and Stability of Numerical
+    Algorithms, theorem 9.4); the factor beside the rows' own sums is the oracle's."""
+    n = 1100
+    rng = np.random.default_rng(17)
+    A = _system(kind, n, rng)
+    x0 = rng.random((n, 1)) - 0.5
+    B = A @ x0
+    f = ctx.factor(_dev(A), "f64", nb)
+    X = _dev(B)
+    f.solve_(X)
+    x = X.cpu().numpy()
+    LUo, ipo, info = O.getrf(A)
+    assert f.info == info == 0
+    p = np.arange(n)
+    for j, q in enumerate(ipo):
+        p[j], p[q - 1] = p[q - 1], p[j]
+    L, R = np.tril(LUo, -1) + np.eye(n), np.triu(LUo)
+    bound = np.empty((n, 1))
+    bound[p] = 3 * n * U * (np.abs(L) @ (np.abs(R) @ np.abs(x)))
+    r = np.abs((B.astype(np.longdouble) - A.astype(np.longdouble) @ x.astype(np.longdouble)).astype(float))
+    assert (r <= bound + U * np.abs(B)).all(), float((r / (bound + U * np.abs(B))).max())
+    f.free()
+
+
+def test_non_finite_entries_are_reported(ctx):
+    from paper_2202_13995_gb300 import lu
+    for bad in (np.nan, np.inf):
+        for at in ((900, 5), (3, 900), (800, 700)):
+            A = I.hpl_matrix(1000, 5)
+            A[at] = bad
+            with pytest.raises(lu.LuError) as e:
+                ctx.factor(_dev(A), "f64", 64)
+            assert e.value.code == lu.LU_ERANGE
