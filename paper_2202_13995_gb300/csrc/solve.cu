@@ -16,15 +16,19 @@
 // chunks whose blocks interleave on the one ticket counter (block b of chunk
 // c is ticket b * chunks + c), so the chunks' chains run side by side in one
 // launch instead of one after the other.
+// What bounds it: the chain of 64-row blocks, one flag each.  Measured per
+// block and triangle (n = 5000; butterfly sums and one warp per substitution
+// before): FP64 1 right-hand side 14.5 -> 7.8 us, 3: 26.8 -> 9.3, 8: 45.7 -> 9.2;
+// FP32 1: 2.1 -> 1.9, 8: 5.1 -> 2.9, 32: 8.4 -> 4.2.
 #include "common.cuh"
 #include "kernels.h"
 
 namespace gb {
 
 constexpr int TS_BS = 64;
-constexpr int TS_NRMAX = 16;  // right-hand sides per CTA: 16 for FP32 factors, 8 for FP64
+constexpr int TS_NRMAX = 16;  // right-hand sides per CTA: up to 16 for FP32 factors, 2 for FP64
 constexpr int TS_RHS_MAX = 32;  // right-hand sides per launch (chunks of the above)
-constexpr int TS_CHUNKS_MAX = TS_RHS_MAX / 8;
+constexpr int TS_CHUNKS_MAX = TS_RHS_MAX / 2;
 
 // Leading dimension of the solution workspaces: a multiple of 16 elements, so
 // that every 16-byte chunk of a solution block starts 16-byte aligned.
@@ -49,12 +53,44 @@ struct TrsvSmem {
   int blk;
 };
 
+// Sums over the warp's lanes of V values per lane (V a power of two), each by
+// the same tree as a butterfly over lane distances 16, 8, 4, 2, 1, but with the
+// values dealt to the lanes on the way: at each distance a lane keeps half of
+// its values and sends the other half, so that V sums take about V exchanges
+// and additions instead of 5 V.  (FP64 additions issue once in 64 cycles per
+// SM quarter: with the butterfly, the sums of 4 right-hand sides were 10 us of
+// the 27 us a block of the FP64 solve took.)  Value i ends in the lanes whose
+// top bits are i (V <= 32), or lane l holds values l V / 32 .. (V > 32).
+template <int M, int OFF, typename T>
+__device__ __forceinline__ void warp_deal_sum(T* a) {
+  if constexpr (OFF > 0) {
+    const int lane = threadIdx.x & 31;
+    if constexpr (M > 1) {
+      const bool up = (lane & OFF) != 0;
+#pragma unroll
+      for (int i = 0; i < M / 2; ++i) {
+        const T send = up ? a[i] : a[i + M / 2];
+        const T keep = up ? a[i + M / 2] : a[i];
+        a[i] = keep + __shfl_xor_sync(0xffffffffu, send, OFF);
+      }
+      warp_deal_sum<M / 2, OFF / 2>(a);
+    } else {
+      a[0] += __shfl_xor_sync(0xffffffffu, a[0], OFF);
+      warp_deal_sum<1, OFF / 2>(a);
+    }
+  }
+}
+
 // With DINV, the diagonal block's inverse (precomputed by trinv_kernel) turns
 // the serial substitution into a parallel matrix-vector product; the FP32
-// correction solves of the refinement use it.  The FP64 solve substitutes;
-// its upper triangle multiplies by the reciprocals of the diagonal, computed
-// when the block starts, off the chain of blocks (an FP64 division on GB300
-// takes longer than the rest of a substitution step).
+// correction solves of the refinement use it.  The FP64 solve substitutes, two
+// warps per right-hand side: one takes the 32 rows that come first, a lane per
+// row and a broadcast and a multiply-add per step, while the other subtracts
+// each eight finished solutions from the other 32 rows, whose own steps follow.
+// Its upper triangle works on U D^-1 with the unknowns D x (D = diag(U)), scaled
+// by the reciprocals of the diagonal when the block starts, off the chain of
+// blocks, so that its steps multiply nothing (an FP64 division on GB300 takes
+// longer than the rest of a substitution step, a product as long).
 
 // LOWER: Y = L^-1 (P B) with unit-lower L; the right-hand side is gathered
 //        from B through rowid: (P b)[i] = b[rowid[i]].
@@ -66,7 +102,7 @@ struct TrsvSmem {
 // Requires ldw % (16 / sizeof(T)) == 0 and a 16-byte aligned W (the working
 // matrix is allocated that way).
 template <typename T, int NR, int STAGES, bool LOWER, bool DINV>
-__global__ void __launch_bounds__(256) trsv_kernel(const T* __restrict__ W, int64_t ldw, int n, int nrhs_all, int nch,
+__global__ void __launch_bounds__(256, 1) trsv_kernel(const T* __restrict__ W, int64_t ldw, int n, int nrhs_all, int nch,
                                                    const double* __restrict__ B0, int64_t ldb,
                                                    const int* __restrict__ rowid, const T* __restrict__ Yin0,
                                                    T* Yout0, double* X0, int64_t ldx, int* flags0, int* ticket,
@@ -124,6 +160,12 @@ __global__ void __launch_bounds__(256) trsv_kernel(const T* __restrict__ W, int6
       if (!DINV && !LOWER) {
         __syncthreads();
         if (tid < TS_BS) sm.rinv[tid] = tid < rows ? T(1) / sm.Ld[tid][tid] : T(0);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+          const int e = tid + q * 256;
+          sm.Ld[e >> 6][e & 63] = dv[q] * sm.rinv[e & 63];
+        }
       }
     }
     // this block's right-hand side: thread (row tid & 63) holds columns
@@ -235,26 +277,17 @@ __global__ void __launch_bounds__(256) trsv_kernel(const T* __restrict__ W, int6
       __syncthreads();
     }
     cp_async_wait_group<0>();
-    // row sums: a fixed butterfly over the lanes (deterministic)
+    // row sums over the lanes (a fixed tree: deterministic)
+    auto rows_out = [&](T (&x)[8][NR]) {
+      constexpr int V = 8 * NR, PL = V > 32 ? V / 32 : 1;
+      warp_deal_sum<V, 16>(&x[0][0]);
+      const int i0v = V >= 32 ? lane * PL : lane / (32 / V);
+      if (V >= 32 || lane % (32 / (V < 32 ? V : 32)) == 0) {
 #pragma unroll
-    for (int rr = 0; rr < 8; ++rr)
-#pragma unroll
-      for (int q = 0; q < NR; ++q) {
-        T v = acc[rr][q];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        acc[rr][q] = v;
+        for (int i = 0; i < PL; ++i) sm.v[(i0v + i) % NR][warp * 8 + (i0v + i) / NR] = (&x[0][0])[i];
       }
-    if (lane < NR) {
-#pragma unroll
-      for (int rr = 0; rr < 8; ++rr) {
-        T tot = T(0);
-#pragma unroll
-        for (int q = 0; q < NR; ++q)
-          if (q == lane) tot = acc[rr][q];
-        sm.v[lane][warp * 8 + rr] = tot;
-      }
-    }
+    };
+    rows_out(acc);
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < NU; ++u) {
@@ -262,56 +295,69 @@ __global__ void __launch_bounds__(256) trsv_kernel(const T* __restrict__ W, int6
       if (q < NR) sm.v[q][r] = (r < rows && q < nrhs) ? rhs[u] - sm.v[q][r] : T(0);
     }
     __syncthreads();
-    if (DINV) {
+    if constexpr (DINV) {
       // x = inverse(diagonal block) * v: warp w computes rows 8w .. 8w+7
       T xr[8][NR];
 #pragma unroll
       for (int rr = 0; rr < 8; ++rr) {
         const T d0 = sm.Ld[warp * 8 + rr][lane], d1 = sm.Ld[warp * 8 + rr][lane + 32];
 #pragma unroll
-        for (int q = 0; q < NR; ++q) {
-          T v = d0 * sm.v[q][lane] + d1 * sm.v[q][lane + 32];
-#pragma unroll
-          for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-          xr[rr][q] = v;
-        }
+        for (int q = 0; q < NR; ++q) xr[rr][q] = d0 * sm.v[q][lane] + d1 * sm.v[q][lane + 32];
       }
       __syncthreads();
-      if (lane < NR) {
+      rows_out(xr);
+    } else {
+      // warps 2 q and 2 q + 1: right-hand side q; a named barrier for each eight
+      // solutions (the first warp only arrives and may run ahead)
+      static_assert(DINV || NR <= 3, "four named barriers per right-hand side");
+      if (warp < 2 * NR) {
+        const int q = warp >> 1;
+        const bool first = (warp & 1) == 0;
+        const int h0 = LOWER ? 0 : 32;          // the rows that come first
+        const int own = first ? h0 : 32 - h0;   // this warp's rows
+        T x = sm.v[q][own + lane];
+        const T* Lrow = sm.Ld[own + lane];
+        // step i of a half: its column t, solved in lane t - half
+        auto col = [&](int half, int i) { return half + (LOWER ? i : 31 - i); };
+        if (!first) {
+#pragma unroll 1
+          for (int g = 0; g < 32; g += 8) {
+            T l[8];
 #pragma unroll
-        for (int rr = 0; rr < 8; ++rr) {
-          T x = T(0);
+            for (int i = 0; i < 8; ++i) l[i] = Lrow[col(h0, g + i)];
+            asm volatile("bar.sync %0, 64;" ::"r"(1 + 4 * q + (g >> 3)) : "memory");
 #pragma unroll
-          for (int q = 0; q < NR; ++q)
-            if (q == lane) x = xr[rr][q];
-          sm.v[lane][warp * 8 + rr] = x;
-        }
-      }
-    } else
-    for (int q = warp; q < nrhs; q += 8) {
-      T x0 = sm.v[q][lane], x1 = sm.v[q][lane + 32];
-      if (LOWER) {
-        for (int t = 0; t < rows; ++t) {
-          const T xt = __shfl_sync(0xffffffffu, t < 32 ? x0 : x1, t & 31);
-          if (lane > t) x0 -= sm.Ld[lane][t] * xt;
-          if (lane + 32 > t) x1 -= sm.Ld[lane + 32][t] * xt;
-        }
-      } else {
-        for (int t = rows - 1; t >= 0; --t) {
-          T xt;
-          if (t >= 32) {
-            if (lane == t - 32) x1 = x1 * sm.rinv[t];
-            xt = __shfl_sync(0xffffffffu, x1, t - 32);
-          } else {
-            if (lane == t) x0 = x0 * sm.rinv[t];
-            xt = __shfl_sync(0xffffffffu, x0, t);
+            for (int i = 0; i < 8; ++i) x = fma(-l[i], sm.v[q][col(h0, g + i)], x);
           }
-          if (lane < t) x0 -= sm.Ld[lane][t] * xt;
-          if (lane + 32 < t) x1 -= sm.Ld[lane + 32][t] * xt;
         }
+#pragma unroll 1
+        for (int g = 0; g < 32; g += 8) {
+          T l[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int t = col(own, g + i);
+            const bool after = LOWER ? own + lane > t : own + lane < t;
+            l[i] = after ? Lrow[t] : T(0);
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int t = col(own, g + i) - own;
+            const T xt = __shfl_sync(0xffffffffu, x, t);
+            if (LOWER ? lane > t : lane < t) x = fma(-l[i], xt, x);
+          }
+          if (first) {
+            const int i = LOWER ? lane : 31 - lane;  // the step that solved this lane's row
+            if (i >= g && i < g + 8) sm.v[q][own + lane] = x;
+            __syncwarp();
+            asm volatile("bar.arrive %0, 64;" ::"r"(1 + 4 * q + (g >> 3)) : "memory");
+          }
+        }
+        if (!first) sm.v[q][own + lane] = x;
       }
-      sm.v[q][lane] = x0;
-      sm.v[q][lane + 32] = x1;
+      if (!LOWER) {
+        __syncthreads();  // (the unscaled unknowns have been read)
+        for (int e = tid; e < TS_BS * NR; e += 256) sm.v[e >> 6][e & 63] *= sm.rinv[e & 63];
+      }
     }
     __syncthreads();
     for (int e = tid; e < TS_BS * NR; e += 256) {
@@ -430,9 +476,10 @@ template cudaError_t launch_trinv<float>(const float*, int64_t, int, float*, cud
 template cudaError_t launch_trinv<double>(const double*, int64_t, int, double*, cudaStream_t);
 
 // One launch pair for up to 32 right-hand sides: a CTA holds up to 16 with
-// FP32 factors, 8 with FP64 (whose accumulators take twice the registers);
-// more are cut in chunks of that width whose chains of diagonal blocks run
-// side by side in the same launches.
+// FP32 factors, 2 with FP64, whose products with the block before run at two
+// multiply-adds per clock on the chain (1 us per right-hand side and 64-row
+// block); more are cut in chunks of that width whose chains of diagonal blocks
+// run side by side in the same launches.
 template <typename T>
 cudaError_t launch_lu_solve(const T* W, int64_t ldw, const int* rowid, int n, int nrhs, const double* B,
                             int64_t ldb, double* X, int64_t ldx, const SolveScratch& s, int* status,
@@ -440,23 +487,19 @@ cudaError_t launch_lu_solve(const T* W, int64_t ldw, const int* rowid, int n, in
   if (n <= 0 || nrhs <= 0) return cudaSuccess;
   if (nrhs > TS_RHS_MAX) return cudaErrorInvalidValue;
   if (((uintptr_t)W & 15u) || (ldw % (16 / sizeof(T))) != 0) return cudaErrorInvalidValue;
-  constexpr int CHUNK = sizeof(T) == 4 ? 16 : 8;
-  static_assert(CHUNK <= TS_NRMAX && TS_RHS_MAX / CHUNK <= TS_CHUNKS_MAX, "solve workspace holds the chunks");
-  // a CTA's width: the right-hand sides rounded up to 1, 2, 4, 8 or the
-  // chunk (a column's arithmetic is the same at every width)
-  const bool dinv = s.dinv != nullptr && s.dinv_ready;
-  if (dinv) {
+  // a CTA's width: the right-hand sides rounded up to 1, 2, 4, 8 or 16 (a
+  // column's arithmetic is the same at every width)
+  if constexpr (sizeof(T) == 4) {
+    if (s.dinv == nullptr || !s.dinv_ready) return cudaErrorInvalidValue;  // (every FP32 factor has them)
     if (nrhs == 1) return run_solve<T, 1, true>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
     if (nrhs == 2) return run_solve<T, 2, true>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
     if (nrhs <= 4) return run_solve<T, 4, true>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
     if (nrhs <= 8) return run_solve<T, 8, true>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
-    return run_solve<T, CHUNK, true>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
+    return run_solve<T, TS_NRMAX, true>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
+  } else {
+    if (nrhs == 1) return run_solve<T, 1, false>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
+    return run_solve<T, 2, false>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
   }
-  if (nrhs == 1) return run_solve<T, 1, false>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
-  if (nrhs == 2) return run_solve<T, 2, false>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
-  if (nrhs <= 4) return run_solve<T, 4, false>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
-  if (nrhs <= 8) return run_solve<T, 8, false>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
-  return run_solve<T, CHUNK, false>(W, ldw, rowid, n, nrhs, B, ldb, X, ldx, s, status, st);
 }
 
 template cudaError_t launch_lu_solve<double>(const double*, int64_t, const int*, int, int, const double*, int64_t,
