@@ -34,6 +34,7 @@ struct PanelScratch {
   int ibmax;
   int wmax;
   int gtarget = 0; // preferred CTA count (0: the default for the element size)
+  void* xres = nullptr;  // panel_resident_bytes(gmax, wmax, tsize) for the resident form, or none
 };
 // Most CTAs one cooperative panel launch may use: every CTA's candidate row
 // of a column must fit the exchange buffer each CTA reads after the barrier.
@@ -70,12 +71,23 @@ cudaError_t launch_panel(T* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv,
 // The panel on one thread-block cluster (panel_cluster.cu): same arguments and
 // outputs as launch_panel without a check; used by launch_panel when the panel
 // fits (panel_cluster_fits: its rows, all w columns, in the shared memory of
-// at most 16 CTAs).
+// at most 16 CTAs; grid: and is not better off on the grid form below).
 template <typename T>
-bool panel_cluster_fits(int m, int w, const DevInfo& dev);
+bool panel_cluster_fits(int m, int w, const DevInfo& dev, bool grid = false);
 template <typename T>
 cudaError_t launch_panel_cluster(T* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv, int* info, int* status,
                                  int* perm, const DevInfo& dev, cudaStream_t st);
+// The panel resident in the shared memory of a cooperative grid (also
+// panel_cluster.cu), for panels that do not fit a cluster: CTAs it would take
+// (0: it does not fit, or the scratch has no xres), and the launch.
+size_t panel_resident_bytes(int gmax, int wmax, int tsize);
+template <typename T>
+int panel_resident_ctas(int m, int w, const DevInfo& dev, const PanelScratch& s);
+template <typename T>
+cudaError_t launch_panel_resident(T* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv, int* info, int* status,
+                                  const PanelScratch& s, const DevInfo& dev, cudaStream_t st);
+// A cooperative launch, retried while other in-flight grids hold the room it needs.
+cudaError_t launch_cooperative(const void* kern, int grid, int threads, void** args, size_t smem, cudaStream_t st);
 // SMs one panel launch occupies (for the lookahead's trailing-update cap).
 int panel_sm_use(int m, int w, int tsize, const DevInfo& dev, const PanelScratch& s);
 

@@ -379,6 +379,23 @@ static int default_nb(int n, lu_prec prec, bool split) {
 
 static int round_up(int v, int a) { return (v + a - 1) / a * a; }
 
+// Records of the grid-resident panels (none when every panel of the
+// factorization goes to a cluster).  Shared contexts keep to the other forms
+// (dev.max_smem_optin = 0): a grid that needs most of every SM's shared memory
+// would wait for the other requests to drain.
+static size_t resident_bytes(int n, lu_prec prec, int nb, const DevInfo& dev) {
+  if (dev.max_smem_optin == 0 || n < nb) return 0;
+  const bool cluster =
+      prec == LU_F64 ? panel_cluster_fits<double>(n, nb, dev, true) : panel_cluster_fits<float>(n, nb, dev, true);
+  return cluster ? 0 : panel_resident_bytes(dev.sm_count, nb, prec == LU_F64 ? 8 : 4);
+}
+// the context's device as the panels see it
+static DevInfo panel_dev(lu_ctx c) {
+  DevInfo d = c->dev;
+  if (c->ev_block != nullptr) d.max_smem_optin = 0;
+  return d;
+}
+
 // ------------------------------------------------------------------ factor
 // The top block solve U12 = L11^-1 A12 with the split update: M = I - L11^-1
 // in FP64, then A12 -= M A12 on the tensor cores (the split reads A12 before
@@ -509,11 +526,14 @@ static int factor_loop(lu_fact f) {
     // with the lookahead, only the next panel's columns of the top block row
     // are solved and cast before the next panel starts; the rest follow on
     // this stream while the next panel runs on the side stream
-    // (a pivoted panel on one cluster waits for a whole GPC, which the update
-    // beside it would hold: it runs after the update instead, and is faster
-    // alone than the cooperative panel beside it)
+    // (a pivoted panel on one cluster waits for a whole GPC, and one resident on
+    // the grid for every SM, which the update beside it would hold: it runs
+    // after the update instead, and is faster alone than the cooperative panel
+    // beside it)
     const bool split_top =
-        tc && lookahead && rest > w2 && !(mode == SPEC_OFF && panel_cluster_fits<T>(rest, w2, c->dev));
+        tc && lookahead && rest > w2 &&
+        !(mode == SPEC_OFF &&
+          (panel_cluster_fits<T>(rest, w2, c->dev) || panel_resident_ctas<T>(rest, w2, c->dev, f->ps) > 0));
     if (f->ozaki) {
       CU_TRY(top_solve_split(f, (double*)Wkk, (double*)U12, ld, w, rest));
     } else if (tc) {
@@ -705,7 +725,9 @@ extern "C" int lu_factor_ex(lu_ctx c, int n, const double* dA, int lda, lu_prec 
   const int nn = n > 0 ? n : 1;
   int rc = LU_OK;
   const int gmax = c->dev.sm_count;
-  size_t pbytes = panel_scratch_bytes(gmax, 32, f->nb, f->tsize);
+  // (the grid-resident panels' records behind the panel scratch)
+  const size_t pbase = (panel_scratch_bytes(gmax, 32, f->nb, f->tsize) + 255) / 256 * 256;
+  const size_t pbytes = pbase + (nopiv ? 0 : resident_bytes(n, prec, f->nb, panel_dev(c)));
   if ((rc = falloc(f, &f->W, (size_t)f->ldw * nn * f->tsize)) ||
       (rc = falloc(f, (void**)&f->ipiv, (size_t)(2 * nn + 64) * sizeof(int))) ||
       (rc = falloc(f, &f->panel_mem, pbytes)) ||
@@ -716,6 +738,7 @@ extern "C" int lu_factor_ex(lu_ctx c, int n, const double* dA, int lda, lu_prec 
   f->rowid = f->ipiv + nn;
   f->info_d = f->rowid + nn;
   panel_scratch_carve(&f->ps, f->panel_mem, gmax, 32, f->nb, f->tsize);
+  if (pbytes > pbase) f->ps.xres = (char*)f->panel_mem + pbase;
   // With the lookahead, the FP32 panel shares the GPU with the update of the
   // rest of the trailing matrix: 5/8 of the SMs for the panel (measured at
   // n = 32768: 96 of 152 SMs, 238 ms per solve against 256 with 64 and 265
@@ -1107,11 +1130,13 @@ extern "C" int lu_step_panel(lu_ctx c, lu_prec prec, int m, int w, void* dP, int
   if (!dInfo) return -8;
   const int tsize = prec == LU_F64 ? 8 : 4;
   const int gmax = c->dev.sm_count;
-  const size_t pbytes = panel_scratch_bytes(gmax, 32, w, tsize);
-  int rc = ensure_step_ws(c, pbytes);
+  const size_t pbase = (panel_scratch_bytes(gmax, 32, w, tsize) + 255) / 256 * 256;
+  const size_t rbytes = resident_bytes(m, prec, w, panel_dev(c));
+  int rc = ensure_step_ws(c, pbase + rbytes);
   if (rc) return rc;
   PanelScratch ps;
   panel_scratch_carve(&ps, c->step_ws, gmax, 32, w, tsize);
+  if (rbytes) ps.xres = (char*)c->step_ws + pbase;
   CU_TRY(cudaMemsetAsync(dInfo, 0x7f, sizeof(int), c->stream));
   if (prec == LU_F64)
     CU_TRY(launch_panel<double>((double*)dP, ld, m, w, 0, dIpiv, dInfo, c->d_status, ps, c->dev, c->stream));
@@ -1219,14 +1244,18 @@ void gb_ctx_free(lu_ctx c, void* p) { dfree(c, p); }
 
 // Bytes lu_factor (+ lu_refine's workspace for nrhs columns) allocates; the
 // server's admission counts requests with it.
-size_t gb_fact_bytes(int n, int nrhs, lu_prec prec, int nb, int sm_count) {
+size_t gb_fact_bytes(int n, int nrhs, lu_prec prec, int nb, int sm_count, int smem_optin) {
   const int nn = n > 0 ? n : 1;
   if (nb == 0) nb = default_nb(n, prec, false);
   nb = nb < nn ? nb : nn;
   const int tsize = prec == LU_F64 ? 8 : 4;
   const size_t ldw = (size_t)round_up(nn, 64);
-  size_t b = ldw * nn * tsize + (size_t)(2 * nn + 64) * sizeof(int) + panel_scratch_bytes(sm_count, 32, nb, tsize) +
-             solve_scratch_bytes(nn, tsize);
+  size_t b = ldw * nn * tsize + (size_t)(2 * nn + 64) * sizeof(int) +
+             (panel_scratch_bytes(sm_count, 32, nb, tsize) + 255) / 256 * 256 + solve_scratch_bytes(nn, tsize);
+  DevInfo dev{};
+  dev.sm_count = sm_count;
+  dev.max_smem_optin = smem_optin;
+  b += resident_bytes(nn, prec, nb, dev);
   if (prec != LU_F64) b += solve_dinv_bytes(nn, tsize);
   if (prec == LU_F64 && cert_applies(nn, nb))  // certified split updates
     b += ozaki_ws_bytes(nn - nb, nn - nb, nb, sm_count, true) + cert_ints(nn, nb) * sizeof(int);
@@ -1270,11 +1299,12 @@ extern "C" int lu_default_nb(int n, lu_prec prec, int flags) {
 
 extern "C" size_t lu_fact_bytes(int n, int nrhs, lu_prec prec, int nb) {
   if (n < 1 || nrhs < 0 || prec < LU_F64 || prec > LU_F32 || nb < 0 || nb > 512) return 0;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
-                                                cudaSuccess) {
+  int dev = 0, sms = 0, optin = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
-  return gb_fact_bytes(n, nrhs, prec, nb, sms);
+  return gb_fact_bytes(n, nrhs, prec, nb, sms, optin);
 }

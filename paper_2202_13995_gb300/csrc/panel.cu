@@ -411,13 +411,32 @@ int panel_sm_use(int m, int w, int tsize, const DevInfo& dev, const PanelScratch
   return panel_grid_size(m, w, tsize, dev, s.gmax, s.gtarget);
 }
 
+// A cooperative launch is refused (without side effects) while other
+// in-flight cooperative grids -- other streams' panels -- hold the resources
+// it needs; those grids always finish, so retry with a short back-off
+// (bounded: 20 s).
+cudaError_t launch_cooperative(const void* kern, int grid, int threads, void** args, size_t smem, cudaStream_t st) {
+  const auto t0 = std::chrono::steady_clock::now();
+  while (true) {
+    const cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), args, smem, st);
+    if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorLaunchOutOfResources) return e;
+    cudaGetLastError();
+    if (std::chrono::steady_clock::now() - t0 > std::chrono::seconds(20)) return e;
+    std::this_thread::sleep_for(std::chrono::microseconds(20));
+  }
+}
+
 template <typename T>
 cudaError_t launch_panel(T* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv, int* info, int* status,
                          const PanelScratch& s, const DevInfo& dev, cudaStream_t st, const int* spec_flag,
                          const T* spec_backup) {
   if (w <= 0 || m < w || w > s.wmax) return cudaErrorInvalidValue;
-  if (spec_flag == nullptr && panel_cluster_fits<T>(m, w, dev))
-    return launch_panel_cluster<T>(Wkk, ldw, m, w, kabs, ipiv, info, status, s.perm, dev, st);
+  if (spec_flag == nullptr) {
+    const bool grid = panel_resident_ctas<T>(m, w, dev, s) > 0;
+    if (panel_cluster_fits<T>(m, w, dev, grid))
+      return launch_panel_cluster<T>(Wkk, ldw, m, w, kabs, ipiv, info, status, s.perm, dev, st);
+    if (grid) return launch_panel_resident<T>(Wkk, ldw, m, w, kabs, ipiv, info, status, s, dev, st);
+  }
   if (s.gmax > PNL_XG) return cudaErrorInvalidValue;  // every candidate row fits the exchange buffer
   const int ib = PNL_IB < s.ibmax ? PNL_IB : s.ibmax;
   const int G0 = panel_grid_size(m, w, sizeof(T), dev, s.gmax, s.gtarget);
@@ -455,18 +474,7 @@ cudaError_t launch_panel(T* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv,
   P.spec = spec_flag;
   P.spec_backup = spec_backup;
   void* args[] = {&P};
-  // A cooperative launch is refused (without side effects) while other
-  // in-flight cooperative grids -- other streams' panels -- hold the resources
-  // it needs; those grids always finish, so retry with a short back-off
-  // (bounded: 20 s).
-  const auto t0 = std::chrono::steady_clock::now();
-  while (true) {
-    e = cudaLaunchCooperativeKernel((const void*)kern, dim3(G), dim3(PNL_THREADS), args, smem, st);
-    if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorLaunchOutOfResources) return e;
-    cudaGetLastError();
-    if (std::chrono::steady_clock::now() - t0 > std::chrono::seconds(20)) return e;
-    std::this_thread::sleep_for(std::chrono::microseconds(20));
-  }
+  return launch_cooperative((const void*)kern, G, PNL_THREADS, args, smem, st);
 }
 
 // ============================================================ laswp

@@ -1,4 +1,6 @@
-// Panel factorization with partial pivoting on one thread-block cluster.
+// Panel factorization with partial pivoting, the panel resident in shared
+// memory: on one thread-block cluster, and for panels that 16 CTAs do not hold
+// or that keep more FP64 pipes busy, on the whole grid (at the end).
 //
 // The same computation as panel_getrf_kernel (the paper's diagonal and left
 // blocks of a block iteration, factored together because partial pivoting
@@ -403,10 +405,12 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
 
 // CTAs of a panel's cluster: rows of 32 (FP64: the FP64 pipes of as many SMs as
 // help) or 64 (FP32) per CTA up to 16 CTAs; -1 when the tile does not fit the
-// shared memory then, or when the cooperative kernel is as fast: an FP64 panel
-// of m w > 360,000 is bound by the FP64 pipes of 16 SMs (3000 x 128: 783 us
-// against 772; 6000 x 64: 358 against 380).
-static int pc_config(int m, int w, int tsize, int optin, int* R, int* nt, size_t* smem) {
+// shared memory then.  grid: the grid form can take the panel instead, which an
+// FP64 panel of m w > 140,000 is faster on, bound as it is by the FP64 pipes of
+// 16 SMs (us per column, cluster and grid: 2048 x 64 3.2 and about 3; 4096 x 64
+// 4.3 and 3.3; 2500 x 128 4.6 and 3.7); without it the line is the cooperative
+// kernel's, 360,000 (3000 x 128: 6.1 and 6.0).
+static int pc_config(int m, int w, int tsize, int optin, bool grid, int* R, int* nt, size_t* smem) {
   if (w < 1 || w > 512 || m < w) return -1;
   const int target = tsize == 8 ? 32 : 64;
   int cl = 1;
@@ -416,7 +420,7 @@ static int pc_config(int m, int w, int tsize, int optin, int* R, int* nt, size_t
   if (*R > PC_NTMAX) return -1;
   *smem = pc_smem_bytes(*R, w, cl, tsize);
   if (*smem + 1024 > (size_t)optin) return -1;
-  if (tsize == 8 && (int64_t)m * w > 360000) return -1;
+  if (tsize == 8 && (int64_t)m * w > (grid ? 140000 : 360000)) return -1;
   return cl;
 }
 
@@ -447,10 +451,10 @@ static cudaError_t pc_prepare() {
 // on the current device (asked of the runtime once per cluster and block size,
 // with the largest shared memory).
 template <typename T>
-bool panel_cluster_fits(int m, int w, const DevInfo& dev) {
+bool panel_cluster_fits(int m, int w, const DevInfo& dev, bool grid) {
   int R = 0, nt = 0;
   size_t smem = 0;
-  const int cl = pc_config(m, w, sizeof(T), dev.max_smem_optin, &R, &nt, &smem);
+  const int cl = pc_config(m, w, sizeof(T), dev.max_smem_optin, grid, &R, &nt, &smem);
   if (cl < 0) return false;
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return false;
@@ -481,7 +485,7 @@ cudaError_t launch_panel_cluster(T* Wkk, int64_t ldw, int m, int w, int kabs, in
   PcParams<T> P;
   int nt = 0;
   size_t smem = 0;
-  const int cl = pc_config(m, w, sizeof(T), dev.max_smem_optin, &P.R, &nt, &smem);
+  const int cl = pc_config(m, w, sizeof(T), dev.max_smem_optin, false, &P.R, &nt, &smem);
   if (cl < 0) return cudaErrorInvalidConfiguration;
   cudaError_t e = pc_prepare<T>();
   if (e != cudaSuccess) return e;
@@ -499,8 +503,381 @@ cudaError_t launch_panel_cluster(T* Wkk, int64_t ldw, int m, int w, int kabs, in
   return cudaLaunchKernelEx(&cfg, panel_cluster_kernel<T>, P);
 }
 
+// ============================================================ the same on the whole grid
+// Panels too large for one cluster: the CTAs of a cooperative launch hold R
+// rows each, all columns, in shared memory, and work as above; only the
+// exchange differs.  A CTA's record lies in global memory: a 16-byte header
+// (key and position) and the row beside it.  Every 8-byte word of either
+// carries the column's stamp next to its data, so readers know a word by
+// itself and no fence orders the stores (a release store that waits for the
+// row's stores cost 1 us a column).  Thread t of every CTA polls CTA t's header,
+// the CTA picks the pivot and reads its row once: two L2 round trips a column,
+// with the update of the other columns under them.  Against the kernel in
+// panel.cu (a counter barrier, every candidate row read by every CTA,
+// sub-panels of 32 columns written back, interchanged and updated through L2)
+// no value but the pivot row crosses L2 twice.
+// Measured (us per column, that kernel -> this one): FP64 6000 x 64 5.9 -> 3.4,
+// 8192 x 128 6.7 -> 3.9, 7000 x 256 7.7 -> 5.1 (there the FP64 pipes set the
+// pace: 256 columns of 46 rows); FP32 8192 x 128 4.5 -> 2.1.  Clock stamps
+// (8192 x 128): the poll 600 cycles, the row 1150, of 8000 (FP64) and 4300 (FP32).
+// The record buffers' stamps are cleared before the launch; a buffer is
+// reused every third column (the argument above).  Every poll is bounded; a CTA whose poll runs
+// out raises ST_TIMEOUT and leaves, and so do the others in their turn.
+
+// A value between its stamps: a double as two 8-byte words {low half, stamp},
+// {high half, stamp}, a float as one; relaxed loads and stores (each 8-byte word
+// is read and written whole).
+__device__ __forceinline__ ulonglong2 pr_load(const ulonglong2* p) {
+  ulonglong2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void pr_store(ulonglong2* p, ulonglong2 v) {
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(v.x), "l"(v.y) : "memory");
+}
+template <typename T>
+struct PrWord;
+template <>
+struct PrWord<double> {
+  using type = ulonglong2;
+  static __device__ __forceinline__ void put(type* p, double v, unsigned stamp) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    pr_store(p, make_ulonglong2((b << 32) | stamp, (b & 0xffffffff00000000ull) | stamp));
+  }
+  static __device__ __forceinline__ bool get(const type* p, double& v, unsigned stamp) {
+    const ulonglong2 x = pr_load(p);
+    v = __longlong_as_double((long long)((x.y & 0xffffffff00000000ull) | (x.x >> 32)));
+    return (unsigned)x.x == stamp && (unsigned)x.y == stamp;
+  }
+};
+template <>
+struct PrWord<float> {
+  using type = unsigned long long;
+  static __device__ __forceinline__ void put(type* p, float v, unsigned stamp) {
+    const unsigned long long x = ((unsigned long long)__float_as_uint(v) << 32) | stamp;
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(x) : "memory");
+  }
+  static __device__ __forceinline__ bool get(const type* p, float& v, unsigned stamp) {
+    unsigned long long x;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(p) : "memory");
+    v = __uint_as_float((unsigned)(x >> 32));
+    return (unsigned)x == stamp;
+  }
+};
+
+template <typename T>
+struct PrParams {
+  T* A;  // W(k, k)
+  int64_t ld;
+  int m, w, R;
+  int kabs;
+  int* ipiv;
+  int* info;
+  int* status;
+  int* perm;
+  ulonglong2* head;  // [PC_NBUF][G]
+  typename PrWord<T>::type* rows;  // [PC_NBUF][G][rstride]: the row's w values, its reciprocal at w
+  int rstride;
+};
+
+__host__ __device__ inline size_t pr_smem_bytes(int R, int w, int tsize) {
+  const size_t tile = ((size_t)w * (R | 1) * tsize + 15) / 16 * 16;
+  return tile + (size_t)PC_NBUF * (w + 1) * tsize + (size_t)R * sizeof(int);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(PC_NTMAX, 1) panel_resident_kernel(PrParams<T> P) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint4 red[PC_NTMAX / 32];   // each row group's best: key, position, row
+  __shared__ uint4 red2[PC_NTMAX / 32];  // each polling warp's best: key, position, CTA
+  __shared__ int abort_flag;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
+  const int cta = blockIdx.x, G = gridDim.x, GW = (G + 31) / 32;
+  const int R = P.R, w = P.w, Rs = R | 1;
+  const int64_t ld = P.ld;
+  const int row0 = cta * R;
+  const int rloc = max(0, min(P.m, row0 + R) - row0);
+  // (row groups, classes and chain warps as in panel_cluster_kernel)
+  const int RG = (R + 31) / 32;
+  const int NC = nw / RG;
+  const int rg = warp % RG, cls = warp / RG;
+  const int r = rg * 32 + lane;
+  const bool live = cls < NC && r < rloc;
+  const bool chain = warp < RG;
+  const size_t tile = ((size_t)w * Rs * sizeof(T) + 15) / 16 * 16;
+  T* S = reinterpret_cast<T*>(smem_raw);
+  T* prow = reinterpret_cast<T*>(smem_raw + tile);  // [PC_NBUF][w + 1]: pivot rows
+  int* sp = reinterpret_cast<int*>(prow + (size_t)PC_NBUF * (w + 1));  // [R] positions, at the end
+  T* Sr = S + r;
+
+  if (tid == 0) {
+    abort_flag = 0;
+    if (cta == 0) P.perm[0] = 0;
+  }
+  for (int rb = warp; rb < rloc; rb += 4 * nw) {
+    for (int c = lane; c < w; c += 32) {
+      T x[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int rr = rb + i * nw;
+        x[i] = rr < rloc ? __ldcg(P.A + (int64_t)(row0 + rr) * ld + c) : T(0);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int rr = rb + i * nw;
+        if (rr < rloc) S[(size_t)c * Rs + rr] = x[i];
+      }
+    }
+  }
+  __syncthreads();
+
+  // this CTA's candidate of column c to global memory (pr as in panel_cluster_kernel)
+  auto publish = [&](int c, int buf, PcKey best, const T* pr) {
+    if (chain) {
+      const bool own = pc_warp_best<T>(best);
+      const unsigned at = __ballot_sync(0xffffffffu, own);
+      if (lane == 0) red[warp] = make_uint4(best.hi, best.lo, (unsigned)best.pos, (unsigned)(rg * 32 + __ffs(at) - 1));
+    }
+    __syncthreads();
+    uint4 e = red[lane < RG ? lane : 0];
+    if (RG > 1) {
+      PcKey k{lane < RG ? e.x : 0u, lane < RG ? e.y : 0u, lane < RG ? (int)e.z : INT_MAX};
+      const bool own = pc_warp_best<T>(k);
+      const unsigned at = __ballot_sync(0xffffffffu, own);
+      e.w = __shfl_sync(0xffffffffu, e.w, at ? __ffs(at) - 1 : 0);
+      e.x = k.hi;
+      e.y = k.lo;
+      e.z = (unsigned)k.pos;
+    }
+    const unsigned stamp = (unsigned)c + 1u;
+    if (tid == nt - 1)
+      pr_store(P.head + (size_t)buf * G + cta,
+               make_ulonglong2(((unsigned long long)e.x << 32) | stamp,
+                               ((unsigned long long)e.y << 32) | ((e.x ? e.z : 0u) << 12) | stamp));
+    if (e.x != 0u) {
+      auto* grow = P.rows + (size_t)(buf * G + cta) * P.rstride;
+      const T* Sk = S + e.w;
+      const T lc = pr != nullptr ? Sk[(size_t)(c - 1) * Rs] : T(0);
+      for (int q = c + tid; q < w; q += nt) {
+        T v = Sk[(size_t)q * Rs];
+        if (pr != nullptr && q > c) v = fma(-lc, pr[q], v);
+        PrWord<T>::put(grow + q, v, stamp);
+      }
+      if (warp == nw - 1) {
+        const T rv = recip_rn(Sk[(size_t)c * Rs]);
+        if (lane == 0) PrWord<T>::put(grow + w, rv, stamp);
+      }
+    }
+    __syncthreads();  // (the candidate's row is read before its columns are updated)
+  };
+  // wait for a stamped value; false (and the CTA's flag) when the wait runs out
+  auto fetch = [&](const typename PrWord<T>::type* q, T& v, unsigned stamp) {
+    if (PrWord<T>::get(q, v, stamp)) return;
+    const uint64_t t0 = gtimer();
+    while (!PrWord<T>::get(q, v, stamp)) {
+      if (*(volatile int*)&abort_flag) return;
+      if (gtimer() - t0 > GB_SPIN_LIMIT_NS) {
+        atomicOr(P.status, ST_TIMEOUT);
+        *(volatile int*)&abort_flag = 1;
+        return;
+      }
+    }
+  };
+
+  int pos = row0 + r;
+  T cur = live ? Sr[0] : T(0);
+  T nxt = live && w > 1 ? Sr[(size_t)Rs] : T(0);
+  publish(0, 0, pc_key(cur, live, pos), nullptr);
+  int buf = 0;
+  bool ok = true;
+  for (int j = 0; j < w; ++j) {
+    const int nbuf = buf + 1 == PC_NBUF ? 0 : buf + 1;
+    if (warp < GW) {
+      PcKey k{0u, 0u, INT_MAX};
+      if (tid < G) {
+        const ulonglong2* hp = P.head + (size_t)buf * G + tid;
+        const unsigned stamp = (unsigned)j + 1u;
+        auto there = [&](const ulonglong2& h) { return (unsigned)h.x == stamp && ((unsigned)h.y & 0xfffu) == stamp; };
+        ulonglong2 h = pr_load(hp);
+        if (!there(h)) {
+          const uint64_t t0 = gtimer();
+          while (!there(h = pr_load(hp))) {
+            if (*(volatile int*)&abort_flag) break;
+            if (gtimer() - t0 > GB_SPIN_LIMIT_NS) {
+              atomicOr(P.status, ST_TIMEOUT);
+              *(volatile int*)&abort_flag = 1;
+              break;
+            }
+          }
+        }
+        k.hi = (unsigned)(h.x >> 32);
+        k.lo = (unsigned)(h.y >> 32);
+        k.pos = k.hi ? (int)((unsigned)h.y >> 12) : INT_MAX;
+      }
+      __syncwarp();
+      const bool own = pc_warp_best<T>(k);
+      const unsigned at = __ballot_sync(0xffffffffu, own);
+      if (lane == 0) red2[warp] = make_uint4(k.hi, k.lo, (unsigned)k.pos, (unsigned)(warp * 32 + (at ? __ffs(at) - 1 : 0)));
+    }
+    __syncthreads();
+    if (abort_flag) {  // (every thread: set before this barrier, by a poll or a fetch of the column before)
+      ok = false;
+      break;
+    }
+    // the pivot, in every warp
+    uint4 e = red2[lane < GW ? lane : 0];
+    PcKey k{lane < GW ? e.x : 0u, lane < GW ? e.y : 0u, lane < GW ? (int)e.z : INT_MAX};
+    const bool own = pc_warp_best<T>(k);
+    const unsigned at = __ballot_sync(0xffffffffu, own);
+    const int win = min((int)__shfl_sync(0xffffffffu, e.w, at ? __ffs(at) - 1 : 0), G - 1);
+    const int p = k.pos;
+    const auto* grow = P.rows + (size_t)(buf * G + win) * P.rstride;
+    T* pr = prow + (size_t)buf * (w + 1);
+    const unsigned stamp = (unsigned)j + 1u;
+    // the pivot row: what the chain needs by its warps, the rest (read after
+    // the next barrier) by the others first
+    T piv = T(0), rinv = T(0), u1 = T(0);
+    if (chain) {
+      bool got = PrWord<T>::get(grow + j, piv, stamp);
+      got &= PrWord<T>::get(grow + w, rinv, stamp);
+      if (j + 1 < w) got &= PrWord<T>::get(grow + j + 1, u1, stamp);
+      if (!got) {
+        fetch(grow + j, piv, stamp);
+        fetch(grow + w, rinv, stamp);
+        if (j + 1 < w) fetch(grow + j + 1, u1, stamp);
+      }
+    }
+    for (int q = j + 1 + (tid + nt - 32 * RG) % nt; q < w; q += nt) {
+      T v = T(0);
+      fetch(grow + q, v, stamp);
+      pr[q] = v;
+    }
+    if (live) {
+      if (pos == p)
+        pos = j;
+      else if (pos == j)
+        pos = p;
+    }
+    const bool act = live && pos > j;
+    PcKey best{0u, 0u, INT_MAX};
+    if (chain) {
+      if (cta == 0 && tid == 0) {
+        P.ipiv[P.kabs + j] = P.kabs + p + 1;
+        if (!nonzero(piv)) atomicMin(P.info, P.kabs + j + 1);
+        if (is_inf_mag(pivot_mag(piv))) atomicOr(P.status, ST_RANGE);
+      }
+      if (act) {
+        const T l = nonzero(piv) ? quot_rn(cur, piv, rinv) : cur;
+        Sr[(size_t)j * Rs] = l;
+        cur = fma(-l, u1, nxt);
+        if (j + 1 < w) {
+          Sr[(size_t)(j + 1) * Rs] = cur;
+          best = pc_key(cur, true, pos);
+        }
+      }
+    }
+    if (j + 1 == w) break;
+    publish(j + 1, nbuf, best, pr);
+    if (act) {
+      const T l = Sr[(size_t)j * Rs];
+      const size_t step = (size_t)NC * Rs;
+      int c = j + 2 + cls;
+      T* x = Sr + (size_t)c * Rs;
+      if (chain && c < w) {
+        nxt = fma(-l, pr[c], x[0]);
+        x[0] = nxt;
+        c += NC;
+        x += step;
+      }
+      for (; c + 3 * NC < w; c += 4 * NC, x += 4 * step) {
+        T v[4], u[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          v[q] = x[q * step];
+          u[q] = pr[c + q * NC];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q * step] = fma(-l, u[q], v[q]);
+      }
+      for (; c < w; c += NC, x += step) x[0] = fma(-l, pr[c], x[0]);
+    }
+    buf = nbuf;
+  }
+  __syncthreads();
+  if (!ok || abort_flag) return;
+  if (chain && live) sp[r] = pos;
+  __syncthreads();
+  for (int rr = warp; rr < rloc; rr += nw) {
+    T* dst = P.A + (int64_t)sp[rr] * ld;
+    for (int c = lane; c < w; c += 32) dst[c] = S[(size_t)c * Rs + rr];
+  }
+  if (chain && live && pos != row0 + r) {
+    const int q = atomicAdd(P.perm, 1);
+    P.perm[1 + q] = pos;
+    P.perm[1 + 2 * w + q] = row0 + r;
+  }
+}
+
+// CTAs of the grid form: at least 32 rows each, at most one per SM; 0 when the
+// tile does not fit.
+static int pr_config(int m, int w, int tsize, const DevInfo& dev, int gmax, int* R, int* nt, size_t* smem) {
+  if (w < 1 || w > 512 || m < w || gmax < 1) return 0;
+  int g = dev.sm_count < gmax ? dev.sm_count : gmax;
+  if (g > 256) g = 256;  // (a polling thread per CTA)
+  if ((int64_t)g * 32 > m) g = (int)cdiv(m, 32);
+  *R = (int)cdiv(m, g);
+  if (*R > PC_NTMAX || m >= (1 << 20)) return 0;
+  *nt = *R <= 64 ? 256 : PC_NTMAX;
+  *smem = pr_smem_bytes(*R, w, tsize);
+  if (*smem + 1024 > (size_t)dev.max_smem_optin) return 0;
+  return (int)cdiv(m, *R);
+}
+
+size_t panel_resident_bytes(int gmax, int wmax, int tsize) {
+  return 256 + (size_t)PC_NBUF * gmax * (sizeof(ulonglong2) + (size_t)(wmax + 2) * 2 * tsize);
+}
+
+template <typename T>
+int panel_resident_ctas(int m, int w, const DevInfo& dev, const PanelScratch& s) {
+  int R = 0, nt = 0;
+  size_t smem = 0;
+  return s.xres == nullptr || w > s.wmax ? 0 : pr_config(m, w, sizeof(T), dev, s.gmax, &R, &nt, &smem);
+}
+
+template <typename T>
+cudaError_t launch_panel_resident(T* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv, int* info, int* status,
+                                  const PanelScratch& s, const DevInfo& dev, cudaStream_t st) {
+  PrParams<T> P;
+  int nt = 0;
+  size_t smem = 0;
+  const int G = s.xres == nullptr ? 0 : pr_config(m, w, sizeof(T), dev, s.gmax, &P.R, &nt, &smem);
+  if (G <= 0 || w > s.wmax) return cudaErrorInvalidConfiguration;
+  cudaError_t e = allow_max_smem((const void*)panel_resident_kernel<T>);
+  if (e != cudaSuccess) return e;
+  P.A = Wkk;
+  P.ld = ldw;
+  P.m = m;
+  P.w = w;
+  P.kabs = kabs;
+  P.ipiv = ipiv;
+  P.info = info;
+  P.status = status;
+  P.perm = s.perm;
+  P.head = (ulonglong2*)s.xres;
+  P.rows = (typename PrWord<T>::type*)((char*)s.xres + ((size_t)PC_NBUF * s.gmax * sizeof(ulonglong2) + 127) / 128 * 128);
+  P.rstride = w + 2;
+  // every stamp cleared: headers and rows
+  e = cudaMemsetAsync(P.head, 0, (char*)(P.rows + (size_t)PC_NBUF * G * P.rstride) - (char*)P.head, st);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&P};
+  return launch_cooperative((const void*)panel_resident_kernel<T>, G, nt, args, smem, st);
+}
+
 #define GB_INST(T)                                                                                            \
-  template bool panel_cluster_fits<T>(int, int, const DevInfo&);                                              \
+  template int panel_resident_ctas<T>(int, int, const DevInfo&, const PanelScratch&);                         \
+  template cudaError_t launch_panel_resident<T>(T*, int64_t, int, int, int, int*, int*, int*,                 \
+                                                const PanelScratch&, const DevInfo&, cudaStream_t);           \
+  template bool panel_cluster_fits<T>(int, int, const DevInfo&, bool);                                              \
   template cudaError_t launch_panel_cluster<T>(T*, int64_t, int, int, int, int*, int*, int*, int*,            \
                                                const DevInfo&, cudaStream_t);
 GB_INST(double)

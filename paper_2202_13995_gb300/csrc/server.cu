@@ -24,7 +24,7 @@
 #include "lu_batched.h"
 #include "lu_server.h"
 
-size_t gb_fact_bytes(int n, int nrhs, lu_prec prec, int nb, int sm_count);
+size_t gb_fact_bytes(int n, int nrhs, lu_prec prec, int nb, int sm_count, int smem_optin);
 void gb_fact_rebind(lu_fact f, lu_ctx c);
 void gb_ctx_set_shared(lu_ctx c, int solve_ctas, int gemm_ctas);
 void gb_ctx_wait(lu_ctx c);
@@ -111,7 +111,7 @@ static int request_nb(lu_server s, int n) {
 }
 
 static size_t request_bytes(lu_server s, const lu_request& r) {
-  return gb_fact_bytes(r.n, r.nrhs, s->prec, request_nb(s, r.n), s->sm_count);
+  return gb_fact_bytes(r.n, r.nrhs, s->prec, request_nb(s, r.n), s->sm_count, 0);
 }
 
 // Evict least-recently-used resident factors not in use until `need` fits.

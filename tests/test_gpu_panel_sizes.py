@@ -1,6 +1,6 @@
-"""Panels at the edges of the cluster kernel's shapes (rows per CTA, CTAs per
-cluster, the last size that fits and the first that goes to the cooperative
-kernel), in arithmetic that is exact in FP32 and FP64, with a zero column and
+"""Panels at the edges of the shapes of the kernels that hold the panel in shared
+memory (rows per CTA, CTAs per cluster, the sizes around the lines between the
+cluster, the grid and the cooperative kernel), in arithmetic that is exact in FP32 and FP64, with a zero column and
 with ties across CTAs: pivots, L and U equal the oracle's bit for bit."""
 import numpy as np
 import pytest
@@ -10,7 +10,8 @@ import oracle as O
 pytestmark = pytest.mark.gpu
 
 SIZES = [(1, 1), (31, 31), (32, 5), (33, 33), (64, 64), (65, 17), (129, 100), (257, 3), (512, 64), (513, 63),
-         (1025, 33), (2049, 128), (5625, 64), (5626, 64), (8192, 32), (8193, 32)]
+         (1025, 33), (2049, 128), (5625, 64), (5626, 64), (8192, 32), (8193, 32),
+         (2187, 64), (2188, 64), (4865, 100), (6240, 128), (7001, 129), (9000, 512)]
 
 
 @pytest.fixture(scope="module")
