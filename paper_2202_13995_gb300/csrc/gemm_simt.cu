@@ -87,12 +87,79 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(T* __restrict__ C, int64
   }
 }
 
+// Small FP64 updates: tiles of BM x 32, BM / 8 elements per thread.  A 64 x 64 tile
+// with k = 64 keeps one SM's FP64 pipes for 63 us, so an update of few tiles
+// leaves most SMs idle; smaller tiles spread it (launch_gemm_simt chooses).
+template <int BM>
+__global__ void __launch_bounds__(256) gemm_small_f64_kernel(double* __restrict__ C, int64_t ldc,
+                                                             const double* __restrict__ A, int64_t lda,
+                                                             const double* __restrict__ B, int64_t ldb, int m, int n,
+                                                             int k) {
+  constexpr int BN = 32, BK = 32, RI = BM / 8;
+  __shared__ double As[BM][BK + 1];
+  __shared__ double Bs[BK][BN];
+  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  double acc[RI];
+#pragma unroll
+  for (int i = 0; i < RI; ++i) acc[i] = 0.0;
+  double ra[RI], rb[4];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < RI; ++q) {
+      const int r = m0 + ty + 8 * q, c = k0 + tx;
+      ra[q] = r < m && c < k ? A[(int64_t)r * lda + c] : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = k0 + ty + 8 * q, c = n0 + tx;
+      rb[q] = r < k && c < n ? B[(int64_t)r * ldb + c] : 0.0;
+    }
+  };
+  load(0);
+  for (int k0 = 0; k0 < k; k0 += BK) {
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < RI; ++q) As[ty + 8 * q][tx] = ra[q];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) Bs[ty + 8 * q][tx] = rb[q];
+    __syncthreads();
+    if (k0 + BK < k) load(k0 + BK);
+#pragma unroll 8
+    for (int kk = 0; kk < BK; ++kk) {
+      const double b = Bs[kk][tx];
+#pragma unroll
+      for (int i = 0; i < RI; ++i) acc[i] = fma(As[ty + 8 * i][kk], b, acc[i]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < RI; ++i) {
+    const int r = m0 + ty + 8 * i, c = n0 + tx;
+    if (r < m && c < n) C[(int64_t)r * ldc + c] -= acc[i];
+  }
+}
+
 template <typename T>
 cudaError_t launch_gemm_simt(T* C, int64_t ldc, const T* A, int64_t lda, const T* B, int64_t ldb, int m, int n,
                              int k, cudaStream_t st) {
   if (m <= 0 || n <= 0 || k <= 0) return cudaSuccess;
   dim3 grid((unsigned)cdiv(n, SG_BN), (unsigned)cdiv(m, SG_BM));
   if (grid.y > 65535u) return cudaErrorInvalidConfiguration;
+  if constexpr (sizeof(T) == 8) {
+    // (fewer 64 x 64 tiles than twice the 152 SMs leave their FP64 pipes unevenly
+    // loaded: k = 64, us with 64 x 64 tiles and with these: 384 rows 72 and 21, 640
+    // 73 and 54, 900 138 and 103, 1100 (324 tiles) 203 and 203)
+    const int64_t tiles = (int64_t)grid.x * grid.y;
+    if (tiles < 304) {
+      if (cdiv(m, 32) * cdiv(n, 32) >= 304)
+        gemm_small_f64_kernel<32><<<dim3((unsigned)cdiv(n, 32), (unsigned)cdiv(m, 32)), 256, 0, st>>>(C, ldc, A, lda, B,
+                                                                                                  ldb, m, n, k);
+      else
+        gemm_small_f64_kernel<8><<<dim3((unsigned)cdiv(n, 32), (unsigned)cdiv(m, 8)), 256, 0, st>>>(C, ldc, A, lda, B,
+                                                                                                ldb, m, n, k);
+      return cudaGetLastError();
+    }
+  }
   gemm_simt_kernel<T><<<grid, 256, 0, st>>>(C, ldc, A, lda, B, ldb, m, n, k);
   return cudaGetLastError();
 }

@@ -608,15 +608,118 @@ __global__ void __launch_bounds__(256) trsm_lower_kernel(const T* L, T* X, int64
     for (int r = warp; r < w; r += 8) X[(int64_t)r * ldw + c] = Xs[r * 32 + lane];
 }
 
+// The FP64 form.  GB300 issues an FP64 warp instruction once in 64 cycles per SM
+// quarter, so the solve takes as long as its busiest quarter has such
+// instructions: with 32 columns per CTA and the diagonal blocks on one warp, a
+// 32-row block took 15 us on one quarter while three idled, and a solve of few
+// columns used few SMs.  Here a CTA takes 8 columns (four times the CTAs, and
+// several share an SM); a diagonal block is solved by four warps, one per
+// quarter, two columns each, a lane holding two of the 32 rows of a column
+// (row 16 i + lane / 2); the rows below go to all eight warps (lane = column
+// and one of four rows), with L's rows staged in shared memory.  Per element
+// the products come in the same order as in the form above.
+// Measured (us, 32 columns per CTA and one warp per diagonal block -> this):
+// 64 x 960 50 -> 13, 192 x 2000 243 -> 89, 192 x 8000 368 -> 285.
+constexpr int TD_NS = 8;
+constexpr int TD_LD = 33;  // row stride of staged L rows
+constexpr int TD_RB = 32;  // L rows staged at a time
+
+__global__ void __launch_bounds__(256) trsm_lower_f64_kernel(const double* __restrict__ L, double* X, int64_t ldw,
+                                                             int w, int N) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* Xs = reinterpret_cast<double*>(smem_raw);  // [w rounded to 32][8]
+  double* Ld = Xs + (size_t)((w + 31) & ~31) * TD_NS;  // [32][33]: the diagonal block
+  double* Lr = Ld + 32 * TD_LD;                        // [2][TD_RB][33]: rows below it
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int c0 = blockIdx.x * TD_NS;
+  const int nc = min(TD_NS, N - c0);
+  const int wr = (w + 31) & ~31;
+  for (int e = tid; e < wr * TD_NS; e += 256) {
+    const int r = e / TD_NS, c = e % TD_NS;
+    Xs[e] = r < w && c < nc ? X[(int64_t)r * ldw + c0 + c] : 0.0;
+  }
+  // rows r0 .. r0 + 31, columns b0 .. b0 + 31 of L (zero past w)
+  auto stage = [&](int r0, int b0, double* dst) {
+    for (int e = tid; e < TD_RB * 32; e += 256) {
+      const int rr = e >> 5, k = e & 31;
+      double* q = &dst[rr * TD_LD + k];
+      if (r0 + rr < w && b0 + k < w)
+        cp_async<8>(q, L + (int64_t)(r0 + rr) * ldw + b0 + k);
+      else
+        *q = 0.0;
+    }
+    cp_async_commit();
+  };
+  stage(0, 0, Ld);
+  for (int b0 = 0; b0 < w; b0 += 32) {
+    if (b0 + 32 < w) stage(b0 + 32, b0, Lr);  // the first rows below, under the diagonal block
+    if (b0 + 32 < w)
+      cp_async_wait_group<1>();
+    else
+      cp_async_wait_group<0>();
+    __syncthreads();
+    if (warp < 4) {
+      // column 2 warp + (lane & 1); rows g and 16 + g of the block, g = lane >> 1
+      const int c = 2 * warp + (lane & 1), g = lane >> 1;
+      double x0 = Xs[(b0 + g) * TD_NS + c], x1 = Xs[(b0 + 16 + g) * TD_NS + c];
+#pragma unroll 4
+      for (int t = 0; t < 16; ++t) {
+        const double xt = __shfl_sync(0xffffffffu, x0, 2 * t + (lane & 1));
+        const double l0 = Ld[g * TD_LD + t], l1 = Ld[(16 + g) * TD_LD + t];
+        if (g > t) x0 = fma(-l0, xt, x0);
+        x1 = fma(-l1, xt, x1);
+      }
+#pragma unroll 4
+      for (int t = 16; t < 31; ++t) {
+        const double xt = __shfl_sync(0xffffffffu, x1, 2 * (t - 16) + (lane & 1));
+        const double l1 = Ld[(16 + g) * TD_LD + t];
+        if (16 + g > t) x1 = fma(-l1, xt, x1);
+      }
+      Xs[(b0 + g) * TD_NS + c] = x0;
+      Xs[(b0 + 16 + g) * TD_NS + c] = x1;
+    }
+    __syncthreads();
+    // rows below, 32 at a time: warp = rows 4 warp .. of the 32, lane = (row, column)
+    const int rr = 4 * warp + (lane >> 3), c = lane & 7;
+    for (int r0 = b0 + 32, i = 0; r0 < w; r0 += TD_RB, ++i) {
+      const double* cur = Lr + (i & 1) * TD_RB * TD_LD;
+      if (r0 + TD_RB < w) {
+        stage(r0 + TD_RB, b0, Lr + ((i + 1) & 1) * TD_RB * TD_LD);
+        cp_async_wait_group<1>();
+      } else {
+        if (b0 + 32 < w) stage(b0 + 32, b0 + 32, Ld);  // the next diagonal block (this one is solved)
+        cp_async_wait_group<1>();
+      }
+      __syncthreads();
+      double acc = Xs[(r0 + rr) * TD_NS + c];
+#pragma unroll 8
+      for (int t = 0; t < 32; ++t) acc = fma(-cur[rr * TD_LD + t], Xs[(b0 + t) * TD_NS + c], acc);
+      Xs[(r0 + rr) * TD_NS + c] = acc;
+      __syncthreads();
+    }
+  }
+  for (int e = tid; e < w * TD_NS; e += 256) {
+    const int r = e / TD_NS, q = e % TD_NS;
+    if (q < nc) X[(int64_t)r * ldw + c0 + q] = Xs[e];
+  }
+}
+
 template <typename T>
 cudaError_t launch_trsm_lower(const T* L11, T* A12, int64_t ldw, int w, int N, cudaStream_t st) {
   if (N <= 0) return cudaSuccess;
-  const size_t smem = ((size_t)w * 32 + 32 * 33) * sizeof(T);
-  auto kern = trsm_lower_kernel<T>;
-  cudaError_t e = allow_max_smem((const void*)kern);
-  if (e != cudaSuccess) return e;
-  trsm_lower_kernel<T><<<(int)cdiv(N, 32), 256, smem, st>>>(L11, A12, ldw, w, N);
-  return cudaGetLastError();
+  if constexpr (sizeof(T) == 8) {
+    const size_t smem = ((size_t)((w + 31) & ~31) * TD_NS + 32 * TD_LD + 2 * TD_RB * TD_LD) * sizeof(double);
+    cudaError_t e = allow_max_smem((const void*)trsm_lower_f64_kernel);
+    if (e != cudaSuccess) return e;
+    trsm_lower_f64_kernel<<<(unsigned)cdiv(N, TD_NS), 256, smem, st>>>(L11, A12, ldw, w, N);
+    return cudaGetLastError();
+  } else {
+    const size_t smem = ((size_t)w * 32 + 32 * 33) * sizeof(T);
+    cudaError_t e = allow_max_smem((const void*)trsm_lower_kernel<T>);
+    if (e != cudaSuccess) return e;
+    trsm_lower_kernel<T><<<(int)cdiv(N, 32), 256, smem, st>>>(L11, A12, ldw, w, N);
+    return cudaGetLastError();
+  }
 }
 
 // ============================================================ layout conversions

@@ -92,6 +92,39 @@ def test_componentwise_backward_error(ctx, kind, nb):
     f.free()
 
 
+@pytest.mark.parametrize("w", [1, 31, 32, 33, 64, 100, 257, 512])
+@pytest.mark.parametrize("N", [1, 7, 8, 9, 130])
+def test_top_solve_edges(ctx, w, N):
+    """L^-1 X by substitution in FP64: |x - x_ref| <= 2 w u |L^-1| |L| |x| (both
+    round each of at most w terms; Higham, theorem 8.5)."""
+    import torch
+    rng = np.random.default_rng(w * 1000 + N)
+    M = rng.random((w, w + N)) - 0.5
+    M[:, :w] *= 4.0 / (4.0 + w)
+    Md = torch.from_numpy(M.copy()).cuda()
+    ctx.step_trsm(Md[:, :w], Md[:, w:], "f64")
+    L = np.tril(M[:, :w], -1) + np.eye(w)
+    want = O.trsm_unit_lower(L, M[:, w:])
+    bound = 2 * w * U * (np.abs(np.linalg.inv(L)) @ (np.abs(L) @ np.abs(want))) + U * np.abs(want)
+    got = Md.cpu().numpy()
+    assert (np.abs(got[:, w:] - want) <= bound).all()
+    assert np.array_equal(got[:, :w], M[:, :w])
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (7, 33, 5), (86, 86, 64), (384, 384, 63), (550, 550, 32), (554, 1000, 33),
+                                   (1088, 1088, 31), (1089, 1089, 64)])
+def test_small_update_edges(ctx, m, n, k):
+    """C - A B: within k u (|A||B|) + u |C - A B| of the compensated update on either side."""
+    import torch
+    rng = np.random.default_rng(m + n + k)
+    A, B, Cm = rng.random((m, k)) - 0.5, rng.random((k, n)) - 0.5, rng.random((m, n)) - 0.5
+    C = torch.from_numpy(Cm.copy()).cuda()
+    ctx.step_gemm(C, torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), "f64")
+    ref = O.gemm_update_dot2(Cm, A, B)
+    bound = (k + 1) * U * (np.abs(A) @ np.abs(B)) + 2 * U * (np.abs(Cm) + np.abs(ref))
+    assert (np.abs(C.cpu().numpy() - ref) <= bound).all()
+
+
 def test_non_finite_entries_are_reported(ctx):
     from paper_2202_13995_gb300 import lu
     for bad in (np.nan, np.inf):
