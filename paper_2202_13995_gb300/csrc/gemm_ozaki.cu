@@ -784,11 +784,35 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       der = rok ? P.ea[row] - (OZ_F + 2 * OZ_BITS) : 0;
     }
     if (ok && dcrow != nullptr) {
-      // the last tile's update
+      // the last tile's update: nothing left to run it under, so its loads go
+      // out four column pairs at a time
 #pragma unroll 1
-      for (int i = 0; i < kn; ++i) {
-        defer_issue(i * kstep + gq);
-        defer_complete();
+      for (int i = 0; i < kn; i += 4) {
+        long long bI[4][2];
+        double bC[4][2];
+        int bF[4][2], bk[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          defer_issue((i + u) * kstep + gq);
+          bk[u] = qk;
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            bI[u][x] = qI[x];
+            bC[u][x] = qC[x];
+            bF[u][x] = qF[x];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          qk = bk[u];
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            qI[x] = bI[u][x];
+            qC[x] = bC[u][x];
+            qF[x] = bF[u][x];
+          }
+          defer_complete();
+        }
       }
     }
   }
