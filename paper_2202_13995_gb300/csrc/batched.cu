@@ -53,9 +53,19 @@ struct BatchSmem {
 };
 // refinement phase views (alias P/Us): x (FP64), r (FP64), y (FP32), 8 x 512 each
 static_assert(sizeof(float) * BT_NB * (BT_NMAX + BT_CW) >=
-                  2 * sizeof(double) * BT_RHSMAX * BT_NMAX + sizeof(float) * BT_RHSMAX * BT_NMAX,
-              "refinement vectors must fit in the factor-phase buffers");
+                  2 * sizeof(double) * BT_RHSMAX * BT_NMAX + sizeof(float) * BT_RHSMAX * BT_NMAX +
+                      sizeof(double) * 8 * BT_RHSMAX * 32,
+              "refinement vectors and the residual's partial sums must fit in the factor-phase buffers");
 static_assert(3 * BT_RHSMAX * 32 >= 16 * 32 + 32, "block_max_many needs 16 warps x 32 + 32 slots");
+
+__device__ __forceinline__ BatchSmem& bt_smem() {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  return *reinterpret_cast<BatchSmem*>(smem_raw);
+}
+// the refinement's vectors, behind one another from P on
+__device__ __forceinline__ double* bt_x(BatchSmem& sm) { return reinterpret_cast<double*>(&sm.P[0][0]); }
+__device__ __forceinline__ double* bt_r(BatchSmem& sm) { return bt_x(sm) + BT_RHSMAX * BT_NMAX; }
+__device__ __forceinline__ float* bt_y(BatchSmem& sm) { return reinterpret_cast<float*>(bt_r(sm) + BT_RHSMAX * BT_NMAX); }
 
 __device__ __forceinline__ void block_argmax_f(float& v, int& i, BatchSmem& sm, int nt) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -206,107 +216,254 @@ __device__ int bt_factor(float* W, int ld, int n, BatchSmem& sm, int* status) {
   return info;
 }
 
-// y <- U^-1 L^-1 (P rhs) in FP32 for nr right-hand sides held in y[q][0..n)
-// (already gathered through perm).  Blocked by 32: one warp per right-hand side
-// solves a diagonal block, then all threads update the rows beyond it.
+// W <- A (FP64 column-major -> FP32 row-major), 32 rows x 128 columns at a time
+// through four 32 x 32 tiles in the (still unused) panel buffer: sixteen loads
+// per thread in flight instead of four.
+// (bt_convert, bt_invert and bt_solve are calls of their own: inlined, their
+// registers and the residual's maxima would not fit two CTAs per SM)
 template <int NT>
-__device__ void bt_solve(const float* W, int ld, int n, int nr, float* y, BatchSmem& sm) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // forward, unit lower
-  for (int b0 = 0; b0 < n; b0 += BT_NB) {
-    const int bw = min(BT_NB, n - b0);
-    for (int e = tid; e < BT_NB * BT_NB; e += NT) {
-      const int r = e / BT_NB, c = e % BT_NB;
-      sm.Ld[r][c] = (r < bw && c < bw) ? W[(int64_t)sm.perm[b0 + r] * ld + b0 + c] : 0.0f;
-    }
-    __syncthreads();
-    for (int q = warp; q < nr; q += NT / 32) {
-      float x = lane < bw ? y[q * BT_NMAX + b0 + lane] : 0.0f;
-      for (int t = 0; t < bw; ++t) {
-        const float xt = __shfl_sync(0xffffffffu, x, t);
-        if (lane > t) x -= sm.Ld[lane][t] * xt;
-      }
-      if (lane < bw) y[q * BT_NMAX + b0 + lane] = x;
-    }
-    __syncthreads();
-    for (int r = b0 + bw + tid; r < n; r += NT) {
-      const float* wr = W + (int64_t)sm.perm[r] * ld + b0;
-      float l[BT_NB];
+__device__ __noinline__ void bt_convert(const double* A, int lda, float* W, int ld, int n) {
+  BatchSmem& sm = bt_smem();
+  const int tid = threadIdx.x;
+  constexpr int TW = BT_NB * (BT_NB + 1);
+  float* T = &sm.P[0][0];  // [4][32][33]
+  constexpr int PER = 4 * BT_NB * BT_NB / NT;
+  for (int i0 = 0; i0 < n; i0 += BT_NB) {
+    for (int j0 = 0; j0 < n; j0 += 4 * BT_NB) {
+      double v[PER];
 #pragma unroll
-      for (int t = 0; t < BT_NB; ++t) l[t] = t < bw ? wr[t] : 0.0f;
-      for (int q = 0; q < nr; ++q) {
-        float v = y[q * BT_NMAX + r];
-#pragma unroll
-        for (int t = 0; t < BT_NB; ++t)
-          if (t < bw) v -= l[t] * y[q * BT_NMAX + b0 + t];
-        y[q * BT_NMAX + r] = v;
+      for (int u = 0; u < PER; ++u) {
+        const int e = tid + u * NT, i = e % BT_NB, j = e / BT_NB;
+        v[u] = (i0 + i < n && j0 + j < n) ? A[(int64_t)(j0 + j) * lda + i0 + i] : 0.0;
       }
-    }
-    __syncthreads();
-  }
-  // backward, upper
-  const int nblk = (n + BT_NB - 1) / BT_NB;
-  for (int bi = nblk - 1; bi >= 0; --bi) {
-    const int b0 = bi * BT_NB;
-    const int bw = min(BT_NB, n - b0);
-    for (int e = tid; e < BT_NB * BT_NB; e += NT) {
-      const int r = e / BT_NB, c = e % BT_NB;
-      sm.Ld[r][c] = (r < bw && c < bw) ? W[(int64_t)sm.perm[b0 + r] * ld + b0 + c] : 0.0f;
-    }
-    __syncthreads();
-    for (int q = warp; q < nr; q += NT / 32) {
-      float x = lane < bw ? y[q * BT_NMAX + b0 + lane] : 0.0f;
-      for (int t = bw - 1; t >= 0; --t) {
-        if (lane == t) x = x / sm.Ld[t][t];
-        const float xt = __shfl_sync(0xffffffffu, x, t);
-        if (lane < t) x -= sm.Ld[lane][t] * xt;
-      }
-      if (lane < bw) y[q * BT_NMAX + b0 + lane] = x;
-    }
-    __syncthreads();
-    for (int r = tid; r < b0; r += NT) {
-      const float* wr = W + (int64_t)sm.perm[r] * ld + b0;
-      float u[BT_NB];
 #pragma unroll
-      for (int t = 0; t < BT_NB; ++t) u[t] = t < bw ? wr[t] : 0.0f;
-      for (int q = 0; q < nr; ++q) {
-        float v = y[q * BT_NMAX + r];
-#pragma unroll
-        for (int t = 0; t < BT_NB; ++t)
-          if (t < bw) v -= u[t] * y[q * BT_NMAX + b0 + t];
-        y[q * BT_NMAX + r] = v;
+      for (int u = 0; u < PER; ++u) {
+        const int e = tid + u * NT, i = e % BT_NB, j = e / BT_NB;
+        T[(j / BT_NB) * TW + (j % BT_NB) * (BT_NB + 1) + i] = (float)v[u];
       }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < PER; ++u) {
+        const int e = tid + u * NT, j = e % (4 * BT_NB), i = e / (4 * BT_NB);
+        if (i0 + i < n && j0 + j < n)
+          W[(int64_t)(i0 + i) * ld + j0 + j] = T[(j / BT_NB) * TW + (j % BT_NB) * (BT_NB + 1) + i];
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
 }
 
-// r = b - A x in FP64 for the rows of this thread (A FP64 column-major), with
-// the column maxima of |r|, |x|, |b| and, on the first pass, the row sums of |A|.
-template <int NR, bool FIRST>
-__device__ __forceinline__ void bt_resid_rows(const BatchDesc& d, int n, const double* xs, double* rs, double& amax,
-                                              double* rmax, double* xmax, double* bmax, int tid, int nt) {
-  for (int i = tid; i < n; i += nt) {
-    double acc[NR];
+// The factors' 32 x 32 diagonal blocks replaced by the inverses of their two
+// triangles (unit lower strictly below the diagonal, upper on and above it),
+// which only the solves below read: their serial substitutions become products
+// (in FP32, as in the refinement's solves of large systems; the refinement
+// corrects the rounding).  A warp per block, a lane per column of the inverses.
+template <int NT>
+__device__ __noinline__ void bt_invert(float* W, int ld, int n) {
+  BatchSmem& sm = bt_smem();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int NW = NT / 32, TW = BT_NB * (BT_NB + 1);
+  static_assert(NW * TW <= BT_NB * (BT_NMAX + BT_CW), "a block per warp in the factor-phase buffers");
+  float* D = &sm.P[0][0] + warp * TW;  // [32][33]
+  const int nblk = (n + BT_NB - 1) / BT_NB;
+  for (int b = warp; b < nblk; b += NW) {
+    const int b0 = b * BT_NB, bw = min(BT_NB, n - b0);
+#pragma unroll 8
+    for (int r = 0; r < BT_NB; ++r)
+      D[r * (BT_NB + 1) + lane] = r < bw && lane < bw ? W[(int64_t)sm.perm[b0 + r] * ld + b0 + lane] : (r == lane ? 1.0f : 0.0f);
+    __syncwarp();
+    // (one triangle after the other: 32 registers of results at a time)
+    float z[BT_NB];
 #pragma unroll
-    for (int q = 0; q < NR; ++q) {
-      acc[q] = d.B[(int64_t)q * d.ldb + i];
-      bmax[q] = fmax(bmax[q], fabs(acc[q]));
-    }
-    double asum = 0.0;
-    for (int j = 0; j < n; ++j) {
-      const double a = d.A[(int64_t)j * d.lda + i];
-      if (FIRST) asum += fabs(a);
+    for (int t = 0; t < BT_NB; ++t) z[t] = t == lane ? 1.0f : 0.0f;
 #pragma unroll
-      for (int q = 0; q < NR; ++q) acc[q] = fma(-a, xs[q * BT_NMAX + j], acc[q]);
-    }
-    amax = fmax(amax, asum);
+    for (int t = 0; t < BT_NB - 1; ++t)
 #pragma unroll
-    for (int q = 0; q < NR; ++q) {
-      rs[q * BT_NMAX + i] = acc[q];
-      rmax[q] = fmax(rmax[q], fabs(acc[q]));
-      xmax[q] = fmax(xmax[q], fabs(xs[q * BT_NMAX + i]));
+      for (int q = t + 1; q < BT_NB; ++q) z[q] = fmaf(-D[q * (BT_NB + 1) + t], z[t], z[q]);
+#pragma unroll
+    for (int t = 0; t < BT_NB; ++t)
+      if (t < bw && t > lane) W[(int64_t)sm.perm[b0 + t] * ld + b0 + lane] = z[t];
+    const float rinv = 1.0f / D[lane * (BT_NB + 1) + lane];
+#pragma unroll
+    for (int t = 0; t < BT_NB; ++t) z[t] = t == lane ? 1.0f : 0.0f;
+#pragma unroll
+    for (int t = BT_NB - 1; t >= 0; --t) {
+      z[t] *= __shfl_sync(0xffffffffu, rinv, t);
+#pragma unroll
+      for (int q = 0; q < t; ++q) z[q] = fmaf(-D[q * (BT_NB + 1) + t], z[t], z[q]);
     }
+#pragma unroll
+    for (int t = 0; t < BT_NB; ++t)
+      if (t <= lane && lane < bw) W[(int64_t)sm.perm[b0 + t] * ld + b0 + lane] = z[t];
+    __syncwarp();
+  }
+  __syncthreads();
+}
+
+// y <- U^-1 L^-1 (P rhs) in FP32 for nr right-hand sides held in y[q][0..n)
+// (already gathered through perm).  Blocked by 32: one warp per right-hand side
+// multiplies by the diagonal block's inverse (bt_invert), then all threads
+// update the rows beyond it, a row per thread, whose entries were loaded
+// before the product; the next diagonal block's are on their way meanwhile.
+template <int NT>
+__device__ __noinline__ void bt_solve(const float* W, int ld, int n, int nr) {
+  BatchSmem& sm = bt_smem();
+  float* y = bt_y(sm);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int PER = BT_NB * BT_NB / NT;
+  const int nblk = (n + BT_NB - 1) / BT_NB;
+#pragma unroll 1
+  for (int dir = 0; dir < 2; ++dir) {  // forward (unit lower), backward (upper)
+    const bool fwd = dir == 0;
+    auto block_at = [&](int i) { return (fwd ? i : nblk - 1 - i) * BT_NB; };
+    float dv[PER];
+    auto load_diag = [&](int b0) {
+      const int bw = min(BT_NB, n - b0);
+#pragma unroll
+      for (int u = 0; u < PER; ++u) {
+        const int e = tid + u * NT, r = e / BT_NB, c = e % BT_NB;
+        dv[u] = (r < bw && c < bw) ? W[(int64_t)sm.perm[b0 + r] * ld + b0 + c] : 0.0f;
+      }
+    };
+    load_diag(block_at(0));
+    for (int ib = 0; ib < nblk; ++ib) {
+      const int b0 = block_at(ib), bw = min(BT_NB, n - b0);
+#pragma unroll
+      for (int u = 0; u < PER; ++u) {
+        const int e = tid + u * NT;
+        sm.Ld[e / BT_NB][e % BT_NB] = dv[u];
+      }
+      // this thread's first row beyond the block
+      const int lo = fwd ? b0 + bw : 0, hi = fwd ? n : b0;
+      float l[BT_NB];
+      auto load_row = [&](int r) {
+        const float* wr = W + (int64_t)sm.perm[r] * ld + b0;  // 16-byte aligned: ld and b0 are multiples of 4
+        if (bw == BT_NB) {
+#pragma unroll
+          for (int t = 0; t < BT_NB; t += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(wr + t);
+            l[t] = v.x;
+            l[t + 1] = v.y;
+            l[t + 2] = v.z;
+            l[t + 3] = v.w;
+          }
+        } else {
+#pragma unroll
+          for (int t = 0; t < BT_NB; ++t) l[t] = t < bw ? wr[t] : 0.0f;
+        }
+      };
+      if (lo + tid < hi) load_row(lo + tid);
+      __syncthreads();
+      for (int q = warp; q < nr; q += NT / 32) {
+        float* yb = y + q * BT_NMAX + b0;
+        const float yl = lane < bw ? yb[lane] : 0.0f;
+        float x[4] = {fwd ? yl : 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int t = 0; t < BT_NB; ++t) {
+          const float m = sm.Ld[lane][t], yt = __shfl_sync(0xffffffffu, yl, t);
+          if (fwd ? t < lane : t >= lane) x[t & 3] = fmaf(m, yt, x[t & 3]);
+        }
+        if (lane < bw) yb[lane] = (x[0] + x[1]) + (x[2] + x[3]);
+      }
+      if (ib + 1 < nblk) load_diag(block_at(ib + 1));
+      __syncthreads();
+      for (int r = lo + tid; r < hi; r += NT) {
+        if (r != lo + tid) load_row(r);
+        for (int q = 0; q < nr; ++q) {
+          const float4* yb = reinterpret_cast<const float4*>(y + q * BT_NMAX + b0);
+          float v = y[q * BT_NMAX + r];
+#pragma unroll
+          for (int t = 0; t < BT_NB; t += 4) {
+            const float4 y4 = yb[t / 4];  // (zero past a ragged block)
+            v = fmaf(-l[t], y4.x, v);
+            v = fmaf(-l[t + 1], y4.y, v);
+            v = fmaf(-l[t + 2], y4.z, v);
+            v = fmaf(-l[t + 3], y4.w, v);
+          }
+          y[q * BT_NMAX + r] = v;
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// r = b - A x in FP64 (A FP64 column-major), with the column maxima of |r|,
+// |x|, |b| and, on the first pass, the row sums of |A|.  Bound by the FP64
+// pipes (two multiply-adds per clock and SM), so every warp gets the same
+// number of warp instructions: 32 rows at a time, the columns in BT_KS slices,
+// a slice per warp, and the slices' sums added in order (a row per thread left
+// most warps idle on the last rows).  The slices do not depend on the launch
+// shape: with 16 warps each half takes every other group of rows.
+constexpr int BT_KS = 8;
+template <int NR, bool FIRST, int NT>
+__device__ __forceinline__ void bt_resid_rows(const BatchDesc& d, int n, const double* xs, double* rs, double* part,
+                                              double* apart, double& amax, double* rmax, double* xmax, double* bmax) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NG = NT / 32 / BT_KS;  // row groups at a time
+  const int ks = warp % BT_KS, g = warp / BT_KS;
+  const int j0 = n * ks / BT_KS, j1 = n * (ks + 1) / BT_KS;
+  for (int i0 = 0; i0 < n; i0 += 32 * NG) {
+    const int i = i0 + 32 * g + lane;
+    double acc[NR], asum = 0.0;
+#pragma unroll
+    for (int q = 0; q < NR; ++q) acc[q] = 0.0;
+    if (i < n) {
+      const double* ap = d.A + (int64_t)j0 * d.lda + i;
+      int j = j0;
+      for (; j + 4 <= j1; j += 4, ap += 4 * (int64_t)d.lda) {
+        double a[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] = ap[u * (int64_t)d.lda];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (FIRST) asum += fabs(a[u]);
+#pragma unroll
+          for (int q = 0; q < NR; ++q) acc[q] = fma(a[u], xs[q * BT_NMAX + j + u], acc[q]);
+        }
+      }
+      for (; j < j1; ++j, ap += d.lda) {
+        const double a = *ap;
+        if (FIRST) asum += fabs(a);
+#pragma unroll
+        for (int q = 0; q < NR; ++q) acc[q] = fma(a, xs[q * BT_NMAX + j], acc[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NR; ++q) part[((g * BT_KS + ks) * NR + q) * 32 + lane] = acc[q];
+    if (FIRST) apart[(g * BT_KS + ks) * 32 + lane] = asum;
+    __syncthreads();
+    for (int e = tid; e < 32 * NG * NR; e += NT) {
+      const int l = e & 31, gq = e >> 5, q = gq % NR, gg = gq / NR;
+      const int r = i0 + 32 * gg + l;
+      if (r < n) {
+        const double bv = d.B[(int64_t)q * d.ldb + r];
+        double sum = part[(gg * BT_KS * NR + q) * 32 + l];
+#pragma unroll
+        for (int k = 1; k < BT_KS; ++k) sum += part[((gg * BT_KS + k) * NR + q) * 32 + l];
+        const double rv = bv - sum;
+        rs[q * BT_NMAX + r] = rv;
+        const double xv = fabs(xs[q * BT_NMAX + r]);
+#pragma unroll
+        for (int u = 0; u < NR; ++u) {  // (a static index into the maxima)
+          if (u == q) {
+            rmax[u] = fmax(rmax[u], fabs(rv));
+            xmax[u] = fmax(xmax[u], xv);
+            bmax[u] = fmax(bmax[u], fabs(bv));
+          }
+        }
+      }
+    }
+    if (FIRST && tid < 32 * NG) {
+      const int gg = tid >> 5;
+      if (i0 + tid < n) {
+        double sum = 0.0;
+#pragma unroll
+        for (int k = 0; k < BT_KS; ++k) sum += apart[(gg * BT_KS + k) * 32 + lane];
+        amax = fmax(amax, sum);
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -336,15 +493,16 @@ __device__ __forceinline__ const double* block_max_many(const double* rmax, cons
 }
 
 template <int NT>
-__global__ void __launch_bounds__(NT) batched_kernel(const BatchDesc* __restrict__ desc, const int* __restrict__ order,
+__global__ void __launch_bounds__(NT, 512 / NT) batched_kernel(const BatchDesc* __restrict__ desc, const int* __restrict__ order,
                                                      int count, int* next, float* scratch, int64_t slot_floats,
                                                      int* info_out, int* iters_out, double* resid_out, double tol,
                                                      int max_iter, int* status) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  BatchSmem& sm = *reinterpret_cast<BatchSmem*>(smem_raw);
-  double* xs = reinterpret_cast<double*>(&sm.P[0][0]);  // [8][512] FP64
-  double* rs = xs + BT_RHSMAX * BT_NMAX;                // [8][512] FP64
-  float* ys = reinterpret_cast<float*>(rs + BT_RHSMAX * BT_NMAX);  // [8][512] FP32
+  BatchSmem& sm = bt_smem();
+  double* xs = bt_x(sm);  // [8][512] FP64
+  double* rs = bt_r(sm);  // [8][512] FP64
+  float* ys = bt_y(sm);   // [8][512] FP32
+  // the residual's partial sums, from y on (y is gathered anew after it)
+  double* part = reinterpret_cast<double*>(ys);
   const int tid = threadIdx.x;
   float* W = scratch + (int64_t)blockIdx.x * slot_floats;
   const double eps = 1.1102230246251565e-16;  // 2^-53
@@ -359,21 +517,7 @@ __global__ void __launch_bounds__(NT) batched_kernel(const BatchDesc* __restrict
     const BatchDesc d = desc[sys];
     const int n = d.n, nr = d.nrhs;
     const int ld = (n + 3) & ~3;
-    // W <- A (FP64 column-major -> FP32 row-major), through 32 x 32 tiles
-    for (int i0 = 0; i0 < n; i0 += BT_NB) {
-      for (int j0 = 0; j0 < n; j0 += BT_NB) {
-        for (int e = tid; e < BT_NB * BT_NB; e += NT) {
-          const int i = e % BT_NB, j = e / BT_NB;
-          sm.Ld[j][i] = (i0 + i < n && j0 + j < n) ? (float)d.A[(int64_t)(j0 + j) * d.lda + i0 + i] : 0.0f;
-        }
-        __syncthreads();
-        for (int e = tid; e < BT_NB * BT_NB; e += NT) {
-          const int j = e % BT_NB, i = e / BT_NB;
-          if (i0 + i < n && j0 + j < n) W[(int64_t)(i0 + i) * ld + j0 + j] = sm.Ld[j][i];
-        }
-        __syncthreads();
-      }
-    }
+    bt_convert<NT>(d.A, d.lda, W, ld, n);
     const int info = bt_factor<NT>(W, ld, n, sm, status);
     if (info != 0) {
       if (tid == 0) {
@@ -384,13 +528,16 @@ __global__ void __launch_bounds__(NT) batched_kernel(const BatchDesc* __restrict
       __syncthreads();
       continue;
     }
+    bt_invert<NT>(W, ld, n);
     // x0 = solve(b)
-    for (int e = tid; e < nr * n; e += NT) {
-      const int q = e / n, r = e % n;
-      ys[q * BT_NMAX + r] = (float)d.B[(int64_t)q * d.ldb + sm.perm[r]];
+    // (zero up to a whole block: bt_solve's products read past a ragged one)
+    const int npad = (n + BT_NB - 1) / BT_NB * BT_NB;
+    for (int e = tid; e < nr * npad; e += NT) {
+      const int q = e / npad, r = e % npad;
+      ys[q * BT_NMAX + r] = r < n ? (float)d.B[(int64_t)q * d.ldb + sm.perm[r]] : 0.0f;
     }
     __syncthreads();
-    bt_solve<NT>(W, ld, n, nr, ys, sm);
+    bt_solve<NT>(W, ld, n, nr);
     for (int e = tid; e < nr * n; e += NT) {
       const int q = e / n, r = e % n;
       xs[q * BT_NMAX + r] = (double)ys[q * BT_NMAX + r];
@@ -411,9 +558,9 @@ __global__ void __launch_bounds__(NT) batched_kernel(const BatchDesc* __restrict
 #define GB_RESID_CASE(NRC)                                                              \
   case NRC:                                                                             \
     if (it == 0)                                                                        \
-      bt_resid_rows<NRC, true>(d, n, xs, rs, amax, rmax, xmax, bmax, tid, NT);          \
+      bt_resid_rows<NRC, true, NT>(d, n, xs, rs, part, sm.redd, amax, rmax, xmax, bmax);          \
     else                                                                                \
-      bt_resid_rows<NRC, false>(d, n, xs, rs, amax, rmax, xmax, bmax, tid, NT);         \
+      bt_resid_rows<NRC, false, NT>(d, n, xs, rs, part, sm.redd, amax, rmax, xmax, bmax);         \
     break;
       switch (nr) {
         GB_RESID_CASE(1)
@@ -454,12 +601,12 @@ __global__ void __launch_bounds__(NT) batched_kernel(const BatchDesc* __restrict
       }
       // d = solve(r) in FP32, x += d for the columns not yet converged
       __syncthreads();
-      for (int e = tid; e < nr * n; e += NT) {
-        const int q = e / n, r = e % n;
-        ys[q * BT_NMAX + r] = (float)rs[q * BT_NMAX + sm.perm[r]];
+      for (int e = tid; e < nr * npad; e += NT) {
+        const int q = e / npad, r = e % npad;
+        ys[q * BT_NMAX + r] = r < n ? (float)rs[q * BT_NMAX + sm.perm[r]] : 0.0f;
       }
       __syncthreads();
-      bt_solve<NT>(W, ld, n, nr, ys, sm);
+      bt_solve<NT>(W, ld, n, nr);
       for (int e = tid; e < nr * n; e += NT) {
         const int q = e / n, r = e % n;
         if ((active >> q) & 1u) xs[q * BT_NMAX + r] += (double)ys[q * BT_NMAX + r];
