@@ -46,8 +46,6 @@ struct BatchSmem {
   float Us[BT_NB][BT_CW];   // U12 chunk
   int perm[BT_NMAX];
   float Ld[BT_NB][BT_NB + 1];
-  float redf[32];
-  int redi[32];
   double redd[3 * BT_RHSMAX * 32];  // >= 16 warps x 32 + 32
   int misc[8];
 };
@@ -67,17 +65,174 @@ __device__ __forceinline__ double* bt_x(BatchSmem& sm) { return reinterpret_cast
 __device__ __forceinline__ double* bt_r(BatchSmem& sm) { return bt_x(sm) + BT_RHSMAX * BT_NMAX; }
 __device__ __forceinline__ float* bt_y(BatchSmem& sm) { return reinterpret_cast<float*>(bt_r(sm) + BT_RHSMAX * BT_NMAX); }
 
-__device__ __forceinline__ void block_argmax_f(float& v, int& i, BatchSmem& sm, int nt) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  warp_argmax(v, i);
-  if (lane == 0) {
-    sm.redf[warp] = v;
-    sm.redi[warp] = i;
+// The panel's scratch in the (in this phase unused) reduction buffer.
+struct BtPanel {
+  uint2 best[2][16];              // per column parity and warp: key, position
+  float cand[2][16][8];           // ... and the candidate row's sub-block
+  float U[BT_NB][8];              // column c: the sub-block's eight U rows
+  int phys[BT_NB];                // pivot j's row
+};
+static_assert(sizeof(BtPanel) <= sizeof(double) * 3 * BT_RHSMAX * 32, "panel scratch");
+
+// The m x kb panel P (column-major in shared memory), rows eliminated with
+// partial pivoting; returns the first zero pivot (1-based within the panel) or
+// 0.  A thread holds its rows' eight columns of a sub-block in registers; rows
+// stay where they are and carry their position, as in the panel kernels.  Per
+// column: the warps' best candidates and their rows go to shared memory, one
+// barrier, and every thread picks the pivot and updates its rows.  Per
+// sub-block: the pivot rows' remaining columns (a thread per column), then a
+// rank-8 update of the other rows.  At the end the rows move to their positions.
+// (Three barriers and a loop over all remaining columns in shared memory per
+// column took 2300 cycles a column with 300 rows; the products of an element
+// come in the same order.)
+template <int NT>
+__device__ __noinline__ int bt_panel(int m, int kb, int k0, int* status) {
+  BatchSmem& sm = bt_smem();
+  constexpr int RPT = BT_NMAX / NT, NW = NT / 32;
+  BtPanel& ps = *reinterpret_cast<BtPanel*>(sm.redd);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int info = 0;
+  int pos[RPT];
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) pos[i] = tid + i * NT < m ? tid + i * NT : -1;
+  for (int jb = 0; jb < kb; jb += 8) {
+    float a[RPT][8];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) a[i][e] = tid + i * NT < m ? sm.P[jb + e][tid + i * NT] : 0.0f;
+#pragma unroll
+    for (int jj = 0; jj < 8; ++jj) {
+      const int j = jb + jj;
+      if (j < kb) {
+        const int par = jj & 1;
+        // this thread's candidate: key (magnitude bits + 1), then the lowest position
+        unsigned key = 0u, kp = 0xffffffffu;
+        int ki = 0;
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+          if (pos[i] >= j) {
+            const float v = a[i][jj];
+            if (v != v) atomicOr(status, ST_RANGE);
+            const unsigned kv = __float_as_uint(pivot_mag(v)) + 1u;
+            if (kv > key || (kv == key && (unsigned)pos[i] < kp)) {
+              key = kv;
+              kp = (unsigned)pos[i];
+              ki = i;
+            }
+          }
+        }
+        const unsigned mk = __reduce_max_sync(0xffffffffu, key);
+        const unsigned mp = __reduce_min_sync(0xffffffffu, key == mk ? kp : 0xffffffffu);
+        if (mk != 0u && key == mk && kp == mp) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            float v = a[0][e];
+#pragma unroll
+            for (int i = 1; i < RPT; ++i) v = ki == i ? a[i][e] : v;
+            ps.cand[par][warp][e] = v;
+          }
+        }
+        if (lane == 0) ps.best[par][warp] = make_uint2(mk, mp);
+        __syncthreads();
+        const uint2 b = ps.best[par][lane < NW ? lane : 0];
+        const unsigned bk = lane < NW ? b.x : 0u;
+        const unsigned gk = __reduce_max_sync(0xffffffffu, bk);
+        const unsigned gp = __reduce_min_sync(0xffffffffu, bk == gk ? b.y : 0xffffffffu);
+        const unsigned at = __ballot_sync(0xffffffffu, bk == gk && b.y == gp);
+        const int win = __ffs(at) - 1;
+        int p = (int)gp;
+        if (!GB_IN_BOUNDS(status, p >= j && p < m)) p = j;
+        float u[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) u[e] = ps.cand[par][win][e];
+        const float piv = u[jj];
+        if (piv == 0.0f && info == 0) info = j + 1;
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+          if (pos[i] == p) {
+            pos[i] = j;
+            ps.phys[j] = tid + i * NT;
+          } else if (pos[i] == j) {
+            pos[i] = p;
+          }
+          if (pos[i] > j) {
+            float l = a[i][jj];
+            if (piv != 0.0f) l = l / piv;
+            a[i][jj] = l;
+#pragma unroll
+            for (int e = jj + 1; e < 8; ++e) a[i][e] = fmaf(-l, u[e], a[i][e]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (tid + i * NT < m) sm.P[jb + e][tid + i * NT] = a[i][e];
+    __syncthreads();
+    if (jb + 8 >= kb) break;
+    // the pivot rows' columns right of the sub-block
+    if (tid < kb - (jb + 8)) {
+      const int c = jb + 8 + tid;
+      float x[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) x[t] = sm.P[c][ps.phys[jb + t]];
+#pragma unroll
+      for (int t = 1; t < 8; ++t)
+#pragma unroll
+        for (int q = 0; q < t; ++q) x[t] = fmaf(-sm.P[jb + q][ps.phys[jb + t]], x[q], x[t]);
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        ps.U[c][t] = x[t];
+        sm.P[c][ps.phys[jb + t]] = x[t];
+      }
+    }
+    __syncthreads();
+    // the rows below them
+#pragma unroll 2
+    for (int c = jb + 8; c < kb; ++c) {
+      float u[8];
+      *reinterpret_cast<float4*>(u) = *reinterpret_cast<const float4*>(&ps.U[c][0]);
+      *reinterpret_cast<float4*>(u + 4) = *reinterpret_cast<const float4*>(&ps.U[c][4]);
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) {
+        if (pos[i] >= jb + 8) {
+          float y = sm.P[c][tid + i * NT];
+#pragma unroll
+          for (int t = 0; t < 8; ++t) y = fmaf(-a[i][t], u[t], y);
+          sm.P[c][tid + i * NT] = y;
+        }
+      }
+    }
+    // (a thread reads its own rows next; the pivot rows are final)
   }
+  // rows to their positions, sixteen columns at a time
+  int pr[RPT];
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) pr[i] = pos[i] >= 0 ? sm.perm[k0 + tid + i * NT] : 0;
+#pragma unroll 1
+  for (int c0 = 0; c0 < kb; c0 += 16) {
+    float v[RPT][16];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+#pragma unroll
+      for (int c = 0; c < 16; ++c) v[i][c] = pos[i] >= 0 ? sm.P[c0 + c][tid + i * NT] : 0.0f;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+      if (pos[i] >= 0) {
+#pragma unroll
+        for (int c = 0; c < 16; ++c) sm.P[c0 + c][pos[i]] = v[i][c];
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < RPT; ++i)
+    if (pos[i] >= 0) sm.perm[k0 + pos[i]] = pr[i];
   __syncthreads();
-  v = lane < nt / 32 ? sm.redf[lane] : -1.0f;
-  i = lane < nt / 32 ? sm.redi[lane] : INT_MAX;
-  warp_argmax(v, i);  // every warp computes the same result
+  return info;
 }
 
 // FP32 LU with partial pivoting of the n x n row-major W (ld), rows through perm.
@@ -108,38 +263,8 @@ __device__ int bt_factor(float* W, int ld, int n, BatchSmem& sm, int* status) {
       }
     }
     __syncthreads();
-    for (int j = 0; j < kb; ++j) {
-      float bv = -1.0f;
-      int bi = INT_MAX;
-      for (int r = j + tid; r < m; r += NT) {
-        const float v = fabsf(sm.P[j][r]);
-        if (v != v) atomicOr(status, ST_RANGE);
-        argmax_merge(bv, bi, v, r);
-      }
-      block_argmax_f(bv, bi, sm, NT);
-      int p = bi;
-      if (!GB_IN_BOUNDS(status, p >= j && p < m)) p = j;
-      if (tid < kb && p != j) {
-        const float t = sm.P[tid][j];
-        sm.P[tid][j] = sm.P[tid][p];
-        sm.P[tid][p] = t;
-      }
-      if (tid == 0 && p != j) {
-        const int t = sm.perm[k0 + j];
-        sm.perm[k0 + j] = sm.perm[k0 + p];
-        sm.perm[k0 + p] = t;
-      }
-      __syncthreads();
-      const float piv = sm.P[j][j];
-      if (piv == 0.0f && info == 0) info = k0 + j + 1;
-      for (int r = j + 1 + tid; r < m; r += NT) {
-        float l = sm.P[j][r];
-        if (piv != 0.0f) l = l / piv;
-        sm.P[j][r] = l;
-        for (int c = j + 1; c < kb; ++c) sm.P[c][r] -= l * sm.P[c][j];
-      }
-      __syncthreads();
-    }
+    const int pinfo = bt_panel<NT>(m, kb, k0, status);
+    if (pinfo != 0 && info == 0) info = k0 + pinfo;
     for (int e = tid; e < m * (BT_NB / 4); e += NT) {
       const int r = e % m, c = (e / m) * 4;
       if (c >= kb) continue;
@@ -216,10 +341,22 @@ __device__ int bt_factor(float* W, int ld, int n, BatchSmem& sm, int* status) {
   return info;
 }
 
+// (float)x by integer operations where the result is a normal number (the
+// conversion instruction runs at the FP64 rate, two a clock and SM): round to
+// nearest even on the 29 bits that drop out.
+__device__ __forceinline__ float bt_float(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned long long m = b & 0x7fffffffffffffffull;
+  const unsigned long long r = m + 0x0fffffffull + ((m >> 29) & 1ull);
+  const unsigned e = (unsigned)(r >> 52);
+  if (e - 897u >= 254u) return (float)x;  // zero, below or above the normal range, not finite
+  return __uint_as_float(((unsigned)(r >> 29) - (896u << 23)) | ((unsigned)(b >> 32) & 0x80000000u));
+}
+
 // W <- A (FP64 column-major -> FP32 row-major), 32 rows x 128 columns at a time
 // through four 32 x 32 tiles in the (still unused) panel buffer: sixteen loads
 // per thread in flight instead of four.
-// (bt_convert, bt_invert and bt_solve are calls of their own: inlined, their
+// (bt_panel, bt_convert, bt_invert and bt_solve are calls of their own: inlined, their
 // registers and the residual's maxima would not fit two CTAs per SM)
 template <int NT>
 __device__ __noinline__ void bt_convert(const double* A, int lda, float* W, int ld, int n) {
@@ -239,7 +376,7 @@ __device__ __noinline__ void bt_convert(const double* A, int lda, float* W, int 
 #pragma unroll
       for (int u = 0; u < PER; ++u) {
         const int e = tid + u * NT, i = e % BT_NB, j = e / BT_NB;
-        T[(j / BT_NB) * TW + (j % BT_NB) * (BT_NB + 1) + i] = (float)v[u];
+        T[(j / BT_NB) * TW + (j % BT_NB) * (BT_NB + 1) + i] = bt_float(v[u]);
       }
       __syncthreads();
 #pragma unroll
