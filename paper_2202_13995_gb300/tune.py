@@ -5,8 +5,8 @@ lu_factor(nb = 0) and lu_fact_bytes read.
 
 nb is the block width of the paper's blocked iteration (its LOCAL_MEM_BLOCK
 blocking parameter): the width of each factored block column and the inner
-dimension of the trailing update.  For each factorization kind (FP64 with the
-CUDA-core update, FP64 with the split tensor-core update, BF16/FP16 mixed
+dimension of the trailing update.  For each factorization kind (plain FP64, FP64
+with the split tensor-core update, BF16/FP16 mixed
 with refinement, FP32) and each size bucket, the sweep times whole solves
 (factor + solve or refinement, CUDA events on the library's stream, the best
 of K after a warm-up) on the seeded HPL-shaped matrices of the benchmarks and
@@ -32,9 +32,10 @@ KINDS = {
     "f32": ("f32", False, 0.25, (64, 128, 256, 384, 512)),
 }
 KIND_ID = {"f64": 0, "f64_split": 1, "mixed": 2, "f32": 3}
-# size buckets (upper bounds) and the size each is measured at; the FP64
-# CUDA-core solve at n = 32768 takes tens of seconds and keeps the n = 16384 choice
-BUCKETS = [(1536, 1024), (3072, 2048), (6144, 4096), (12288, 8192), (24576, 16384), (1 << 30, 32768)]
+# size buckets (upper bounds) and the size each is measured at; the plain FP64
+# solve at n = 32768 takes seconds and keeps the n = 16384 choice
+BUCKETS = [(800, 600), (1280, 1024), (3072, 2048), (4608, 4096), (7168, 6000), (12288, 8192), (24576, 16384),
+           (1 << 30, 32768)]
 SKIP = {("f64", 32768)}
 
 
