@@ -800,7 +800,15 @@ template <typename T>
 static cudaError_t launch_below(const T* U, const T* uinv, T* X, int64_t ld, int m, int ws, int wt,
                                 const SpecDev<T>& sp, int first, int tag, cudaStream_t st) {
   const int optin = device_smem_optin();
-  if (ls_smem(64, wt, sizeof(T)) <= (size_t)optin)
+  // Fewer rows per CTA while two CTAs per SM still take all rows at once: the
+  // launch is then as short as one CTA's chain of blocks, whose length grows
+  // with its rows (slab of 128 x 256, 1400 rows below: 64 rows per CTA 37 us, 16
+  // rows 21; slab of 128 x 128: 22 and 14; 5400 rows, 256 wide: 37 and 33 with
+  // 32); a longer launch takes 64, which read U least often.
+  const bool short_launch = cdiv(m, 32) <= 304;
+  if (cdiv(m, 16) <= 304 && ls_smem(16, wt, sizeof(T)) <= (size_t)optin)
+    return launch_ls<T, 16>(U, uinv, X, ld, m, ws, wt, sp, first, tag, st);
+  if (!short_launch && ls_smem(64, wt, sizeof(T)) <= (size_t)optin)
     return launch_ls<T, 64>(U, uinv, X, ld, m, ws, wt, sp, first, tag, st);
   if (ls_smem(32, wt, sizeof(T)) <= (size_t)optin)
     return launch_ls<T, 32>(U, uinv, X, ld, m, ws, wt, sp, first, tag, st);
