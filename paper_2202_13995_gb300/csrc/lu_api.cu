@@ -441,6 +441,38 @@ static cudaError_t panel_step(lu_fact f, int mode, T* Wkk, int m, int w, int kab
                                                     c->dev, s, f->spec_flag, (const T*)f->spec_backup));
 }
 
+// The first panel's check: the host waits for its verdict anyway, so a failed
+// check is undone here (the rows it changed come back from the copy) and the
+// panel goes to the pivoted kernel of its size, not to the cooperative kernel
+// on spec_sms CTAs that a later panel's failure is left to (FP32, 2500 x 128:
+// 519 -> 195 us).
+template <typename T>
+static cudaError_t try_panel(lu_fact f, T* Wkk, int m, int w, int kabs, cudaStream_t s, int* hflag, int* mode) {
+  lu_ctx c = f->ctx;
+  SpecArgs sa;
+  sa.flag = f->spec_flag;
+  sa.backup = f->spec_backup;
+  sa.ipiv = f->ipiv;
+  sa.perm = f->ps.perm;
+  cudaError_t e = PHASE_ON(c, s, PH_PANEL, block_column_launches(m, w, sizeof(T)),
+                           launch_block_column<T>(Wkk, f->ldw, m, w, kabs, nullptr, (T*)f->uinv, s, sa));
+  if (e != cudaSuccess) return e;
+  e = cudaMemcpyAsync(hflag, f->spec_flag, 4 * sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = ctx_wait(c, s);
+  if (e != cudaSuccess) return e;
+  *mode = (hflag[0] == 0 && hflag[3] == 0) ? SPEC_ON : SPEC_OFF;
+  if (*mode == SPEC_ON) return cudaSuccess;
+  const int tag = kabs + 1;
+  const int rows = hflag[3] == tag ? m : (hflag[1] == tag ? (hflag[2] < m ? hflag[2] : m) : 0);
+  if (rows > 0) {
+    e = cudaMemcpy2DAsync(Wkk, (size_t)f->ldw * sizeof(T), f->spec_backup, (size_t)w * sizeof(T), (size_t)w * sizeof(T),
+                          rows, cudaMemcpyDeviceToDevice, s);
+    if (e != cudaSuccess) return e;
+  }
+  return PHASE_ON(c, s, PH_PANEL, 1, launch_panel<T>(Wkk, f->ldw, m, w, kabs, f->ipiv, f->info_d, c->d_status, f->ps,
+                                                    c->dev, s));
+}
+
 // Persistent CTAs of a trailing update that has the device to itself: all
 // SMs; a shared context's (server slots) keep to gemm_ctas.
 static int gemm_cap(lu_ctx c) { return c->gemm_ctas > 0 ? c->gemm_ctas : c->dev.sm_count; }
@@ -508,12 +540,11 @@ static int factor_loop(lu_fact f) {
       // must all be resident at once) keeps to spec_sms CTAs: it returns at
       // once when the check passed, and a launch across the whole device
       // would wait for the device to drain whenever other work shares it
-      CU_TRY(panel_step<T>(f, mode, Wkk, n - k, w, k, st, mode != SPEC_OFF ? spec_sms : 0));
       if (mode == SPEC_TRY) {
-        CU_TRY(cudaMemcpyAsync(hflag, f->spec_flag, 4 * sizeof(int), cudaMemcpyDeviceToHost, st));
-        CU_TRY(ctx_wait(c, st));
-        mode = (hflag[0] == 0 && hflag[3] == 0) ? SPEC_ON : SPEC_OFF;
+        CU_TRY(try_panel<T>(f, Wkk, n - k, w, k, st, hflag, &mode));
         hflag[4] = hflag[7] = 0;
+      } else {
+        CU_TRY(panel_step<T>(f, mode, Wkk, n - k, w, k, st, mode != SPEC_OFF ? spec_sms : 0));
       }
     }
     CU_TRY(PHASE(c, PH_LASWP, 1, launch_laswp<T>(W, ld, n, k, w, f->ps.perm, f->rowid, st)));
