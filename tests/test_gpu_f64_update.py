@@ -3,6 +3,8 @@ with the FP64 CUDA cores where the certificate fails or the update is small):
 factors against the oracle at the edges of the rule that chooses it, and the
 componentwise backward error of badly scaled, banded and sparse systems, which
 a split update without the certificate loses."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -98,11 +100,15 @@ def test_top_solve_edges(ctx, w, N):
     """L^-1 X by substitution in FP64: |x - x_ref| <= 2 w u |L^-1| |L| |x| (both
     round each of at most w terms; Higham, theorem 8.5)."""
     import torch
+    from paper_2202_13995_gb300 import lu
     rng = np.random.default_rng(w * 1000 + N)
     M = rng.random((w, w + N)) - 0.5
     M[:, :w] *= 4.0 / (4.0 + w)
     Md = torch.from_numpy(M.copy()).cuda()
-    ctx.step_trsm(Md[:, :w], Md[:, w:], "f64")
+    # (the C entry itself: Context.step_trsm takes a one-row operand's width for its row stride)
+    assert lu.load().lu_step_trsm(ctx._h, lu._prec("f64"), w, N, C.c_void_p(Md.data_ptr()), w + N,
+                                  C.c_void_p(Md.data_ptr() + 8 * w), w + N) == 0
+    ctx.stream.synchronize()
     L = np.tril(M[:, :w], -1) + np.eye(w)
     want = O.trsm_unit_lower(L, M[:, w:])
     bound = 2 * w * U * (np.abs(np.linalg.inv(L)) @ (np.abs(L) @ np.abs(want))) + U * np.abs(want)
