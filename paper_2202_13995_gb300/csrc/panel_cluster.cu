@@ -21,18 +21,18 @@
 //    through distributed shared memory, no grid barrier and no L2 round trip;
 //  - what the exchange needs of column j + 1 comes first (the multipliers of
 //    column j, column j + 1's update and search, the candidate row's values);
-//    the update of the other columns runs while the candidates travel.
+//    the update of the other columns runs while the candidates travel;
+//  - the warps have roles: those of the chain (one per 32 rows) read the
+//    records and take the multipliers, the next two columns and the search, the
+//    others update the rest, so the FP64 pipes work through the chain's waits
+//    (all warps in step: 2.5 us a column of 512 x 64, 2.9 of 1024 x 128).
 // Quotients come from the pivot's reciprocal by P. Markstein's correction
 // (see quot_rn), three multiply-adds instead of a division: GB300 issues an
 // FP64 warp instruction once in 64 cycles per SM quarter, and a division takes
 // nine of them.
 // Measured (us per column, step call, cooperative kernel -> this one): FP64
-// 512 x 64 5.1 -> 2.2, 1023 x 64 5.5 -> 2.5, 4096 x 64 5.9 -> 4.4, 2500 x 128
-// 6.0 -> 4.6; FP32 512 x 64 3.6 -> 1.6, 2500 x 128 4.0 -> 1.8, 6000 x 64
-// 4.3 -> 2.2.  Clock stamps (1024 x 64): the wait for the records is 130 cycles
-// of a column's 2700 (FP32) and 4600 (FP64); the rest is the CTA's own chain
-// (search 550, multipliers 300 / 780, sending 600 / 880) and the update of
-// the other columns (400 / 1500).
+// 512 x 64 5.1 -> 2.0, 1023 x 64 5.5 -> 2.4, 1024 x 128 5.5 -> 2.7; FP32
+// 512 x 64 3.6 -> 1.6, 2500 x 128 4.0 -> 1.6, 6000 x 64 4.3 -> 2.2.
 //
 // A record's buffer is reused every third column: its pivot row is read until
 // a CTA has finished column j, a peer sends column j + 3 only after it has
@@ -145,12 +145,74 @@ __device__ __forceinline__ bool pc_try(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// A CTA's rows (at A, row stride ld) to shared memory, four of a warp's rows in
+// flight at a time
+template <typename T>
+__device__ __forceinline__ void pc_load_rows(T* S, int Rs, const T* A, int64_t ld, int rows, int w) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int rb = warp; rb < rows; rb += 4 * nw) {
+    for (int c = lane; c < w; c += 32) {
+      T x[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int rr = rb + i * nw;
+        x[i] = rr < rows ? __ldcg(A + (int64_t)rr * ld + c) : T(0);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int rr = rb + i * nw;
+        if (rr < rows) S[(size_t)c * Rs + rr] = x[i];
+      }
+    }
+  }
+}
+
+// ... and back, row rr to position sp[rr] of the panel at A
+template <typename T>
+__device__ __forceinline__ void pc_store_rows(T* A, int64_t ld, const T* S, int Rs, const int* sp, int rows, int w) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int rr = warp; rr < rows; rr += nw) {
+    T* dst = A + (int64_t)sp[rr] * ld;
+    for (int c = lane; c < w; c += 32) dst[c] = S[(size_t)c * Rs + rr];
+  }
+}
+
+// Columns c, c + step, .. below w of this lane's row (at Sr, column stride Rs) -= l
+// times the pivot row
+template <typename T>
+__device__ __forceinline__ void pc_update(T* Sr, int Rs, const T* pr, T l, int c, int step, int w) {
+  const size_t st = (size_t)step * Rs;
+  T* x = Sr + (size_t)c * Rs;
+  for (; c + 3 * step < w; c += 4 * step, x += 4 * st) {
+    T v[4], u[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      v[q] = x[q * st];
+      u[q] = pr[c + q * step];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) x[q * st] = fma(-l, u[q], v[q]);
+  }
+  T v[3], u[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (c + q * step < w) {
+      v[q] = x[q * st];
+      u[q] = pr[c + q * step];
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q)
+    if (c + q * step < w) x[q * st] = fma(-l, u[q], v[q]);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> P) {
   constexpr int VN = PcRec<T>::VN, HC = PcRec<T>::HC;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bars[PC_NBUF];
   __shared__ uint4 red[PC_NTMAX / 32];  // each row group's best: key, position, row
+  __shared__ int sel[2];  // the current column's pivot: position, CTA
   __shared__ int abort_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
   const int cta = (int)cluster_rank(), CL = (int)gridDim.x;
@@ -158,15 +220,20 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
   const int64_t ld = P.ld;
   const int row0 = cta * R;
   const int rloc = max(0, min(P.m, row0 + R) - row0);
-  // A warp serves one group of 32 rows, a lane per row: class 0 of the group's
-  // warps takes the chain (multipliers, the next column, the search), and
-  // every class its share of the other columns.
+  // A warp serves one group of 32 rows, a lane per row.  Class 0 of the group's
+  // warps takes the chain: the records, the multipliers, the next two columns,
+  // the search.  The other classes update the other columns meanwhile; they
+  // learn of the pivot at the barrier that ends the search.  (A CTA of so many
+  // rows that every warp is a chain warp updates them itself.)
   const int RG = (R + 31) / 32;
   const int NC = nw / RG;  // classes; warps past NC * RG only help with the records
   const int rg = warp % RG, cls = warp / RG;
   const int r = rg * 32 + lane;
   const bool live = cls < NC && r < rloc;
   const bool chain = warp < RG;
+  const bool all_upd = NC == 1;
+  const int c_off = all_upd ? 3 + cls : 2 + cls, c_step = all_upd ? NC : NC - 1;  // columns j + c_off, + c_step, ..
+  const bool upd = cls < NC && (all_upd || !chain);
   const int pieces = pc_pieces(w, sizeof(T));
   const size_t tile = ((size_t)w * Rs * sizeof(T) + 15) / 16 * 16;
   T* S = reinterpret_cast<T*>(smem_raw);  // [w][Rs]: column c of the tile, row r
@@ -181,22 +248,7 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
     abort_flag = 0;
     if (cta == 0) P.perm[0] = 0;
   }
-  // the rows, four of a warp's rows in flight at a time
-  for (int rb = warp; rb < rloc; rb += 4 * nw) {
-    for (int c = lane; c < w; c += 32) {
-      T x[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int rr = rb + i * nw;
-        x[i] = rr < rloc ? __ldcg(P.A + (int64_t)(row0 + rr) * ld + c) : T(0);
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int rr = rb + i * nw;
-        if (rr < rloc) S[(size_t)c * Rs + rr] = x[i];
-      }
-    }
-  }
+  pc_load_rows(S, Rs, P.A + (int64_t)row0 * ld, ld, rloc, w);
   __syncthreads();
   cluster_sync();  // every peer's barriers are set up, and the count of perm is zero
 
@@ -212,10 +264,22 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
     pdst[i] = cluster_map(dst0, (uint32_t)(peer < CL ? peer : 0));
   }
 
+  int pos = row0 + r;  // this lane's row's position
+  bool act = live;     // ... and whether the row is below the current column's diagonal
+  // column j's pivot moved to row j: positions p and j change places
+  auto move = [&](int j, int p) {
+    if (live) {
+      if (pos == p)
+        pos = j;
+      else if (pos == j)
+        pos = p;
+    }
+    act = live && pos > j;
+  };
   // The CTA's candidate of column c (key `best` of this lane's row, chain
-  // warps): its record to every peer.  pr: the pivot row of column c - 1, by
-  // which the columns right of c still lack their update (null: none).
-  auto publish = [&](int c, int buf, PcKey best, const T* pr) {
+  // warps): its record to every peer.  With c > 0 the columns right of c still
+  // lack their update by column c - 1, whose pivot row (sel) pr is set to.
+  auto publish = [&](int c, int buf, int pbuf, PcKey best, const T*& pr) {
     if (chain) {
       const bool own = pc_warp_best<T>(best);
       const unsigned at = __ballot_sync(0xffffffffu, own);
@@ -223,6 +287,10 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
     }
     __syncthreads();
     if (abort_flag) return false;
+    if (c > 0) {
+      pr = reinterpret_cast<const T*>(recs + (size_t)pbuf * CL * pieces * 16 + (size_t)sel[1] * pieces * 16 + 16 * HC);
+      if (!chain) move(c - 1, sel[0]);
+    }
     uint4 e = red[lane < RG ? lane : 0];
     if (RG > 1) {
       PcKey k{lane < RG ? e.x : 0u, lane < RG ? e.y : 0u, lane < RG ? (int)e.z : INT_MAX};
@@ -236,10 +304,10 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
     const bool any = e.x != 0u;
     if (any) {
       const T* Sk = S + e.w;
-      const T lc = pr != nullptr ? Sk[(size_t)(c - 1) * Rs] : T(0);
+      const T lc = c > 0 ? Sk[(size_t)(c - 1) * Rs] : T(0);
       for (int q = c + tid; q < w; q += nt) {
         T v = Sk[(size_t)q * Rs];
-        if (pr != nullptr && q > c) v = fma(-lc, pr[q], v);
+        if (c > 0 && q > c) v = fma(-lc, pr[q], v);
         mrow[q] = v;
       }
     }
@@ -270,18 +338,20 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
   };
   // arm the barrier of column c's records (its previous phase is complete)
   auto arm = [&](int c, int buf) {
-    if (tid == nt - 1) mbar_expect_tx(bar0 + 8u * (uint32_t)buf, (uint32_t)(CL * (pieces - c / VN) * 16));
+    if (tid == 0) mbar_expect_tx(bar0 + 8u * (uint32_t)buf, (uint32_t)(CL * (pieces - c / VN) * 16));
   };
 
-  int pos = row0 + r;        // this lane's row's position
   T cur = live ? Sr[0] : T(0);                                    // chain warps: column j of the row,
   T nxt = live && w > 1 ? Sr[(size_t)Rs] : T(0);                  // and column j + 1 before column j's update
+  const T* pr = nullptr;
   arm(0, 0);
-  bool ok = publish(0, 0, pc_key(cur, live, pos), nullptr);
+  bool ok = publish(0, 0, 0, pc_key(cur, live, pos), pr);
   int buf = 0;
   uint32_t par = 0;
   for (int j = 0; j < w && ok; ++j) {
-    {
+    const int nbuf = buf + 1 == PC_NBUF ? 0 : buf + 1;
+    PcKey best{0u, 0u, INT_MAX};
+    if (chain) {
       const uint32_t bar = bar0 + 8u * (uint32_t)buf;
       if (!pc_try(bar, par)) {
         const uint64_t t0 = gtimer();
@@ -295,40 +365,33 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
         }
       }
       __syncwarp();
-    }
-    const int nbuf = buf + 1 == PC_NBUF ? 0 : buf + 1;
-    if (j + 1 < w) arm(j + 1, nbuf);
-    // the pivot: the best of the CTAs' candidates, in every warp
-    const unsigned char* rb = recs + (size_t)buf * bufstep;
-    PcKey k{0u, 0u, INT_MAX};
-    if (lane < CL) {
-      const unsigned* h = reinterpret_cast<const unsigned*>(rb + (size_t)lane * pieces * 16);
-      k = {h[0], sizeof(T) == 8 ? h[2] : 0u, (int)h[1]};
-    }
-    const bool kown = pc_warp_best<T>(k);
-    const unsigned bal = __ballot_sync(0xffffffffu, kown);
-    const int win = bal ? __ffs(bal) - 1 : 0;
-    const int p = k.pos;
-    const unsigned char* rec = rb + (size_t)win * pieces * 16;
-    const T* pr = reinterpret_cast<const T*>(rec + 16 * HC);  // the pivot row, columns j .. w
-    if (live) {
-      if (pos == p)
-        pos = j;
-      else if (pos == j)
-        pos = p;
-    }
-    const bool act = live && pos > j;  // the row is below the diagonal
-    // chain warps: multipliers, column j + 1 and its search
-    PcKey best{0u, 0u, INT_MAX};
-    if (chain) {
+      if (j + 1 < w) arm(j + 1, nbuf);
+      // the pivot: the best of the CTAs' candidates
+      const unsigned char* rb = recs + (size_t)buf * bufstep;
+      PcKey k{0u, 0u, INT_MAX};
+      if (lane < CL) {
+        const unsigned* h = reinterpret_cast<const unsigned*>(rb + (size_t)lane * pieces * 16);
+        k = {h[0], sizeof(T) == 8 ? h[2] : 0u, (int)h[1]};
+      }
+      const bool kown = pc_warp_best<T>(k);
+      const unsigned bal = __ballot_sync(0xffffffffu, kown);
+      const int win = bal ? __ffs(bal) - 1 : 0;
+      const unsigned char* rec = rb + (size_t)win * pieces * 16;
+      pr = reinterpret_cast<const T*>(rec + 16 * HC);  // the pivot row, columns j .. w
       const T rinv = reinterpret_cast<const T*>(rec)[2];
       const T piv = pr[j];
       const T u1 = j + 1 < w ? pr[j + 1] : T(0);
-      if (cta == 0 && tid == 0) {
-        P.ipiv[P.kabs + j] = P.kabs + p + 1;
-        if (!nonzero(piv)) atomicMin(P.info, P.kabs + j + 1);
-        if (is_inf_mag(pivot_mag(piv))) atomicOr(P.status, ST_RANGE);  // a non-finite candidate
+      if (tid == 0) {
+        sel[0] = k.pos;
+        sel[1] = win;
+        if (cta == 0) {
+          P.ipiv[P.kabs + j] = P.kabs + k.pos + 1;
+          if (!nonzero(piv)) atomicMin(P.info, P.kabs + j + 1);
+          if (is_inf_mag(pivot_mag(piv))) atomicOr(P.status, ST_RANGE);  // a non-finite candidate
+        }
       }
+      move(j, k.pos);
+      // multipliers, column j + 1 and its search
       if (act) {
         const T l = nonzero(piv) ? quot_rn(cur, piv, rinv) : cur;
         Sr[(size_t)j * Rs] = l;
@@ -340,42 +403,18 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
       }
     }
     if (j + 1 == w) break;
-    ok = publish(j + 1, nbuf, best, pr);
+    ok = publish(j + 1, nbuf, buf, best, pr);
     if (!ok) break;
-    // the other columns while the candidates travel: class q takes columns
-    // j + 2 + q, + NC, ... (column j + 2, which the chain needs next, is class 0's)
+    // while the candidates travel: column j + 2, which the chain needs next,
+    // by the chain warps, the columns after it by the others
     if (act) {
       const T l = Sr[(size_t)j * Rs];
-      const size_t step = (size_t)NC * Rs;
-      int c = j + 2 + cls;
-      T* x = Sr + (size_t)c * Rs;
-      if (chain && c < w) {
-        nxt = fma(-l, pr[c], x[0]);
+      if (chain && j + 2 < w) {
+        T* x = Sr + (size_t)(j + 2) * Rs;
+        nxt = fma(-l, pr[j + 2], x[0]);
         x[0] = nxt;
-        c += NC;
-        x += step;
       }
-      for (; c + 3 * NC < w; c += 4 * NC, x += 4 * step) {
-        T v[4], u[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          v[q] = x[q * step];
-          u[q] = pr[c + q * NC];
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) x[q * step] = fma(-l, u[q], v[q]);
-      }
-      T v[3], u[3];
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        if (c + q * NC < w) {
-          v[q] = x[q * step];
-          u[q] = pr[c + q * NC];
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < 3; ++q)
-        if (c + q * NC < w) x[q * step] = fma(-l, u[q], v[q]);
+      if (upd) pc_update(Sr, Rs, pr, l, j + c_off, c_step, w);
     }
     buf = nbuf;
     if (buf == 0) par ^= 1u;
@@ -386,10 +425,7 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
     int* sp = reinterpret_cast<int*>(recs);  // [R] (the records are all read)
     if (chain && live) sp[r] = pos;
     __syncthreads();
-    for (int rr = warp; rr < rloc; rr += nw) {
-      T* dst = P.A + (int64_t)sp[rr] * ld;
-      for (int c = lane; c < w; c += 32) dst[c] = S[(size_t)c * Rs + rr];
-    }
+    pc_store_rows(P.A, ld, S, Rs, sp, rloc, w);
     if (chain && live && pos != row0 + r) {
       const int q = atomicAdd(P.perm, 1);
       P.perm[1 + q] = pos;
@@ -406,21 +442,22 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
 // CTAs of a panel's cluster: rows of 32 (FP64: the FP64 pipes of as many SMs as
 // help) or 64 (FP32) per CTA up to 16 CTAs; -1 when the tile does not fit the
 // shared memory then.  grid: the grid form can take the panel instead, which an
-// FP64 panel of m w > 140,000 is faster on, bound as it is by the FP64 pipes of
-// 16 SMs (us per column, cluster and grid: 2048 x 64 3.2 and about 3; 4096 x 64
-// 4.3 and 3.3; 2500 x 128 4.6 and 3.7); without it the line is the cooperative
-// kernel's, 360,000 (3000 x 128: 6.1 and 6.0).
+// FP64 panel of m w > 100,000 is faster on, bound as it is by the FP64 pipes of
+// 16 SMs (us, cluster and grid: 1500 x 64 167 and 180, 2048 x 64 188 and 178,
+// 2048 x 32 96 and 105, 3000 x 32 102 and 103, 4096 x 32 117 and 102, 1024 x 128
+// 348 and 341); without it the line is the cooperative kernel's, 360,000
+// (3000 x 128: 6.1 and 6.0 us a column).
 static int pc_config(int m, int w, int tsize, int optin, bool grid, int* R, int* nt, size_t* smem) {
   if (w < 1 || w > 512 || m < w) return -1;
   const int target = tsize == 8 ? 32 : 64;
   int cl = 1;
   while (cl < PC_CLMAX && cl * target < m) cl *= 2;
   *R = (int)cdiv(m, cl);
-  *nt = *R <= 64 ? 256 : PC_NTMAX;  // (a warp per 32 rows at least)
+  *nt = *R <= target ? 256 : PC_NTMAX;  // (a warp per 32 rows at least)
   if (*R > PC_NTMAX) return -1;
   *smem = pc_smem_bytes(*R, w, cl, tsize);
   if (*smem + 1024 > (size_t)optin) return -1;
-  if (tsize == 8 && (int64_t)m * w > (grid ? 140000 : 360000)) return -1;
+  if (tsize == 8 && (int64_t)m * w > (grid ? 100000 : 360000)) return -1;
   return cl;
 }
 
@@ -510,16 +547,15 @@ cudaError_t launch_panel_cluster(T* Wkk, int64_t ldw, int m, int w, int kabs, in
 // (key and position) and the row beside it.  Every 8-byte word of either
 // carries the column's stamp next to its data, so readers know a word by
 // itself and no fence orders the stores (a release store that waits for the
-// row's stores cost 1 us a column).  Thread t of every CTA polls CTA t's header,
-// the CTA picks the pivot and reads its row once: two L2 round trips a column,
-// with the update of the other columns under them.  Against the kernel in
+// row's stores cost 1 us a column).  Every CTA polls all headers, picks the
+// pivot and reads its row once: two L2 round trips a column, with the update of
+// the other columns under them.  Against the kernel in
 // panel.cu (a counter barrier, every candidate row read by every CTA,
 // sub-panels of 32 columns written back, interchanged and updated through L2)
 // no value but the pivot row crosses L2 twice.
-// Measured (us per column, that kernel -> this one): FP64 6000 x 64 5.9 -> 3.4,
-// 8192 x 128 6.7 -> 3.9, 7000 x 256 7.7 -> 5.1 (there the FP64 pipes set the
-// pace: 256 columns of 46 rows); FP32 8192 x 128 4.5 -> 2.1.  Clock stamps
-// (8192 x 128): the poll 600 cycles, the row 1150, of 8000 (FP64) and 4300 (FP32).
+// Measured (us per column, that kernel -> this one): FP64 6000 x 64 5.9 -> 3.3,
+// 8192 x 128 6.7 -> 3.1, 7000 x 256 7.7 -> 3.6 (there the FP64 pipes set the
+// pace: 256 columns of 47 rows); FP32 8192 x 128 4.5 -> 2.2.
 // The record buffers' stamps are cleared before the launch; a buffer is
 // reused every third column (the argument above).  Every poll is bounded; a CTA whose poll runs
 // out raises ST_TIMEOUT and leaves, and so do the others in their turn.
@@ -565,6 +601,22 @@ struct PrWord<float> {
   }
 };
 
+// wait for a stamped value; *abort_flag is set when the wait runs out
+template <typename T>
+__device__ __forceinline__ void pr_fetch(const typename PrWord<T>::type* q, T& v, unsigned stamp, int* abort_flag,
+                                         int* status) {
+  if (PrWord<T>::get(q, v, stamp)) return;
+  const uint64_t t0 = gtimer();
+  while (!PrWord<T>::get(q, v, stamp)) {
+    if (*(volatile int*)abort_flag) return;
+    if (gtimer() - t0 > GB_SPIN_LIMIT_NS) {
+      atomicOr(status, ST_TIMEOUT);
+      *(volatile int*)abort_flag = 1;
+      return;
+    }
+  }
+}
+
 template <typename T>
 struct PrParams {
   T* A;  // W(k, k)
@@ -585,8 +637,243 @@ __host__ __device__ inline size_t pr_smem_bytes(int R, int w, int tsize) {
   return tile + (size_t)PC_NBUF * (w + 1) * tsize + (size_t)R * sizeof(int);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(PC_NTMAX, 1) panel_resident_kernel(PrParams<T> P) {
+constexpr int PR_HL = 5;  // headers per polling lane: up to 160 CTAs
+constexpr int PR_RL = 4;  // pivot row values per chain lane in flight
+
+__global__ void __launch_bounds__(PC_NTMAX, 1) panel_grid_f64_kernel(PrParams<double> P) {
+  using T = double;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint4 red[PC_NTMAX / 32];   // each row group's best: key, position, row
+  __shared__ int sel[2];  // the current column's pivot: position, CTA
+  __shared__ int abort_flag;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
+  const int cta = blockIdx.x, G = gridDim.x;
+  const int R = P.R, w = P.w, Rs = R | 1;
+  const int64_t ld = P.ld;
+  const int row0 = cta * R;
+  const int rloc = max(0, min(P.m, row0 + R) - row0);
+  // (row groups, classes and chain warps as in panel_cluster_kernel)
+  const int RG = (R + 31) / 32;
+  const int NC = nw / RG;
+  const int rg = warp % RG, cls = warp / RG;
+  const int r = rg * 32 + lane;
+  const bool live = cls < NC && r < rloc;
+  const bool chain = warp < RG;
+  const bool all_upd = NC == 1;
+  const int c_off = all_upd ? 3 + cls : 2 + cls, c_step = all_upd ? NC : NC - 1;
+  const bool upd = cls < NC && (all_upd || !chain);
+  const size_t tile = ((size_t)w * Rs * sizeof(T) + 15) / 16 * 16;
+  T* S = reinterpret_cast<T*>(smem_raw);
+  T* prow = reinterpret_cast<T*>(smem_raw + tile);  // [PC_NBUF][w + 1]: pivot rows
+  int* sp = reinterpret_cast<int*>(prow + (size_t)PC_NBUF * (w + 1));  // [R] positions, at the end
+  T* Sr = S + r;
+
+  if (tid == 0) {
+    abort_flag = 0;
+    if (cta == 0) P.perm[0] = 0;
+  }
+  pc_load_rows(S, Rs, P.A + (int64_t)row0 * ld, ld, rloc, w);
+  __syncthreads();
+
+  int pos = row0 + r;
+  bool act = live;
+  auto move = [&](int j, int p) {
+    if (live) {
+      if (pos == p)
+        pos = j;
+      else if (pos == j)
+        pos = p;
+    }
+    act = live && pos > j;
+  };
+  // this CTA's candidate of column c to global memory (pr: the pivot row of
+  // column c - 1, which the columns right of c still lack)
+  auto publish = [&](int c, int buf, PcKey best, const T* pr) {
+    if (chain) {
+      const bool own = pc_warp_best<T>(best);
+      const unsigned at = __ballot_sync(0xffffffffu, own);
+      if (lane == 0) red[warp] = make_uint4(best.hi, best.lo, (unsigned)best.pos, (unsigned)(rg * 32 + __ffs(at) - 1));
+    }
+    __syncthreads();
+    if (abort_flag) return false;
+    if (c > 0 && !chain) move(c - 1, sel[0]);
+    uint4 e = red[lane < RG ? lane : 0];
+    if (RG > 1) {
+      PcKey k{lane < RG ? e.x : 0u, lane < RG ? e.y : 0u, lane < RG ? (int)e.z : INT_MAX};
+      const bool own = pc_warp_best<T>(k);
+      const unsigned at = __ballot_sync(0xffffffffu, own);
+      e.w = __shfl_sync(0xffffffffu, e.w, at ? __ffs(at) - 1 : 0);
+      e.x = k.hi;
+      e.y = k.lo;
+      e.z = (unsigned)k.pos;
+    }
+    const unsigned stamp = (unsigned)c + 1u;
+    if (tid == nt - 1)
+      pr_store(P.head + (size_t)buf * G + cta,
+               make_ulonglong2(((unsigned long long)e.x << 32) | stamp,
+                               ((unsigned long long)e.y << 32) | ((e.x ? e.z : 0u) << 12) | stamp));
+    if (e.x != 0u) {
+      auto* grow = P.rows + (size_t)(buf * G + cta) * P.rstride;
+      const T* Sk = S + e.w;
+      const T lc = pr != nullptr ? Sk[(size_t)(c - 1) * Rs] : T(0);
+      for (int q = c + tid; q < w; q += nt) {
+        T v = Sk[(size_t)q * Rs];
+        if (pr != nullptr && q > c) v = fma(-lc, pr[q], v);
+        PrWord<T>::put(grow + q, v, stamp);
+      }
+      if (warp == nw - 1) {
+        const T rv = recip_rn(Sk[(size_t)c * Rs]);
+        if (lane == 0) PrWord<T>::put(grow + w, rv, stamp);
+      }
+    }
+    __syncthreads();  // (the candidate's row is read before its columns are updated)
+    return true;
+  };
+  auto fetch = [&](const typename PrWord<T>::type* q, T& v, unsigned stamp) {
+    pr_fetch<T>(q, v, stamp, &abort_flag, P.status);
+  };
+
+  T cur = live ? Sr[0] : T(0);
+  T nxt = live && w > 1 ? Sr[(size_t)Rs] : T(0);
+  bool ok = publish(0, 0, pc_key(cur, live, pos), nullptr);
+  int buf = 0;
+  for (int j = 0; j < w && ok; ++j) {
+    const int nbuf = buf + 1 == PC_NBUF ? 0 : buf + 1;
+    const unsigned stamp = (unsigned)j + 1u;
+    T* pr = prow + (size_t)buf * (w + 1);
+    PcKey best{0u, 0u, INT_MAX};
+    if (chain) {
+      // every chain warp polls all headers, PR_HL per lane, and picks the pivot
+      PcKey k{0u, 0u, INT_MAX};
+      int kc = 0;
+      {
+        ulonglong2 h[PR_HL];
+        auto there = [&](const ulonglong2& v) { return (unsigned)v.x == stamp && ((unsigned)v.y & 0xfffu) == stamp; };
+        auto all = [&]() {
+          bool got = true;
+#pragma unroll
+          for (int i = 0; i < PR_HL; ++i) {
+            const int t = lane + 32 * i;
+            if (t < G) {
+              h[i] = pr_load(P.head + (size_t)buf * G + t);
+              got &= there(h[i]);
+            }
+          }
+          return got;
+        };
+        if (!all()) {
+          const uint64_t t0 = gtimer();
+          while (!all()) {
+            if (*(volatile int*)&abort_flag) break;
+            if (gtimer() - t0 > GB_SPIN_LIMIT_NS) {
+              atomicOr(P.status, ST_TIMEOUT);
+              *(volatile int*)&abort_flag = 1;  // seen by every thread after the CTA's next barrier
+              break;
+            }
+          }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < PR_HL; ++i) {
+          const int t = lane + 32 * i;
+          if (t < G) {
+            PcKey q;
+            q.hi = (unsigned)(h[i].x >> 32);
+            q.lo = (unsigned)(h[i].y >> 32);
+            q.pos = q.hi ? (int)((unsigned)h[i].y >> 12) : INT_MAX;
+            if (pc_better(q, k)) {
+              k = q;
+              kc = t;
+            }
+          }
+        }
+      }
+      const bool own = pc_warp_best<T>(k);
+      const unsigned at = __ballot_sync(0xffffffffu, own);
+      const int win = __shfl_sync(0xffffffffu, kc, at ? __ffs(at) - 1 : 0);
+      const auto* grow = P.rows + (size_t)(buf * G + win) * P.rstride;
+      // the pivot row: what the chain needs, and the rest to shared memory
+      // (read after the next barrier), its loads in flight together
+      T piv = T(0), rinv = T(0), u1 = T(0);
+      T rest[PR_RL];
+      bool got = PrWord<T>::get(grow + j, piv, stamp);
+      got &= PrWord<T>::get(grow + w, rinv, stamp);
+      if (j + 1 < w) got &= PrWord<T>::get(grow + j + 1, u1, stamp);
+      const int q0 = j + 1 + tid, qs = 32 * RG;
+      bool gotr = true;
+#pragma unroll
+      for (int i = 0; i < PR_RL; ++i) {
+        rest[i] = T(0);
+        if (q0 + i * qs < w) gotr &= PrWord<T>::get(grow + q0 + i * qs, rest[i], stamp);
+      }
+      if (!got) {
+        fetch(grow + j, piv, stamp);
+        fetch(grow + w, rinv, stamp);
+        if (j + 1 < w) fetch(grow + j + 1, u1, stamp);
+      }
+      if (tid == 0) {
+        sel[0] = k.pos;
+        sel[1] = win;
+        if (cta == 0) {
+          P.ipiv[P.kabs + j] = P.kabs + k.pos + 1;
+          if (!nonzero(piv)) atomicMin(P.info, P.kabs + j + 1);
+          if (is_inf_mag(pivot_mag(piv))) atomicOr(P.status, ST_RANGE);
+        }
+      }
+      move(j, k.pos);
+      if (act) {
+        const T l = nonzero(piv) ? quot_rn(cur, piv, rinv) : cur;
+        Sr[(size_t)j * Rs] = l;
+        cur = fma(-l, u1, nxt);
+        if (j + 1 < w) {
+          Sr[(size_t)(j + 1) * Rs] = cur;
+          best = pc_key(cur, true, pos);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < PR_RL; ++i) {
+        if (q0 + i * qs < w) {
+          if (!gotr) fetch(grow + q0 + i * qs, rest[i], stamp);
+          pr[q0 + i * qs] = rest[i];
+        }
+      }
+      for (int q = q0 + PR_RL * qs; q < w; q += qs) {
+        T v = T(0);
+        fetch(grow + q, v, stamp);
+        pr[q] = v;
+      }
+    }
+    if (j + 1 == w) break;
+    ok = publish(j + 1, nbuf, best, pr);
+    if (!ok) break;
+    if (act) {
+      const T l = Sr[(size_t)j * Rs];
+      if (chain && j + 2 < w) {
+        T* x = Sr + (size_t)(j + 2) * Rs;
+        nxt = fma(-l, pr[j + 2], x[0]);
+        x[0] = nxt;
+      }
+      if (upd) pc_update(Sr, Rs, pr, l, j + c_off, c_step, w);
+    }
+    buf = nbuf;
+  }
+  __syncthreads();
+  if (!ok || abort_flag) return;
+  if (chain && live) sp[r] = pos;
+  __syncthreads();
+  pc_store_rows(P.A, ld, S, Rs, sp, rloc, w);
+  if (chain && live && pos != row0 + r) {
+    const int q = atomicAdd(P.perm, 1);
+    P.perm[1 + q] = pos;
+    P.perm[1 + 2 * w + q] = row0 + r;
+  }
+}
+
+// The FP32 form: bound by the exchange, not by its pipes, so every thread polls a
+// header, reads the pivot row and updates (in the roles above an 8192 x 128
+// panel takes 328 us, in these 290; for FP64 it is 403 and 447)
+__global__ void __launch_bounds__(PC_NTMAX, 1) panel_grid_f32_kernel(PrParams<float> P) {
+  using T = float;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint4 red[PC_NTMAX / 32];   // each row group's best: key, position, row
   __shared__ uint4 red2[PC_NTMAX / 32];  // each polling warp's best: key, position, CTA
@@ -614,21 +901,7 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_resident_kernel(PrParams<T>
     abort_flag = 0;
     if (cta == 0) P.perm[0] = 0;
   }
-  for (int rb = warp; rb < rloc; rb += 4 * nw) {
-    for (int c = lane; c < w; c += 32) {
-      T x[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int rr = rb + i * nw;
-        x[i] = rr < rloc ? __ldcg(P.A + (int64_t)(row0 + rr) * ld + c) : T(0);
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int rr = rb + i * nw;
-        if (rr < rloc) S[(size_t)c * Rs + rr] = x[i];
-      }
-    }
-  }
+  pc_load_rows(S, Rs, P.A + (int64_t)row0 * ld, ld, rloc, w);
   __syncthreads();
 
   // this CTA's candidate of column c to global memory (pr as in panel_cluster_kernel)
@@ -670,18 +943,8 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_resident_kernel(PrParams<T>
     }
     __syncthreads();  // (the candidate's row is read before its columns are updated)
   };
-  // wait for a stamped value; false (and the CTA's flag) when the wait runs out
   auto fetch = [&](const typename PrWord<T>::type* q, T& v, unsigned stamp) {
-    if (PrWord<T>::get(q, v, stamp)) return;
-    const uint64_t t0 = gtimer();
-    while (!PrWord<T>::get(q, v, stamp)) {
-      if (*(volatile int*)&abort_flag) return;
-      if (gtimer() - t0 > GB_SPIN_LIMIT_NS) {
-        atomicOr(P.status, ST_TIMEOUT);
-        *(volatile int*)&abort_flag = 1;
-        return;
-      }
-    }
+    pr_fetch<T>(q, v, stamp, &abort_flag, P.status);
   };
 
   int pos = row0 + r;
@@ -807,10 +1070,7 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_resident_kernel(PrParams<T>
   if (!ok || abort_flag) return;
   if (chain && live) sp[r] = pos;
   __syncthreads();
-  for (int rr = warp; rr < rloc; rr += nw) {
-    T* dst = P.A + (int64_t)sp[rr] * ld;
-    for (int c = lane; c < w; c += 32) dst[c] = S[(size_t)c * Rs + rr];
-  }
+  pc_store_rows(P.A, ld, S, Rs, sp, rloc, w);
   if (chain && live && pos != row0 + r) {
     const int q = atomicAdd(P.perm, 1);
     P.perm[1 + q] = pos;
@@ -818,16 +1078,21 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_resident_kernel(PrParams<T>
   }
 }
 
+template <typename T>
+static const void* pr_kernel() {
+  return sizeof(T) == 8 ? (const void*)panel_grid_f64_kernel : (const void*)panel_grid_f32_kernel;
+}
+
 // CTAs of the grid form: at least 32 rows each, at most one per SM; 0 when the
 // tile does not fit.
 static int pr_config(int m, int w, int tsize, const DevInfo& dev, int gmax, int* R, int* nt, size_t* smem) {
   if (w < 1 || w > 512 || m < w || gmax < 1) return 0;
   int g = dev.sm_count < gmax ? dev.sm_count : gmax;
-  if (g > 256) g = 256;  // (a polling thread per CTA)
+  if (g > 32 * PR_HL) g = 32 * PR_HL;
   if ((int64_t)g * 32 > m) g = (int)cdiv(m, 32);
   *R = (int)cdiv(m, g);
   if (*R > PC_NTMAX || m >= (1 << 20)) return 0;
-  *nt = *R <= 64 ? 256 : PC_NTMAX;
+  *nt = *R <= (tsize == 8 ? 32 : 64) ? 256 : PC_NTMAX;
   *smem = pr_smem_bytes(*R, w, tsize);
   if (*smem + 1024 > (size_t)dev.max_smem_optin) return 0;
   return (int)cdiv(m, *R);
@@ -852,7 +1117,7 @@ cudaError_t launch_panel_resident(T* Wkk, int64_t ldw, int m, int w, int kabs, i
   size_t smem = 0;
   const int G = s.xres == nullptr ? 0 : pr_config(m, w, sizeof(T), dev, s.gmax, &P.R, &nt, &smem);
   if (G <= 0 || w > s.wmax) return cudaErrorInvalidConfiguration;
-  cudaError_t e = allow_max_smem((const void*)panel_resident_kernel<T>);
+  cudaError_t e = allow_max_smem(pr_kernel<T>());
   if (e != cudaSuccess) return e;
   P.A = Wkk;
   P.ld = ldw;
@@ -870,7 +1135,7 @@ cudaError_t launch_panel_resident(T* Wkk, int64_t ldw, int m, int w, int kabs, i
   e = cudaMemsetAsync(P.head, 0, (char*)(P.rows + (size_t)PC_NBUF * G * P.rstride) - (char*)P.head, st);
   if (e != cudaSuccess) return e;
   void* args[] = {&P};
-  return launch_cooperative((const void*)panel_resident_kernel<T>, G, nt, args, smem, st);
+  return launch_cooperative(pr_kernel<T>(), G, nt, args, smem, st);
 }
 
 #define GB_INST(T)                                                                                            \

@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 SIZES = [(1, 1), (31, 31), (32, 5), (33, 33), (64, 64), (65, 17), (129, 100), (257, 3), (512, 64), (513, 63),
          (1025, 33), (2049, 128), (5625, 64), (5626, 64), (8192, 32), (8193, 32),
-         (2187, 64), (2188, 64), (4865, 100), (6240, 128), (7001, 129), (9000, 512)]
+         (1562, 64), (1563, 64), (2187, 64), (2188, 64), (4865, 100), (6240, 128), (7001, 129), (9000, 512)]
 
 
 @pytest.fixture(scope="module")
