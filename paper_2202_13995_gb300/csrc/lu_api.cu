@@ -482,9 +482,11 @@ static int gemm_cap(lu_ctx c) { return c->gemm_ctas > 0 ? c->gemm_ctas : c->dev.
 // certificate's sum is short and fails on dense matrices too) and from
 // kCertRest remaining rows on, where they win over the FP64 CUDA cores (all
 // updates of a factorization: n = 8192, nb = 192, 290 -> 26 ms; n = 2048,
-// nb = 64, 6.0 -> 3.1 ms; n = 600, nb = 64, where two updates lie above the
-// line, 0.7 ms either way); the CUDA cores otherwise.
-constexpr int kCertNb = 64, kCertRest = 384;
+// nb = 64, 6.0 -> 3.1 ms); the CUDA cores otherwise.  The line, by whole
+// factorizations (ms with it at 384, 512, 640, 768, 900): n = 1023, nb = 64
+// 2.95 2.86 2.81 2.79 2.83; n = 1280, nb = 128 3.93 3.89 3.85 3.87 4.03;
+// n = 2048, nb = 128 6.83 6.79 6.77 6.79 6.95.
+constexpr int kCertNb = 64, kCertRest = 640;
 static bool cert_applies(int n, int nb) { return nb >= kCertNb && nb <= 256 && n - nb >= kCertRest; }
 static size_t cert_ints(int n, int nb) { return 1 + (size_t)(n / nb + 1) + oz_cert_blocks(n, n); }
 

@@ -15,18 +15,18 @@ struct NbEntry {
 };
 
 constexpr NbEntry kNbTable[] = {
-    {0, 800, 32},  // f64, measured at n = 600: nb 32: 1.727, nb 64: 1.832, nb 96: 1.822, nb 128: 1.822, nb 192: 2.119, nb 256: 2.215
-    {0, 1280, 64},  // f64, measured at n = 1023: nb 32: 3.372, nb 64: 3.378, nb 96: 3.405, nb 128: 3.399, nb 192: 3.890, nb 256: 4.052
-    {0, 3072, 128},  // f64, measured at n = 2048: nb 32: 11.491, nb 64: 8.497, nb 96: 8.119, nb 128: 7.863, nb 192: 8.313, nb 256: 8.813
-    {0, 4608, 128},  // f64, measured at n = 4096: nb 32: 54.039, nb 64: 24.168, nb 96: 21.382, nb 128: 19.882, nb 192: 19.895, nb 256: 20.440
-    {0, 7168, 192},  // f64, measured at n = 6000: nb 32: 145.503, nb 64: 50.987, nb 96: 42.636, nb 128: 37.990, nb 192: 36.308, nb 256: 36.872
-    {0, 12288, 256},  // f64, measured at n = 8192: nb 32: 340.574, nb 64: 101.188, nb 96: 80.685, nb 128: 69.635, nb 192: 63.104, nb 256: 62.336
+    {0, 800, 64},  // f64, measured at n = 600: nb 32: 1.680, nb 64: 1.585, nb 96: 1.600, nb 128: 1.640, nb 192: 1.852, nb 256: 2.035
+    {0, 1280, 64},  // f64, measured at n = 1023: nb 32: 3.286, nb 64: 3.083, nb 96: 3.131, nb 128: 3.314, nb 192: 3.611, nb 256: 3.920
+    {0, 3072, 128},  // f64, measured at n = 2048: nb 32: 11.199, nb 64: 7.896, nb 96: 7.569, nb 128: 7.360, nb 192: 7.743, nb 256: 8.409
+    {0, 4608, 128},  // f64, measured at n = 4096: nb 32: 53.185, nb 64: 23.485, nb 96: 20.599, nb 128: 19.022, nb 192: 18.948, nb 256: 19.644
+    {0, 7168, 192},  // f64, measured at n = 6000: nb 32: 145.067, nb 64: 50.690, nb 96: 41.958, nb 128: 36.996, nb 192: 34.807, nb 256: 35.107
+    {0, 12288, 256},  // f64, measured at n = 8192: nb 32: 340.921, nb 64: 101.347, nb 96: 79.956, nb 128: 68.142, nb 192: 60.611, nb 256: 59.217
     {0, 24576, 256},  // f64, measured at n = 16384: nb 32: 2521.305, nb 64: 608.801, nb 96: 447.020, nb 128: 361.227, nb 192: 289.931, nb 256: 260.948
     {0, 1073741824, 256},  // f64, measured at n = 32768: not measured: n = 32768 keeps the smaller size's choice
-    {1, 1280, 128},  // f64_split, measured at n = 1024: nb 64: 4.817, nb 128: 4.150, nb 192: 4.416, nb 256: 4.354
-    {1, 3072, 128},  // f64_split, measured at n = 2048: nb 64: 10.953, nb 128: 9.130, nb 192: 9.128, nb 256: 9.207
-    {1, 4608, 256},  // f64_split, measured at n = 4096: nb 64: 28.511, nb 128: 21.894, nb 192: 20.868, nb 256: 20.433
-    {1, 7168, 256},  // f64_split, measured at n = 7001: nb 64: 77.134, nb 128: 53.242, nb 192: 47.253, nb 256: 45.692
+    {1, 1280, 128},  // f64_split, measured at n = 1024: nb 64: 4.663, nb 128: 4.065, nb 192: 4.094, nb 256: 4.206
+    {1, 3072, 128},  // f64_split, measured at n = 2048: nb 64: 10.488, nb 128: 8.692, nb 192: 8.566, nb 256: 8.808
+    {1, 4608, 256},  // f64_split, measured at n = 4096: nb 64: 27.908, nb 128: 21.090, nb 192: 19.890, nb 256: 19.625
+    {1, 7168, 256},  // f64_split, measured at n = 7001: nb 64: 76.885, nb 128: 51.887, nb 192: 45.207, nb 256: 43.258
     {1, 12288, 256},  // f64_split, measured at n = 8192: nb 64: 107.476, nb 128: 71.496, nb 192: 61.973, nb 256: 58.585
     {1, 24576, 256},  // f64_split, measured at n = 16384: nb 64: 607.516, nb 128: 353.454, nb 192: 274.128, nb 256: 237.480
     {1, 1073741824, 256},  // f64_split, measured at n = 32768: nb 64: 4066.466, nb 128: 2244.717, nb 192: 1653.813, nb 256: 1410.500

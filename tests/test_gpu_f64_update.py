@@ -35,7 +35,7 @@ def _dev(a):
 
 # one step, the first size that takes the split update, the last that does not, ragged last blocks,
 # widths below, at and above the certificate's least and most
-@pytest.mark.parametrize("n,nb", [(447, 64), (448, 64), (449, 64), (449, 63), (600, 65), (1030, 64), (777, 128),
+@pytest.mark.parametrize("n,nb", [(703, 64), (704, 64), (705, 64), (705, 63), (600, 65), (1030, 64), (777, 128),
                                   (900, 256), (1000, 257)])
 @pytest.mark.parametrize("nopiv", [False, True])
 def test_factors_at_the_edges_of_the_rule(ctx, n, nb, nopiv):
