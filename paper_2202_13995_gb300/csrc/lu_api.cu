@@ -164,7 +164,7 @@ struct lu_fact_s {
   bool ozaki = false;   // FP64 trailing update by error-free splitting
   void* oz_ws = nullptr;
   double* oz_minv = nullptr;  // nb x nb: I - L11^-1 of the current block
-  int* oz_cert = nullptr;     // plain FP64 with certified split updates: flag, counts per step, block list
+  int* oz_cert = nullptr;     // plain FP64 with certified split updates: two flags, two counts per step, block list
   int* spec_flag = nullptr;   // diagonal-pivot check flags (SpecArgs), FP32 panels
   void* spec_backup = nullptr;  // n x nb FP32: a checked panel's rows before the check
   void* uinv = nullptr;         // nb x 32: inverses of the diagonal blocks of a block column's U
@@ -488,7 +488,52 @@ static int gemm_cap(lu_ctx c) { return c->gemm_ctas > 0 ? c->gemm_ctas : c->dev.
 // n = 2048, nb = 128 6.83 6.79 6.77 6.79 6.95.
 constexpr int kCertNb = 64, kCertRest = 640;
 static bool cert_applies(int n, int nb) { return nb >= kCertNb && nb <= 256 && n - nb >= kCertRest; }
-static size_t cert_ints(int n, int nb) { return 1 + (size_t)(n / nb + 1) + oz_cert_blocks(n, n); }
+static size_t cert_heads(int n, int nb) { return 2 + 2 * (size_t)(n / nb + 1); }
+static size_t cert_ints(int n, int nb) { return cert_heads(n, nb) + oz_cert_blocks(n, n); }
+
+// C (m x cols) -= A B in certified split products, an update of step `step`: the
+// trailing one (top = 0) or the one inside the top solve (top = 1), which have
+// their own flag and count.
+static cudaError_t update_cert(lu_fact f, int ph, double* C, const double* A, const double* B, int m, int cols, int k,
+                               int step, int top) {
+  lu_ctx c = f->ctx;
+  cudaStream_t st = c->stream;
+  const int64_t ld = f->ldw;
+  OzCert cert;
+  cert.off = f->oz_cert + top;
+  cert.cnt = f->oz_cert + 2 + 2 * step + top;
+  cert.list = f->oz_cert + cert_heads(f->n, f->nb);
+  cert.tag = step + 1;
+  cudaError_t e = PHASE(c, ph == PH_GEMM ? PH_CAST : ph, 2,
+                        ozaki_split(A, ld, B, ld, m, cols, k, f->oz_ws, c->d_status, st, &cert));
+  if (e == cudaSuccess)
+    e = PHASE(c, ph, 1, ozaki_gemm(C, ld, f->oz_ws, m, cols, k, 0, cols, c->d_status, c->dev, st, 0, &cert));
+  if (e == cudaSuccess) e = PHASE(c, ph, 1, launch_gemm_list(C, ld, A, ld, B, ld, m, cols, k, cert, c->dev, st));
+  return e;
+}
+
+// The plain FP64 factorization's top solve: for blocks of 256 and from kTopRest
+// columns on in two halves of L11, whose off-diagonal block is a certified split
+// update: the substitution, bound by the FP64 pipes, then has half of the
+// products.  Whole factorizations, ms without and with the line at 6000, 4500,
+// 3000, 2000, 1000: n = 8192, nb = 256 56.2, 55.3 54.9 54.8 54.8 54.9; n = 16384
+// 243.2, 234.9 234.4 234.3 234.4 234.5.  Narrower blocks leave too little to
+// halve (n = 8192, nb = 192 57.4, 57.3 57.4 57.6; n = 4096, nb = 128 17.7, 17.7
+// 17.7 18.1).
+constexpr int kTopW = 256, kTopRest = 3000;
+static cudaError_t top_solve_f64(lu_fact f, const double* L11, double* U12, int w, int rest, int step) {
+  lu_ctx c = f->ctx;
+  const int64_t ld = f->ldw;
+  if (f->oz_cert == nullptr || w < kTopW || rest < kTopRest)
+    return PHASE(c, PH_TRSM, 1, launch_trsm_lower<double>(L11, U12, ld, w, rest, c->stream));
+  const int h = (w / 2 + 63) / 64 * 64;
+  double* X2 = U12 + (int64_t)h * ld;
+  const double* L21 = L11 + (int64_t)h * ld;
+  cudaError_t e = PHASE(c, PH_TRSM, 1, launch_trsm_lower<double>(L11, U12, ld, h, rest, c->stream));
+  if (e == cudaSuccess) e = update_cert(f, PH_TRSM, X2, L21, U12, w - h, rest, h, step, 1);
+  if (e == cudaSuccess) e = PHASE(c, PH_TRSM, 1, launch_trsm_lower<double>(L21 + h, X2, ld, w - h, rest, c->stream));
+  return e;
+}
 
 static int update_f64(lu_fact f, double* A22, const double* L21, const double* U12, int rest, int w, int step) {
   lu_ctx c = f->ctx;
@@ -498,14 +543,7 @@ static int update_f64(lu_fact f, double* A22, const double* L21, const double* U
     CU_TRY(PHASE(c, PH_GEMM, 1, launch_gemm_simt<double>(A22, ld, L21, ld, U12, ld, rest, rest, w, st)));
     return LU_OK;
   }
-  OzCert cert;
-  cert.off = f->oz_cert;
-  cert.cnt = f->oz_cert + 1 + step;
-  cert.list = f->oz_cert + 1 + (f->n / f->nb + 1);
-  cert.tag = step + 1;
-  CU_TRY(PHASE(c, PH_CAST, 2, ozaki_split(L21, ld, U12, ld, rest, rest, w, f->oz_ws, c->d_status, st, &cert)));
-  CU_TRY(PHASE(c, PH_GEMM, 1, ozaki_gemm(A22, ld, f->oz_ws, rest, rest, w, 0, rest, c->d_status, c->dev, st, 0, &cert)));
-  CU_TRY(PHASE(c, PH_GEMM, 1, launch_gemm_list(A22, ld, L21, ld, U12, ld, rest, rest, w, cert, c->dev, st)));
+  CU_TRY(update_cert(f, PH_GEMM, A22, L21, U12, rest, rest, w, step, 0));
   return LU_OK;
 }
 
@@ -573,6 +611,8 @@ static int factor_loop(lu_fact f) {
       // (the tensor-core form also writes the solved columns' B operand)
       CU_TRY(PHASE(c, PH_TRSM, 1, launch_trsm_inv((const float*)Wkk, (float*)U12, ld, w, split_top ? w2 : rest, kind,
                                                    f->bop, f->kpad, c->d_status, st)));
+    } else if constexpr (sizeof(T) == 8) {
+      CU_TRY(top_solve_f64(f, Wkk, U12, w, rest, k / nb));
     } else {
       CU_TRY(PHASE(c, PH_TRSM, 1, launch_trsm_lower<T>(Wkk, U12, ld, w, split_top ? w2 : rest, st)));
     }
@@ -828,7 +868,7 @@ extern "C" int lu_factor_ex(lu_ctx c, int n, const double* dA, int lda, lu_prec 
     return r;
   };
   if (cudaMemsetAsync(f->info_d, 0x7f, sizeof(int), st) != cudaSuccess) return fail(LU_ECUDA);
-  if (f->oz_cert && cudaMemsetAsync(f->oz_cert, 0, (2 + (size_t)(n / f->nb)) * sizeof(int), st) != cudaSuccess)
+  if (f->oz_cert && cudaMemsetAsync(f->oz_cert, 0, cert_heads(n, f->nb) * sizeof(int), st) != cudaSuccess)
     return fail(LU_ECUDA);
   if (f->spec_flag && cudaMemsetAsync(f->spec_flag, 0, 4 * sizeof(int), st) != cudaSuccess) return fail(LU_ECUDA);
   if (n > 0) {

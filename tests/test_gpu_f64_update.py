@@ -36,7 +36,9 @@ def _dev(a):
 # one step, the first size that takes the split update, the last that does not, ragged last blocks,
 # widths below, at and above the certificate's least and most
 @pytest.mark.parametrize("n,nb", [(703, 64), (704, 64), (705, 64), (705, 63), (600, 65), (1030, 64), (777, 128),
-                                  (900, 256), (1000, 257)])
+                                  (900, 256), (1000, 257),
+                                  # the top solve in halves: from 3000 columns on, blocks of 256
+                                  (3255, 256), (3256, 256), (3301, 256), (3301, 255)])
 @pytest.mark.parametrize("nopiv", [False, True])
 def test_factors_at_the_edges_of_the_rule(ctx, n, nb, nopiv):
     A = I.hpl_matrix(n, 300 + n + nb, diag_shift=n / 4 if nopiv else 0.0)
@@ -66,13 +68,12 @@ def _system(kind, n, rng):
     return A
 
 
-@pytest.mark.parametrize("nb", [64, 128])
+@pytest.mark.parametrize("n,nb", [(1100, 64), (1100, 128), (3301, 256)])
 @pytest.mark.parametrize("kind", ["row_scaled", "rows_far_apart", "column_scaled", "banded", "sparse", "half_scaled"])
-def test_componentwise_backward_error(ctx, kind, nb):
+def test_componentwise_backward_error(ctx, kind, n, nb):
     """|b - A x| <= c (|A||x| + |b|) row by row.  Partial pivoting gives
     |b - A x| <= 3 n u |P^T L||U||x| (N. Higham, Accuracy and Stability of Numerical
     Algorithms, theorem 9.4); the factor beside the rows' own sums is the oracle's."""
-    n = 1100
     rng = np.random.default_rng(17)
     A = _system(kind, n, rng)
     x0 = rng.random((n, 1)) - 0.5
