@@ -228,16 +228,6 @@ __device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ float cluster_ld(uint32_t addr, float) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ double cluster_ld(uint32_t addr, double) {
-  double v;
-  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
-  return v;
-}
 // the hardware cluster barrier, release / acquire at cluster scope: every
 // CTA's prior shared and global writes are visible to every peer after it
 __device__ __forceinline__ void cluster_sync() {

@@ -78,7 +78,8 @@ template <typename T>
 cudaError_t launch_panel_cluster(T* Wkk, int64_t ldw, int m, int w, int kabs, int* ipiv, int* info, int* status,
                                  int* perm, const DevInfo& dev, cudaStream_t st);
 // The panel resident in the shared memory of a cooperative grid (also
-// panel_cluster.cu), for panels that do not fit a cluster: CTAs it would take
+// panel_cluster.cu), for panels that do not fit a cluster and FP64 ones that
+// more SMs' FP64 pipes finish sooner: CTAs it would take
 // (0: it does not fit, or the scratch has no xres), and the launch.
 size_t panel_resident_bytes(int gmax, int wmax, int tsize);
 template <typename T>

@@ -14,7 +14,7 @@
 // factored by one CTA in shared memory -- the LU of the slab's h x h diagonal
 // block and its U rows to the right -- and then every row below the slab gets
 // its L columns (X <- X U^-1 for the slab's h columns) and the update of the
-// block column's remaining columns, a CTA per 64 rows.  The next slab starts
+// block column's remaining columns, a CTA per 16 to 64 rows.  The next slab starts
 // h rows and h columns further down.  The same two kernels serve the
 // diagonal-pivot check of a pivoted panel (SpecArgs in kernels.h).
 #include "common.cuh"

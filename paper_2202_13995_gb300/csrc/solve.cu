@@ -473,7 +473,6 @@ cudaError_t launch_trinv(const T* W, int64_t ldw, int n, T* Dinv, cudaStream_t s
   return cudaGetLastError();
 }
 template cudaError_t launch_trinv<float>(const float*, int64_t, int, float*, cudaStream_t);
-template cudaError_t launch_trinv<double>(const double*, int64_t, int, double*, cudaStream_t);
 
 // One launch pair for up to 32 right-hand sides: a CTA holds up to 16 with
 // FP32 factors, 2 with FP64, whose products with the block before run at two
