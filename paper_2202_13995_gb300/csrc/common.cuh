@@ -228,6 +228,12 @@ __device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
+// Programmatic dependent launch: a kernel launched with it may start once every
+// CTA of the kernel before it has called dependents_launch (or ended), and
+// previous_wait returns when that kernel has ended and its writes are visible
+// (at once for an ordinary launch).
+__device__ __forceinline__ void previous_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // the hardware cluster barrier, release / acquire at cluster scope: every
 // CTA's prior shared and global writes are visible to every peer after it
 __device__ __forceinline__ void cluster_sync() {

@@ -526,6 +526,7 @@ __global__ void __launch_bounds__(SL_THREADS) slab_lu_kernel(T* D, int64_t ld, i
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool spec = sp.flag != nullptr;
   bool bad = false;
+  previous_wait();
   if (spec) {
     const int f0 = __ldcg(sp.flag), f3 = __ldcg(sp.flag + 3);
     if (f0 != 0 || f3 != 0) {
@@ -579,6 +580,7 @@ __global__ void __launch_bounds__(SL_THREADS) slab_lu_kernel(T* D, int64_t ld, i
       __syncthreads();
     }
   }
+  dependents_launch();
   // (iii) on the first warps while the others write the slab back
   const int nblk = uinv != nullptr ? (hs + 31) / 32 : 0;
   const int w0 = nblk < SL_WARPS ? nblk : 0;
@@ -622,7 +624,7 @@ __global__ void __launch_bounds__(SL_THREADS) slab_lu_kernel(T* D, int64_t ld, i
 constexpr int LS_THREADS = 256;
 
 template <typename T, int RB>
-__global__ void __launch_bounds__(LS_THREADS) below_solve_kernel(const T* __restrict__ U, const T* __restrict__ uinv,
+__global__ void __launch_bounds__(LS_THREADS) below_solve_kernel(const T* U, const T* uinv,
                                                                  T* X, int64_t ld, int m, int ws, int wt,
                                                                  SpecDev<T> sp, int first, int tag) {
   static_assert(RB % 16 == 0 && RB <= LS_THREADS, "RB rows: 16 row groups, one thread per row");
@@ -640,6 +642,7 @@ __global__ void __launch_bounds__(LS_THREADS) below_solve_kernel(const T* __rest
   const int r0 = blockIdx.x * RB;
   const int rows = min(RB, m - r0);
   const bool spec = sp.flag != nullptr;
+  previous_wait();
   if (spec) {
     const bool stop = first ? __ldcg(sp.flag) != 0 : (__ldcg(sp.flag) != 0 || __ldcg(sp.flag + 3) != 0);
     if (stop) return;
@@ -749,6 +752,7 @@ __global__ void __launch_bounds__(LS_THREADS) below_solve_kernel(const T* __rest
     }
   }
   __syncthreads();
+  dependents_launch();
   for (int r = warp; r < rows; r += LS_THREADS / 32)
     for (int c = lane; c < wt; c += 32) X[(int64_t)(r0 + r) * ld + c] = Xs[r * wx + c];
   if (spec && __syncthreads_or(bad) && tid == 0) sp.flag[3] = tag;
@@ -785,15 +789,37 @@ static size_t ls_smem(int rb, int wt, int tsize) {
   return (32 * wu + 32 * 32 + (size_t)rb * (wt | 1) + 32 * (size_t)rb) * tsize;
 }
 
+// One launch of the block column's chain.  dependent: the launch before it in
+// the stream is the chain's own, whose kernels let the next one start while they
+// still write their results (the next one waits for them at its start): it hides
+// the launch, not the work (mixed n = 1500 1.39 -> 1.36 ms, no-pivot n = 6000 6.68
+// -> 6.61).  Only up to 16 * 304 rows, where the rows below are one wave: the
+// waiting CTAs of a larger launch keep the trailing update beside the panel off
+// their SMs (mixed n = 32768 114.3 -> 116.5 ms).
+template <typename... P, typename... A>
+static cudaError_t launch_chain(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st,
+                                bool dependent, A... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 template <typename T, int RB>
 static cudaError_t launch_ls(const T* U, const T* uinv, T* X, int64_t ld, int m, int ws, int wt,
                              const SpecDev<T>& sp, int first, int tag, cudaStream_t st) {
   auto kern = below_solve_kernel<T, RB>;
   cudaError_t e = allow_max_smem((const void*)kern);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)cdiv(m, RB), LS_THREADS, ls_smem(RB, wt, sizeof(T)), st>>>(U, uinv, X, ld, m, ws, wt, sp, first,
-                                                                               tag);
-  return cudaGetLastError();
+  return launch_chain(kern, (unsigned)cdiv(m, RB), LS_THREADS, ls_smem(RB, wt, sizeof(T)), st, m <= 16 * 304,
+                      U, uinv, X, ld, m, ws, wt, sp, first, tag);
 }
 
 template <typename T>
@@ -820,13 +846,12 @@ static cudaError_t launch_below(const T* U, const T* uinv, T* X, int64_t ld, int
 // One slab: a CTA with the slab in shared memory.
 template <typename T>
 static cudaError_t launch_slab(T* D, int64_t ld, int hs, int wt, int kabs, int* info, const SpecDev<T>& sp,
-                               int first, int tag, int restore, T* uinv, cudaStream_t st) {
+                               int first, int tag, int restore, T* uinv, cudaStream_t st, bool dependent) {
   auto kern = slab_lu_kernel<T>;
   cudaError_t e = allow_max_smem((const void*)kern);
   if (e != cudaSuccess) return e;
-  kern<<<1, SL_THREADS, slab_smem_bytes(hs, wt, sizeof(T)), st>>>(D, ld, hs, wt, kabs, info, sp, first, tag, restore,
-                                                                   uinv);
-  return cudaGetLastError();
+  return launch_chain(kern, 1, SL_THREADS, slab_smem_bytes(hs, wt, sizeof(T)), st, dependent, D, ld, hs, wt, kabs, info,
+                      sp, first, tag, restore, uinv);
 }
 
 template <typename T>
@@ -848,7 +873,7 @@ cudaError_t launch_block_column(T* P, int64_t ld, int m, int w, int kabs, int* i
     const int below = m - s0 - hs;
     T* ui = uinv + (size_t)(s0 / 32) * 1024;  // the slab's diagonal blocks' inverses (for the rows below)
     if ((e = launch_slab<T>(D, ld, hs, wt, kabs + s0, info, spec_dev<T>(spec, 0), first, tag, restore,
-                            below > 0 ? ui : nullptr, st)) != cudaSuccess)
+                            below > 0 ? ui : nullptr, st, !first && m <= 16 * 304)) != cudaSuccess)
       return e;
     if (below > 0) {
       // the first slab's rows below it follow its rows in the backup (row stride w)
