@@ -547,6 +547,14 @@ static int update_f64(lu_fact f, double* A22, const double* L21, const double* U
   return LU_OK;
 }
 
+// The mixed factorizations' lookahead stops when fewer rows than this remain:
+// the update is then too short to hide a panel, and the two streams' events cost
+// more than they give.  Factorizations, ms with the line at 0, 800, 1500, 2200,
+// 3000, 4500: n = 1024 0.694 0.663 0.668 0.666 0.666 0.663; n = 2048 1.364 1.342
+// 1.337 1.310 1.311 1.313; n = 4096 2.901 2.878 2.876 2.858 2.886 2.929;
+// n = 8192 6.565 6.541 6.501 6.492 6.522 6.597.
+constexpr int kLookRest = 2200;
+
 template <typename T>
 static int factor_loop(lu_fact f) {
   lu_ctx c = f->ctx;
@@ -602,7 +610,7 @@ static int factor_loop(lu_fact f) {
     // after the update instead, and is faster alone than the cooperative panel
     // beside it)
     const bool split_top =
-        tc && lookahead && rest > w2 &&
+        tc && lookahead && rest > w2 && rest >= kLookRest &&
         !(mode == SPEC_OFF &&
           (panel_cluster_fits<T>(rest, w2, c->dev) || panel_resident_ctas<T>(rest, w2, c->dev, f->ps) > 0));
     if (f->ozaki) {
@@ -711,7 +719,7 @@ static int factor_loop_nopiv(lu_fact f) {
     T* L21 = Wkk + (int64_t)w * ld;
     T* A22 = L21 + w;
     const int w2 = rest < nb ? rest : nb;
-    const bool split_top = tc && lookahead && rest > w2;  // as in factor_loop
+    const bool split_top = tc && lookahead && rest > w2 && rest >= kLookRest;  // as in factor_loop
     if (f->ozaki) {
       CU_TRY(top_solve_split(f, (double*)Wkk, (double*)U12, ld, w, rest));
     } else if (tc) {
