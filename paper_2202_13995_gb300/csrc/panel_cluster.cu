@@ -557,8 +557,13 @@ cudaError_t launch_panel_cluster(T* Wkk, int64_t ldw, int m, int w, int kabs, in
 // 8192 x 128 6.7 -> 3.1, 7000 x 256 7.7 -> 3.6 (there the FP64 pipes set the
 // pace: 256 columns of 47 rows); FP32 8192 x 128 4.5 -> 2.2.
 // The record buffers' stamps are cleared before the launch; a buffer is
-// reused every third column (the argument above).  Every poll is bounded; a CTA whose poll runs
-// out raises ST_TIMEOUT and leaves, and so do the others in their turn.
+// reused every third column (the argument above).  What is not stamped, the rows
+// that a CTA loads before its first header and others overwrite at the end and the
+// count of the permutation record, is ordered once a panel: the thread that writes
+// the headers fences before its first one, every thread after the last column,
+// when its CTA has read every CTA's first header.  Every poll is bounded; a CTA
+// whose poll runs out raises ST_TIMEOUT and leaves, and so do the others in their
+// turn.
 
 // A value between its stamps: a double as two 8-byte words {low half, stamp},
 // {high half, stamp}, a float as one; relaxed loads and stores (each 8-byte word
@@ -708,6 +713,7 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_grid_f64_kernel(PrParams<do
       e.z = (unsigned)k.pos;
     }
     const unsigned stamp = (unsigned)c + 1u;
+    if (c == 0 && tid == nt - 1) __threadfence();  // (the CTA's row loads and the count's zero, before the barrier above)
     if (tid == nt - 1)
       pr_store(P.head + (size_t)buf * G + cta,
                make_ulonglong2(((unsigned long long)e.x << 32) | stamp,
@@ -857,6 +863,7 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_grid_f64_kernel(PrParams<do
     }
     buf = nbuf;
   }
+  __threadfence();  // (after every CTA's first header: their row loads and the count's zero)
   __syncthreads();
   if (!ok || abort_flag) return;
   if (chain && live) sp[r] = pos;
@@ -923,6 +930,7 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_grid_f32_kernel(PrParams<fl
       e.z = (unsigned)k.pos;
     }
     const unsigned stamp = (unsigned)c + 1u;
+    if (c == 0 && tid == nt - 1) __threadfence();  // (the CTA's row loads and the count's zero, before the barrier above)
     if (tid == nt - 1)
       pr_store(P.head + (size_t)buf * G + cta,
                make_ulonglong2(((unsigned long long)e.x << 32) | stamp,
@@ -1066,6 +1074,7 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_grid_f32_kernel(PrParams<fl
     }
     buf = nbuf;
   }
+  __threadfence();  // (after every CTA's first header: their row loads and the count's zero)
   __syncthreads();
   if (!ok || abort_flag) return;
   if (chain && live) sp[r] = pos;

@@ -92,3 +92,27 @@ def test_permutation_record_reaches_the_other_columns(ctx):
         d = np.abs(f.lu().cpu().numpy() - LUo).max()
         assert d <= 256 * n * 2.0 ** -53 * np.abs(LUo).max()
         f.free()
+
+
+@pytest.mark.parametrize("n,nb,prec", [(8300, 1, "f32"), (8300, 2, "f32"), (6400, 16, "f64")])
+def test_permutation_record_of_narrow_grid_panels(ctx, n, nb, prec):
+    """Panels of few columns on the grid, where the permutation record's count is zeroed
+    and counted up within a column or two: |P A - L U| <= n u |L||U| (Higham, theorem 9.3)
+    in every column, which a row missing from the record would break by O(1)."""
+    import torch
+    from paper_2202_13995_gb300 import inputs as I
+    A = I.hpl_matrix_torch(n, 19 + nb, device="cuda")
+    f = ctx.factor(A, prec, nb)
+    assert f.info == 0
+    p = np.arange(n)
+    for j, q in enumerate(f.ipiv().cpu().numpy()):
+        p[j], p[q - 1] = p[q - 1], p[j]
+    LU = f.lu().double()
+    f.free()
+    if prec == "f32":
+        A = A.float().double()
+    L, R = torch.tril(LU, -1), torch.triu(LU)
+    L.diagonal().fill_(1.0)
+    d = (A[torch.from_numpy(p).cuda()] - L @ R).abs()
+    u = 2.0 ** -24 if prec == "f32" else 2.0 ** -53
+    assert bool((d <= n * u * (L.abs() @ R.abs())).all())
