@@ -364,10 +364,12 @@ __device__ __forceinline__ unsigned long long oz_corr(int t) {
 }
 
 // C - I 2^E: I converted to FP64 (one rounding), scaled by 2^E through its
-// exponent field (exact; two exact power-of-two products outside the normal
-// range), then subtracted (one rounding).
+// exponent field (exact; two power-of-two products outside the normal range, of
+// which only the second can round), then subtracted (one rounding).  Below
+// 2^-1138 the product, |I| < 2^63, rounds to zero, and 2^(E/2) may have no
+// exponent field (all-zero lines come here too, with I = 0).
 __device__ __forceinline__ double oz_sub(double c, long long I, int E) {
-  if (I == 0) return c;
+  if (I == 0 || E < -1138) return c;
   double d = __ll2double_rn(I);
   const long long bits = __double_as_longlong(d);
   const int ex = (int)((bits >> 52) & 0x7ff) + E;

@@ -95,6 +95,23 @@ def test_componentwise_backward_error(ctx, kind, n, nb):
     f.free()
 
 
+@pytest.mark.parametrize("nopiv", [False, True])
+@pytest.mark.parametrize("s", [1e-295, 1e-302, 1e-307])
+def test_blocks_far_apart(ctx, s, nopiv):
+    """Two clusters with a coupling so small that its products with itself underflow
+    (the split's scale 2^(e_i + f_j - 54) is then below every FP64 number)."""
+    n, nb = 900, 64
+    A = I.hpl_matrix(n, 3, diag_shift=n / 4)
+    A[:450, 450:] *= s
+    A[450:, :450] *= s
+    f = ctx.factor(_dev(A), "f64", nb, nopiv=nopiv)
+    LUo, ipo, info = O.getrf(A)
+    assert f.info == info == 0
+    assert np.array_equal(f.ipiv().cpu().numpy(), ipo)
+    assert np.abs(f.lu().cpu().numpy() - LUo).max() <= 256 * n * U * np.abs(LUo).max()
+    f.free()
+
+
 @pytest.mark.parametrize("w", [1, 31, 32, 33, 64, 100, 257, 512])
 @pytest.mark.parametrize("N", [1, 7, 8, 9, 130])
 def test_top_solve_edges(ctx, w, N):

@@ -117,6 +117,25 @@ def test_wide_dynamic_range_zero_lines(ctx):
     assert np.array_equal(got[:, 11], Cm[:, 11])
 
 
+@pytest.mark.parametrize("ea,eb", [(-500, -500), (-510, -540), (-520, -560), (-1000, -993), (-1000, -995), (-1020, -1020),
+                                   (500, -1060)])
+def test_products_at_the_end_of_the_exponent_range(ctx, ea, eb):
+    """Products that are normal, subnormal or below every FP64 number, with an accumulator of
+    their size and one that hides them: the bound of above plus two roundings of subnormals."""
+    m, n, k = 160, 140, 64
+    rng = np.random.default_rng(9)
+    Am = np.ldexp(rng.random((m, k)) - 0.5, ea)
+    Bm = np.ldexp(rng.random((k, n)) - 0.5, eb)
+    for Cm in (np.ldexp(rng.random((m, n)) - 0.5, max(ea + eb, -1000)), rng.random((m, n)) - 0.5):
+        LD = np.longdouble  # (the compensated update's own error terms underflow here)
+        ref = (Cm.astype(LD) - Am.astype(LD) @ Bm.astype(LD))
+        err = np.abs(_run(ctx, Cm, Am, Bm).astype(LD) - ref)
+        sc = np.ldexp(LD(1.0), (_expo(Am, 1)[:, None] + _expo(Bm, 0)[None, :]).astype(np.int64))
+        bound = LD(EPS) * ((1.13 * k + 4) * sc + np.abs(Am).astype(LD) @ np.abs(Bm).astype(LD) + 2 * np.abs(ref)) + \
+            2 * np.ldexp(LD(1.0), -1074)
+        assert (err <= bound).all()
+
+
 def test_non_finite_operand_is_reported(ctx):
     from paper_2202_13995_gb300 import lu
     m, n, k = 64, 64, 16
