@@ -165,6 +165,11 @@ __device__ __forceinline__ bool is_inf_mag(double v) {
   return (unsigned long long)__double_as_longlong(v) == 0x7ff0000000000000ull;
 }
 
+// neither zero, subnormal, infinite nor NaN (on the exponent field)
+__device__ __forceinline__ bool normal_number(double v) {
+  return (((unsigned)__double2hiint(v) >> 20) & 0x7ffu) - 1u < 2046u;
+}
+
 // a / p from r = 1 / p (rounded): P. Markstein's quotient correction ("Computation
 // of elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
 // Develop. 34, 1990): q = a r, then q + (a - p q) r, which rounds as the division

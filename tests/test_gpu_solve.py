@@ -325,3 +325,42 @@ def test_full_size_mixed_n32768_vs_oracle(ctx, mixed_n32768, prec):
     xo = ref["x"][:, 0]
     err = np.abs(X.cpu().numpy()[:, 0] - xo).max() / np.abs(xo).max()
     assert err <= max(1e-10, 10 * float(ref["kappa1_est"]) * EPS), err
+
+
+@pytest.mark.parametrize("A", [((1e200, 1e200), (0.0, 1e-150)), ((1.0, 3.0), (0.0, 1e-308)),
+                               ((1e-160, 1e-160), (0.0, 1e160)), ((1e-163, 1e-163), (0.0, 1e163))])
+def test_solve_where_u_over_its_pivot_leaves_the_normal_range(ctx, A):
+    """u_01 / u_11 overflows or is subnormal, the solution (1, 1) is ordinary: a product, a
+    subtraction and a quotient each round once or twice."""
+    A = np.array(A)
+    f = ctx.factor(_dev(A), "f64", 0)
+    X = _dev(A @ np.ones((2, 1)))
+    f.solve_(X)
+    assert np.abs(X.cpu().numpy() - 1.0).max() <= 8 * EPS
+    f.free()
+
+
+@pytest.mark.parametrize("n", [64, 65, 700])
+@pytest.mark.parametrize("scale", ["rows rising", "rows falling", "rows", "columns"])
+def test_solve_scaled_far_apart(ctx, n, scale):
+    """Upper triangular systems with rows or columns scaled by 10^-160 to 10^160: |b - U x| <=
+    (n + 4) u |U||x| + u |b| row by row (Higham, theorem 8.5; the reciprocals add two roundings)."""
+    rng = np.random.default_rng(n)
+    A = np.triu((rng.random((n, n)) - 0.5) / n) + np.diag(1 + rng.random(n))
+    e = 320 * rng.random(n) - 160
+    if scale.startswith("rows "):
+        e = np.sort(e)[:: 1 if scale.endswith("rising") else -1]
+    s = (10.0 ** e)[:, None]
+    A = A * (s.T if scale == "columns" else s)
+    x0 = (rng.random((n, 2)) - 0.5) / (s if scale == "columns" else 1.0)
+    B = A @ x0
+    f = ctx.factor(_dev(A), "f64", 64)
+    assert f.info == 0
+    X = _dev(B)
+    f.solve_(X)
+    x = X.cpu().numpy()
+    assert np.isfinite(x).all()
+    LD = np.longdouble
+    r = np.abs((B.astype(LD) - A.astype(LD) @ x.astype(LD)).astype(float))
+    assert (r <= (n + 4) * EPS * (np.abs(A) @ np.abs(x)) + EPS * np.abs(B)).all()
+    f.free()
