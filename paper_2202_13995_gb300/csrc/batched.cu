@@ -395,6 +395,10 @@ __device__ __noinline__ void bt_convert(const double* A, int lda, float* W, int 
 // which only the solves below read: their serial substitutions become products
 // (in FP32, as in the refinement's solves of large systems; the refinement
 // corrects the rounding).  A warp per block, a lane per column of the inverses.
+// An upper block whose inverse is not finite or reaches BT_INV_MAX (subnormal or
+// far smaller pivots than the rows beside them: products with it could overflow
+// where a substitution does not) stays, with its bit in misc[1], and is substituted.
+constexpr float BT_INV_MAX = 7.9228163e28f;  // 2^96
 template <int NT>
 __device__ __noinline__ void bt_invert(float* W, int ld, int n) {
   BatchSmem& sm = bt_smem();
@@ -403,6 +407,9 @@ __device__ __noinline__ void bt_invert(float* W, int ld, int n) {
   static_assert(NW * TW <= BT_NB * (BT_NMAX + BT_CW), "a block per warp in the factor-phase buffers");
   float* D = &sm.P[0][0] + warp * TW;  // [32][33]
   const int nblk = (n + BT_NB - 1) / BT_NB;
+  static_assert(BT_NMAX / BT_NB <= 32, "a bit per block in misc[1]");
+  if (threadIdx.x == 0) sm.misc[1] = 0;
+  __syncthreads();
   for (int b = warp; b < nblk; b += NW) {
     const int b0 = b * BT_NB, bw = min(BT_NB, n - b0);
 #pragma unroll 8
@@ -429,9 +436,16 @@ __device__ __noinline__ void bt_invert(float* W, int ld, int n) {
 #pragma unroll
       for (int q = 0; q < t; ++q) z[q] = fmaf(-D[q * (BT_NB + 1) + t], z[t], z[q]);
     }
+    bool fit = true;
 #pragma unroll
-    for (int t = 0; t < BT_NB; ++t)
-      if (t <= lane && lane < bw) W[(int64_t)sm.perm[b0 + t] * ld + b0 + lane] = z[t];
+    for (int t = 0; t < BT_NB; ++t) fit = fit && (t > lane || fabsf(z[t]) < BT_INV_MAX);
+    if (__all_sync(0xffffffffu, fit)) {
+#pragma unroll
+      for (int t = 0; t < BT_NB; ++t)
+        if (t <= lane && lane < bw) W[(int64_t)sm.perm[b0 + t] * ld + b0 + lane] = z[t];
+    } else if (lane == 0) {
+      atomicOr(&sm.misc[1], 1 << b);
+    }
     __syncwarp();
   }
   __syncthreads();
@@ -493,7 +507,16 @@ __device__ __noinline__ void bt_solve(const float* W, int ld, int n, int nr) {
       __syncthreads();
       for (int q = warp; q < nr; q += NT / 32) {
         float* yb = y + q * BT_NMAX + b0;
-        const float yl = lane < bw ? yb[lane] : 0.0f;
+        float yl = lane < bw ? yb[lane] : 0.0f;
+        if (!fwd && ((sm.misc[1] >> (b0 / BT_NB)) & 1)) {  // (a block left by bt_invert)
+          for (int t = bw - 1; t >= 0; --t) {
+            if (lane == t) yl = yl / sm.Ld[t][t];
+            const float yt = __shfl_sync(0xffffffffu, yl, t);
+            if (lane < t) yl = fmaf(-sm.Ld[lane][t], yt, yl);
+          }
+          if (lane < bw) yb[lane] = yl;
+          continue;
+        }
         float x[4] = {fwd ? yl : 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int t = 0; t < BT_NB; ++t) {

@@ -132,3 +132,39 @@ def test_solve_batched_in_place(ctx):
         xo, _, _, _ = O.solve(A, B)
         x = xd.cpu().numpy()
         assert np.abs(x - xo).max() / np.abs(xo).max() <= 1e-10
+
+
+def _block(u, at, n):
+    """A well-conditioned upper system of size n with the 2 x 2 block u on its diagonal at `at`."""
+    A = np.triu(np.full((n, n), 0.25 / n)) + np.eye(n)
+    A[at:at + 2, :] = A[:, at:at + 2] = 0.0
+    A[at:at + 2, at:at + 2] = u
+    return A
+
+
+def test_pivots_whose_reciprocal_overflows_fp32(ctx):
+    """Upper 32 x 32 blocks without a finite FP32 inverse (subnormal pivots, or pivots far below the
+    entry beside them) are substituted: alone, in a first, a middle and a ragged last block."""
+    tiny, far = np.diag([2.0 ** -130, 2.0 ** -129]), np.array([[1e-20, 1.0], [0.0, 1e-20]])
+    As = [np.array([[2e-39]]), far] + [_block(u, at, n) for u in (tiny, far) for at, n in ((0, 40), (40, 100), (96, 99))]
+    x0 = [np.array([[0.5]]), np.array([[0.0], [1.0]])]
+    for A in As[2:]:
+        x = np.linspace(-1.0, 1.0, 2 * A.shape[0]).reshape(-1, 2)
+        at = np.flatnonzero(np.diag(A) < 1e-10)
+        x[at] = [[0.0, 0.0], [1.0, -2.0]]
+        x0.append(x)
+    X, info, _, resid, _ = run_batch(ctx, As, [A @ x for A, x in zip(As, x0)])
+    assert np.all(info == 0), info
+    for x, want in zip(X, x0):
+        assert np.abs(x - want).max() <= 1e-10
+
+
+def test_wide_range_pivots_keep_their_products(ctx):
+    """Inverses on both sides of the line below which a block is inverted (2^96)."""
+    for d in (2.0 ** -94, 2.0 ** -97):
+        A = np.eye(70)
+        A[5, 5] = A[66, 66] = d
+        x = np.linspace(0.5, 2.0, 70).reshape(-1, 1)
+        X, info, _, _, _ = run_batch(ctx, [A], [A @ x])
+        assert info[0] == 0
+        assert np.abs(X[0] - x).max() <= 1e-10
