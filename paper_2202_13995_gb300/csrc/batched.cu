@@ -548,6 +548,13 @@ __device__ __noinline__ void bt_solve(const float* W, int ld, int n, int nr) {
   }
 }
 
+// The larger of two magnitudes, a NaN above every number (on the bit patterns: a
+// NaN that a maximum drops would make its system look converged)
+__device__ __forceinline__ double bt_max_mag(double a, double b) {
+  const unsigned long long ua = (unsigned long long)__double_as_longlong(a), ub = (unsigned long long)__double_as_longlong(b);
+  return __longlong_as_double((long long)(ua > ub ? ua : ub));
+}
+
 // r = b - A x in FP64 (A FP64 column-major), with the column maxima of |r|,
 // |x|, |b| and, on the first pass, the row sums of |A|.  Bound by the FP64
 // pipes (two multiply-adds per clock and SM), so every warp gets the same
@@ -607,9 +614,9 @@ __device__ __forceinline__ void bt_resid_rows(const BatchDesc& d, int n, const d
 #pragma unroll
         for (int u = 0; u < NR; ++u) {  // (a static index into the maxima)
           if (u == q) {
-            rmax[u] = fmax(rmax[u], fabs(rv));
-            xmax[u] = fmax(xmax[u], xv);
-            bmax[u] = fmax(bmax[u], fabs(bv));
+            rmax[u] = bt_max_mag(rmax[u], fabs(rv));
+            xmax[u] = bt_max_mag(xmax[u], xv);
+            bmax[u] = bt_max_mag(bmax[u], fabs(bv));
           }
         }
       }
@@ -620,7 +627,7 @@ __device__ __forceinline__ void bt_resid_rows(const BatchDesc& d, int n, const d
         double sum = 0.0;
 #pragma unroll
         for (int k = 0; k < BT_KS; ++k) sum += apart[(gg * BT_KS + k) * 32 + lane];
-        amax = fmax(amax, sum);
+        amax = bt_max_mag(amax, sum);
       }
     }
     __syncthreads();
@@ -639,13 +646,13 @@ __device__ __forceinline__ const double* block_max_many(const double* rmax, cons
   for (int k = 0; k < K; ++k) {
     double v = k < nr ? rmax[k] : k < 2 * nr ? xmax[k - nr] : k < 3 * nr ? bmax[k - 2 * nr] : amax;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, off));
+    for (int off = 16; off > 0; off >>= 1) v = bt_max_mag(v, __shfl_xor_sync(0xffffffffu, v, off));
     if (lane == 0) red[warp * 32 + k] = v;
   }
   __syncthreads();
   if ((int)threadIdx.x < K) {
     double m = 0.0;
-    for (int w = 0; w < nt / 32; ++w) m = fmax(m, red[w * 32 + threadIdx.x]);
+    for (int w = 0; w < nt / 32; ++w) m = bt_max_mag(m, red[w * 32 + threadIdx.x]);
     red[16 * 32 + threadIdx.x] = m;
   }
   __syncthreads();
@@ -746,8 +753,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) batched_kernel(const BatchDesc* 
         const double xn = cm[nr + q];
         const double bn = cm[2 * nr + q];
         const double den = eps * (anorm * xn + bn) * (double)n;
-        const double sc = den > 0.0 ? rn / den : (rn > 0.0 ? INFINITY : 0.0);
-        worst = fmax(worst, sc);
+        const double sc = den > 0.0 ? rn / den : (rn == 0.0 && den == 0.0 ? 0.0 : INFINITY);
+        worst = sc == sc ? fmax(worst, sc) : INFINITY;  // (fmax keeps an infinity)
         if (!(sc < tol)) still |= 1u << q;
       }
       active = still;

@@ -168,3 +168,17 @@ def test_wide_range_pivots_keep_their_products(ctx):
         X, info, _, _, _ = run_batch(ctx, [A], [A @ x])
         assert info[0] == 0
         assert np.abs(X[0] - x).max() <= 1e-10
+
+
+@pytest.mark.parametrize("where", ["A", "B"])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_non_finite_systems_are_not_reported_as_solved(ctx, bad, where):
+    As, Bs = make_batch(5, 8, nmin=30, nmax=100)
+    (As if where == "A" else Bs)[2][7, 0] = bad
+    X, info, _, resid, _ = run_batch(ctx, As, Bs)
+    assert info[2] != 0 and not resid[2] < 16.0
+    keep = [0, 1, 3, 4]
+    assert np.all(info[keep] == 0) and np.all(resid[keep] < 16.0)
+    for i in keep:
+        assert np.all(O.scaled_residual(As[i], X[i], Bs[i]) < 16.0)
+    assert ctx.status() in (0, 4)  # (a NaN that a panel meets is a range status too)
