@@ -37,8 +37,9 @@ extern "C" {
 /* Factor precision.  LU_F64: FP64 panel, FP64 trailing update (the plain
  * FP64 solve; large updates run as certified split products, see
  * LU_FACTOR_OZAKI: an element whose split error bound would exceed the FP64
- * dot product's, k 2^-53 sum_k |a b|, is updated on the FP64 CUDA cores).  LU_BF16 / LU_FP16: FP32 working matrix and panel, trailing
- * update on the tensor cores with BF16 / FP16 operands and FP32 accumulation;
+ * dot product's, k 2^-53 sum_k |a b|, is updated on the FP64 CUDA cores, as
+ * every element is with LU_FACTOR_DFMA).  LU_BF16 / LU_FP16: FP32 working
+ * matrix and panel, trailing update on the tensor cores with BF16 / FP16 operands and FP32 accumulation;
  * solutions are brought to FP64 accuracy by lu_refine.  LU_F32: FP32 panel and
  * FP32 trailing update on the CUDA cores. */
 typedef enum { LU_F64 = 0, LU_BF16 = 1, LU_FP16 = 2, LU_F32 = 3 } lu_prec;
@@ -124,8 +125,11 @@ int lu_factor(lu_ctx ctx, int n, const double *dA, int lda, lu_prec prec, int nb
  * 2^-53 * ((0.35 k + 4) * 2^(e_i + f_j) + sum_k |a b| + |result|), with 2^e_i and
  * 2^f_j the powers of two just above the largest |L21| of row i and |U12| of
  * column j: the order of an FP64 dot product's error bound.  Non-finite
- * operands fail with LU_ERANGE. */
-enum { LU_FACTOR_NOPIV = 1, LU_FACTOR_OZAKI = 2 };
+ * operands fail with LU_ERANGE.
+ * LU_FACTOR_DFMA (prec = LU_F64 only, not with LU_FACTOR_OZAKI): every update
+ * as FP64 multiply-adds on the CUDA cores, never as split products (n = 8192
+ * 340 ms instead of 55). */
+enum { LU_FACTOR_NOPIV = 1, LU_FACTOR_OZAKI = 2, LU_FACTOR_DFMA = 4 };
 int lu_factor_ex(lu_ctx ctx, int n, const double *dA, int lda, lu_prec prec, int nb, int flags, lu_fact *out,
                  int *info);
 

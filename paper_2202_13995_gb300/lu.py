@@ -24,7 +24,7 @@ LIB_PATH = os.environ.get("GB300LU_LIB") or os.path.join(_HERE, "libgb300lu.so")
 LU_F64, LU_BF16, LU_FP16, LU_F32 = 0, 1, 2, 3
 PRECS = {"f64": LU_F64, "bf16": LU_BF16, "fp16": LU_FP16, "f32": LU_F32}
 LU_OK, LU_ESINGULAR, LU_ENOMEM, LU_ENOTCONV, LU_ERANGE, LU_ETIMEOUT, LU_EAGAIN, LU_ECUDA, LU_EINTERNAL = range(9)
-LU_FACTOR_NOPIV, LU_FACTOR_OZAKI = 1, 2
+LU_FACTOR_NOPIV, LU_FACTOR_OZAKI, LU_FACTOR_DFMA = 1, 2, 4
 
 EXPORTED = [
     "lu_create", "lu_destroy", "lu_strerror", "lu_factor", "lu_fact_info", "lu_fact_ipiv", "lu_fact_lu",
@@ -289,17 +289,18 @@ class Context:
         return {p: (ms[i], int(nl[i])) for i, p in enumerate(PHASES)}
 
     def factor(self, A, prec="f64", nb: int = 0, sync: bool = True, nopiv: bool = False,
-               ozaki: bool = False) -> "Factor":
+               ozaki: bool = False, dfma: bool = False) -> "Factor":
         """Factor P A = L U of the column-major FP64 (n, n) tensor A (nopiv: the
         paper's no-pivot variant for diagonally dominant A; ozaki: FP64 trailing
-        update on the BF16 tensor cores by error-free splitting, prec f64)."""
+        update on the BF16 tensor cores by error-free splitting, prec f64; dfma:
+        every FP64 update as multiply-adds on the CUDA cores, prec f64)."""
         ptr, lda, ncol = _colmajor(A, "A")
         n = A.shape[0]
         if ncol != n:
             raise ValueError("A must be square")
         f = C.c_void_p()
         info = C.c_int(-1)
-        flags = (LU_FACTOR_NOPIV if nopiv else 0) | (LU_FACTOR_OZAKI if ozaki else 0)
+        flags = (LU_FACTOR_NOPIV if nopiv else 0) | (LU_FACTOR_OZAKI if ozaki else 0) | (LU_FACTOR_DFMA if dfma else 0)
         rc = load().lu_factor_ex(self._h, n, C.c_void_p(ptr), lda, _prec(prec), int(nb), flags,
                                  C.byref(f), C.byref(info) if sync else None)
         if f.value:

@@ -158,3 +158,33 @@ def test_non_finite_entries_are_reported(ctx):
             with pytest.raises(lu.LuError) as e:
                 ctx.factor(_dev(A), "f64", 64)
             assert e.value.code == lu.LU_ERANGE
+
+
+@pytest.mark.parametrize("nopiv", [False, True])
+@pytest.mark.parametrize("n,nb", [(900, 64), (3300, 256)])
+def test_update_on_the_fp64_cores_by_flag(ctx, n, nb, nopiv):
+    """LU_FACTOR_DFMA: the oracle's factors, without one split launch (the cast phase), where the
+    default splits."""
+    A = I.hpl_matrix(n, 31 + n, diag_shift=n / 4 if nopiv else 0.0)
+    LUo, ipo, info = O.getrf(A)
+    casts = {}
+    for dfma in (False, True):
+        ctx.profile(True)
+        ctx.profile_read()
+        f = ctx.factor(_dev(A), "f64", nb, nopiv=nopiv, dfma=dfma)
+        casts[dfma] = ctx.profile_read()["cast"][1]
+        ctx.profile(False)
+        assert f.info == info == 0
+        assert np.array_equal(f.ipiv().cpu().numpy(), ipo)
+        assert np.abs(f.lu().cpu().numpy() - LUo).max() <= 256 * n * U * np.abs(LUo).max()
+        f.free()
+    assert casts[True] == 0 < casts[False]
+
+
+def test_flag_combinations_that_are_refused(ctx):
+    from paper_2202_13995_gb300 import lu
+    A = _dev(I.hpl_matrix(64, 1))
+    for prec, kw in (("bf16", {}), ("f32", {}), ("f64", {"ozaki": True})):
+        with pytest.raises(lu.LuError) as e:
+            ctx.factor(A, prec, 0, dfma=True, **kw)
+        assert e.value.code == -7
