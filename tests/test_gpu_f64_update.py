@@ -188,3 +188,24 @@ def test_flag_combinations_that_are_refused(ctx):
         with pytest.raises(lu.LuError) as e:
             ctx.factor(A, prec, 0, dfma=True, **kw)
         assert e.value.code == -7
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("at", [(900, 5), (3, 900), (3, 3), (700, 850)])
+def test_non_finite_entries_without_pivoting(ctx, bad, at):
+    """Without pivoting nothing is searched and nothing refused: a non-finite entry spreads to the
+    same entries by the certified update as by multiply-adds, across a zero row and column too."""
+    n = 1000
+    A = I.hpl_matrix(n, 5, diag_shift=n / 4)
+    A[495, :495] = 0.0
+    A[:505, 505] = 0.0
+    A[at] = bad
+    out = []
+    for dfma in (False, True):
+        f = ctx.factor(_dev(A), "f64", 64, nopiv=True, dfma=dfma)
+        assert f.info == 0
+        out.append(f.lu().cpu().numpy())
+        f.free()
+    ok = np.isfinite(out[1])
+    assert not ok.all() and np.array_equal(np.isfinite(out[0]), ok)
+    assert np.abs(out[0][ok] - out[1][ok]).max() <= 256 * n * U * np.abs(out[1][ok]).max()
