@@ -65,7 +65,9 @@
 // sum_k |a b| >= G 2^(e_i + f_j - 14), so G >= (0.35 + 4 / 64) 2^14 makes the
 // bound at most k 2^-53 sum_k |a b|, the dot product's own (k >= 64).  A block of 32
 // rows x 64 columns with an element below that is left alone and listed, and
-// gemm_list_kernel updates the listed blocks in plain FP64.  When nearly every
+// gemm_list_kernel updates the listed blocks in plain FP64.  So are the blocks of a
+// line with an infinity or a NaN, which therefore spreads as in a plain FP64 update
+// (the form without a certificate reports it instead).  When nearly every
 // block of an update failed, the rest of the factorization goes to that kernel
 // whole (a device flag, which the split and product kernels read first).
 // Every mbarrier
@@ -87,6 +89,7 @@ constexpr int OZ_KMAX = 256;   // exactness bound on k (k * 128^2 <= 2^22)
 constexpr int OZ_MAG = OZ_S;   // the ninth slice of a certified update: magnitudes of slice 0
 constexpr float OZ_CERT_MIN = 6759.0f;  // (0.35 + 4 / 64) 2^14, rounded up
 constexpr int OZ_ZERO_LINE = -(1 << 20);  // exponent that marks an all-zero line
+constexpr int OZ_BAD_LINE = 1 << 20;      // ... and a line with an infinity or a NaN (its digits are all 0)
 constexpr int OZ_F = 40;       // fraction bits of the integer sum below the t = 0 term
 constexpr int OZ_BM = 128, OZ_BN = 128, OZ_BK = 64;
 constexpr int OZ_CHUNK = OZ_BM * OZ_BK * 2;          // 16 KB: one 128 x 64 BF16 box (A or B)
@@ -187,8 +190,8 @@ __global__ void __launch_bounds__(256) oz_split_rows_kernel(const double* __rest
     mx = o > mx ? o : mx;
   }
   const bool zero = __any_sync(0xffffffffu, bad);
-  if (zero && lane == 0) atomicOr(status, ST_RANGE);
-  const int e = zero ? 0 : oz_expo(mx);
+  if (zero && !mag && lane == 0) atomicOr(status, ST_RANGE);
+  const int e = zero ? OZ_BAD_LINE : oz_expo(mx);
   if (lane == 0) ea[i] = e;
   uint32_t* out = reinterpret_cast<uint32_t*>(As);
 #pragma unroll
@@ -253,8 +256,8 @@ __global__ void __launch_bounds__(256, 3) oz_split_cols_kernel(const double* __r
       b2 |= o == ~0ull;
       if (o != ~0ull) mx = o > mx ? o : mx;
     }
-    if (b2) atomicOr(status, ST_RANGE);
-    const int e = b2 ? 0 : oz_expo(mx);
+    if (b2 && !mag) atomicOr(status, ST_RANGE);
+    const int e = b2 ? OZ_BAD_LINE : oz_expo(mx);
     fe[lane] = (b2 || mx == 0) ? ZERO_COL : e;
     if (j < n) fb[j] = e;
   }
@@ -693,9 +696,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           const int tt = p + gq + q;
           if (p == OZ_MAG) {
             // G of this warp's 32 rows x 64 columns: all of them large enough, or
-            // the block goes to the list (all-zero lines pass: their part is 0)
+            // the block goes to the list (all-zero lines pass, as their part is 0,
+            // but not across a line with an infinity or a NaN, which fails)
             const uint32_t taddr = tmem_base + lane_addr + (uint32_t)(acc * OZ_BN + half * 64);
-            const bool zrow = rok && P.ea[row] == OZ_ZERO_LINE;
+            const int er = rok ? P.ea[row] : 0;
             bool small = false;
 #pragma unroll 1
             for (int h = 0; h < 64; h += 32) {
@@ -703,14 +707,17 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
               TMEM_LD_X16(taddr + h, v);
               TMEM_LD_X16(taddr + h + 16, (v + 16));
               tmem_wait_ld();
-              const int nc = rok && !zrow ? P.n - col0 - h : 0;
+              const int nc = rok ? P.n - col0 - h : 0;
               bool low = false;
 #pragma unroll
               for (int j = 0; j < 32; ++j) low |= j < nc && __uint_as_float(v[j]) < OZ_CERT_MIN;
               if (low) {
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
-                  if (j < nc && __uint_as_float(v[j]) < OZ_CERT_MIN) small |= P.fb[col0 + h + j] != OZ_ZERO_LINE;
+                  if (j < nc && __uint_as_float(v[j]) < OZ_CERT_MIN) {
+                    const int fc = P.fb[col0 + h + j];
+                    small |= er == OZ_ZERO_LINE ? fc == OZ_BAD_LINE : fc != OZ_ZERO_LINE || er == OZ_BAD_LINE;
+                  }
               }
             }
             tc_fence_before();
