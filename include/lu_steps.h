@@ -80,10 +80,21 @@ int lu_step_gemm(lu_ctx ctx, lu_prec prec, int m, int n, int k, void *dC, int ld
  * A m x k, B k x n, 1 <= k <= 256) with the products on the BF16 tensor cores
  * by error-free splitting, as lu_factor_ex's LU_FACTOR_OZAKI (same error
  * bound).  Workspace: the context's step scratch (grown as needed).  Returns
- * -5 for k outside 1..256, LU_ERANGE (at the next lu_ctx_status) for
+ * -4 for k outside 1..256, LU_ERANGE (at the next lu_ctx_status) for
  * non-finite operands. */
 int lu_step_gemm_ozaki(lu_ctx ctx, int m, int n, int k, double *dC, int ldc, const double *dA, int lda,
                        const double *dB, int ldb);
+
+/* The same update as plain LU_F64 factorizations run it from 640 remaining rows
+ * on, 64 <= k <= 256 (-4 otherwise): split products where a certificate proves
+ * that an element's error is at most the FP64 dot product's bound, k 2^-53
+ * sum_k |a b| + 2^-53 |result|, and FP64 multiply-adds in the blocks of 32 rows x
+ * 64 columns where it does not.  whole != 0: as after an update that raised the
+ * flag, every block by multiply-adds.  *listed receives the number of refused
+ * blocks, *raised whether this update raised the flag (more than nine in ten
+ * refused); either may be NULL.  Synchronizes. */
+int lu_step_gemm_cert(lu_ctx ctx, int m, int n, int k, double *dC, int ldc, const double *dA, int lda,
+                      const double *dB, int ldb, int whole, int *listed, int *raised);
 
 /* Failure-path probe: runs one of the library's bounded device waits on a
  * condition that nothing ever satisfies -- kind 0: a triangular solve's wait

@@ -62,8 +62,9 @@
 // sum_k |a b|, which badly scaled rows can leave far below.  The certified
 // form therefore takes one more product first, of the leading digits'
 // magnitudes (a ninth slice of each operand): G = sum_k |d_0 g_0| gives
-// sum_k |a b| >= G 2^(e_i + f_j - 14), so G >= (0.35 + 4 / 64) 2^14 makes the
-// bound at most k 2^-53 sum_k |a b|, the dot product's own (k >= 64).  A block of 32
+// sum_k |a b| >= G 2^(e_i + f_j - 14), so G >= (0.35 k + 4) / (k - 1) 2^14 makes the
+// bound, with the conversion's part, at most k 2^-53 sum_k |a b|, the dot product's
+// own; the line is that of k = 64, the least k, and more than any larger k needs.  A block of 32
 // rows x 64 columns with an element below that is left alone and listed, and
 // gemm_list_kernel updates the listed blocks in plain FP64.  So are the blocks of a
 // line with an infinity or a NaN, which therefore spreads as in a plain FP64 update
@@ -87,7 +88,7 @@ constexpr int OZ_S = 8;        // slices per operand
 constexpr int OZ_BITS = 7;     // bits per slice
 constexpr int OZ_KMAX = 256;   // exactness bound on k (k * 128^2 <= 2^22)
 constexpr int OZ_MAG = OZ_S;   // the ninth slice of a certified update: magnitudes of slice 0
-constexpr float OZ_CERT_MIN = 6759.0f;  // (0.35 + 4 / 64) 2^14, rounded up
+constexpr float OZ_CERT_MIN = 6866.0f;  // (0.35 * 64 + 4) / 63 * 2^14, rounded up
 constexpr int OZ_ZERO_LINE = -(1 << 20);  // exponent that marks an all-zero line
 constexpr int OZ_BAD_LINE = 1 << 20;      // ... and a line with an infinity or a NaN (its digits are all 0)
 constexpr int OZ_F = 40;       // fraction bits of the integer sum below the t = 0 term

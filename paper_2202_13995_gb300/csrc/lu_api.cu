@@ -1316,6 +1316,43 @@ extern "C" int lu_step_gemm_ozaki(lu_ctx c, int m, int n, int k, double* dC, int
   return LU_OK;
 }
 
+extern "C" int lu_step_gemm_cert(lu_ctx c, int m, int n, int k, double* dC, int ldc, const double* dA, int lda,
+                                 const double* dB, int ldb, int whole, int* listed, int* raised) {
+  if (!c) return -1;
+  if (m < 0) return -2;
+  if (n < 0) return -3;
+  if (k < kCertNb || k > 256) return -4;
+  if (listed) *listed = 0;
+  if (raised) *raised = 0;
+  if (m == 0 || n == 0) return LU_OK;
+  if (!dC) return -5;
+  if (ldc < n) return -6;
+  if (!dA) return -7;
+  if (lda < k) return -8;
+  if (!dB) return -9;
+  if (ldb < n) return -10;
+  const size_t wbytes = (ozaki_ws_bytes(m, n, k, c->dev.sm_count, true) + 255) / 256 * 256;
+  int rc = ensure_step_ws(c, wbytes + (2 + oz_cert_blocks(m, n)) * sizeof(int));
+  if (rc) return rc;
+  OzCert cert;
+  cert.off = (int*)((char*)c->step_ws + wbytes);
+  cert.cnt = cert.off + 1;
+  cert.list = cert.off + 2;
+  cert.tag = 2;
+  c->h_pinned[9] = whole ? 1 : 0;  // (an earlier update's tag)
+  c->h_pinned[10] = 0;
+  CU_TRY(cudaMemcpyAsync(cert.off, c->h_pinned + 9, 2 * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+  CU_TRY(ozaki_split(dA, lda, dB, ldb, m, n, k, c->step_ws, c->d_status, c->stream, &cert));
+  CU_TRY(ozaki_gemm(dC, ldc, c->step_ws, m, n, k, 0, n, c->d_status, c->dev, c->stream, 0, &cert));
+  CU_TRY(launch_gemm_list(dC, ldc, dA, lda, dB, ldb, m, n, k, cert, c->dev, c->stream));
+  c->launches += 4;
+  CU_TRY(cudaMemcpyAsync(c->h_pinned + 9, cert.off, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  CU_TRY(cudaStreamSynchronize(c->stream));
+  if (listed) *listed = c->h_pinned[10];
+  if (raised) *raised = c->h_pinned[9] == cert.tag;
+  return LU_OK;
+}
+
 // ------------------------------------------------------------------ context accessors (batched / server files)
 cudaStream_t gb_ctx_stream(lu_ctx c) { return c->stream; }
 int gb_ctx_sm_count(lu_ctx c) { return c->dev.sm_count; }

@@ -33,7 +33,7 @@ EXPORTED = [
     "lu_create_ex", "lu_peak_probe", "lu_default_nb", "lu_generate", "lu_profile_enable", "lu_profile_select", "lu_profile_read", "lu_launch_count", "lu_step_panel_static",
     "lu_batch_create", "lu_batch_run", "lu_batch_shape", "lu_batch_free", "lu_solve_batched",
     "lu_server_create", "lu_server_submit", "lu_server_poll", "lu_server_wait", "lu_server_stats",
-    "lu_server_destroy", "lu_fact_bytes", "lu_factor_ex", "lu_step_gemm_ozaki", "lu_step_wait_probe",
+    "lu_server_destroy", "lu_fact_bytes", "lu_factor_ex", "lu_step_gemm_ozaki", "lu_step_gemm_cert", "lu_step_wait_probe",
 ]
 PHASES = ["panel", "laswp", "trsm", "cast", "gemm", "solve", "residual", "other"]
 
@@ -101,6 +101,7 @@ def load():
             "lu_step_trsm": (I, [P, I, I, I, P, I, P, I]),
             "lu_step_gemm": (I, [P, I, I, I, I, P, I, P, I, P, I]),
             "lu_step_gemm_ozaki": (I, [P, I, I, I, P, I, P, I, P, I]),
+            "lu_step_gemm_cert": (I, [P, I, I, I, P, I, P, I, P, I, I, IP, IP]),
             "lu_step_wait_probe": (I, [P, I]),
             "lu_ctx_status": (I, [P]),
             "lu_device_sm_count": (I, [P]),
@@ -380,6 +381,19 @@ class Context:
         n = B.shape[1]
         _check(load().lu_step_gemm_ozaki(self._h, m, n, k, C.c_void_p(pc), ldc, C.c_void_p(pa), lda,
                                          C.c_void_p(pb), ldb), "lu_step_gemm_ozaki")
+
+    def step_gemm_cert(self, Cm, A, B, whole: bool = False):
+        """C -= A B in FP64 as the plain FP64 factorizations' large updates (row-major FP64,
+        64 <= k <= 256; whole: every block by multiply-adds).  Returns (refused blocks, flag raised)."""
+        pc, ldc = _rowmajor(Cm, "C")
+        pa, lda = _rowmajor(A, "A")
+        pb, ldb = _rowmajor(B, "B")
+        m, k = A.shape
+        n = B.shape[1]
+        listed, raised = C.c_int(-1), C.c_int(-1)
+        _check(load().lu_step_gemm_cert(self._h, m, n, k, C.c_void_p(pc), ldc, C.c_void_p(pa), lda, C.c_void_p(pb), ldb,
+                                        int(whole), C.byref(listed), C.byref(raised)), "lu_step_gemm_cert")
+        return listed.value, bool(raised.value)
 
 
 class Factor:

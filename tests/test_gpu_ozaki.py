@@ -4,13 +4,15 @@
 Bars:
   - operands that the slices represent exactly (7-bit integers times a power
     of two): the update equals C - A B bit for bit (every step is exact);
-  - any FP64 operands: |C_oz - C_ref| <= u ((1.13 k + 4) 2^(e_i + f_j)
+  - any FP64 operands: |C_oz - C_ref| <= u ((0.35 k + 4) 2^(e_i + f_j)
     + (|A||B|)_ij) + 2u |C_ref|, C_ref the compensated (Dot2) update of the
     oracle, u = 2^-53 and 2^e_i, 2^f_j the powers of two just above the
-    largest |A(i, :)| and |B(:, j)|: dropped slice pairs (p + q >= 8) < 0.87 k,
-    splitting remainders < 0.25 k, the 15 rounded right shifts <= 3.75 (in
+    largest |A(i, :)| and |B(:, j)|: dropped slice pairs (p + q >= 8) < 0.222 k,
+    splitting remainders < 0.126 k, the 15 rounded right shifts <= 3.82 (in
     units of u 2^(e_i + f_j)), then the conversion of the integer sum and the
     subtraction round once each;
+  - the certified form: within the FP64 dot product's k u (|A||B|)_ij + u |C|
+    everywhere, refusing exactly the blocks that its rule refuses;
   - the factorization with this update: the FP64 bars (pivots equal to the
     oracle's, factors and x within the roundoff bounds, scaled residual < 16).
 """
@@ -60,7 +62,7 @@ def _expo(x, axis):
 def _bound(Am, Bm, ref):
     k = Am.shape[1]
     sc = np.ldexp(1.0, (_expo(Am, 1)[:, None] + _expo(Bm, 0)[None, :]).astype(np.int64))
-    return EPS * ((1.13 * k + 4) * sc + np.abs(Am) @ np.abs(Bm)) + 2 * EPS * np.abs(ref)
+    return EPS * ((0.35 * k + 4) * sc + np.abs(Am) @ np.abs(Bm)) + 2 * EPS * np.abs(ref)
 
 
 def _run(ctx, Cm, Am, Bm):
@@ -131,7 +133,7 @@ def test_products_at_the_end_of_the_exponent_range(ctx, ea, eb):
         ref = (Cm.astype(LD) - Am.astype(LD) @ Bm.astype(LD))
         err = np.abs(_run(ctx, Cm, Am, Bm).astype(LD) - ref)
         sc = np.ldexp(LD(1.0), (_expo(Am, 1)[:, None] + _expo(Bm, 0)[None, :]).astype(np.int64))
-        bound = LD(EPS) * ((1.13 * k + 4) * sc + np.abs(Am).astype(LD) @ np.abs(Bm).astype(LD) + 2 * np.abs(ref)) + \
+        bound = LD(EPS) * ((0.35 * k + 4) * sc + np.abs(Am).astype(LD) @ np.abs(Bm).astype(LD) + 2 * np.abs(ref)) + \
             2 * np.ldexp(LD(1.0), -1074)
         assert (err <= bound).all()
 
@@ -146,10 +148,91 @@ def test_non_finite_operand_is_reported(ctx):
     assert ctx.status() == lu.LU_ERANGE
 
 
+def _lead(x, axis):
+    """The magnitudes' leading base-128 digits of the lines along axis (of |x| 2^-e rounded to 56 bits)."""
+    e = np.expand_dims(_expo(x, axis), axis)
+    return np.floor(np.rint(np.ldexp(np.abs(x), 56 - e)) / 2.0 ** 49)
+
+
+CERT_LINE = 6866  # (0.35 * 64 + 4) / 63 * 2^14
+
+
+def _refused(Am, Bm):
+    """Blocks of 32 x 64 with an element whose magnitude product is below the line (zero lines pass)."""
+    m, n = Am.shape[0], Bm.shape[1]
+    small = _lead(Am, 1) @ _lead(Bm, 0) < CERT_LINE
+    small &= np.abs(Am).max(1)[:, None] > 0
+    small &= np.abs(Bm).max(0)[None, :] > 0
+    pad = np.zeros(((m + 31) // 32 * 32, (n + 63) // 64 * 64), dtype=bool)
+    pad[:m, :n] = small
+    return pad.reshape(pad.shape[0] // 32, 32, -1, 64).any(axis=(1, 3))
+
+
+def _peaked(rng, m, k, s):
+    """Rows of entries of size s with one of size 1: sum |a b| is far below the lines' maxima."""
+    X = (rng.random((m, k)) - 0.5) * 2 * s
+    X[np.arange(m), rng.integers(0, k, m)] = rng.choice([-1.0, 1.0], m) * (0.5 + 0.5 * rng.random(m))
+    return X * 2.0 ** rng.integers(-30, 30, (m, 1))
+
+
+# sizes of the smaller entries from "every block refused" to "none"; ragged blocks, k of 1 to 4 chunks
+@pytest.mark.parametrize("m,n,k", [(333, 517, 64), (129, 65, 64), (32, 700, 100), (640, 640, 128), (300, 260, 256)])
+def test_certificate_on_either_side_of_its_line(ctx, m, n, k):
+    rng = np.random.default_rng(m + n + k)
+    shares = []
+    for s in np.array([0.02, 0.12, 0.13, 0.137, 0.14, 0.143, 0.146, 0.15, 0.16, 0.5]) * (64.0 / k) ** 0.5 * 1.3:
+        Am, Bm = _peaked(rng, m, k, s), _peaked(rng, n, k, s).T.copy()
+        Am[m // 3] = 0.0
+        Bm[:, n // 2] = 0.0
+        Cm = (rng.random((m, n)) - 0.5) * np.abs(Am).max(1)[:, None] * np.abs(Bm).max(0)[None, :]
+        Cm[m // 3], Cm[:, n // 2] = 1.5, 2.5
+        want = _refused(Am, Bm)
+        ref = O.gemm_update_dot2(Cm, Am, Bm)
+        bound = k * EPS * (np.abs(Am) @ np.abs(Bm)) * (1 + 1e-9) + 2 * EPS * np.abs(ref)
+        c, d, w = _rm(Cm), _rm(Cm), _rm(Cm)
+        listed, raised = ctx.step_gemm_cert(c, _rm(Am), _rm(Bm))
+        assert listed == want.sum() and raised == (want.sum() * 10 > want.size * 9)
+        got = c.cpu().numpy()
+        assert (np.abs(got - ref) <= bound).all(), float((np.abs(got - ref) / np.maximum(bound, 1e-300)).max())
+        assert np.array_equal(got[m // 3], Cm[m // 3]) and np.array_equal(got[:, n // 2], Cm[:, n // 2])
+        # refused blocks are the multiply-add update's, bit for bit, and with the flag every block is
+        ctx.step_gemm(d, _rm(Am), _rm(Bm), "f64")
+        plain = d.cpu().numpy()
+        mask = np.kron(want, np.ones((32, 64), dtype=bool))[:m, :n]
+        assert np.array_equal(got[mask], plain[mask])
+        listed, raised = ctx.step_gemm_cert(w, _rm(Am), _rm(Bm), whole=True)
+        assert (listed, raised) == (0, False) and np.array_equal(w.cpu().numpy(), plain)
+        shares.append(want.mean())
+    assert shares[0] == 1.0 and shares[-1] == 0.0 and any(0 < x < 1 for x in shares), shares
+    assert ctx.status() == 0
+
+
+def test_certificate_and_non_finite_lines(ctx):
+    """A line with an infinity or a NaN has its blocks refused, across a zero line too."""
+    rng = np.random.default_rng(2)
+    m, n, k = 100, 200, 64
+    for bad in (np.nan, np.inf):
+        Am, Bm, Cm = rng.random((m, k)) - 0.5, rng.random((k, n)) - 0.5, rng.random((m, n)) - 0.5
+        Am[40, 3] = Bm[5, 150] = bad
+        Am[90] = 0.0
+        Bm[:, 20] = 0.0
+        c, d = _rm(Cm), _rm(Cm)
+        listed, raised = ctx.step_gemm_cert(c, _rm(Am), _rm(Bm))
+        ctx.step_gemm(d, _rm(Am), _rm(Bm), "f64")
+        # block row 1 (row 40: 4 blocks) and block column 2 (column 150: 4 blocks), one shared
+        assert (listed, raised) == (7, False)
+        assert np.array_equal(np.isfinite(c.cpu().numpy()), np.isfinite(d.cpu().numpy()))
+        assert ctx.status() == 0
+
+
 def test_k_out_of_range_is_rejected(ctx):
     from paper_2202_13995_gb300 import lu
     with pytest.raises(lu.LuError):
         ctx.step_gemm_ozaki(_rm(np.zeros((4, 4))), _rm(np.zeros((4, 257))), _rm(np.zeros((257, 4))))
+    for k in (63, 257):
+        with pytest.raises(lu.LuError) as e:
+            ctx.step_gemm_cert(_rm(np.zeros((4, 4))), _rm(np.zeros((4, k))), _rm(np.zeros((k, 4))))
+        assert e.value.code == -4
 
 
 @pytest.mark.parametrize("n,nb", [(1, 64), (65, 64), (500, 64), (777, 100), (1500, 256), (2048, 128)])
