@@ -100,10 +100,11 @@ int lu_step_gemm_cert(lu_ctx ctx, int m, int n, int k, double *dC, int ldc, cons
  * condition that nothing ever satisfies -- kind 0: a triangular solve's wait
  * for a solution block that is never published; 1: a panel's grid barrier
  * that the other CTA never reaches; 2: a tensor-core kernel's mbarrier wait
- * for a copy that never lands.  The wait gives up after the library's
+ * for a copy that never lands; 3: a cluster panel's wait for a record that no
+ * CTA sends; 4: a grid panel's wait for a stamped word that no CTA writes.  The wait gives up after the library's
  * compiled-in limit (2 s), the kernel sets the timeout bit and returns, and
  * the call returns LU_ETIMEOUT with the status cleared; the context stays
- * usable.  Synchronizes.  Returns -1 (ctx NULL), -2 (kind not 0..2). */
+ * usable.  Synchronizes.  Returns -1 (ctx NULL), -2 (kind not 0..4). */
 int lu_step_wait_probe(lu_ctx ctx, int kind);
 
 /* The seeded synthetic input of the benchmarks, generated on the device

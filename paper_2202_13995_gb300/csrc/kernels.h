@@ -254,7 +254,8 @@ cudaError_t launch_add_update(double* X, int64_t ldx, const double* D, int64_t l
                               const int* active, cudaStream_t st);
 
 // Bounded-wait probe (waitprobe.cu): kind 0 flag wait, 1 grid barrier, 2
-// mbarrier wait, each on a condition nothing satisfies; 8 bytes of scratch.
+// mbarrier wait, 3 a cluster panel's record, 4 a grid panel's stamped word, each
+// on a condition nothing satisfies; 32 bytes of scratch.
 cudaError_t launch_wait_probe(int kind, void* scratch, int* status, cudaStream_t st);
 
 }  // namespace gb

@@ -46,6 +46,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "panel_wait.cuh"
 #include "tc_ptx.cuh"
 
 namespace gb {
@@ -132,17 +133,6 @@ __device__ __forceinline__ void pc_send16(uint32_t dst, longlong2 v, uint32_t ba
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(dst),
                "l"(v.x), "l"(v.y), "r"(bar)
                : "memory");
-}
-__device__ __forceinline__ bool pc_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
 }
 
 // A CTA's rows (at A, row stride ld) to shared memory, four of a warp's rows in
@@ -353,17 +343,7 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
     PcKey best{0u, 0u, INT_MAX};
     if (chain) {
       const uint32_t bar = bar0 + 8u * (uint32_t)buf;
-      if (!pc_try(bar, par)) {
-        const uint64_t t0 = gtimer();
-        while (!pc_try(bar, par)) {
-          if (*(volatile int*)&abort_flag) break;
-          if (gtimer() - t0 > GB_SPIN_LIMIT_NS) {
-            atomicOr(P.status, ST_TIMEOUT);
-            *(volatile int*)&abort_flag = 1;  // seen by every thread after the CTA's next barrier
-            break;
-          }
-        }
-      }
+      pc_wait(bar, par, &abort_flag, P.status);
       __syncwarp();
       if (j + 1 < w) arm(j + 1, nbuf);
       // the pivot: the best of the CTAs' candidates
@@ -381,6 +361,7 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
       const T rinv = reinterpret_cast<const T*>(rec)[2];
       const T piv = pr[j];
       const T u1 = j + 1 < w ? pr[j + 1] : T(0);
+      if (!GB_IN_BOUNDS(P.status, k.hi == 0u || (k.pos >= j && k.pos < P.m))) k.pos = j;
       if (tid == 0) {
         sel[0] = k.pos;
         sel[1] = win;
@@ -423,13 +404,15 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_cluster_kernel(PcParams<T> 
   if (!abort_flag) {
     // each row to its position; the rows that moved to the permutation record
     int* sp = reinterpret_cast<int*>(recs);  // [R] (the records are all read)
-    if (chain && live) sp[r] = pos;
+    if (chain && live) sp[r] = GB_IN_BOUNDS(P.status, pos >= 0 && pos < P.m) ? pos : row0 + r;
     __syncthreads();
     pc_store_rows(P.A, ld, S, Rs, sp, rloc, w);
     if (chain && live && pos != row0 + r) {
       const int q = atomicAdd(P.perm, 1);
-      P.perm[1 + q] = pos;
-      P.perm[1 + 2 * w + q] = row0 + r;
+      if (GB_IN_BOUNDS(P.status, q < 2 * w)) {
+        P.perm[1 + q] = pos;
+        P.perm[1 + 2 * w + q] = row0 + r;
+      }
     }
   } else {
     // records may still be on their way to a CTA whose wait ran out
@@ -565,63 +548,6 @@ cudaError_t launch_panel_cluster(T* Wkk, int64_t ldw, int m, int w, int kabs, in
 // whose poll runs out raises ST_TIMEOUT and leaves, and so do the others in their
 // turn.
 
-// A value between its stamps: a double as two 8-byte words {low half, stamp},
-// {high half, stamp}, a float as one; relaxed loads and stores (each 8-byte word
-// is read and written whole).
-__device__ __forceinline__ ulonglong2 pr_load(const ulonglong2* p) {
-  ulonglong2 v;
-  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void pr_store(ulonglong2* p, ulonglong2 v) {
-  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(v.x), "l"(v.y) : "memory");
-}
-template <typename T>
-struct PrWord;
-template <>
-struct PrWord<double> {
-  using type = ulonglong2;
-  static __device__ __forceinline__ void put(type* p, double v, unsigned stamp) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    pr_store(p, make_ulonglong2((b << 32) | stamp, (b & 0xffffffff00000000ull) | stamp));
-  }
-  static __device__ __forceinline__ bool get(const type* p, double& v, unsigned stamp) {
-    const ulonglong2 x = pr_load(p);
-    v = __longlong_as_double((long long)((x.y & 0xffffffff00000000ull) | (x.x >> 32)));
-    return (unsigned)x.x == stamp && (unsigned)x.y == stamp;
-  }
-};
-template <>
-struct PrWord<float> {
-  using type = unsigned long long;
-  static __device__ __forceinline__ void put(type* p, float v, unsigned stamp) {
-    const unsigned long long x = ((unsigned long long)__float_as_uint(v) << 32) | stamp;
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(x) : "memory");
-  }
-  static __device__ __forceinline__ bool get(const type* p, float& v, unsigned stamp) {
-    unsigned long long x;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(p) : "memory");
-    v = __uint_as_float((unsigned)(x >> 32));
-    return (unsigned)x == stamp;
-  }
-};
-
-// wait for a stamped value; *abort_flag is set when the wait runs out
-template <typename T>
-__device__ __forceinline__ void pr_fetch(const typename PrWord<T>::type* q, T& v, unsigned stamp, int* abort_flag,
-                                         int* status) {
-  if (PrWord<T>::get(q, v, stamp)) return;
-  const uint64_t t0 = gtimer();
-  while (!PrWord<T>::get(q, v, stamp)) {
-    if (*(volatile int*)abort_flag) return;
-    if (gtimer() - t0 > GB_SPIN_LIMIT_NS) {
-      atomicOr(status, ST_TIMEOUT);
-      *(volatile int*)abort_flag = 1;
-      return;
-    }
-  }
-}
-
 template <typename T>
 struct PrParams {
   T* A;  // W(k, k)
@@ -649,7 +575,7 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_grid_f64_kernel(PrParams<do
   using T = double;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint4 red[PC_NTMAX / 32];   // each row group's best: key, position, row
-  __shared__ int sel[2];  // the current column's pivot: position, CTA
+  __shared__ int sel;  // the current column's pivot: position
   __shared__ int abort_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
   const int cta = blockIdx.x, G = gridDim.x;
@@ -701,7 +627,7 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_grid_f64_kernel(PrParams<do
     }
     __syncthreads();
     if (abort_flag) return false;
-    if (c > 0 && !chain) move(c - 1, sel[0]);
+    if (c > 0 && !chain) move(c - 1, sel);
     uint4 e = red[lane < RG ? lane : 0];
     if (RG > 1) {
       PcKey k{lane < RG ? e.x : 0u, lane < RG ? e.y : 0u, lane < RG ? (int)e.z : INT_MAX};
@@ -817,9 +743,9 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_grid_f64_kernel(PrParams<do
         fetch(grow + w, rinv, stamp);
         if (j + 1 < w) fetch(grow + j + 1, u1, stamp);
       }
+      if (!GB_IN_BOUNDS(P.status, k.hi == 0u || (k.pos >= j && k.pos < P.m))) k.pos = j;
       if (tid == 0) {
-        sel[0] = k.pos;
-        sel[1] = win;
+        sel = k.pos;
         if (cta == 0) {
           P.ipiv[P.kabs + j] = P.kabs + k.pos + 1;
           if (!nonzero(piv)) atomicMin(P.info, P.kabs + j + 1);
@@ -866,13 +792,15 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_grid_f64_kernel(PrParams<do
   __threadfence();  // (after every CTA's first header: their row loads and the count's zero)
   __syncthreads();
   if (!ok || abort_flag) return;
-  if (chain && live) sp[r] = pos;
+  if (chain && live) sp[r] = GB_IN_BOUNDS(P.status, pos >= 0 && pos < P.m) ? pos : row0 + r;
   __syncthreads();
   pc_store_rows(P.A, ld, S, Rs, sp, rloc, w);
   if (chain && live && pos != row0 + r) {
     const int q = atomicAdd(P.perm, 1);
-    P.perm[1 + q] = pos;
-    P.perm[1 + 2 * w + q] = row0 + r;
+    if (GB_IN_BOUNDS(P.status, q < 2 * w)) {
+      P.perm[1 + q] = pos;
+      P.perm[1 + 2 * w + q] = row0 + r;
+    }
   }
 }
 
@@ -1001,7 +929,8 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_grid_f32_kernel(PrParams<fl
     const bool own = pc_warp_best<T>(k);
     const unsigned at = __ballot_sync(0xffffffffu, own);
     const int win = min((int)__shfl_sync(0xffffffffu, e.w, at ? __ffs(at) - 1 : 0), G - 1);
-    const int p = k.pos;
+    int p = k.pos;
+    if (!GB_IN_BOUNDS(P.status, k.hi == 0u || (p >= j && p < P.m))) p = j;
     const auto* grow = P.rows + (size_t)(buf * G + win) * P.rstride;
     T* pr = prow + (size_t)buf * (w + 1);
     const unsigned stamp = (unsigned)j + 1u;
@@ -1077,13 +1006,15 @@ __global__ void __launch_bounds__(PC_NTMAX, 1) panel_grid_f32_kernel(PrParams<fl
   __threadfence();  // (after every CTA's first header: their row loads and the count's zero)
   __syncthreads();
   if (!ok || abort_flag) return;
-  if (chain && live) sp[r] = pos;
+  if (chain && live) sp[r] = GB_IN_BOUNDS(P.status, pos >= 0 && pos < P.m) ? pos : row0 + r;
   __syncthreads();
   pc_store_rows(P.A, ld, S, Rs, sp, rloc, w);
   if (chain && live && pos != row0 + r) {
     const int q = atomicAdd(P.perm, 1);
-    P.perm[1 + q] = pos;
-    P.perm[1 + 2 * w + q] = row0 + r;
+    if (GB_IN_BOUNDS(P.status, q < 2 * w)) {
+      P.perm[1 + q] = pos;
+      P.perm[1 + 2 * w + q] = row0 + r;
+    }
   }
 }
 

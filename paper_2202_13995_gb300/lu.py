@@ -366,7 +366,7 @@ class Context:
 
     def wait_probe(self, kind: int) -> int:
         """Run one bounded device wait on a condition nothing satisfies (0 flag,
-        1 grid barrier, 2 mbarrier); returns the library's code (LU_ETIMEOUT)."""
+        1 grid barrier, 2 mbarrier, 3 cluster record, 4 stamped word); returns the library's code (LU_ETIMEOUT)."""
         rc = load().lu_step_wait_probe(self._h, int(kind))
         if rc < 0:
             _check(rc, "lu_step_wait_probe")

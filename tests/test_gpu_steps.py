@@ -225,11 +225,11 @@ def test_gemm_fp16_overflow_is_reported(ctx):
     assert ctx.status() == 0  # cleared by the read
 
 
-@pytest.mark.parametrize("kind", [0, 1, 2])
+@pytest.mark.parametrize("kind", [0, 1, 2, 3, 4])
 def test_bounded_wait_times_out_and_context_survives(ctx, kind):
     """Failure detection without a fault: a solve's flag wait, a panel's grid
-    barrier and a tensor-core mbarrier wait, each on a condition nothing
-    satisfies, give up after the library's limit with LU_ETIMEOUT; the status
+    barrier, a tensor-core mbarrier wait, a cluster panel's record and a grid
+    panel's stamped word, each on a condition nothing satisfies, give up after the library's limit with LU_ETIMEOUT; the status
     is cleared and the same context then factors and solves correctly."""
     import time
     from paper_2202_13995_gb300 import lu
