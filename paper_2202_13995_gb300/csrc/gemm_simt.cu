@@ -141,17 +141,18 @@ __global__ void __launch_bounds__(256) gemm_small_f64_kernel(double* __restrict_
 
 template <typename T>
 cudaError_t launch_gemm_simt(T* C, int64_t ldc, const T* A, int64_t lda, const T* B, int64_t ldb, int m, int n,
-                             int k, cudaStream_t st) {
+                             int k, const DevInfo& dev, cudaStream_t st) {
   if (m <= 0 || n <= 0 || k <= 0) return cudaSuccess;
   dim3 grid((unsigned)cdiv(n, SG_BN), (unsigned)cdiv(m, SG_BM));
   if (grid.y > 65535u) return cudaErrorInvalidConfiguration;
   if constexpr (sizeof(T) == 8) {
-    // (fewer 64 x 64 tiles than twice the 152 SMs leave their FP64 pipes unevenly
+    // (fewer 64 x 64 tiles than twice the SMs, 304 on GB300, leave their FP64 pipes unevenly
     // loaded: k = 64, us with 64 x 64 tiles and with these: 384 rows 72 and 21, 640
     // 73 and 54, 900 138 and 103, 1100 (324 tiles) 203 and 203)
     const int64_t tiles = (int64_t)grid.x * grid.y;
-    if (tiles < 304) {
-      if (cdiv(m, 32) * cdiv(n, 32) >= 304)
+    const int64_t wave = 2 * dev.sm_count;
+    if (tiles < wave) {
+      if (cdiv(m, 32) * cdiv(n, 32) >= wave)
         gemm_small_f64_kernel<32><<<dim3((unsigned)cdiv(n, 32), (unsigned)cdiv(m, 32)), 256, 0, st>>>(C, ldc, A, lda, B,
                                                                                                   ldb, m, n, k);
       else
@@ -247,8 +248,8 @@ cudaError_t launch_gemm_list(double* C, int64_t ldc, const double* A, int64_t ld
 }
 
 template cudaError_t launch_gemm_simt<double>(double*, int64_t, const double*, int64_t, const double*, int64_t, int,
-                                              int, int, cudaStream_t);
+                                              int, int, const DevInfo&, cudaStream_t);
 template cudaError_t launch_gemm_simt<float>(float*, int64_t, const float*, int64_t, const float*, int64_t, int, int,
-                                             int, cudaStream_t);
+                                             int, const DevInfo&, cudaStream_t);
 
 }  // namespace gb

@@ -162,7 +162,7 @@ int block_column_launches(int m, int w, int tsize);
 // C (m x n) -= A (m x k) * B (k x n), all row-major in T, CUDA-core FMA.
 template <typename T>
 cudaError_t launch_gemm_simt(T* C, int64_t ldc, const T* A, int64_t lda, const T* B, int64_t ldb, int m, int n,
-                             int k, cudaStream_t st);
+                             int k, const DevInfo& dev, cudaStream_t st);
 
 // The listed 32 x 64 blocks of C -= A B in FP64 (every block when cert.off is set).
 struct OzCert;

@@ -543,7 +543,7 @@ static int update_f64(lu_fact f, double* A22, const double* L21, const double* U
   cudaStream_t st = c->stream;
   const int64_t ld = f->ldw;
   if (f->oz_cert == nullptr || w < kCertNb || rest < kCertRest) {
-    CU_TRY(PHASE(c, PH_GEMM, 1, launch_gemm_simt<double>(A22, ld, L21, ld, U12, ld, rest, rest, w, st)));
+    CU_TRY(PHASE(c, PH_GEMM, 1, launch_gemm_simt<double>(A22, ld, L21, ld, U12, ld, rest, rest, w, c->dev, st)));
     return LU_OK;
   }
   CU_TRY(update_cert(f, PH_GEMM, A22, L21, U12, rest, rest, w, step, 0));
@@ -640,7 +640,7 @@ static int factor_loop(lu_fact f) {
       continue;
     }
     if (!tc) {
-      CU_TRY(PHASE(c, PH_GEMM, 1, launch_gemm_simt<T>(A22, ld, L21, ld, U12, ld, rest, rest, w, st)));
+      CU_TRY(PHASE(c, PH_GEMM, 1, launch_gemm_simt<T>(A22, ld, L21, ld, U12, ld, rest, rest, w, c->dev, st)));
       continue;
     }
     CU_TRY(PHASE(c, PH_CAST, 1, launch_cast_a(kind, (const float*)L21, ld, rest, w, f->aop, f->kpad, c->d_status, st)));
@@ -762,7 +762,7 @@ static int factor_loop_nopiv(lu_fact f) {
       const int rc = update_f64(f, A22, L21, U12, rest, w, k / nb);
       if (rc) return rc;
     } else {
-      CU_TRY(PHASE(c, PH_GEMM, 1, launch_gemm_simt<T>(A22, ld, L21, ld, U12, ld, rest, rest, w, st)));
+      CU_TRY(PHASE(c, PH_GEMM, 1, launch_gemm_simt<T>(A22, ld, L21, ld, U12, ld, rest, rest, w, c->dev, st)));
     }
   }
   if (panel_ready) CU_TRY(cudaStreamWaitEvent(st, c->ev_panel, 0));
@@ -1261,11 +1261,12 @@ extern "C" int lu_step_gemm(lu_ctx c, lu_prec prec, int m, int n, int k, void* d
   if (m == 0 || n == 0 || k == 0) return LU_OK;
   if (prec == LU_F64) {
     CU_TRY(launch_gemm_simt<double>((double*)dC, ldc, (const double*)dA, lda, (const double*)dB, ldb, m, n, k,
-                                    c->stream));
+                                    c->dev, c->stream));
     return LU_OK;
   }
   if (prec == LU_F32) {
-    CU_TRY(launch_gemm_simt<float>((float*)dC, ldc, (const float*)dA, lda, (const float*)dB, ldb, m, n, k, c->stream));
+    CU_TRY(launch_gemm_simt<float>((float*)dC, ldc, (const float*)dA, lda, (const float*)dB, ldb, m, n, k, c->dev,
+                                   c->stream));
     return LU_OK;
   }
   // tensor-core path: the cast kernel reads A (m x k) and B (k x n) with one

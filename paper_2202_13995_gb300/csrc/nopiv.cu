@@ -769,11 +769,19 @@ static SpecDev<T> spec_dev(const SpecArgs& a, int64_t backup_offset) {
   return d;
 }
 
-static int device_smem_optin() {
-  int dev = 0, optin = 0;
+// The rows-below launches' view of the device: shared memory per CTA, and the CTAs
+// of one wave (two per SM: 304 on GB300).
+struct BelowDev {
+  int optin, wave;
+};
+static BelowDev below_dev() {
+  int dev = 0, sms = 0;
+  BelowDev d{0, 0};
   cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  return optin;
+  cudaDeviceGetAttribute(&d.optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  d.wave = 2 * sms;
+  return d;
 }
 
 // Slab height: the largest multiple of 32, at most 128, whose slab fits in
@@ -793,7 +801,8 @@ static size_t ls_smem(int rb, int wt, int tsize) {
 // the stream is the chain's own, whose kernels let the next one start while they
 // still write their results (the next one waits for them at its start): it hides
 // the launch, not the work (mixed n = 1500 1.39 -> 1.36 ms, no-pivot n = 6000 6.68
-// -> 6.61).  Only up to 16 * 304 rows, where the rows below are one wave: the
+// -> 6.61).  Only where the rows below the first slab are one wave in CTAs of 16
+// rows (4864 rows on GB300), and then for the whole chain: the
 // waiting CTAs of a larger launch keep the trailing update beside the panel off
 // their SMs (mixed n = 32768 114.3 -> 116.5 ms).
 template <typename... P, typename... A>
@@ -814,32 +823,33 @@ static cudaError_t launch_chain(void (*kern)(P...), unsigned grid, unsigned thre
 
 template <typename T, int RB>
 static cudaError_t launch_ls(const T* U, const T* uinv, T* X, int64_t ld, int m, int ws, int wt,
-                             const SpecDev<T>& sp, int first, int tag, cudaStream_t st) {
+                             const SpecDev<T>& sp, int first, int tag, bool dependent, cudaStream_t st) {
   auto kern = below_solve_kernel<T, RB>;
   cudaError_t e = allow_max_smem((const void*)kern);
   if (e != cudaSuccess) return e;
-  return launch_chain(kern, (unsigned)cdiv(m, RB), LS_THREADS, ls_smem(RB, wt, sizeof(T)), st, m <= 16 * 304,
+  return launch_chain(kern, (unsigned)cdiv(m, RB), LS_THREADS, ls_smem(RB, wt, sizeof(T)), st, dependent,
                       U, uinv, X, ld, m, ws, wt, sp, first, tag);
 }
 
 template <typename T>
 static cudaError_t launch_below(const T* U, const T* uinv, T* X, int64_t ld, int m, int ws, int wt,
-                                const SpecDev<T>& sp, int first, int tag, cudaStream_t st) {
-  const int optin = device_smem_optin();
+                                const SpecDev<T>& sp, int first, int tag, const BelowDev& dv, bool dependent,
+                                cudaStream_t st) {
+  const int optin = dv.optin;
   // Fewer rows per CTA while two CTAs per SM still take all rows at once: the
   // launch is then as short as one CTA's chain of blocks, whose length grows
   // with its rows (slab of 128 x 256, 1400 rows below: 64 rows per CTA 37 us, 16
   // rows 21; slab of 128 x 128: 22 and 14; 5400 rows, 256 wide: 37 and 33 with
   // 32); a longer launch takes 64, which read U least often.
-  const bool short_launch = cdiv(m, 32) <= 304;
-  if (cdiv(m, 16) <= 304 && ls_smem(16, wt, sizeof(T)) <= (size_t)optin)
-    return launch_ls<T, 16>(U, uinv, X, ld, m, ws, wt, sp, first, tag, st);
+  const bool short_launch = cdiv(m, 32) <= dv.wave;
+  if (cdiv(m, 16) <= dv.wave && ls_smem(16, wt, sizeof(T)) <= (size_t)optin)
+    return launch_ls<T, 16>(U, uinv, X, ld, m, ws, wt, sp, first, tag, dependent, st);
   if (!short_launch && ls_smem(64, wt, sizeof(T)) <= (size_t)optin)
-    return launch_ls<T, 64>(U, uinv, X, ld, m, ws, wt, sp, first, tag, st);
+    return launch_ls<T, 64>(U, uinv, X, ld, m, ws, wt, sp, first, tag, dependent, st);
   if (ls_smem(32, wt, sizeof(T)) <= (size_t)optin)
-    return launch_ls<T, 32>(U, uinv, X, ld, m, ws, wt, sp, first, tag, st);
+    return launch_ls<T, 32>(U, uinv, X, ld, m, ws, wt, sp, first, tag, dependent, st);
   if (ls_smem(16, wt, sizeof(T)) <= (size_t)optin)
-    return launch_ls<T, 16>(U, uinv, X, ld, m, ws, wt, sp, first, tag, st);
+    return launch_ls<T, 16>(U, uinv, X, ld, m, ws, wt, sp, first, tag, dependent, st);
   return cudaErrorInvalidValue;
 }
 
@@ -860,6 +870,8 @@ cudaError_t launch_block_column(T* P, int64_t ld, int m, int w, int kabs, int* i
   if (w <= 0) return cudaSuccess;
   if (m < w) return cudaErrorInvalidValue;
   const int h = slab_rows(w, sizeof(T));
+  const BelowDev dv = below_dev();
+  const bool dependent = cdiv(m - (w < h ? w : h), 16) <= dv.wave;
   cudaError_t e = cudaSuccess;
   const int tag = kabs + 1;
   for (int s0 = 0; s0 < w; s0 += h) {
@@ -873,12 +885,12 @@ cudaError_t launch_block_column(T* P, int64_t ld, int m, int w, int kabs, int* i
     const int below = m - s0 - hs;
     T* ui = uinv + (size_t)(s0 / 32) * 1024;  // the slab's diagonal blocks' inverses (for the rows below)
     if ((e = launch_slab<T>(D, ld, hs, wt, kabs + s0, info, spec_dev<T>(spec, 0), first, tag, restore,
-                            below > 0 ? ui : nullptr, st, !first && m <= 16 * 304)) != cudaSuccess)
+                            below > 0 ? ui : nullptr, st, !first && dependent)) != cudaSuccess)
       return e;
     if (below > 0) {
       // the first slab's rows below it follow its rows in the backup (row stride w)
       e = launch_below<T>(D, ui, D + (int64_t)hs * ld, ld, below, hs, wt, spec_dev<T>(spec, (int64_t)hs * w), first,
-                          tag, st);
+                          tag, dv, dependent, st);
       if (e != cudaSuccess) return e;
     }
   }
