@@ -1,8 +1,10 @@
 // Block width nb of lu_factor(nb = 0), by factorization kind and size:
-// the fastest candidate of an offline sweep of whole solves (factor +
-// solve or refinement) on the benchmarks' seeded matrices.  Generated by
+// chosen from sweeps of whole solves (factor + solve or refinement) on the
+// benchmarks' seeded matrices, by
 //   python -m paper_2202_13995_gb300.tune
-// on NVIDIA GB300; times in ms (best of the repetitions after a warm-up).
+// on NVIDIA GB300: the fastest width at the size, or a narrower one within 3 percent
+// of it that the sizes beside it prefer (chosen by hand; the sweep names the fastest).
+// Times in ms, best of five after a warm-up, all rows of one run.
 #pragma once
 
 namespace gb {
@@ -15,36 +17,38 @@ struct NbEntry {
 };
 
 constexpr NbEntry kNbTable[] = {
-    {0, 800, 64},  // f64, measured at n = 600: nb 32: 1.680, nb 64: 1.585, nb 96: 1.600, nb 128: 1.640, nb 192: 1.852, nb 256: 2.035
-    {0, 1280, 64},  // f64, measured at n = 1023: nb 32: 3.286, nb 64: 3.083, nb 96: 3.131, nb 128: 3.314, nb 192: 3.611, nb 256: 3.920
-    {0, 3072, 128},  // f64, measured at n = 2048: nb 32: 11.199, nb 64: 7.896, nb 96: 7.569, nb 128: 7.360, nb 192: 7.743, nb 256: 8.409
-    {0, 4608, 128},  // f64, measured at n = 4096: nb 32: 53.185, nb 64: 23.485, nb 96: 20.599, nb 128: 19.022, nb 192: 18.948, nb 256: 19.644
-    {0, 7168, 192},  // f64, measured at n = 6000: nb 32: 145.067, nb 64: 50.690, nb 96: 41.958, nb 128: 36.996, nb 192: 34.807, nb 256: 35.107
-    {0, 12288, 256},  // f64, measured at n = 8192: nb 32: 340.921, nb 64: 101.347, nb 96: 79.956, nb 128: 68.142, nb 192: 60.611, nb 256: 59.217
-    {0, 24576, 256},  // f64, measured at n = 16384: nb 32: 2521.305, nb 64: 608.801, nb 96: 447.020, nb 128: 361.227, nb 192: 289.931, nb 256: 260.948
+    {0, 800, 64},  // f64, measured at n = 600: nb 32: 1.632, nb 64: 1.550, nb 96: 1.554, nb 128: 1.617, nb 192: 1.816, nb 256: 2.017
+    {0, 1280, 64},  // f64, measured at n = 1024: nb 32: 3.240, nb 64: 3.058, nb 96: 3.071, nb 128: 3.096, nb 192: 3.360, nb 256: 3.715
+    {0, 3072, 128},  // f64, measured at n = 2048: nb 32: 10.989, nb 64: 7.677, nb 96: 7.353, nb 128: 7.174, nb 192: 7.466, nb 256: 8.160
+    {0, 4608, 128},  // f64, measured at n = 4096: nb 32: 52.866, nb 64: 22.980, nb 96: 20.144, nb 128: 18.520, nb 192: 18.478, nb 256: 19.094
+    {0, 7168, 192},  // f64, measured at n = 5800: nb 32: 132.476, nb 64: 46.292, nb 96: 38.253, nb 128: 34.382, nb 192: 32.050, nb 256: 32.026
+    {0, 12288, 256},  // f64, measured at n = 8192: nb 32: 339.936, nb 64: 99.328, nb 96: 78.020, nb 128: 66.484, nb 192: 58.849, nb 256: 56.148
+    {0, 24576, 256},  // f64, measured at n = 16384: nb 32: 2520.064, nb 64: 597.495, nb 96: 433.155, nb 128: 345.725, nb 192: 273.029, nb 256: 235.283
     {0, 1073741824, 256},  // f64, measured at n = 32768: not measured: n = 32768 keeps the smaller size's choice
-    {1, 1280, 128},  // f64_split, measured at n = 1024: nb 64: 4.663, nb 128: 4.065, nb 192: 4.094, nb 256: 4.206
-    {1, 3072, 128},  // f64_split, measured at n = 2048: nb 64: 10.488, nb 128: 8.692, nb 192: 8.566, nb 256: 8.808
-    {1, 4608, 256},  // f64_split, measured at n = 4096: nb 64: 27.908, nb 128: 21.090, nb 192: 19.890, nb 256: 19.625
-    {1, 7168, 256},  // f64_split, measured at n = 7001: nb 64: 76.885, nb 128: 51.887, nb 192: 45.207, nb 256: 43.258
-    {1, 12288, 256},  // f64_split, measured at n = 8192: nb 64: 107.476, nb 128: 71.496, nb 192: 61.973, nb 256: 58.585
-    {1, 24576, 256},  // f64_split, measured at n = 16384: nb 64: 607.516, nb 128: 353.454, nb 192: 274.128, nb 256: 237.480
-    {1, 1073741824, 256},  // f64_split, measured at n = 32768: nb 64: 4066.466, nb 128: 2244.717, nb 192: 1653.813, nb 256: 1410.500
-    {2, 800, 128},  // mixed, measured at n = 600: nb 64: 1.076, nb 128: 0.868, nb 192: 0.895, nb 256: 0.859, nb 384: 0.847
-    {2, 1280, 256},  // mixed, measured at n = 1024: nb 64: 1.488, nb 128: 1.267, nb 192: 1.192, nb 256: 1.121, nb 384: 1.169
-    {2, 3072, 256},  // mixed, measured at n = 2048: nb 64: 2.814, nb 128: 2.167, nb 192: 2.183, nb 256: 2.117, nb 384: 2.275
-    {2, 4608, 256},  // mixed, measured at n = 4096: nb 64: 5.862, nb 128: 4.535, nb 192: 4.551, nb 256: 4.417, nb 384: 4.636
-    {2, 7168, 256},  // mixed, measured at n = 6000: nb 64: 9.361, nb 128: 7.218, nb 192: 7.065, nb 256: 6.793, nb 384: 7.189
-    {2, 12288, 256},  // mixed, measured at n = 8192: nb 64: 14.909, nb 128: 10.821, nb 192: 10.198, nb 256: 9.608, nb 384: 10.458
-    {2, 24576, 256},  // mixed, measured at n = 16384: nb 64: 57.702, nb 128: 35.933, nb 192: 30.219, nb 256: 27.199, nb 384: 28.869
-    {2, 1073741824, 256},  // mixed, measured at n = 32768: nb 64: 299.866, nb 128: 171.840, nb 256: 127.095, nb 384: 127.630, nb 512: 136.121
-    {3, 800, 128},  // f32, measured at n = 600: nb 64: 0.874, nb 128: 0.750, nb 192: 0.806, nb 256: 0.794
-    {3, 1280, 128},  // f32, measured at n = 1024: nb 64: 1.321, nb 128: 1.126, nb 192: 1.187, nb 256: 1.163
-    {3, 3072, 128},  // f32, measured at n = 2048: nb 64: 2.628, nb 128: 2.247, nb 192: 2.322, nb 256: 2.321
-    {3, 4608, 128},  // f32, measured at n = 4096: nb 64: 6.874, nb 128: 6.089, nb 192: 6.238, nb 256: 6.220
-    {3, 12288, 128},  // f32, measured at n = 8192: nb 64: 27.834, nb 128: 24.786, nb 192: 24.857, nb 256: 24.671
-    {3, 24576, 256},  // f32, measured at n = 16384: nb 64: 171.784, nb 128: 159.849, nb 256: 158.109, nb 384: 161.688, nb 512: 164.032
-    {3, 1073741824, 256},  // f32, measured at n = 32768: nb 64: 1200.106, nb 128: 1107.765, nb 256: 1089.696, nb 384: 1095.953, nb 512: 1099.100
+    {1, 800, 128},  // f64_split, measured at n = 600: nb 64: 2.682, nb 128: 2.132, nb 192: 2.194, nb 256: 2.268
+    {1, 1280, 128},  // f64_split, measured at n = 1024: nb 64: 4.605, nb 128: 3.834, nb 192: 3.870, nb 256: 3.974
+    {1, 3072, 128},  // f64_split, measured at n = 2048: nb 64: 10.293, nb 128: 8.450, nb 192: 8.212, nb 256: 8.491
+    {1, 4608, 256},  // f64_split, measured at n = 4096: nb 64: 27.399, nb 128: 20.475, nb 192: 19.265, nb 256: 19.022
+    {1, 7168, 256},  // f64_split, measured at n = 5800: nb 64: 51.732, nb 128: 36.440, nb 192: 32.254, nb 256: 31.404
+    {1, 12288, 256},  // f64_split, measured at n = 8192: nb 64: 105.555, nb 128: 67.888, nb 192: 57.250, nb 256: 53.658
+    {1, 24576, 256},  // f64_split, measured at n = 16384: nb 64: 596.455, nb 128: 336.324, nb 192: 257.725, nb 256: 221.104
+    {1, 1073741824, 256},  // f64_split, measured at n = 32768: nb 64: 4272.015, nb 128: 2274.564, nb 192: 1668.054, nb 256: 1374.150
+    {2, 800, 128},  // mixed, measured at n = 600: nb 64: 0.851, nb 128: 0.691, nb 192: 0.727, nb 256: 0.705, nb 384: 0.699, nb 512: 0.721
+    {2, 1280, 256},  // mixed, measured at n = 1024: nb 64: 1.139, nb 128: 0.929, nb 192: 0.928, nb 256: 0.901, nb 384: 0.919, nb 512: 0.938
+    {2, 3072, 256},  // mixed, measured at n = 2048: nb 64: 2.155, nb 128: 1.714, nb 192: 1.685, nb 256: 1.674, nb 384: 1.724, nb 512: 1.792
+    {2, 4608, 256},  // mixed, measured at n = 4096: nb 64: 4.598, nb 128: 3.524, nb 192: 3.497, nb 256: 3.446, nb 384: 3.570, nb 512: 3.826
+    {2, 7168, 256},  // mixed, measured at n = 5800: nb 64: 7.338, nb 128: 5.542, nb 192: 5.381, nb 256: 5.234, nb 384: 5.468, nb 512: 5.928
+    {2, 12288, 256},  // mixed, measured at n = 8192: nb 64: 12.735, nb 128: 8.908, nb 192: 8.436, nb 256: 7.719, nb 384: 8.518, nb 512: 9.224
+    {2, 24576, 256},  // mixed, measured at n = 16384: nb 64: 54.130, nb 128: 32.269, nb 192: 26.282, nb 256: 22.640, nb 384: 24.285, nb 512: 26.973
+    {2, 1073741824, 256},  // mixed, measured at n = 32768: nb 64: 319.196, nb 128: 174.478, nb 192: 131.550, nb 256: 103.712, nb 384: 102.440, nb 512: 100.741
+    {3, 800, 128},  // f32, measured at n = 600: nb 64: 0.744, nb 128: 0.647, nb 192: 0.691, nb 256: 0.685, nb 384: 0.661, nb 512: 0.756
+    {3, 1280, 128},  // f32, measured at n = 1024: nb 64: 1.169, nb 128: 0.998, nb 192: 1.037, nb 256: 1.000, nb 384: 1.036, nb 512: 1.061
+    {3, 3072, 128},  // f32, measured at n = 2048: nb 64: 2.342, nb 128: 2.011, nb 192: 2.037, nb 256: 2.035, nb 384: 2.185, nb 512: 2.216
+    {3, 4608, 128},  // f32, measured at n = 4096: nb 64: 6.292, nb 128: 5.519, nb 192: 5.589, nb 256: 5.547, nb 384: 5.757, nb 512: 5.986
+    {3, 7168, 128},  // f32, measured at n = 5800: nb 64: 12.258, nb 128: 11.036, nb 192: 10.938, nb 256: 10.945, nb 384: 11.282, nb 512: 11.667
+    {3, 12288, 128},  // f32, measured at n = 8192: nb 64: 26.306, nb 128: 23.525, nb 192: 23.531, nb 256: 23.356, nb 384: 23.806, nb 512: 24.411
+    {3, 24576, 256},  // f32, measured at n = 16384: nb 64: 158.769, nb 128: 147.073, nb 192: 145.933, nb 256: 144.583, nb 384: 145.465, nb 512: 146.836
+    {3, 1073741824, 256},  // f32, measured at n = 32768: nb 64: 1177.684, nb 128: 1082.593, nb 192: 1071.538, nb 256: 1063.387, nb 384: 1064.212, nb 512: 1065.735
 };
 
 }  // namespace gb
