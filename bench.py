@@ -192,6 +192,15 @@ def default_nb(n: int, prec: str, ozaki: bool = False) -> int:
     return lu.default_nb(n, prec, ozaki)
 
 
+# the rule by which plain FP64 factorizations take the certified split update
+# (update_f64 in csrc/lu_api.cu): block widths, least remaining rows
+CERT_NB, CERT_REST = (64, 256), 640
+UPDATES = {"split": "exact BF16 slice products (LU_FACTOR_OZAKI)",
+           "certified": "BF16 slice products with a certificate of the FP64 dot product's error bound, FP64 multiply-adds "
+                        "where it fails (plain LU_F64)",
+           "dfma": "FP64 multiply-adds on the CUDA cores (LU_FACTOR_DFMA, and small plain LU_F64)"}
+
+
 def gemm_roofline(prof: dict, n: int, nb: int, prec: str, steps: int, peaks: dict, wname: str,
                   ozaki: bool = False, cert: bool = False) -> dict:
     """Roofline of the dominant kernel, the trailing update, from its summed
@@ -203,15 +212,19 @@ def gemm_roofline(prof: dict, n: int, nb: int, prec: str, steps: int, peaks: dic
     tensor ridge); algorithmic bytes per launch = 8 m' n' (C read + write)
     + 2 (m' + n') kpad (the 16-bit operands).  FP64 by error-free splitting
     (tcgen05, BF16 slices): bound by the tensor pipe; algorithmic FLOPs per
-    launch = 36 slice pairs x 2 m' n' kpad.  cert: the certified form of the
-    plain FP64 factorizations, 37 products; its launches include the kernel
-    that updates the blocks the certificate refused (none on dense random
-    matrices)."""
-    ozaki = ozaki or cert
+    launch = 36 slice pairs x 2 m' n' kpad.  cert: the plain FP64
+    factorizations, whose updates of 640 rows and more (nb 64 to 256) take the
+    certified form, 37 products.  The time is that of the whole update phase,
+    which also holds the launches that update the blocks the certificate refused
+    (none on dense random matrices: a few us each) and the smaller updates on the
+    FP64 cores; their operations are not counted as products
+    (`cores_gflop_per_step` has them), so that `achieved` is a lower bound."""
     gemm_ms, gemm_n = prof["gemm"]
     nbx = nb or default_nb(n, prec, ozaki)
+    cert = cert and prec == "f64" and not ozaki and CERT_NB[0] <= nbx <= CERT_NB[1] and n - nbx >= CERT_REST
+    ozaki = ozaki or cert
     kpad = -(-nbx // 64) * 64
-    flops = bytes_ = 0.0
+    flops = bytes_ = split_flops = 0.0
     dram_alg = 0.0  # algorithmic DRAM bytes of the kernel's own data type, all launches of one step
     nlaunch = 0
     for k in range(0, n, nbx):
@@ -219,18 +232,22 @@ def gemm_roofline(prof: dict, n: int, nb: int, prec: str, steps: int, peaks: dic
         rest = n - k - w
         if rest > 0:
             flops += 2.0 * rest * rest * w
+            if cert and (rest < CERT_REST or w < CERT_NB[0]):
+                continue  # on the FP64 cores
+            split_flops += 2.0 * rest * rest * w
             bytes_ += 8.0 * rest * rest + 2.0 * (2 * rest) * kpad
-            if ozaki:  # FP64 C read + write, 8 BF16 slices of both operands
-                dram_alg += 16.0 * rest * rest + 16.0 * (2 * rest) * kpad
+            if ozaki:  # FP64 C read + write, 8 (certified: 9) BF16 slices of both operands
+                dram_alg += 16.0 * rest * rest + (18.0 if cert else 16.0) * (2 * rest) * kpad
             elif prec == "f64":  # FP64 C read + write, FP64 operands
                 dram_alg += 16.0 * rest * rest + 8.0 * (2 * rest) * w
             else:
                 dram_alg += 8.0 * rest * rest + 2.0 * (2 * rest) * kpad
             nlaunch += 1
     flops *= steps
+    split_flops *= steps
     bytes_ *= steps
     sec = gemm_ms * 1e-3
-    kernel = "oz_gemm_kernel" if ozaki else ("gemm_simt_kernel<double>" if prec == "f64" else "tc_gemm_kernel")
+    kernel = "oz_gemm_kernel (certified)" if cert else "oz_gemm_kernel" if ozaki else ("gemm_simt_kernel<double>" if prec == "f64" else "tc_gemm_kernel")
     # traffic per launch: the ratio of ncu DRAM bytes to algorithmic bytes of
     # launches captured on a small case of the same kernel (profiles/traffic.json,
     # one entry per kernel; counters beyond the launch time are collected only
@@ -249,9 +266,11 @@ def gemm_roofline(prof: dict, n: int, nb: int, prec: str, steps: int, peaks: dic
             "traffic_over_algorithmic": traffic_ratio,
             "tflops": flops / sec / 1e12 if sec > 0 else None}
     if ozaki:
-        tflops_bf16 = (37.0 if cert else 36.0) * flops / nbx * kpad / sec / 1e12 if sec > 0 else None
+        tflops_bf16 = (37.0 if cert else 36.0) * split_flops / nbx * kpad / sec / 1e12 if sec > 0 else None
         peak = peaks.get("bf16_tflops_sustained", 1701.1)
-        return dict(base, bound="tensor", kernel="oz_gemm_kernel", achieved=tflops_bf16, peak=peak,
+        if cert:
+            base["cores_gflop_per_step"] = (flops - split_flops) / steps / 1e9
+        return dict(base, bound="tensor", kernel=kernel, achieved=tflops_bf16, peak=peak,
                     unit="TFLOP/s", frac=(tflops_bf16 / peak) if tflops_bf16 else None,
                     peak_source=f"bf16_tflops_sustained of {peaks['_source']}",
                     fp64_equiv_tflops=base["tflops"])
@@ -371,8 +390,10 @@ def timed_solves(ctx, stream, cfg: dict, nb, steps: int, warmup: int, rank: int,
     ozaki = bool(cfg.get("ozaki", False))
     refine = mixed and not cfg.get("norefine", False)
 
+    dfma = bool(cfg.get("dfma", False))
+
     def step():
-        f = ctx.factor(A, prec, nb, sync=False, nopiv=nopiv, ozaki=ozaki)
+        f = ctx.factor(A, prec, nb, sync=False, nopiv=nopiv, ozaki=ozaki, dfma=dfma)
         if refine:
             iters.append(f.refine(A, B, X, 16.0, 50)[0])
         else:
@@ -582,6 +603,9 @@ def run_ours(args, cfg, wname):
     phases_ms, profiled_ms = r["phases_ms"], r["profiled_ms"]
     ozaki = bool(cfg.get("ozaki", False))
     roofline = gemm_roofline(prof, n, nb, prec, args.steps, peaks, wname, ozaki, prec == "f64" and not ozaki)
+    update = None
+    if not mixed:
+        update = "split" if ozaki else "certified" if "certified" in roofline["kernel"] else "dfma"
 
     # ---- end to end through the public API with host buffers
     e2e = None
@@ -687,6 +711,21 @@ def run_ours(args, cfg, wname):
         del orr
         torch.cuda.empty_cache()
 
+    dfma_line = None
+    if not mixed and not args.no_mixed and wname == DEFAULT:
+        # the same FP64 configuration with every update as FP64 multiply-adds (LU_FACTOR_DFMA)
+        dc = dict(cfg, dfma=True)
+        dsteps = min(args.steps, 2)
+        dr = timed_solves(ctx, stream, dc, nb, dsteps, 3, rank, ws)
+        dv = flops * ws / (dr["ms"] * 1e-3) / 1e12
+        dfma_line = {"workload": wname, "update": UPDATES["dfma"], "value": dv, "unit": "TFLOP/s", "steps": dsteps,
+                     "warmup": 3, "ms_per_step": dr["ms"], "scaled_residual": dr["res"],
+                     "roofline": gemm_roofline(dr["prof"], n, nb, prec, dsteps, peaks, wname),
+                     "phases_ms_per_step": dr["phases_ms"], "profiled_ms_per_step": dr["profiled_ms"]}
+        launches += dr["launches"]
+        del dr
+        torch.cuda.empty_cache()
+
     # arithmetic-rate probes of this GPU (the denominators of the CUDA-core
     # kernels: the FP32 batched factor; the FP64 update keeps the rate derived
     # from unit counts and clock, which it reaches, above the probe's)
@@ -728,8 +767,11 @@ def run_ours(args, cfg, wname):
             "metric": METRIC,
             "value": flops * ws / (ms * 1e-3) / 1e12, "unit": "TFLOP/s", "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": ("f64 (bf16-split products)" if ozaki else "f64") if not mixed else f"{prec}+f32acc+f64refine", "data": "synthetic",
+            "vs_baseline": None, "dtype": {"split": "f64 (bf16-split products)", "certified": "f64 (certified bf16-split update)",
+                                            "dfma": "f64"}[update] if not mixed else f"{prec}+f32acc+f64refine", "data": "synthetic",
             "config": {"workload": wname, "n": n, "nb": nb or "auto", "nrhs": nrhs, "precision": prec,
+                       "update": UPDATES.get(update, "16-bit operands, FP32 accumulation (tcgen05)" if prec != "f32"
+                                             else "FP32 multiply-adds"),
                        "matrix": "uniform[-0.5,0.5]" + (f" + {cfg['shift']}*n*I" if shift else ""),
                        "l2": (f"inputs larger than L2 (A = {n * n * 8 / 2 ** 30:.1f} GiB FP64)" if n * n * 8 > 129e6
                               else f"inputs smaller than L2 (A = {n * n * 8 / 2 ** 20:.0f} MiB FP64), not flushed"),
@@ -746,6 +788,7 @@ def run_ours(args, cfg, wname):
             "mixed": mixed_line,
             "paper_nopiv": nopiv_line,
             "f64_ozaki": ozaki_line,
+            "f64_dfma": dfma_line,
             "batched": batched_line,
             "served": served_line,
             "measured_rates": rates,

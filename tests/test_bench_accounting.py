@@ -65,6 +65,29 @@ def test_split_update_roofline_counts_36_products():
     assert r["bound"] == "tensor"
 
 
+def test_certified_update_roofline_counts_its_own_updates():
+    """37 products of the updates of 640 rows and more; the width of the plain table; none for a
+    factorization that the rule leaves to the FP64 cores."""
+    import json
+    from paper_2202_13995_gb300 import lu
+    n = 4096
+    peaks = {"bf16_tflops_sustained": 1701.1, "_source": "measured"}
+    nb = lu.default_nb(n, "f64")
+    assert nb != lu.default_nb(n, "f64", True)
+    kpad = -(-nb // 64) * 64
+    r = bench.gemm_roofline(_prof(20.0, 60), n, 0, "f64", 1, peaks, "x", cert=True)
+    rest = [n - k - nb for k in range(0, n, nb) if n - k - nb > 0]
+    split = [m for m in rest if m >= 640]
+    assert math.isclose(r["achieved"], 37.0 * sum(2.0 * m * m * kpad for m in split) / 0.020 / 1e12, rel_tol=1e-12)
+    assert math.isclose(r["cores_gflop_per_step"], sum(2.0 * m * m * nb for m in rest if m < 640) / 1e9, rel_tol=1e-9)
+    assert math.isclose(r["tflops"], sum(2.0 * m * m * nb for m in rest) / 0.020 / 1e12, rel_tol=1e-12)
+    ratio = json.load(open(os.path.join(ROOT, "profiles", "traffic.json")))["oz_gemm_kernel (certified)"]["ratio"]
+    alg = [16.0 * m * m + 18.0 * 2 * m * kpad for m in split]
+    assert math.isclose(r["traffic"], ratio * sum(alg) / len(alg), rel_tol=1e-12)
+    for small in ((600, 64), (4096, 32), (4096, 512)):
+        assert bench.gemm_roofline(_prof(20.0, 60), *small, "f64", 1, peaks, "x", cert=True)["bound"] == "alu"
+
+
 def test_traffic_scales_the_measured_ratio():
     """traffic per launch = measured DRAM bytes / algorithmic bytes of the
     captured launches x this step's mean algorithmic bytes per update."""
