@@ -128,7 +128,7 @@ int lu_factor(lu_ctx ctx, int n, const double *dA, int lda, lu_prec prec, int nb
  * operands fail with LU_ERANGE.
  * LU_FACTOR_DFMA (prec = LU_F64 only, not with LU_FACTOR_OZAKI): every update
  * as FP64 multiply-adds on the CUDA cores, never as split products (n = 8192
- * 340 ms instead of 55). */
+ * 320 ms instead of 54). */
 enum { LU_FACTOR_NOPIV = 1, LU_FACTOR_OZAKI = 2, LU_FACTOR_DFMA = 4 };
 int lu_factor_ex(lu_ctx ctx, int n, const double *dA, int lda, lu_prec prec, int nb, int flags, lu_fact *out,
                  int *info);

@@ -486,9 +486,10 @@ static int gemm_cap(lu_ctx c) { return c->gemm_ctas > 0 ? c->gemm_ctas : c->dev.
 // factorizations (ms with it at 384, 512, 640, 768, 900): n = 1023, nb = 64
 // 2.95 2.86 2.81 2.79 2.83; n = 1280, nb = 128 3.93 3.89 3.85 3.87 4.03;
 // n = 2048, nb = 128 6.83 6.79 6.77 6.79 6.95.  The error of whole solves against
-// systems with a known solution, certified over CUDA cores (LU_FACTOR_DFMA), 220
-// general matrices of n = 704 to 8192: 0.97 +- 0.06 (geometric mean); dominant ones
-// the same to three digits; residuals 0.87 to 1.00.
+// systems with a known solution, certified over CUDA cores (LU_FACTOR_DFMA,
+// geometric means): n = 1023 0.99 +- 0.06 (300 general matrices), 2500 1.00 +- 0.06
+// (200), 4096 0.98 +- 0.08 (150), 7000 0.96 +- 0.09 (100), 8192 0.84 +- 0.08 (100);
+// residuals 0.95 to 0.99; dominant matrices the same to three digits.
 constexpr int kCertNb = 64, kCertRest = 640;
 static bool cert_applies(int n, int nb) { return nb >= kCertNb && nb <= 256 && n - nb >= kCertRest; }
 static size_t cert_heads(int n, int nb) { return 2 + 2 * (size_t)(n / nb + 1); }
